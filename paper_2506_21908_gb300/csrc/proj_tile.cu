@@ -474,37 +474,61 @@ k_tile_gather(const float2* __restrict__ psi, int N, int comps_per_k, int groups
 }
 
 // Sum the partial products of every (brick, slot) of atom a in a fixed order with the phase
-// exp(i q.delta), times dV: c[kb][a][2p + sigma]; then D c with the atom's block.
-__global__ void __launch_bounds__(64)
+// exp(i q.delta), times dV: c[kb][a][2p + sigma]; then D c with the atom's block.  Thread (p, t):
+// projector p of component t, so a CTA has 64 nlm threads; the phases of up to kRedPh pairs at a
+// time are formed once per CTA, and four pairs' partial products are requested before the first
+// is used.  Bound by the latency of those loads: with one thread per component looping over the
+// projectors (64 threads, one pair at a time, 3 % of the warp slots) it took 241 us at the large
+// supercell with 32 spinors and 107 us at 64^3 with 48; gather and reduction together went from
+// 869 to 677 us per launch at the large supercell with 128 spinors.
+constexpr int kRedPh = 256;
+__global__ void __launch_bounds__(64 * kMaxNLM)
 k_tile_reduce(const float* __restrict__ part, TileDev td, int groups, int comps_per_k, int nstates, int natoms,
               float dV, EpiParams ep, const float* __restrict__ Dmat, float2* __restrict__ c_out,
               float2* __restrict__ dc_out) {
   const int a = blockIdx.x, kg = blockIdx.y;
   const int k = kg / groups, comp0 = (kg % groups) * 64;
   const int nlm = td.nlm;
-  const int t = threadIdx.x;
+  const int t = threadIdx.x & 63, p = threadIdx.x >> 6;
   __shared__ float2 cs[64][kMaxNLM];
-  float2 acc[kMaxNLM];
-#pragma unroll
-  for (int p = 0; p < kMaxNLM; ++p) acc[p] = make_float2(0.f, 0.f);
+  __shared__ float2 ph[kRedPh];
+  __shared__ long long so[kRedPh];
   const double* q = ep.shift[k];
-  for (int e = td.a_ptr[a]; e < td.a_ptr[a + 1]; ++e) {
-    const int it = td.a_item[e], sl = td.a_slot[e];
-    const float4 dl = td.slot_delta[(size_t)it * td.smax + sl];
-    float sn, cs_;
-    sincosf((float)(q[0] * dl.x + q[1] * dl.y + q[2] * dl.z), &sn, &cs_);
-    const float* src = part + (size_t)kg * td.part_layer + td.it_poff[it] + (size_t)sl * nlm * 128;
+  const int e0 = td.a_ptr[a], e1 = td.a_ptr[a + 1];
+  const float* base = part + (size_t)kg * td.part_layer + (size_t)p * 128 + t;
+  float2 acc = make_float2(0.f, 0.f);
+  for (int b0 = e0; b0 < e1; b0 += kRedPh) {
+    const int nb = min(kRedPh, e1 - b0);
+    __syncthreads();
+    for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+      const int it = td.a_item[b0 + i], sl = td.a_slot[b0 + i];
+      const float4 dl = td.slot_delta[(size_t)it * td.smax + sl];
+      float sn, cs_;
+      sincosf((float)(q[0] * dl.x + q[1] * dl.y + q[2] * dl.z), &sn, &cs_);
+      ph[i] = make_float2(cs_, sn);
+      so[i] = td.it_poff[it] + (long long)sl * nlm * 128;
+    }
+    __syncthreads();
+    for (int i = 0; i < nb; i += 4) {
+      float re[4], im[4];
 #pragma unroll
-    for (int p = 0; p < kMaxNLM; ++p) {
-      if (p < nlm) {
-        const float re = src[(size_t)p * 128 + t], im = src[(size_t)p * 128 + 64 + t];
-        acc[p].x += re * cs_ - im * sn;
-        acc[p].y += re * sn + im * cs_;
+      for (int j = 0; j < 4; ++j) {
+        re[j] = im[j] = 0.f;
+        if (i + j < nb) {
+          const float* src = base + so[i + j];
+          re[j] = __ldg(src);
+          im[j] = __ldg(src + 64);
+        }
       }
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (i + j < nb) {
+          acc.x += re[j] * ph[i + j].x - im[j] * ph[i + j].y;
+          acc.y += re[j] * ph[i + j].y + im[j] * ph[i + j].x;
+        }
     }
   }
-#pragma unroll
-  for (int p = 0; p < kMaxNLM; ++p) cs[t][p] = make_float2(acc[p].x * dV, acc[p].y * dV);
+  cs[t][p] = make_float2(acc.x * dV, acc.y * dV);
   __syncthreads();
   const int comp = comp0 + t;
   if (comp >= comps_per_k) return;
@@ -513,19 +537,17 @@ k_tile_reduce(const float* __restrict__ part, TileDev td, int groups, int comps_
   const size_t kb = (size_t)k * nstates + sp;
   const int M = 2 * nlm;
   const float* D = Dmat + (size_t)a * M * M * 2;
-  for (int p = 0; p < nlm; ++p) {
-    const int row = 2 * p + sig;
-    float re = 0.f, im = 0.f;
-    for (int u = 0; u < M; ++u) {
-      const float2 cu = cs[pair + (u & 1)][u >> 1];
-      const float dr = D[(row * M + u) * 2], di = D[(row * M + u) * 2 + 1];
-      re += dr * cu.x - di * cu.y;
-      im += dr * cu.y + di * cu.x;
-    }
-    const size_t o = (kb * natoms + a) * M + row;
-    c_out[o] = cs[t][p];
-    dc_out[o] = make_float2(re, im);
+  const int row = 2 * p + sig;
+  float re = 0.f, im = 0.f;
+  for (int u = 0; u < M; ++u) {
+    const float2 cu = cs[pair + (u & 1)][u >> 1];
+    const float dr = D[(row * M + u) * 2], di = D[(row * M + u) * 2 + 1];
+    re += dr * cu.x - di * cu.y;
+    im += dr * cu.y + di * cu.x;
   }
+  const size_t o = (kb * natoms + a) * M + row;
+  c_out[o] = cs[t][p];
+  dc_out[o] = make_float2(re, im);
 }
 
 // ============================================================================ scatter
@@ -886,8 +908,9 @@ static cudaError_t gather_et(cudaStream_t st, int N, const void* psi, int nk, in
   kf<<<dim3(nk * groups, td.nitems), PT_NT, smem, st>>>((const float2*)psi, N, comps_per_k, groups, td, ep, part, err);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_tile_reduce<<<dim3(td.natoms, nk * groups), 64, 0, st>>>(part, td, groups, comps_per_k, nstates, td.natoms,
-                                                             (float)dV, ep, Dmat, (float2*)c_out, (float2*)dc_out);
+  k_tile_reduce<<<dim3(td.natoms, nk * groups), 64 * td.nlm, 0, st>>>(part, td, groups, comps_per_k, nstates,
+                                                                      td.natoms, (float)dV, ep, Dmat, (float2*)c_out,
+                                                                      (float2*)dc_out);
   return cudaGetLastError();
 }
 
