@@ -181,6 +181,10 @@ struct tddft_ctx {
   double t = 0, emin = 0, emax = 0, nl_bound = 0, kin_max = 0;
   int K_full = 0, K_half = 0;
   std::vector<cd> cf_full, cf_half;
+  // Chebyshev exponential: cf[k] = ph (-i)^k rf[k] with real rf and one phase ph per series
+  bool real_series = false;
+  std::vector<double> rf_full, rf_half;
+  cd ph_full, ph_half;
   bool use_tma = false;      // FP32 xy passes fed by bulk asynchronous copies
   bool epi_pairs = false;    // epilogue threads take one point of two spinors
   bool epi_fuse = false;     // tensor-core projectors: scatter and Chebyshev epilogue in one kernel
@@ -875,22 +879,27 @@ template <typename R> ProjTables<R> epi_tables(const tddft_ctx* c) {
 // epilogue k has T_{k-1}, T_k and T_{k+1} in registers, so the accumulator is touched only
 // when three terms are pending or T_{k+1} is its last term (one read-modify-write per three
 // terms instead of one per term).  `done` is the first term not yet added; the first update
-// writes without reading.  Coefficients go to cm (T_{k-1}), c0 (T_k) and c1 (T_{k+1}).
-static void acc_schedule(int k, int Ka, const std::vector<cd>& cf, int& done, int& use, int& init, double* cm,
-                         double* c0, double* c1) {
+// writes without reading.  Coefficients go to cm (T_{k-1}), c0 (T_k) and c1 (T_{k+1}); for a real
+// series (rf not null) to r[0..2], with the sign of (-i)^i: i = 0, 1 mod 4 positive, 2, 3
+// negative (odd i add (t.y, -t.x)), and fin marks the last update, which applies the phase.
+static void acc_schedule(int k, int Ka, const std::vector<cd>& cf, const double* rf, int& done, int& use, int& init,
+                         int& fin, double* cm, double* c0, double* c1, double* r) {
   use = 0;
   init = 0;
-  cm[0] = cm[1] = c0[0] = c0[1] = c1[0] = c1[1] = 0.0;
+  fin = 0;
+  cm[0] = cm[1] = c0[0] = c0[1] = c1[0] = c1[1] = r[0] = r[1] = r[2] = 0.0;
   const int last = k + 1;
   if (done > Ka || last > Ka) return;
   if (last - done + 1 < 3 && last != Ka) return;
   use = 1;
   init = (done == 0);
+  fin = (last == Ka);
   double* slot[3] = {cm, c0, c1};
   for (int i = done; i <= last; ++i) {
     double* d = slot[i - (k - 1)];
     d[0] = cf[i].real();
     d[1] = cf[i].imag();
+    if (rf) r[i - (k - 1)] = (i & 2) ? -rf[i] : rf[i];
   }
   done = last + 1;
 }
@@ -914,6 +923,15 @@ tddft_status cheb_series(tddft_ctx* c, const void* in, const R* Vr, const double
   int done1 = 0, done2 = 0;
   // tensor-core projectors: the scatter and the epilogue run as one kernel
   const bool fuse = c->tile && c->epi_fuse && std::is_same<R, float>::value;
+  // cf1, cf2 are cf_full or cf_half: their real factors and phases
+  const auto real_of = [&](const std::vector<cd>& cf) {
+    return !c->real_series ? nullptr : (&cf == &c->cf_full ? c->rf_full.data() : c->rf_half.data());
+  };
+  const auto phase_of = [&](const std::vector<cd>& cf) { return &cf == &c->cf_full ? c->ph_full : c->ph_half; };
+  const double *rf1 = real_of(cf1), *rf2 = real_of(cf2);
+  ep.real_coef = c->real_series ? 1 : 0;
+  ep.ph1[0] = phase_of(cf1).real(); ep.ph1[1] = phase_of(cf1).imag();
+  ep.ph2[0] = phase_of(cf2).real(); ep.ph2[1] = phase_of(cf2).imag();
   for (int k = 0; k < K; ++k) {
     if ((s = kinetic_and_gather<R>(c, cur, A, !fuse))) return s;
     void* out;
@@ -922,8 +940,9 @@ tddft_status cheb_series(tddft_ctx* c, const void* in, const R* Vr, const double
     else if (prev == in) out = (cur == c->Ta) ? c->Tb : c->Ta;
     else out = const_cast<void*>(prev);
     ep.mode = (k == 0) ? EPI_FIRST : EPI_RECUR;
-    acc_schedule(k, K1, cf1, done1, ep.use_acc1, ep.init1, ep.am, ep.a0, ep.a1);
-    if (acc2) acc_schedule(k, K2, cf2, done2, ep.use_acc2, ep.init2, ep.bm, ep.b0, ep.b1);
+    ep.odd = k & 1;
+    acc_schedule(k, K1, cf1, rf1, done1, ep.use_acc1, ep.init1, ep.fin1, ep.am, ep.a0, ep.a1, ep.ra);
+    if (acc2) acc_schedule(k, K2, cf2, rf2, done2, ep.use_acc2, ep.init2, ep.fin2, ep.bm, ep.b0, ep.b1, ep.rb);
     else ep.use_acc2 = 0;
     const void* tkm1 = (k == 0) ? nullptr : prev;
     const double streams = 3.0 + (k == 0 ? 0.0 : 1.0) + (ep.use_acc1 ? (ep.init1 ? 1.0 : 2.0) : 0.0) +
@@ -1433,19 +1452,22 @@ void set_orders(tddft_ctx* c) {
       c->K_full = chebyshev_order(c->dt * dlt, tol);
       c->K_half = chebyshev_order(0.5 * c->dt * dlt, tol);
     }
-    auto coefs = [&](double tau, int K) {
+    auto coefs = [&](double tau, int K, std::vector<double>& r, cd& ph) {
       std::vector<cd> a(K + 1);
       auto J = bessel_j(K, tau * dlt);
-      const cd ph = std::exp(cd(0.0, -tau * cc));
+      r.resize(K + 1);
+      ph = std::exp(cd(0.0, -tau * cc));
       cd mi(1.0, 0.0);
       for (int k = 0; k <= K; ++k) {
-        a[k] = (k == 0 ? 1.0 : 2.0) * mi * J[k] * ph;
+        r[k] = (k == 0 ? 1.0 : 2.0) * J[k];
+        a[k] = r[k] * mi * ph;
         mi *= cd(0.0, -1.0);
       }
       return a;
     };
-    c->cf_full = coefs(c->dt, c->K_full);
-    c->cf_half = coefs(0.5 * c->dt, c->K_half);
+    c->cf_full = coefs(c->dt, c->K_full, c->rf_full, c->ph_full);
+    c->cf_half = coefs(0.5 * c->dt, c->K_half, c->rf_half, c->ph_half);
+    c->real_series = true;
   } else if (c->exp_kind == TDDFT_EXP_CRANK_NICOLSON) {
     // Chebyshev coefficients of the Cayley transform f(E) = (1 - i tau E/2) / (1 + i tau E/2) on
     // [emin, emax]: a_k = (2 - delta_k0)/Q sum_j f(c + Delta cos th_j) cos(k th_j), th_j = pi (j + 1/2)/Q

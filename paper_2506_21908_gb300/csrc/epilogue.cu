@@ -21,10 +21,14 @@ __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefe
 // projector scatter then walks the point's entries once for both.  The D c of the CTA's
 // spinor(s) for every atom is staged in shared memory when it is small.
 // AK selects the accumulator code compiled in: 0 = Chebyshev term without accumulator update,
-// 1 = Chebyshev term updating accumulator 1 only, 2 = every mode with run-time flags.  The
-// Chebyshev recurrence touches its accumulators on every third term only, so most launches take
-// the AK = 0 form, which carries the least code.  FP32 forms are held to 64 registers (four
-// CTAs per SM; the few bytes of spill in the AK = 1, 2 forms cost less than the lost occupancy).
+// 1 = Chebyshev term updating accumulator 1, 2 = both, with the exponential's real coefficients;
+// 3 = every mode and complex coefficients with run-time flags.  The Chebyshev recurrence touches
+// its accumulators on every third term only, so most launches take the AK = 0 form, which
+// carries the least code.  FP32 forms are held to 64 registers (four CTAs per SM; the few bytes
+// of spill in the accumulator forms cost less than the lost occupancy).  The float-float updates
+// bound those forms by instruction issue (83 % issued with complex coefficients and two
+// accumulators, 346 us for 48 spinors at 64^3 against 165 us without accumulators); the real
+// coefficients halve their products (mean launch 443 -> 411 us at 64^3 x 104 spinors).
 template <typename R, int AK> struct EpiMinBlocks { static constexpr int value = 1; };
 template <int AK> struct EpiMinBlocks<float, AK> { static constexpr int value = 4; };
 
@@ -72,7 +76,7 @@ k_epilogue(const typename CT<R>::type* __restrict__ kin, const typename CT<R>::t
     kd2 = {cadd(kd2.a, vd.a), cadd(kd2.b, vd.b)};
   }
   // Chebyshev terms: every input is requested before any arithmetic (more loads in flight)
-  const bool cheb = AK < 2 || ep.mode == EPI_RECUR || ep.mode == EPI_FIRST;
+  const bool cheb = AK < 3 || ep.mode == EPI_RECUR || ep.mode == EPI_FIRST;
   const bool rec = ep.mode == EPI_RECUR;
   const bool use1 = AK >= 1 && ep.use_acc1, use2 = AK >= 2 && ep.use_acc2;
   const C zc = cmake<C>((R)0, (R)0);
@@ -112,12 +116,12 @@ k_epilogue(const typename CT<R>::type* __restrict__ kin, const typename CT<R>::t
     if constexpr (sizeof(R) == 4) return cmul_split(a, zf);
     else return cmulr(a, (R)z[0], (R)z[1]);
   };
-  if (AK == 2 && ep.mode == EPI_APPLY) {
+  if (AK == 3 && ep.mode == EPI_APPLY) {
     st(Tout, ou, hu[0], hu[1]);
     st(Tout, od, hd[0], hd[1]);
     return;
   }
-  if (AK == 2 && ep.mode == EPI_TAYLOR) {
+  if (AK == 3 && ep.mode == EPI_TAYLOR) {
     C tu[2], td[2];
     for (int j = 0; j < 2; ++j) { tu[j] = ccoef(hu[j], ep.a1, ep.f_a1); td[j] = ccoef(hd[j], ep.a1, ep.f_a1); }
     st(Tout, ou, tu[0], tu[1]);
@@ -127,7 +131,7 @@ k_epilogue(const typename CT<R>::type* __restrict__ kin, const typename CT<R>::t
     st(acc1, od, cadd(ad.a, td[0]), cadd(ad.b, td[1]));
     return;
   }
-  if (AK == 2 && (ep.mode == EPI_ADJ || ep.mode == EPI_ADJ0)) {
+  if (AK == 3 && (ep.mode == EPI_ADJ || ep.mode == EPI_ADJ0)) {
     // Clenshaw-type adjoint recurrence: S_k = f (H - c)/Delta S_{k+1} - S_{k+2} + seeds,
     // f = 2 (k >= 1) or 1 (k = 0); Tk holds S_{k+1}, Tkm1 holds S_{k+2} (may be null),
     // acc1/acc2 hold the seed cotangents with coefficients a1, b1.
@@ -174,11 +178,45 @@ k_epilogue(const typename CT<R>::type* __restrict__ kin, const typename CT<R>::t
   st(Tout, od, td[0], td[1]);
   // Accumulators take up to three terms at once (T_{k-1}, T_k, T_{k+1}, all in registers here),
   // so the host updates each of them on every third term only.
-  auto upd = [&](C* acc, int init, const Pair<C>& au, const Pair<C>& ad, const double* cm, const float* cmf,
-                 const double* c0, const float* c0f, const double* c1, const float* c1f) {
+  auto upd = [&](C* acc, int init, int fin, const Pair<C>& au, const Pair<C>& ad, const double* cm, const float* cmf,
+                 const double* c0, const float* c0f, const double* c1, const float* c1f, const double* rc,
+                 const float* rf, const double* ph, const float* phf) {
     const C qus[2] = {qu0.a, qu0.b}, qds[2] = {qd0.a, qd0.b};
     C nu[2], nd[2];
-    if constexpr (sizeof(R) == 4) {
+    if constexpr (AK < 3) {
+      // real coefficients: terms k - 1 and k + 1 have the other parity than k
+      const bool odd = ep.odd;
+      const C aus[2] = {au.a, au.b}, ads[2] = {ad.a, ad.b};
+      const C z2 = cmake<C>((R)0, (R)0);
+      for (int j = 0; j < 2; ++j) {
+        C xu = init ? z2 : aus[j], xd = init ? z2 : ads[j];
+        if constexpr (sizeof(R) == 4) {
+          C lu = z2, ld = z2;  // float-float update, rounded once
+          ff_rmadd(xu, lu, tu[j], rf + 4, !odd);
+          ff_rmadd(xd, ld, td[j], rf + 4, !odd);
+          ff_rmadd(xu, lu, pu[j], rf + 2, odd);
+          ff_rmadd(xd, ld, pd[j], rf + 2, odd);
+          if (rec) {
+            ff_rmadd(xu, lu, qus[j], rf, !odd);
+            ff_rmadd(xd, ld, qds[j], rf, !odd);
+          }
+          nu[j] = fin ? ff_phase(xu, lu, phf) : cadd(xu, lu);
+          nd[j] = fin ? ff_phase(xd, ld, phf) : cadd(xd, ld);
+        } else {
+          auto add = [](C a, C t2, R s, bool swap) {
+            return cmake<C>(a.x + s * (swap ? t2.y : t2.x), a.y + s * (swap ? -t2.x : t2.y));
+          };
+          xu = add(add(xu, tu[j], (R)rc[2], !odd), pu[j], (R)rc[1], odd);
+          xd = add(add(xd, td[j], (R)rc[2], !odd), pd[j], (R)rc[1], odd);
+          if (rec) {
+            xu = add(xu, qus[j], (R)rc[0], !odd);
+            xd = add(xd, qds[j], (R)rc[0], !odd);
+          }
+          nu[j] = fin ? cmulr(xu, (R)ph[0], (R)ph[1]) : xu;
+          nd[j] = fin ? cmulr(xd, (R)ph[0], (R)ph[1]) : xd;
+        }
+      }
+    } else if constexpr (sizeof(R) == 4) {
       // float-float update, rounded once (ff_cmadd)
       const C aus[2] = {au.a, au.b}, ads[2] = {ad.a, ad.b};
       const C z2 = cmake<C>(0.f, 0.f);
@@ -212,15 +250,20 @@ k_epilogue(const typename CT<R>::type* __restrict__ kin, const typename CT<R>::t
     st(acc, ou, nu[0], nu[1]);
     st(acc, od, nd[0], nd[1]);
   };
-  if (use1) upd(acc1, ep.init1, au1, ad1, ep.am, ep.f_am, ep.a0, ep.f_a0, ep.a1, ep.f_a1);
-  if (use2) upd(acc2, ep.init2, au2, ad2, ep.bm, ep.f_bm, ep.b0, ep.f_b0, ep.b1, ep.f_b1);
+  if (use1)
+    upd(acc1, ep.init1, ep.fin1, au1, ad1, ep.am, ep.f_am, ep.a0, ep.f_a0, ep.a1, ep.f_a1, ep.ra, ep.f_ra, ep.ph1,
+        ep.f_ph1);
+  if (use2)
+    upd(acc2, ep.init2, ep.fin2, au2, ad2, ep.bm, ep.f_bm, ep.b0, ep.f_b0, ep.b1, ep.f_b1, ep.rb, ep.f_rb, ep.ph2,
+        ep.f_ph2);
 }
 
 template <typename R, int NLM, int SP, typename... A>
 static void epi_ak(int ak, dim3 grid, size_t smem, cudaStream_t st, A... args) {
   if (ak == 0) k_epilogue<R, NLM, 0, SP><<<grid, 256, smem, st>>>(args...);
   else if (ak == 1) k_epilogue<R, NLM, 1, SP><<<grid, 256, smem, st>>>(args...);
-  else k_epilogue<R, NLM, 2, SP><<<grid, 256, smem, st>>>(args...);
+  else if (ak == 2) k_epilogue<R, NLM, 2, SP><<<grid, 256, smem, st>>>(args...);
+  else k_epilogue<R, NLM, 3, SP><<<grid, 256, smem, st>>>(args...);
 }
 template <typename R, int NLM, typename... A>
 static void epi_sp(bool sp, int ak, dim3 grid, size_t smem, cudaStream_t st, A... args) {
@@ -244,7 +287,8 @@ cudaError_t launch_epilogue(cudaStream_t st, int N, const void* kin, const void*
   epx.dc_staged = (nlm > 0 && dcb <= 32 * 1024) ? 1 : 0;
   const size_t smem = epx.dc_staged ? dcb : 0;
   const bool cheb = ep.mode == EPI_FIRST || ep.mode == EPI_RECUR;
-  const int ak = !cheb ? 2 : (ep.use_acc2 ? 2 : (ep.use_acc1 ? 1 : 0));
+  const bool acc = ep.use_acc1 || ep.use_acc2;
+  const int ak = (!cheb || (acc && !ep.real_coef)) ? 3 : (ep.use_acc2 ? 2 : (ep.use_acc1 ? 1 : 0));
 #define EPI_ARGS (const C*)kin, (const C*)kin2, (const C*)Tk, (const C*)Tkm1, (C*)Tout, (C*)acc1, (C*)acc2, V, N3, pt, (const C*)dc, epx
   switch (nlm) {
     case 0: epi_sp<R, 0>(sp, ak, grid, smem, st, EPI_ARGS); break;

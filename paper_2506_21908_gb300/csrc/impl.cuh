@@ -37,6 +37,13 @@ struct EpiParams {
   double am[2], bm[2];          // unfused recurrence: coefficients on T_{k-1} (accumulators 1, 2)
   int use_acc1, use_acc2;
   int init1, init2;             // unfused recurrence: write the accumulator without reading it
+  // Chebyshev exponential: a_i = phase (-i)^i r_i with real r_i and one phase per series, so the
+  // accumulators sum (-i)^i r_i T_i with real coefficients and take the phase at their last update.
+  // ra, rb: signed r_i on T_{k-1}, T_k, T_{k+1} (accumulators 1, 2; see acc_schedule).
+  int real_coef;
+  int odd;                      // k is odd: (-i)^i swaps the parts of T_k, else those of T_{k-1}, T_{k+1}
+  int fin1, fin2;               // last update of the accumulator: apply ph1, ph2
+  double ra[3], rb[3], ph1[2], ph2[2];
   double shift[kMaxK][3];       // k + A(t), for projector phases
   int nstates;
   int dc_staged;                // fused kernel: D c copied to shared memory (set by its launcher)
@@ -45,6 +52,8 @@ struct EpiParams {
   // (hi = the value rounded to float, lo = the rounded remainder; set by split_constants)
   float f_c[2], f_id[2];
   float f_a0[4], f_a1[4], f_b0[4], f_b1[4], f_am[4], f_bm[4];
+  float f_ra[6], f_rb[6];       // {hi, lo} of ra, rb
+  float f_ph1[4], f_ph2[4];
 };
 
 // The series constants are applied identically at every term, every step and every grid point, so
@@ -71,6 +80,12 @@ inline void split_constants(EpiParams& e) {
   s4(e.b1, e.f_b1);
   s4(e.am, e.f_am);
   s4(e.bm, e.f_bm);
+  for (int i = 0; i < 3; ++i) {
+    s2(e.ra[i], e.f_ra + 2 * i);
+    s2(e.rb[i], e.f_rb + 2 * i);
+  }
+  s4(e.ph1, e.f_ph1);
+  s4(e.ph2, e.f_ph2);
 }
 
 // Device-side projector tables.

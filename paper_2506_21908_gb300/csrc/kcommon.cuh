@@ -55,6 +55,24 @@ __device__ __forceinline__ void ff_cmadd(float2& hi, float2& lo, float2 t, const
   lo.y += z[2] * t.y + z[3] * t.x;
 }
 
+// (hi, lo) += s (-i)^i t up to the sign in s = {hi, lo}: the parts of t as they are (i even) or
+// (t.y, -t.x) (i odd, swap).  Half the products of ff_cmadd.
+__device__ __forceinline__ void ff_rmadd(float2& hi, float2& lo, float2 t, const float* s, bool swap) {
+  const float a = swap ? t.y : t.x, b = swap ? -t.x : t.y;
+  ff_madd(hi.x, lo.x, s[0], a);
+  ff_madd(hi.y, lo.y, s[0], b);
+  lo.x += s[1] * a;
+  lo.y += s[1] * b;
+}
+// z (hi + lo) rounded to FP32 once, z = {re hi, im hi, re lo, im lo}.
+__device__ __forceinline__ float2 ff_phase(float2 hi, float2 lo, const float* z) {
+  float2 h = make_float2(0.f, 0.f), l = make_float2(0.f, 0.f);
+  ff_cmadd(h, l, hi, z);
+  l.x += z[0] * lo.x - z[1] * lo.y;
+  l.y += z[0] * lo.y + z[1] * lo.x;
+  return make_float2(h.x + l.x, h.y + l.y);
+}
+
 #define TDDFT_DISPATCH_N(N, CALL)          \
   switch (N) {                             \
     case 8: { constexpr int NN = 8; return CALL; }   \

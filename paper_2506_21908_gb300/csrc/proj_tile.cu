@@ -18,9 +18,9 @@
 // 128 bytes with the 128-byte swizzle), as one rounded part (TF32) or as hi + lo parts (TF32 x3,
 // BF16 x3, FP16 x3: hi*hi + hi*lo + lo*hi with FP32 accumulation, the split-precision product).
 //
-// Each CTA (320 threads): warps 0-7 stage psi (phase, split, swizzled stores) or X and drain the
-// tensor memory, warp 8 issues the MMAs (one elected thread), warp 9 the bulk copies of the
-// projector tables; two shared-memory stages between them, full / empty mbarriers.  Every
+// Each CTA: worker warps (8 in the gather, 16 in the scatter) stage psi (phase, split, swizzled
+// stores) or X and drain the tensor memory, one warp issues the MMAs (one elected thread), one the
+// bulk copies of the projector tables; two shared-memory stages between them, full / empty mbarriers.  Every
 // mbarrier wait has an iteration limit: on expiry the CTA sets bit 1 of the error word, stops
 // issuing work, waits (with a limit) for its copies and MMAs in flight and frees its tensor memory.
 #include <cstdint>
@@ -152,12 +152,20 @@ __device__ __forceinline__ void tmem_ld16_async(uint32_t taddr, uint32_t* r) {
         "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
 }
+__device__ __forceinline__ void tmem_ld8_async(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // After tmem_wait_ld: ties the loaded registers to a point after the wait, so that no use of them
 // is scheduled before it.
 __device__ __forceinline__ void tmem_regs_ready(uint32_t* r) {
   asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
                "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]));
+}
+__device__ __forceinline__ void tmem_regs_ready8(uint32_t* r) {
+  asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]));
 }
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float* v) {
   asm volatile(
@@ -553,14 +561,25 @@ k_tile_reduce(const float* __restrict__ part, TileDev td, int groups, int comps_
 // ============================================================================ scatter
 
 // CTA (kg, brick): SC components (X, the B operand, resident) against the brick's points in
-// tiles of 128 (the A operand, streamed).  FUSED = 0: out = exp(-i q.(r - r_b)) (beta^T X) at every
+// tiles of 128 (the A operand, streamed).  AK < 0: out = exp(-i q.(r - r_b)) (beta^T X) at every
 // point of a brick with projectors (the points of other bricks are never written and keep their
-// zeros).  FUSED = 1: the drain runs the Chebyshev epilogue of every point of the brick itself
+// zeros).  AK >= 0: the drain runs the Chebyshev epilogue of every point of the brick itself
 // (kinetic part from io.kin, V_NL from the tensor memory, the 2x2 local potential, T_{k+1} and the
 // accumulators) with the arithmetic of k_epilogue, so V_NL never crosses HBM; bricks without
-// projectors take the same path with V_NL = 0.
-template <int EK, int TERMS, int FUSED>
-__global__ void __launch_bounds__(PT_NT, 1)
+// projectors take the same path with V_NL = 0.  AK as in k_epilogue: 0 no accumulator, 1 and 2
+// real coefficients on one or both, 3 complex coefficients with run-time flags.
+//
+// Bound by HBM as long as enough loads are in flight: one CTA holds the SM (its 512
+// tensor-memory columns), so 16 worker warps drain it, four to each lane quarter of the tensor
+// memory, and the first spinors of a tile are requested before the wait for its products.
+// At the large supercell with 128 spinors the mean launch went from 2676 us (3.2 TB/s, 8 warps,
+// complex coefficients) to 1927 us (4.5 TB/s).
+constexpr int ST_WARPS = 16;                  // worker warps
+constexpr int ST_NT = 32 * (ST_WARPS + 2);    // + MMA warp + copy warp
+constexpr int ST_MMA_WARP = ST_WARPS, ST_COPY_WARP = ST_WARPS + 1;
+
+template <int EK, int TERMS, int AK>
+__global__ void __launch_bounds__(ST_NT, 1)
 k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, int natoms, TileDev td, EpiParams ep,
                const float2* __restrict__ dc, int* __restrict__ err, EpiIO io) {
   constexpr int EPR = PT_ROWB / Elt<EK>::bytes;    // projector indices per K chunk
@@ -580,7 +599,7 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
   const int kg = blockIdx.x, it = blockIdx.y;
   const int k = kg / sgroups, comp0 = (kg % sgroups) * SC;
   const int nslot = td.it_nslot[it], kch = td.it_kch[it];
-  if (!FUSED && nslot == 0) return;  // nothing to add at this brick
+  if (AK < 0 && nslot == 0) return;  // nothing to add at this brick
   const bool has_nl = nslot > 0;
   const int BX = td.BX;
   const int brick = td.it_brick[it];
@@ -601,7 +620,7 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
       bar_init(sm_addr(&bar_full[s]), 1);
       bar_init(sm_addr(&bar_empty[s]), 1);
       bar_init(sm_addr(&bar_accf[s]), 1);
-      bar_init(sm_addr(&bar_acce[s]), 32 * PT_WARPS);
+      bar_init(sm_addr(&bar_acce[s]), 32 * ST_WARPS);
     }
     bar_init(sm_addr(&bar_fin), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -618,7 +637,7 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
   // hi x lo and lo x hi products go to a second pair at column 256, so the rounding of the tensor
   // cores' accumulation (biased toward zero) sees a third of the MMAs at full magnitude
   constexpr uint32_t TMEM_COLS = (TERMS == 3) ? 512u : 256u;
-  if (warp == PT_MMA_WARP) {
+  if (warp == ST_MMA_WARP) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sm_addr(&tmem_base)),
                  "r"(TMEM_COLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -630,17 +649,17 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
 
   // ---- X: rows cl (re) and SC + cl (im), K element j = slot * nlm + p.  One 16-byte load of D c
   // gives both spin components of one spinor at one projector (index 2 p + sigma).
-  if (warp < PT_WARPS) {
+  if (warp < ST_WARPS) {
     const int tid = threadIdx.x;
     constexpr int SPG = SC / 2;                    // spinors per CTA
     const int total = nslot * SPG * nlm;
     const float4* dc4 = reinterpret_cast<const float4*>(dc);
-    for (int b0 = 0; b0 < total; b0 += 4 * 32 * PT_WARPS) {
+    for (int b0 = 0; b0 < total; b0 += 4 * 32 * ST_WARPS) {
       float4 f[4];
       int ee[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const int e = b0 + u * 32 * PT_WARPS + tid;
+        const int e = b0 + u * 32 * ST_WARPS + tid;
         ee[u] = e;
         f[u] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (e < total) {
@@ -674,7 +693,7 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
     }
     // padding of the last K chunk
     const int j0 = nslot * nlm, pad = kch * EPR - j0;
-    for (int i = tid; i < pad * 2 * SC; i += 32 * PT_WARPS) {
+    for (int i = tid; i < pad * 2 * SC; i += 32 * ST_WARPS) {
       const int row = i % (2 * SC), j = j0 + i / (2 * SC);
       put<EK>(xpart(j / EPR, 0), row, j % EPR, 0u);
       if constexpr (TERMS == 3) put<EK>(xpart(j / EPR, 1), row, j % EPR, 0u);
@@ -684,7 +703,7 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
   __syncthreads();
 
   const int nchunk = ntile * kch;
-  if (warp == PT_COPY_WARP) {
+  if (warp == ST_COPY_WARP) {
     if (lane == 0 && has_nl) {
       const unsigned char* src = td.s_tab + td.it_soff[it];
       int issued = 0;
@@ -700,7 +719,7 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
       for (int j = (issued > 2 ? issued - 2 : 0); j < issued; ++j)
         if (!pt_wait(sm_addr(&bar_full[j & 1]), (j >> 1) & 1)) atomicOr(err, 1);
     }
-  } else if (warp == PT_MMA_WARP) {
+  } else if (warp == ST_MMA_WARP) {
     if (lane == 0 && has_nl) {
       const uint32_t id = idesc<EK>(2 * SC);
       for (int t = 0; t < ntile && !abort_flag; ++t) {
@@ -732,99 +751,100 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
       if (!pt_wait(sm_addr(&bar_fin), 0)) atomicOr(err, 1);
     }
   } else {
-    // ---- drain: thread = point of the tile (lane quarter of the warp); the two warps of a
-    // quarter take one half of the components each; V_NL = exp(-i q.(r - r_b)) (re + i im)
-    const int quarter = warp & 3, half = warp >> 2;
+    // ---- drain: thread = point of the tile (lane quarter of the warp); the four warps of a
+    // quarter take a fourth of the components each, eight (four spinors) at a time;
+    // V_NL = exp(-i q.(r - r_b)) (re + i im)
+    const int quarter = warp & 3;
     const int row = quarter * 32 + lane;
-    const int cbeg = half * (SC / 2), cend = (half + 1) * (SC / 2);
+    const int cbeg = (warp >> 2) * (SC / 4), cend = cbeg + SC / 4;
     // epilogue constants (Chebyshev term k: T_{k+1} = f (H - c) T_k / Delta - T_{k-1}, f = 1 or 2)
     const bool rec = ep.mode == EPI_RECUR;
-    const bool use1 = ep.use_acc1, use2 = ep.use_acc2;
+    const bool use1 = AK >= 1 && ep.use_acc1, use2 = AK >= 2 && ep.use_acc2;
     const bool ld1 = use1 && !ep.init1, ld2 = use2 && !ep.init2;
+    // spinors loaded at a time; the accumulator forms hold fewer, for registers
+    constexpr int NB = AK == 0 ? 4 : 2;
+    float2 pu[NB], pd[NB], ku[NB], kd[NB], qu[NB], qd[NB], au[NB], ad[NB], bu[NB], bd[NB];
     for (int t = 0; t < ntile; ++t) {
       const int acc = t & 1;
-      if (has_nl) {
-        if (!pt_wait(sm_addr(&bar_accf[acc]), (t >> 1) & 1)) abort_flag = 1;
-        if (abort_flag) break;
-        asm volatile("tcgen05.fence::after_thread_sync;");
-      }
       const int p = t * 128 + row;
       const int lx = p % BX, ly = (p / BX) & 7, lz = p / (BX * 8);
       const size_t idx = ((size_t)(z0 + lz) * N + (y0 + ly)) * N + (x0 + lx);
-      const float2 ph = cm(cm(px[lx], py[ly]), pz[lz]);
-      const float2 phc = make_float2(ph.x, -ph.y);
       const uint32_t tb = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * 2 * SC);
       const size_t base = ((size_t)k * comps_per_k + comp0) * N3 + idx;  // component comp0 at this point
+      const float2 z2 = make_float2(0.f, 0.f);
+      // every input of NB spinors from component cu0 on
+      auto load = [&](int cu0) {
+#pragma unroll
+        for (int j = 0; j < NB; ++j) {
+          const int cu = cu0 + 2 * j;
+          pu[j] = pd[j] = ku[j] = kd[j] = qu[j] = qd[j] = au[j] = ad[j] = bu[j] = bd[j] = z2;
+          if (comp0 + cu < comps_per_k) {
+            const size_t ou = base + (size_t)cu * N3, od = ou + N3;
+            pu[j] = io.Tk[ou]; pd[j] = io.Tk[od];
+            ku[j] = io.kin[ou]; kd[j] = io.kin[od];
+            if (rec) { qu[j] = io.Tkm1[ou]; qd[j] = io.Tkm1[od]; }
+            if (ld1) { au[j] = io.acc1[ou]; ad[j] = io.acc1[od]; }
+            if (ld2) { bu[j] = io.acc2[ou]; bd[j] = io.acc2[od]; }
+          }
+        }
+      };
       float V0 = 0.f, V1 = 0.f, hx = 0.f, hy = 0.f;
-      if constexpr (FUSED) {
+      if constexpr (AK >= 0) {
+        load(cbeg);
         V0 = io.V[idx];
         V1 = io.V[N3 + idx];
         hx = 0.5f * io.V[2 * N3 + idx];
         hy = 0.5f * io.V[3 * N3 + idx];
       }
-      for (int c0 = cbeg; c0 < cend; c0 += 16) {
-        float re[16], im[16];
+      const float2 ph = cm(cm(px[lx], py[ly]), pz[lz]);
+      const float2 phc = make_float2(ph.x, -ph.y);
+      if (has_nl) {
+        if (!pt_wait(sm_addr(&bar_accf[acc]), (t >> 1) & 1)) abort_flag = 1;
+        if (__any_sync(0xffffffffu, abort_flag != 0)) break;
+        asm volatile("tcgen05.fence::after_thread_sync;");
+      }
+#pragma unroll 1
+      for (int c0 = cbeg; c0 < cend; c0 += 8) {
+        float re[8], im[8];
         if (has_nl) {
-          uint32_t hr[16], hi_[16];
-          tmem_ld16_async(tb + (uint32_t)c0, hr);
-          tmem_ld16_async(tb + (uint32_t)(SC + c0), hi_);
-          if constexpr (TERMS == 3) {
-            uint32_t lr[16], li[16];
-            tmem_ld16_async(tb + 256u + (uint32_t)c0, lr);
-            tmem_ld16_async(tb + 256u + (uint32_t)(SC + c0), li);
-            tmem_wait_ld();
-            tmem_regs_ready(hr);
-            tmem_regs_ready(hi_);
-            tmem_regs_ready(lr);
-            tmem_regs_ready(li);
+          auto part = [&](uint32_t col, float* o) {
+            uint32_t h[8];
+            tmem_ld8_async(tb + col, h);
+            if constexpr (TERMS == 3) {
+              uint32_t l[8];
+              tmem_ld8_async(tb + 256u + col, l);
+              tmem_wait_ld();
+              tmem_regs_ready8(h);
+              tmem_regs_ready8(l);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              re[j] = __uint_as_float(hr[j]) + __uint_as_float(lr[j]);
-              im[j] = __uint_as_float(hi_[j]) + __uint_as_float(li[j]);
-            }
-          } else {
-            tmem_wait_ld();
-            tmem_regs_ready(hr);
-            tmem_regs_ready(hi_);
+              for (int j = 0; j < 8; ++j) o[j] = __uint_as_float(h[j]) + __uint_as_float(l[j]);
+            } else {
+              tmem_wait_ld();
+              tmem_regs_ready8(h);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              re[j] = __uint_as_float(hr[j]);
-              im[j] = __uint_as_float(hi_[j]);
+              for (int j = 0; j < 8; ++j) o[j] = __uint_as_float(h[j]);
             }
-          }
-          if (c0 + 16 >= cend) {
+          };
+          part((uint32_t)c0, re);
+          part((uint32_t)(SC + c0), im);
+          if (c0 + 8 >= cend) {
             asm volatile("tcgen05.fence::before_thread_sync;");
             pt_arrive(sm_addr(&bar_acce[acc]));
           }
         } else {
 #pragma unroll
-          for (int j = 0; j < 16; ++j) re[j] = im[j] = 0.f;
+          for (int j = 0; j < 8; ++j) re[j] = im[j] = 0.f;
         }
-        if constexpr (!FUSED) {
+        if constexpr (AK < 0) {
 #pragma unroll
-          for (int j = 0; j < 16; ++j)
+          for (int j = 0; j < 8; ++j)
             if (comp0 + c0 + j < comps_per_k) out[base + (size_t)(c0 + j) * N3] = cm(make_float2(re[j], im[j]), phc);
         } else {
-          // four spinors at a time: every input is requested before any arithmetic
 #pragma unroll
-          for (int b = 0; b < 16; b += 8) {
-            float2 pu[4], pd[4], ku[4], kd[4], qu[4], qd[4], au[4], ad[4], bu[4], bd[4];
-            const float2 z2 = make_float2(0.f, 0.f);
+          for (int b = 0; b < 8; b += 2 * NB) {
+            if (c0 + b != cbeg) load(c0 + b);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const int cu = c0 + b + 2 * j;
-              pu[j] = pd[j] = ku[j] = kd[j] = qu[j] = qd[j] = au[j] = ad[j] = bu[j] = bd[j] = z2;
-              if (comp0 + cu < comps_per_k) {
-                const size_t ou = base + (size_t)cu * N3, od = ou + N3;
-                pu[j] = io.Tk[ou]; pd[j] = io.Tk[od];
-                ku[j] = io.kin[ou]; kd[j] = io.kin[od];
-                if (rec) { qu[j] = io.Tkm1[ou]; qd[j] = io.Tkm1[od]; }
-                if (ld1) { au[j] = io.acc1[ou]; ad[j] = io.acc1[od]; }
-                if (ld2) { bu[j] = io.acc2[ou]; bd[j] = io.acc2[od]; }
-              }
-            }
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; j < NB; ++j) {
               const int cu = c0 + b + 2 * j;
               if (comp0 + cu >= comps_per_k) continue;
               const size_t ou = base + (size_t)cu * N3, od = ou + N3;
@@ -835,38 +855,51 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
               const float2 u = pu[j], d = pd[j];
               hu = make_float2(hu.x + V0 * u.x + hx * d.x - hy * d.y, hu.y + V0 * u.y + hx * d.y + hy * d.x);
               hd = make_float2(hd.x + V1 * d.x + hx * u.x + hy * u.y, hd.y + V1 * d.y + hx * u.y - hy * u.x);
-              float2 tu, td;
-              // the series constants as float pairs (split_constants)
-              if (!rec) {
-                tu = make_float2(shifted_f(hu.x, u.x, ep.f_c, ep.f_id), shifted_f(hu.y, u.y, ep.f_c, ep.f_id));
-                td = make_float2(shifted_f(hd.x, d.x, ep.f_c, ep.f_id), shifted_f(hd.y, d.y, ep.f_c, ep.f_id));
-              } else {
-                tu = make_float2(2.f * shifted_f(hu.x, u.x, ep.f_c, ep.f_id) - qu[j].x,
-                                 2.f * shifted_f(hu.y, u.y, ep.f_c, ep.f_id) - qu[j].y);
-                td = make_float2(2.f * shifted_f(hd.x, d.x, ep.f_c, ep.f_id) - qd[j].x,
-                                 2.f * shifted_f(hd.y, d.y, ep.f_c, ep.f_id) - qd[j].y);
-              }
+              // the series constants as float pairs (split_constants); T_1 without the factor 2 and
+              // without T_{-1} (zero here)
+              const float f = rec ? 2.f : 1.f;
+              const float2 tu = make_float2(f * shifted_f(hu.x, u.x, ep.f_c, ep.f_id) - qu[j].x,
+                                            f * shifted_f(hu.y, u.y, ep.f_c, ep.f_id) - qu[j].y);
+              const float2 td = make_float2(f * shifted_f(hd.x, d.x, ep.f_c, ep.f_id) - qd[j].x,
+                                            f * shifted_f(hd.y, d.y, ep.f_c, ep.f_id) - qd[j].y);
               io.Tout[ou] = tu;
               io.Tout[od] = td;
-              // accumulators: up to three terms (T_{k-1}, T_k, T_{k+1}) at once
-              // float-float update, rounded once (ff_cmadd), as in k_epilogue
-              auto upd = [&](float2* accp, int init, float2 ou_old, float2 od_old, const float* cmf, const float* c0f,
-                             const float* c1f) {
-                const float2 z2 = make_float2(0.f, 0.f);
-                float2 hu2 = init ? z2 : ou_old, hd2 = init ? z2 : od_old, lu = z2, ld = z2;
-                ff_cmadd(hu2, lu, tu, c1f);
-                ff_cmadd(hd2, ld, td, c1f);
-                ff_cmadd(hu2, lu, u, c0f);
-                ff_cmadd(hd2, ld, d, c0f);
-                if (rec) {
-                  ff_cmadd(hu2, lu, qu[j], cmf);
-                  ff_cmadd(hd2, ld, qd[j], cmf);
+              // accumulators: up to three terms (T_{k-1}, T_k, T_{k+1}) at once in float-float
+              // arithmetic, rounded once, as in k_epilogue
+              auto upd = [&](float2* accp, int init, int fin, float2 xu, float2 xd, const float* cmf, const float* c0f,
+                             const float* c1f, const float* rf, const float* phf) {
+                if (init) xu = xd = z2;
+                float2 lu = z2, ld = z2;
+                if constexpr (AK < 3) {
+                  const bool odd = ep.odd;
+                  ff_rmadd(xu, lu, tu, rf + 4, !odd);
+                  ff_rmadd(xd, ld, td, rf + 4, !odd);
+                  ff_rmadd(xu, lu, u, rf + 2, odd);
+                  ff_rmadd(xd, ld, d, rf + 2, odd);
+                  if (rec) {
+                    ff_rmadd(xu, lu, qu[j], rf, !odd);
+                    ff_rmadd(xd, ld, qd[j], rf, !odd);
+                  }
+                  if (fin) {
+                    accp[ou] = ff_phase(xu, lu, phf);
+                    accp[od] = ff_phase(xd, ld, phf);
+                    return;
+                  }
+                } else {
+                  ff_cmadd(xu, lu, tu, c1f);
+                  ff_cmadd(xd, ld, td, c1f);
+                  ff_cmadd(xu, lu, u, c0f);
+                  ff_cmadd(xd, ld, d, c0f);
+                  if (rec) {
+                    ff_cmadd(xu, lu, qu[j], cmf);
+                    ff_cmadd(xd, ld, qd[j], cmf);
+                  }
                 }
-                accp[ou] = make_float2(hu2.x + lu.x, hu2.y + lu.y);
-                accp[od] = make_float2(hd2.x + ld.x, hd2.y + ld.y);
+                accp[ou] = make_float2(xu.x + lu.x, xu.y + lu.y);
+                accp[od] = make_float2(xd.x + ld.x, xd.y + ld.y);
               };
-              if (use1) upd(io.acc1, ep.init1, au[j], ad[j], ep.f_am, ep.f_a0, ep.f_a1);
-              if (use2) upd(io.acc2, ep.init2, bu[j], bd[j], ep.f_bm, ep.f_b0, ep.f_b1);
+              if (use1) upd(io.acc1, ep.init1, ep.fin1, au[j], ad[j], ep.f_am, ep.f_a0, ep.f_a1, ep.f_ra, ep.f_ph1);
+              if (use2) upd(io.acc2, ep.init2, ep.fin2, bu[j], bd[j], ep.f_bm, ep.f_b0, ep.f_b1, ep.f_rb, ep.f_ph2);
             }
           }
         }
@@ -876,7 +909,7 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
-  if (warp == PT_MMA_WARP)
+  if (warp == ST_MMA_WARP)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS));
 }
 
@@ -914,7 +947,7 @@ static cudaError_t gather_et(cudaStream_t st, int N, const void* psi, int nk, in
   return cudaGetLastError();
 }
 
-template <int EK, int TERMS, int FUSED>
+template <int EK, int TERMS, int AK>
 static cudaError_t scatter_et(cudaStream_t st, int N, void* out, int nk, int nstates, const TileDev& td,
                               const EpiParams& ep, const void* dc, int* err, const EpiIO& io) {
   constexpr int SC = (Elt<EK>::bytes == 4) ? 32 : 64;
@@ -922,21 +955,21 @@ static cudaError_t scatter_et(cudaStream_t st, int N, void* out, int nk, int nst
   const int sgroups = (comps_per_k + SC - 1) / SC;
   const size_t smem = tile_scatter_smem(EK, TERMS, td.kch_max);
   if (smem > 227 * 1024) return cudaErrorInvalidConfiguration;
-  auto kf = k_tile_scatter<EK, TERMS, FUSED>;
+  auto kf = k_tile_scatter<EK, TERMS, AK>;
   cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  kf<<<dim3(nk * sgroups, td.nitems), PT_NT, smem, st>>>((float2*)out, N, comps_per_k, sgroups, nstates, td.natoms,
+  kf<<<dim3(nk * sgroups, td.nitems), ST_NT, smem, st>>>((float2*)out, N, comps_per_k, sgroups, nstates, td.natoms,
                                                          td, ep, (const float2*)dc, err, io);
   return cudaGetLastError();
 }
 
-template <int FUSED>
+template <int AK>
 static cudaError_t scatter_dispatch(cudaStream_t st, int N, void* out, int nk, int nstates, const TileDev& td,
                                     const EpiParams& ep, const void* dc, int* err, const EpiIO& io) {
   switch (td.ek * 4 + td.terms) {
-    case TILE_TF32 * 4 + 1: return scatter_et<TILE_TF32, 1, FUSED>(st, N, out, nk, nstates, td, ep, dc, err, io);
-    case TILE_TF32 * 4 + 3: return scatter_et<TILE_TF32, 3, FUSED>(st, N, out, nk, nstates, td, ep, dc, err, io);
-    case TILE_BF16 * 4 + 3: return scatter_et<TILE_BF16, 3, FUSED>(st, N, out, nk, nstates, td, ep, dc, err, io);
-    case TILE_F16 * 4 + 3: return scatter_et<TILE_F16, 3, FUSED>(st, N, out, nk, nstates, td, ep, dc, err, io);
+    case TILE_TF32 * 4 + 1: return scatter_et<TILE_TF32, 1, AK>(st, N, out, nk, nstates, td, ep, dc, err, io);
+    case TILE_TF32 * 4 + 3: return scatter_et<TILE_TF32, 3, AK>(st, N, out, nk, nstates, td, ep, dc, err, io);
+    case TILE_BF16 * 4 + 3: return scatter_et<TILE_BF16, 3, AK>(st, N, out, nk, nstates, td, ep, dc, err, io);
+    case TILE_F16 * 4 + 3: return scatter_et<TILE_F16, 3, AK>(st, N, out, nk, nstates, td, ep, dc, err, io);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -957,7 +990,7 @@ cudaError_t launch_tile_gather(cudaStream_t st, int N, const void* psi, int nk, 
 cudaError_t launch_tile_scatter(cudaStream_t st, int N, void* out, int nk, int nstates, const TileDev& td,
                                 const EpiParams& ep, const void* dc, int* err) {
   if (td.nitems == 0) return cudaSuccess;
-  return scatter_dispatch<0>(st, N, out, nk, nstates, td, ep, dc, err, EpiIO{});
+  return scatter_dispatch<-1>(st, N, out, nk, nstates, td, ep, dc, err, EpiIO{});
 }
 
 cudaError_t launch_tile_epilogue(cudaStream_t st, int N, int nk, int nstates, const TileDev& td, const EpiParams& ep,
@@ -966,7 +999,10 @@ cudaError_t launch_tile_epilogue(cudaStream_t st, int N, int nk, int nstates, co
   if (td.nitems == 0) return cudaSuccess;
   EpiParams epx = ep;
   split_constants(epx);
-  return scatter_dispatch<1>(st, N, nullptr, nk, nstates, td, epx, dc, err, io);
+  if (!ep.use_acc1 && !ep.use_acc2) return scatter_dispatch<0>(st, N, nullptr, nk, nstates, td, epx, dc, err, io);
+  if (!ep.real_coef) return scatter_dispatch<3>(st, N, nullptr, nk, nstates, td, epx, dc, err, io);
+  if (!ep.use_acc2) return scatter_dispatch<1>(st, N, nullptr, nk, nstates, td, epx, dc, err, io);
+  return scatter_dispatch<2>(st, N, nullptr, nk, nstates, td, epx, dc, err, io);
 }
 
 cudaError_t set_first_wait_tile(unsigned polls) { return cudaMemcpyToSymbol(g_first_wait, &polls, sizeof(polls)); }
