@@ -337,17 +337,19 @@ cudaError_t launch_accum_parts(cudaStream_t st, size_t count, const double* part
 // and since beta is real this equals, per atom and spinor, one pass over the sphere entries:
 //   sum_e d_alpha Im( e^{-i phi} [conj(S) w_T + conj(T) w_S] ) dV,  w_X = sum_p beta_p (D c_X)_p,
 // summed over both spin components.  The caller's 1/dV cancels the dV.  Partials per (spinor,
-// atom) are added over atoms in a fixed order by k_nl_agrad_sum.
+// atom, chunk of its entries) are added in a fixed order by k_nl_agrad_sum.  Phases and (FP64)
+// projector values come from the tables of the gather; the chunks fill the chip where atoms and
+// spinors alone do not (proj_chunks).
 template <typename R, int NLM>
 __global__ void __launch_bounds__(256)
 k_nl_agrad_fused(const typename CT<R>::type* __restrict__ S, const typename CT<R>::type* __restrict__ T, size_t N3,
-                 ProjTables<R> pt, EpiParams ep, const typename CT<R>::type* __restrict__ dcS,
+                 ProjTables<R> pt, EpiParams ep, int chunks, const typename CT<R>::type* __restrict__ dcS,
                  const typename CT<R>::type* __restrict__ dcT, double* __restrict__ part) {
   using C = typename CT<R>::type;
-  const int a = blockIdx.x;
+  const int a = blockIdx.x / chunks, ch = blockIdx.x - a * chunks;
   const int kb = blockIdx.y;
   const int k = kb / ep.nstates;
-  const R sx = (R)ep.shift[k][0], sy = (R)ep.shift[k][1], sz = (R)ep.shift[k][2];
+  const C* ph = reinterpret_cast<const C*>(pt.g_ph) + (size_t)k * pt.nent;
   __shared__ C dS[2 * NLM], dT[2 * NLM];
   __shared__ double red[8][3];
   const size_t cof = ((size_t)kb * pt.natoms + a) * 2 * NLM;
@@ -356,21 +358,20 @@ k_nl_agrad_fused(const typename CT<R>::type* __restrict__ S, const typename CT<R
     dT[threadIdx.x] = dcT[cof + threadIdx.x];
   }
   __syncthreads();
-  R nl[4];
-  load_row<R, 4>(pt.nrm + (size_t)a * 4, nl);
   const C* su_ = S + (size_t)(2 * kb) * N3;
   const C* sd_ = su_ + N3;
   const C* tu_ = T + (size_t)(2 * kb) * N3;
   const C* td_ = tu_ + N3;
   double acc[3] = {0.0, 0.0, 0.0};
-  const int e0 = pt.g_ptr[a], e1 = pt.g_ptr[a + 1];
+  const int g0 = pt.g_ptr[a], ng = pt.g_ptr[a + 1] - g0;
+  const int e0 = g0 + (int)((long long)ng * ch / chunks), e1 = g0 + (int)((long long)ng * (ch + 1) / chunks);
   for (int e = e0 + threadIdx.x; e < e1; e += 256) {
     const int r = pt.g_idx[e];
-    R t[4], bt[NLM];
+    R t[4], bt[beta_pitch(NLM)];
     load_row<R, 4>(pt.g_row + (size_t)e * 4, t);
-    beta_values<R, NLM>(t[0], t[1], t[2], t[3], nl, pt.yc, bt);
-    R sn, cs;
-    sincos_r<R>(sx * t[0] + sy * t[1] + sz * t[2], &sn, &cs);
+    entry_beta<R, NLM>(e, a, pt.g_row, pt.g_beta, pt, bt);
+    const C pe = ph[e];
+    const R cs = pe.x, sn = pe.y;
     const C su = su_[r], sd = sd_[r], tu = tu_[r], td = td_[r];
     R wtu_x = 0, wtu_y = 0, wtd_x = 0, wtd_y = 0, wsu_x = 0, wsu_y = 0, wsd_x = 0, wsd_y = 0;
 #pragma unroll
@@ -401,17 +402,17 @@ k_nl_agrad_fused(const typename CT<R>::type* __restrict__ S, const typename CT<R
   if (threadIdx.x < 3) {
     double tsum = 0.0;
     for (int w = 0; w < 8; ++w) tsum += red[w][threadIdx.x];
-    part[((size_t)kb * pt.natoms + a) * 3 + threadIdx.x] = tsum;
+    part[(((size_t)kb * pt.natoms + a) * chunks + ch) * 3 + threadIdx.x] = tsum;
   }
 }
 
-// out[3 kb + i] += f sum_a part[kb][a][i], atoms in order.
-__global__ void k_nl_agrad_sum(int nkb, int natoms, const double* __restrict__ part, double f, double* out) {
+// out[3 kb + i] += f sum_p part[kb][p][i] over the (atom, chunk) pairs p in order.
+__global__ void k_nl_agrad_sum(int nkb, int nparts, const double* __restrict__ part, double f, double* out) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= 3 * nkb) return;
   const int kb = j / 3, i = j - 3 * kb;
   double t = 0.0;
-  for (int a = 0; a < natoms; ++a) t += part[((size_t)kb * natoms + a) * 3 + i];
+  for (int p = 0; p < nparts; ++p) t += part[((size_t)kb * nparts + p) * 3 + i];
   out[j] += f * t;
 }
 
@@ -421,8 +422,9 @@ cudaError_t launch_nl_agrad_fused(cudaStream_t st, int N, const void* S, const v
                                   double f, double* part, double* out) {
   using C = typename CT<R>::type;
   const size_t N3 = (size_t)N * N * N;
-  dim3 grid(pt.natoms, nkb);
-#define NLA_ARGS (const C*)S, (const C*)T, N3, pt, ep, (const C*)dcS, (const C*)dcT, part
+  const int chunks = proj_chunks(pt.natoms, nkb, pt.nent);
+  dim3 grid(pt.natoms * chunks, nkb);
+#define NLA_ARGS (const C*)S, (const C*)T, N3, pt, ep, chunks, (const C*)dcS, (const C*)dcT, part
   switch (pt.nlm) {
     case 1: k_nl_agrad_fused<R, 1><<<grid, 256, 0, st>>>(NLA_ARGS); break;
     case 4: k_nl_agrad_fused<R, 4><<<grid, 256, 0, st>>>(NLA_ARGS); break;
@@ -432,7 +434,7 @@ cudaError_t launch_nl_agrad_fused(cudaStream_t st, int N, const void* S, const v
 #undef NLA_ARGS
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_nl_agrad_sum<<<(3 * nkb + 127) / 128, 128, 0, st>>>(nkb, pt.natoms, part, f, out);
+  k_nl_agrad_sum<<<(3 * nkb + 127) / 128, 128, 0, st>>>(nkb, pt.natoms * chunks, part, f, out);
   return cudaGetLastError();
 }
 

@@ -219,8 +219,13 @@ struct tddft_ctx {
   float* tile_part = nullptr;  // gather partial products, nk * groups * td.part_layer floats
   void* vnl = nullptr;         // V_NL T_k from the tensor-core scatter (spinor layout)
   int* tc_err = nullptr;     // wait errors: bit 1 tensor-core projector, bit 2 bulk-copy FFT pass
-  void *g_tab = nullptr, *s_tab = nullptr, *Dmat = nullptr;
-  void *g_row = nullptr, *s_row = nullptr, *nrm = nullptr;
+  void *g_row = nullptr, *s_row = nullptr, *nrm = nullptr, *Dmat = nullptr;
+  void *g_ph = nullptr, *s_ph = nullptr;      // phases exp(i (k + A).d) at A = ph_A
+  void *g_beta = nullptr, *s_beta = nullptr;  // FP64 projector values
+  bool ph_valid = false;
+  double ph_A[3] = {0, 0, 0};
+  void* gpart = nullptr;                      // gather partial sums of the chunks, and their counters
+  int* gcount = nullptr;
   // bookkeeping
   std::string err;
   long long launches = 0;
@@ -237,17 +242,19 @@ struct tddft_ctx {
     ProjTables<R> p;
     p.natoms = natoms;
     p.nlm = nlm;
-    p.ntab = 3 + nlm;
+    p.nent = n_entries;
     p.g_ptr = g_ptr;
     p.g_idx = g_idx;
-    p.g_tab = (const R*)g_tab;
     p.s_ptr = s_ptr;
     p.s_atom = s_atom;
-    p.s_tab = (const R*)s_tab;
     p.Dmat = (const R*)Dmat;
     p.g_row = (const R*)g_row;
     p.s_row = (const R*)s_row;
     p.nrm = (const R*)nrm;
+    p.g_ph = g_ph;
+    p.s_ph = s_ph;
+    p.g_beta = (const R*)g_beta;
+    p.s_beta = (const R*)s_beta;
     const double pi = 3.14159265358979323846;  // the constants of solid_harmonics()
     p.yc[0] = (R)(0.5 / std::sqrt(pi));
     p.yc[1] = (R)std::sqrt(3.0 / (4.0 * pi));
@@ -814,6 +821,22 @@ template <typename R> tddft_status kinetic(tddft_ctx* c, const void* in, void* o
   return c->launch(KC_FFT_XY, "ifft xy", [&] { return xy_pass<R>(c, out, out, nbatch, true); }, by);
 }
 
+// The phase tables of the CUDA-core projector kernels for this A, filled on the gather's stream: every
+// kernel that reads them follows a gather at the same A (on that stream or after its join).  They
+// depend on A, the k-points and the atoms only, so an unchanged A keeps them.
+template <typename R> tddft_status phases(tddft_ctx* c, const double A[3], const EpiParams& ep, cudaStream_t sg) {
+  if (c->ph_valid && A[0] == c->ph_A[0] && A[1] == c->ph_A[1] && A[2] == c->ph_A[2]) return TDDFT_OK;
+  c->ph_valid = false;
+  tddft_status s = c->launch_on(sg, KC_PROJ, "projector phases", [&] {
+    cudaError_t e = launch_phase_table<R>(sg, c->n_entries, c->nk, (const R*)c->g_row, ep, c->g_ph);
+    return e != cudaSuccess ? e : launch_phase_table<R>(sg, c->n_entries, c->nk, (const R*)c->s_row, ep, c->s_ph);
+  });
+  if (s) return s;
+  for (int a = 0; a < 3; ++a) c->ph_A[a] = A[a];
+  c->ph_valid = true;
+  return TDDFT_OK;
+}
+
 template <typename R> tddft_status gather(tddft_ctx* c, const void* in, const double A[3], cudaStream_t sg = nullptr) {
   if (c->natoms == 0) return TDDFT_OK;
   if (!sg) sg = c->st;
@@ -829,8 +852,9 @@ template <typename R> tddft_status gather(tddft_ctx* c, const void* in, const do
                                 c->cbuf, c->dcbuf, c->tc_err);
     }, byt);
   }
+  if (tddft_status s = phases<R>(c, A, ep, sg)) return s;
   return c->launch_on(sg, KC_PROJ, "projector gather", [&] {
-    return launch_proj_gather<R>(sg, c->N, in, c->nkb, pt, c->dV, ep, c->cbuf, c->dcbuf);
+    return launch_proj_gather<R>(sg, c->N, in, c->nkb, pt, c->dV, ep, c->gpart, c->gcount, c->cbuf, c->dcbuf);
   }, by);
 }
 
@@ -1102,8 +1126,9 @@ tddft_status gather_into(tddft_ctx* c, const void* in, const double A[3], void* 
   ep.nstates = c->nb;
   fill_shifts(c, A, ep.shift);
   ProjTables<R> pt = c->tables<R>();
+  if (tddft_status s = phases<R>(c, A, ep, c->st)) return s;
   return c->launch(KC_PROJ, "adjoint gather", [&] {
-    return launch_proj_gather<R>(c->st, c->N, in, c->nkb, pt, c->dV, ep, cb, dcb);
+    return launch_proj_gather<R>(c->st, c->N, in, c->nkb, pt, c->dV, ep, c->gpart, c->gcount, cb, dcb);
   });
 }
 
@@ -1373,7 +1398,7 @@ tddft_status do_backward(tddft_ctx* c, int nsteps, int ckpt, const double* dL_dr
   w.ncoef = (size_t)c->nkb * std::max(1, c->natoms) * 2 * c->nlm;
   const size_t cb = w.ncoef * 2 * sizeof(R);
   if ((s = tmp_alloc(c, db, &w.cS, cb, "cS")) || (s = tmp_alloc(c, db, &w.dcS, cb, "dcS")) ||
-      (s = tmp_alloc(c, db, &w.apart, (size_t)c->nkb * std::max(c->natoms, 1) * 3 * 8, "agrad parts")) ||
+      (s = tmp_alloc(c, db, &w.apart, (size_t)c->nkb * std::max(c->natoms, 1) * proj_chunks(c->natoms, c->nkb, c->n_entries) * 3 * 8, "agrad parts")) ||
       (s = tmp_alloc(c, db, &w.cT, cb, "cT")) || (s = tmp_alloc(c, db, &w.dcT, cb, "dcT")))
     return s;
   const int nck = (nsteps + ckpt - 1) / ckpt;
@@ -1954,8 +1979,7 @@ tddft_status create_impl(tddft_ctx* c, const tddft_cell* cell, const tddft_grid*
       if ((s = upload_typed<double>(c, reinterpret_cast<void**>(&Td), T, "soc torque"))) return s;
       c->Tsoc = reinterpret_cast<double2*>(Td);
     }
-    // the full tables (d and the nlm projector values per entry) only feed the tensor-core
-    // gather; the CUDA-core gather and the scatter evaluate beta from the compact rows
+    // compact rows (d, exp(-|d|^2 / (2 w^2))); FP64 also tabulates the projector values below
     if (c->prec == TDDFT_FP64) {
       if ((s = upload_typed<double>(c, &c->g_row, ht.g_row, "g_row")) || (s = upload_typed<double>(c, &c->s_row, ht.s_row, "s_row")) ||
           (s = upload_typed<double>(c, &c->nrm, ht.nrm, "nrm")) || (s = upload_typed<double>(c, &c->Dmat, ht.Dmat, "D")))
@@ -1963,6 +1987,24 @@ tddft_status create_impl(tddft_ctx* c, const tddft_cell* cell, const tddft_grid*
     } else {
       if ((s = upload_typed<float>(c, &c->g_row, ht.g_row, "g_row")) || (s = upload_typed<float>(c, &c->s_row, ht.s_row, "s_row")) ||
           (s = upload_typed<float>(c, &c->nrm, ht.nrm, "nrm")) || (s = upload_typed<float>(c, &c->Dmat, ht.Dmat, "D")))
+        return s;
+    }
+    const size_t ne = c->n_entries;
+    const size_t part_bytes = proj_gather_part_bytes(c->natoms, c->nlm, c->nk, c->nb, ne, rs);
+    const size_t ncnt = proj_gather_counters(c->natoms, c->nk, c->nb) * sizeof(int);
+    if ((s = c->alloc(&c->g_ph, ne * c->nk * 2 * rs, "phases")) || (s = c->alloc(&c->s_ph, ne * c->nk * 2 * rs, "phases")) ||
+        (s = c->alloc(&c->gpart, part_bytes, "gather partials")) || (s = c->alloc(&c->gcount, ncnt, "gather counters")) ||
+        (s = c->cuda(cudaMemset(c->gcount, 0, ncnt), "gather counters init")))
+      return s;
+    if (c->prec == TDDFT_FP64) {
+      const size_t bb = ne * beta_pitch(c->nlm) * sizeof(double);
+      if ((s = c->alloc(&c->g_beta, bb, "projector values")) || (s = c->alloc(&c->s_beta, bb, "projector values"))) return s;
+      const ProjTables<double> pt = c->tables<double>();
+      if ((s = c->launch(KC_OTHER, "projector values", [&] {
+             cudaError_t e = launch_beta_table<double>(c->st, ne, (const double*)c->g_row, nullptr, pt, (double*)c->g_beta);
+             return e != cudaSuccess ? e
+                                     : launch_beta_table<double>(c->st, ne, (const double*)c->s_row, c->s_atom, pt, (double*)c->s_beta);
+           })))
         return s;
     }
     if (c->tile) {

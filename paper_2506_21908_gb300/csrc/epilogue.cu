@@ -91,15 +91,15 @@ k_epilogue(const typename CT<R>::type* __restrict__ kin, const typename CT<R>::t
   const C pu[2] = {pu2.a, pu2.b}, pd[2] = {pd2.a, pd2.b};
   C hu[2] = {ku2.a, ku2.b}, hd[2] = {kd2.a, kd2.b};
   {
-    const R sx = (R)ep.shift[k][0], sy = (R)ep.shift[k][1], sz = (R)ep.shift[k][2];
+    const C* ph = reinterpret_cast<const C*>(pt.s_ph) + (size_t)k * pt.nent;
     if constexpr (SP) {
       const R v0 = V[r], v1 = V[N3 + r], v2 = V[2 * N3 + r], v3 = V[3 * N3 + r];
-      h_point_2sp<R, NLM>(hu, hd, pu, pd, v0, v1, (R)0.5 * v2, (R)0.5 * v3, r, pt, dcb, dcb + ncoef, sx, sy, sz);
+      h_point_2sp<R, NLM>(hu, hd, pu, pd, v0, v1, (R)0.5 * v2, (R)0.5 * v3, r, pt, dcb, dcb + ncoef, ph);
     } else {
       const C v0 = *reinterpret_cast<const C*>(V + r), v1 = *reinterpret_cast<const C*>(V + N3 + r);
       const C v2 = *reinterpret_cast<const C*>(V + 2 * N3 + r), v3 = *reinterpret_cast<const C*>(V + 3 * N3 + r);
-      h_point<R, NLM>(hu[0], hd[0], pu[0], pd[0], v0.x, v1.x, (R)0.5 * v2.x, (R)0.5 * v3.x, r, pt, dcb, sx, sy, sz);
-      h_point<R, NLM>(hu[1], hd[1], pu[1], pd[1], v0.y, v1.y, (R)0.5 * v2.y, (R)0.5 * v3.y, r + 1, pt, dcb, sx, sy, sz);
+      h_point<R, NLM>(hu[0], hd[0], pu[0], pd[0], v0.x, v1.x, (R)0.5 * v2.x, (R)0.5 * v3.x, r, pt, dcb, ph);
+      h_point<R, NLM>(hu[1], hd[1], pu[1], pd[1], v0.y, v1.y, (R)0.5 * v2.y, (R)0.5 * v3.y, r + 1, pt, dcb, ph);
     }
   }
   if (rec) { qu0 = ld(Tkm1, ou); qd0 = ld(Tkm1, od); }

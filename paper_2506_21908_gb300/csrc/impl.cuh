@@ -90,21 +90,30 @@ inline void split_constants(EpiParams& e) {
 
 // Device-side projector tables.
 template <typename R> struct ProjTables {
-  int natoms = 0, nlm = 0, ntab = 0;        // ntab = 3 + nlm reals per entry
+  int natoms = 0, nlm = 0;
+  size_t nent = 0;                          // entries (sphere points of all atoms)
   const int* g_ptr = nullptr;               // [natoms + 1] entries of each atom (gather order)
   const int* g_idx = nullptr;               // grid point of each gather entry
-  const R* g_tab = nullptr;                 // [entries][3 + nlm]: d, beta
   const int* s_ptr = nullptr;               // [N^3 + 1] entries of each grid point (scatter order)
   const int* s_atom = nullptr;              // atom of each scatter entry
-  const R* s_tab = nullptr;                 // [entries][3 + nlm]
   const R* Dmat = nullptr;                  // [natoms][2 nlm][2 nlm] complex (re, im)
   // Compact rows for the CUDA-core gather and the scatter: beta is evaluated from d as
   // N_l(w_a) g S_lm(d) with g = exp(-|d|^2 / (2 w_a^2)) and S_lm the real solid harmonics.
   const R* g_row = nullptr;                 // [entries][4]: d, g (gather order)
   const R* s_row = nullptr;                 // [entries][4] (scatter order)
   const R* nrm = nullptr;                   // [natoms][4]: N_0, N_1, N_2 of the atom's width, 0
+  // Phases exp(i (k + A).d) of every entry at the current A, per k-point ([nk][entries] complex), in
+  // gather and scatter order; and in FP64, where their arithmetic would cost more than the loads
+  // (the FP64 pipe is the bound), the projector values [entries][beta_pitch(nlm)].
+  const void* g_ph = nullptr;
+  const void* s_ph = nullptr;
+  const R* g_beta = nullptr;
+  const R* s_beta = nullptr;
   R yc[4] = {};                             // solid-harmonic constants: l = 0, l = 1, l = 2 (xy, ...), l = 2 (3z^2 - r^2)
 };
+
+// Row length of the FP64 projector value tables: rows of whole 16-byte loads.
+__host__ __device__ constexpr int beta_pitch(int nlm) { return nlm == 1 ? 1 : (nlm + 1) / 2 * 2; }
 
 // ---------------------------------------------------------------- launchers
 template <typename R>
@@ -118,9 +127,21 @@ cudaError_t launch_fft_xy_tma(cudaStream_t st, int N, const void* src, void* dst
 template <typename R>
 cudaError_t launch_fft_z(cudaStream_t st, int N, void* data, int nbatch, const void* tw, int mode,
                          const ZParams& zp);
+// out[k][e] = exp(i shift_k.d_e) from the compact rows; beta tables [entries][beta_pitch(nlm)], the
+// entries of atom a at g_ptr[a] (atom == null) or with their atom listed (scatter order).
+template <typename R>
+cudaError_t launch_phase_table(cudaStream_t st, size_t nent, int nk, const R* rows, const EpiParams& ep, void* out);
+template <typename R>
+cudaError_t launch_beta_table(cudaStream_t st, size_t nent, const R* rows, const int* atom, const ProjTables<R>& pt,
+                              R* out);
+// CTAs that share one (atom, spinor group) of the projector gather and of the projector-phase
+// gradient, and the scratch they need: partial sums (bytes) and zeroed counters (ints).
+int proj_chunks(int natoms, int ngroups, size_t nent);
+size_t proj_gather_part_bytes(int natoms, int nlm, int nk, int nstates, size_t nent, size_t rsize);
+size_t proj_gather_counters(int natoms, int nk, int nstates);
 template <typename R>
 cudaError_t launch_proj_gather(cudaStream_t st, int N, const void* psi, int nkb, const ProjTables<R>& pt,
-                               double dV, const EpiParams& ep, void* c_out, void* dc_out);
+                               double dV, const EpiParams& ep, void* part, int* counters, void* c_out, void* dc_out);
 template <typename R>
 // kin: the kinetic part of H T_k; kin2 (may be null): V_NL T_k from the tensor-core scatter.
 cudaError_t launch_epilogue(cudaStream_t st, int N, const void* kin, const void* kin2, const void* Tk,
@@ -240,7 +261,7 @@ cudaError_t launch_fft_z_current(cudaStream_t st, int N, void* U, const void* W,
                                  const ZParams& zp, double* part);
 // Projector-phase A-gradient in one pass over the entries (replaces the moment gathers and
 // launch_nl_agrad): out[kb][a] += f sum_atoms sum_e d_a Im(e^{-i phi}[conj(S) w_T + conj(T) w_S]).
-// part: natoms x nkb x 3 doubles of scratch.
+// part: natoms x nkb x 3 doubles of scratch for each of proj_chunks(natoms, nkb, entries) chunks.
 template <typename R>
 cudaError_t launch_nl_agrad_fused(cudaStream_t st, int N, const void* S, const void* T, int nkb,
                                   const ProjTables<R>& pt, const EpiParams& ep, const void* dcS, const void* dcT,

@@ -62,19 +62,26 @@ __device__ __forceinline__ void beta_values(R x, R y, R z, R g, const R* nl, con
   }
 }
 
-// phase exp(-i arg): FP32 reduces the argument to [-pi, pi] and uses the fast intrinsic
-__device__ __forceinline__ void phase_sincos(float x, float* sn, float* cs) {
-  const float r = x - 6.28318530717958647692f * rintf(x * 0.15915494309189533577f);
-  __sincosf(r, sn, cs);
+// Projector values of entry e: FP64 reads its table row, FP32 evaluates them from the compact row.
+template <typename R, int NLM>
+__device__ __forceinline__ void entry_beta(size_t e, int a, const R* rows, const R* beta, const ProjTables<R>& pt, R* bt) {
+  if constexpr (sizeof(R) == 8) {
+    load_row<R, beta_pitch(NLM)>(beta + e * beta_pitch(NLM), bt);
+  } else {
+    R t[4], nl[4];
+    load_row<R, 4>(rows + e * 4, t);
+    load_row<R, 4>(pt.nrm + (size_t)a * 4, nl);
+    beta_values<R, NLM>(t[0], t[1], t[2], t[3], nl, pt.yc, bt);
+  }
 }
-__device__ __forceinline__ void phase_sincos(double x, double* sn, double* cs) { sincos(x, sn, cs); }
 
 // Hamiltonian at one point for both spinor components: (hu, hd) holds the kinetic part on
 // entry; the 2x2 local potential and the projector scatter are added.
 template <typename R, int NLM>
 __device__ __forceinline__ void h_point(typename CT<R>::type& hu, typename CT<R>::type& hd, typename CT<R>::type pu,
                                         typename CT<R>::type pd, R V0, R V1, R hx, R hy, size_t r,
-                                        const ProjTables<R>& pt, const typename CT<R>::type* dcb, R sx, R sy, R sz) {
+                                        const ProjTables<R>& pt, const typename CT<R>::type* dcb,
+                                        const typename CT<R>::type* ph) {
   using C = typename CT<R>::type;
   hu = cmake<C>(hu.x + V0 * pu.x + hx * pd.x - hy * pd.y, hu.y + V0 * pu.y + hx * pd.y + hy * pd.x);
   hd = cmake<C>(hd.x + V1 * pd.x + hx * pu.x + hy * pu.y, hd.y + V1 * pd.y + hx * pu.y - hy * pu.x);
@@ -82,10 +89,9 @@ __device__ __forceinline__ void h_point(typename CT<R>::type& hu, typename CT<R>
     const int e0 = pt.s_ptr[r], e1 = pt.s_ptr[r + 1];
     for (int e = e0; e < e1; ++e) {
       const int a = pt.s_atom[e];
-      R t[4], nl[4], bt[NLM];
-      load_row<R, 4>(pt.s_row + (size_t)e * 4, t);
-      load_row<R, 4>(pt.nrm + (size_t)a * 4, nl);
-      beta_values<R, NLM>(t[0], t[1], t[2], t[3], nl, pt.yc, bt);
+      R bt[beta_pitch(NLM)];
+      const C pe = ph[e];
+      entry_beta<R, NLM>(e, a, pt.s_row, pt.s_beta, pt, bt);
       const C* dca = dcb + (size_t)a * 2 * NLM;  // this spinor's D c of atom a, (up, dn) per p
       R vux = 0, vuy = 0, vdx = 0, vdy = 0;
 #pragma unroll
@@ -95,8 +101,7 @@ __device__ __forceinline__ void h_point(typename CT<R>::type& hu, typename CT<R>
         vux += bp * cc.a.x; vuy += bp * cc.a.y;
         vdx += bp * cc.b.x; vdy += bp * cc.b.y;
       }
-      R sn, cs;
-      phase_sincos(sx * t[0] + sy * t[1] + sz * t[2], &sn, &cs);
+      const R cs = pe.x, sn = pe.y;
       hu.x += vux * cs + vuy * sn; hu.y += vuy * cs - vux * sn;
       hd.x += vdx * cs + vdy * sn; hd.y += vdy * cs - vdx * sn;
     }
@@ -110,8 +115,8 @@ template <typename R, int NLM>
 __device__ __forceinline__ void h_point_2sp(typename CT<R>::type (&hu)[2], typename CT<R>::type (&hd)[2],
                                             const typename CT<R>::type (&pu)[2], const typename CT<R>::type (&pd)[2],
                                             R V0, R V1, R hx, R hy, size_t r, const ProjTables<R>& pt,
-                                            const typename CT<R>::type* dcb0, const typename CT<R>::type* dcb1, R sx,
-                                            R sy, R sz) {
+                                            const typename CT<R>::type* dcb0, const typename CT<R>::type* dcb1,
+                                            const typename CT<R>::type* ph) {
   using C = typename CT<R>::type;
 #pragma unroll
   for (int g = 0; g < 2; ++g) {
@@ -124,12 +129,10 @@ __device__ __forceinline__ void h_point_2sp(typename CT<R>::type (&hu)[2], typen
     const int e0 = pt.s_ptr[r], e1 = pt.s_ptr[r + 1];
     for (int e = e0; e < e1; ++e) {
       const int a = pt.s_atom[e];
-      R t[4], nl[4], bt[NLM];
-      load_row<R, 4>(pt.s_row + (size_t)e * 4, t);
-      load_row<R, 4>(pt.nrm + (size_t)a * 4, nl);
-      beta_values<R, NLM>(t[0], t[1], t[2], t[3], nl, pt.yc, bt);
-      R sn, cs;
-      phase_sincos(sx * t[0] + sy * t[1] + sz * t[2], &sn, &cs);
+      R bt[beta_pitch(NLM)];
+      const C pe = ph[e];
+      entry_beta<R, NLM>(e, a, pt.s_row, pt.s_beta, pt, bt);
+      const R cs = pe.x, sn = pe.y;
 #pragma unroll
       for (int g = 0; g < 2; ++g) {
         const C* dca = (g ? dcb1 : dcb0) + (size_t)a * 2 * NLM;

@@ -9,6 +9,7 @@
 //   k_density    rho_v = sum_k w_k sum_i f_i {|u|^2, |d|^2, Re u d*, Im u d*}  (Eqs. rho1-rho3)
 //   k_potential  locally collinear LSDA (Eqs. LC+ALDA2, LC+ALDA) and assembly of V_v
 //   reductions   deterministic fixed-order block reductions for energies and norms
+#include <algorithm>
 #include <cstdint>
 
 #include "fft.cuh"
@@ -416,117 +417,267 @@ cudaError_t launch_fft_z(cudaStream_t st, int N, void* data, int nbatch, const v
 
 // ============================================================================ projectors
 
-// One CTA per (atom, spinor): c[p][sigma] = sum_e beta_p exp(+i s.d) psi_sigma(r_e) dV, then D c.
-template <typename R> struct GatherMinBlocks { static constexpr int value = 1; };
-template <> struct GatherMinBlocks<float> { static constexpr int value = 3; };
-
-template <typename R, int NLM>
-__global__ void __launch_bounds__(256, GatherMinBlocks<R>::value)
-k_proj_gather(const typename CT<R>::type* __restrict__ psi, size_t N3, ProjTables<R> pt, R dV, EpiParams ep,
-              typename CT<R>::type* __restrict__ c_out, typename CT<R>::type* __restrict__ dc_out) {
+// exp(i s.d) of every entry, per k-point: evaluated once per A(t) instead of once per entry, spinor
+// and Chebyshev term (in FP64 the sine and cosine were 110 of the 181 FP64 instructions an entry
+// cost the gather, whose bound is the FP64 pipe).
+template <typename R>
+__global__ void __launch_bounds__(256)
+k_phase_table(size_t nent, const R* __restrict__ rows, EpiParams ep, typename CT<R>::type* __restrict__ out) {
   using C = typename CT<R>::type;
-  constexpr int NV = 4 * NLM;  // reals: (re, im) x (up, dn) x NLM
-  const int a = blockIdx.x;
-  const int kb = blockIdx.y;
-  const int k = kb / ep.nstates;
-  const R sx = (R)ep.shift[k][0], sy = (R)ep.shift[k][1], sz = (R)ep.shift[k][2];
+  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= nent) return;
+  const int k = blockIdx.y;
+  R t[4];
+  load_row<R, 4>(rows + e * 4, t);
+  R sn, cs;
+  sincos_r<R>((R)ep.shift[k][0] * t[0] + (R)ep.shift[k][1] * t[1] + (R)ep.shift[k][2] * t[2], &sn, &cs);
+  out[(size_t)k * nent + e] = cmake<C>(cs, sn);
+}
+template <typename R>
+cudaError_t launch_phase_table(cudaStream_t st, size_t nent, int nk, const R* rows, const EpiParams& ep, void* out) {
+  if (nent == 0) return cudaSuccess;
+  k_phase_table<R><<<dim3((unsigned)((nent + 255) / 256), nk), 256, 0, st>>>(nent, rows, ep, (typename CT<R>::type*)out);
+  return cudaGetLastError();
+}
+
+// Projector values of every entry (once, at creation).
+template <typename R, int NLM>
+__global__ void __launch_bounds__(256)
+k_beta_table(size_t nent, const R* __restrict__ rows, const int* __restrict__ atom, ProjTables<R> pt, R* __restrict__ out) {
+  const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= nent) return;
+  int a = 0;
+  if (atom) a = atom[e];
+  else
+    while (a + 1 < pt.natoms && (size_t)pt.g_ptr[a + 1] <= e) ++a;
+  R t[4], nl[4], b[NLM];
+  load_row<R, 4>(rows + e * 4, t);
+  load_row<R, 4>(pt.nrm + (size_t)a * 4, nl);
+  beta_values<R, NLM>(t[0], t[1], t[2], t[3], nl, pt.yc, b);
+  R* o = out + e * beta_pitch(NLM);
+#pragma unroll
+  for (int p = 0; p < beta_pitch(NLM); ++p) o[p] = p < NLM ? b[p] : (R)0;
+}
+template <typename R>
+cudaError_t launch_beta_table(cudaStream_t st, size_t nent, const R* rows, const int* atom, const ProjTables<R>& pt,
+                              R* out) {
+  if (nent == 0) return cudaSuccess;
+  const unsigned grid = (unsigned)((nent + 255) / 256);
+  switch (pt.nlm) {
+    case 1: k_beta_table<R, 1><<<grid, 256, 0, st>>>(nent, rows, atom, pt, out); break;
+    case 4: k_beta_table<R, 4><<<grid, 256, 0, st>>>(nent, rows, atom, pt, out); break;
+    case 9: k_beta_table<R, 9><<<grid, 256, 0, st>>>(nent, rows, atom, pt, out); break;
+    default: return cudaErrorInvalidValue;
+  }
+  return cudaGetLastError();
+}
+
+// Sum of v[0..NV) over the lanes of a warp, NV values at once: each of the five steps exchanges
+// half of the values a lane still holds, so it takes about NV additions where NV separate
+// butterflies take 5 NV (FP64 additions are the bound of a small gather).  On return the lane
+// holds the sums of the values lane_sum_index(j) in v[j]; indices out of range are negative.
+__host__ __device__ constexpr int lane_sum_count(int nv) {
+  for (int o = 0; o < 5; ++o) nv = (nv + 1) / 2;
+  return nv;
+}
+template <int N, int O, typename R>
+__device__ __forceinline__ void lane_sums(R* v, int lane) {
+  constexpr int H = (N + 1) / 2;
+  const bool up = (lane & O) != 0;
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    const R hi = (i + H < N) ? v[i + H] : (R)0;
+    const R mine = up ? hi : v[i], other = up ? v[i] : hi;
+    v[i] = mine + __shfl_xor_sync(0xffffffffu, other, O);
+  }
+  if constexpr (O > 1) lane_sums<H, O / 2>(v, lane);
+}
+// Index of the sum that slot j holds after lane_sums<N, O> (negative: none).
+template <int N, int O>
+__device__ __forceinline__ int lane_sum_index(int j, int lane) {
+  constexpr int H = (N + 1) / 2;
+  int pos = j;
+  if constexpr (O > 1) pos = lane_sum_index<H, O / 2>(j, lane);
+  if (pos < 0) return -1;
+  if (lane & O) pos += H;
+  return pos < N ? pos : -1;
+}
+
+// CTA (atom, chunk; spinor group): c[p][sigma] = sum_e beta_p exp(+i s.d) psi_sigma(r_e) dV over the
+// chunk's entries, SPN spinors of one k-point per thread (they share the entry's tables); with
+// several chunks the last CTA of the group to finish adds the partial sums in chunk order (the
+// result does not depend on which one that is), then D c.
+//
+// Bound by the FP64 pipe in FP64 (44 instructions an entry and spinor with the phases and projector
+// values read from tables, 181 when they were evaluated here) and by the latency of the entry ->
+// psi loads in FP32; one CTA per (atom, spinor) left the chip idle for few of either (4 CTAs,
+// 126 us, at 24^3 with one atom and four spinors).
+constexpr int PG_NT = 128;
+template <typename R> struct GatherMinBlocks { static constexpr int value = 3; };
+template <> struct GatherMinBlocks<float> { static constexpr int value = 4; };
+
+template <typename R, int NLM, int SPN>
+__global__ void __launch_bounds__(PG_NT, GatherMinBlocks<R>::value)
+k_proj_gather(const typename CT<R>::type* __restrict__ psi, size_t N3, ProjTables<R> pt, R dV, int nstates, int chunks,
+              R* __restrict__ part, int* __restrict__ counters, typename CT<R>::type* __restrict__ c_out,
+              typename CT<R>::type* __restrict__ dc_out) {
+  using C = typename CT<R>::type;
+  constexpr int NS = 4 * NLM;    // reals per spinor: (re, im) x (up, dn) x NLM
+  constexpr int NV = SPN * NS;
+  const int a = blockIdx.x / chunks, ch = blockIdx.x - a * chunks;
+  const int kb = blockIdx.y * SPN;
+  const int k = kb / nstates;
   const C* up = psi + (size_t)(2 * kb) * N3;
-  const C* dn = up + N3;
+  const C* ph = reinterpret_cast<const C*>(pt.g_ph) + (size_t)k * pt.nent;
   R acc[NV];
 #pragma unroll
   for (int i = 0; i < NV; ++i) acc[i] = (R)0;
-  const int e0 = pt.g_ptr[a], e1 = pt.g_ptr[a + 1];
-  R nl[4];
-  load_row<R, 4>(pt.nrm + (size_t)a * 4, nl);
-  // Software pipeline over this thread's entries e, e + 256, ...: the grid index of the entry
-  // after next, and the table row and psi values of the next entry, are requested before the
-  // current entry is processed, so two dependent load chains are in flight at a time.
+  const int g0 = pt.g_ptr[a], ng = pt.g_ptr[a + 1] - g0;
+  const int e0 = g0 + (int)((long long)ng * ch / chunks), e1 = g0 + (int)((long long)ng * (ch + 1) / chunks);
+  // Software pipeline over this thread's entries e, e + PG_NT, ...: the grid index of the entry
+  // after next, and the psi values and phase of the next entry, are requested before the current
+  // entry is processed, so two dependent load chains are in flight at a time.
   const C zc = cmake<C>((R)0, (R)0);
   int e = e0 + threadIdx.x;
-  int r1 = (e + 256 < e1) ? pt.g_idx[e + 256] : 0;  // index of the next entry
-  R tc[4] = {(R)0, (R)0, (R)0, (R)0};
-  C uc = zc, dc = zc;
+  int r1 = (e + PG_NT < e1) ? pt.g_idx[e + PG_NT] : 0;  // index of the next entry
+  C pc = zc, w[2 * SPN];
+#pragma unroll
+  for (int j = 0; j < 2 * SPN; ++j) w[j] = zc;
   if (e < e1) {
     const int r0 = pt.g_idx[e];
-    load_row<R, 4>(pt.g_row + (size_t)e * 4, tc);
-    uc = up[r0];
-    dc = dn[r0];
+    pc = ph[e];
+#pragma unroll
+    for (int j = 0; j < 2 * SPN; ++j) w[j] = up[(size_t)j * N3 + r0];
   }
-  for (; e < e1; e += 256) {
-    R tn[4] = {(R)0, (R)0, (R)0, (R)0};
-    C un = zc, dn_ = zc;
+  for (; e < e1; e += PG_NT) {
+    C pn = zc, wn[2 * SPN];
     int r2 = 0;
-    if (e + 256 < e1) {
-      load_row<R, 4>(pt.g_row + (size_t)(e + 256) * 4, tn);
-      un = up[r1];
-      dn_ = dn[r1];
-      if (e + 512 < e1) r2 = pt.g_idx[e + 512];
+#pragma unroll
+    for (int j = 0; j < 2 * SPN; ++j) wn[j] = zc;
+    if (e + PG_NT < e1) {
+      pn = ph[e + PG_NT];
+#pragma unroll
+      for (int j = 0; j < 2 * SPN; ++j) wn[j] = up[(size_t)j * N3 + r1];
+      if (e + 2 * PG_NT < e1) r2 = pt.g_idx[e + 2 * PG_NT];
     }
-    R t[4] = {tc[0], tc[1], tc[2], tc[3]}, bt[NLM];
-    beta_values<R, NLM>(t[0], t[1], t[2], t[3], nl, pt.yc, bt);
-    R sn, cs;
-    sincos_r<R>(sx * t[0] + sy * t[1] + sz * t[2], &sn, &cs);
-    const C u = uc, d = dc;
-    for (int i = 0; i < 4; ++i) tc[i] = tn[i];
-    uc = un;
-    dc = dn_;
+    R bt[beta_pitch(NLM)];
+    entry_beta<R, NLM>(e, a, pt.g_row, pt.g_beta, pt, bt);
+#pragma unroll
+    for (int s = 0; s < SPN; ++s) {
+      const C u = cmul(w[2 * s], pc), d = cmul(w[2 * s + 1], pc);  // psi exp(+i arg)
+#pragma unroll
+      for (int p = 0; p < NLM; ++p) {
+        acc[s * NS + 4 * p + 0] += bt[p] * u.x;
+        acc[s * NS + 4 * p + 1] += bt[p] * u.y;
+        acc[s * NS + 4 * p + 2] += bt[p] * d.x;
+        acc[s * NS + 4 * p + 3] += bt[p] * d.y;
+      }
+    }
+    pc = pn;
+#pragma unroll
+    for (int j = 0; j < 2 * SPN; ++j) w[j] = wn[j];
     r1 = r2;
-    const R pux = u.x * cs - u.y * sn, puy = u.x * sn + u.y * cs;  // u exp(+i arg)
-    const R pdx = d.x * cs - d.y * sn, pdy = d.x * sn + d.y * cs;
-#pragma unroll
-    for (int p = 0; p < NLM; ++p) {
-      const R bp = bt[p];
-      acc[4 * p + 0] += bp * pux;
-      acc[4 * p + 1] += bp * puy;
-      acc[4 * p + 2] += bp * pdx;
-      acc[4 * p + 3] += bp * pdy;
-    }
   }
-  __shared__ R red[8][NV];
-  __shared__ C cv[2 * NLM];
+  __shared__ R red[PG_NT / 32][NV];
+  __shared__ C cv[SPN * 2 * NLM];
+  __shared__ int last;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  lane_sums<NV, 16>(acc, lane);
 #pragma unroll
-  for (int i = 0; i < NV; ++i) {
-    const R v = warp_sum(acc[i]);
-    if (lane == 0) red[warp][i] = v;
+  for (int j = 0; j < lane_sum_count(NV); ++j) {
+    const int i = lane_sum_index<NV, 16>(j, lane);
+    if (i >= 0) red[warp][i] = acc[j];
   }
   __syncthreads();
-  if (threadIdx.x < 2 * NLM) {
-    R re = 0, im = 0;
-    for (int w = 0; w < 8; ++w) {
-      re += red[w][2 * threadIdx.x];
-      im += red[w][2 * threadIdx.x + 1];
+  const size_t grp = (size_t)blockIdx.y * pt.natoms + a;
+  if (threadIdx.x < NV) {
+    R s = red[0][threadIdx.x];
+#pragma unroll
+    for (int v = 1; v < PG_NT / 32; ++v) s += red[v][threadIdx.x];
+    if (chunks == 1) red[0][threadIdx.x] = s;
+    else part[(grp * chunks + ch) * NV + threadIdx.x] = s;
+  }
+  if (chunks > 1) {
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      last = atomicAdd(counters + grp, 1) == chunks - 1;
+      if (last) counters[grp] = 0;  // for the next launch
     }
-    C c = cmake<C>(re * dV, im * dV);
-    cv[threadIdx.x] = c;
-    c_out[((size_t)kb * pt.natoms + a) * 2 * NLM + threadIdx.x] = c;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (threadIdx.x < NV) {
+      R s = (R)0;
+      for (int i = 0; i < chunks; ++i) s += __ldcg(part + (grp * chunks + i) * NV + threadIdx.x);
+      red[0][threadIdx.x] = s;
+    }
   }
   __syncthreads();
-  if (threadIdx.x < 2 * NLM) {
-    const R* D = pt.Dmat + ((size_t)a * 2 * NLM + threadIdx.x) * 2 * NLM * 2;
+  for (int i = threadIdx.x; i < SPN * 2 * NLM; i += PG_NT) {
+    const C c = cmake<C>(red[0][2 * i] * dV, red[0][2 * i + 1] * dV);
+    cv[i] = c;
+    const int s = i / (2 * NLM), q = i - s * 2 * NLM;
+    c_out[((size_t)(kb + s) * pt.natoms + a) * 2 * NLM + q] = c;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < SPN * 2 * NLM; i += PG_NT) {
+    const int s = i / (2 * NLM), q = i - s * 2 * NLM;
+    const R* D = pt.Dmat + ((size_t)a * 2 * NLM + q) * 2 * NLM * 2;
     R re = 0, im = 0;
     for (int u = 0; u < 2 * NLM; ++u) {
       const R dr = D[2 * u], di = D[2 * u + 1];
-      re += dr * cv[u].x - di * cv[u].y;
-      im += dr * cv[u].y + di * cv[u].x;
+      const C c = cv[s * 2 * NLM + u];
+      re += dr * c.x - di * c.y;
+      im += dr * c.y + di * c.x;
     }
-    dc_out[((size_t)kb * pt.natoms + a) * 2 * NLM + threadIdx.x] = cmake<C>(re, im);
+    dc_out[((size_t)(kb + s) * pt.natoms + a) * 2 * NLM + q] = cmake<C>(re, im);
   }
 }
 
+// Spinors per thread: two in FP32 where a k-point's states pair up, else one (FP64: registers).
+static int gather_spn(size_t rsize, int nstates) { return rsize == 4 && nstates % 2 == 0 ? 2 : 1; }
+
+// Enough CTAs for four per SM (608 on this chip), at least 256 entries each (two per thread).
+int proj_chunks(int natoms, int ngroups, size_t nent) {
+  const long long have = (long long)natoms * ngroups;
+  if (have <= 0) return 1;
+  const long long want = (608 + have - 1) / have, most = (long long)(nent / (size_t)natoms) / 256;
+  return (int)std::max(1LL, std::min(want, std::min(most, 64LL)));
+}
+size_t proj_gather_part_bytes(int natoms, int nlm, int nk, int nstates, size_t nent, size_t rsize) {
+  const int spn = gather_spn(rsize, nstates), groups = nk * nstates / spn;
+  return (size_t)groups * natoms * proj_chunks(natoms, groups, nent) * spn * 4 * nlm * rsize;
+}
+size_t proj_gather_counters(int natoms, int nk, int nstates) { return (size_t)natoms * nk * nstates; }
+
 template <typename R>
 cudaError_t launch_proj_gather(cudaStream_t st, int N, const void* psi, int nkb, const ProjTables<R>& pt,
-                               double dV, const EpiParams& ep, void* c_out, void* dc_out) {
+                               double dV, const EpiParams& ep, void* part, int* counters, void* c_out, void* dc_out) {
   using C = typename CT<R>::type;
   if (pt.natoms == 0) return cudaSuccess;
-  dim3 grid(pt.natoms, nkb);
+  const int spn = gather_spn(sizeof(R), ep.nstates), groups = nkb / spn;
+  const int chunks = proj_chunks(pt.natoms, groups, pt.nent);
+  dim3 grid(pt.natoms * chunks, groups);
   const size_t N3 = (size_t)N * N * N;
+#define PG_ARGS (const C*)psi, N3, pt, (R)dV, ep.nstates, chunks, (R*)part, counters, (C*)c_out, (C*)dc_out
+#define PG_CASE(NLM)                                                                         \
+  if constexpr (sizeof(R) == 4) {                                                            \
+    if (spn == 2) {                                                                          \
+      k_proj_gather<R, NLM, 2><<<grid, PG_NT, 0, st>>>(PG_ARGS);                             \
+      break;                                                                                 \
+    }                                                                                        \
+  }                                                                                          \
+  k_proj_gather<R, NLM, 1><<<grid, PG_NT, 0, st>>>(PG_ARGS);                                 \
+  break
   switch (pt.nlm) {
-    case 1: k_proj_gather<R, 1><<<grid, 256, 0, st>>>((const C*)psi, N3, pt, (R)dV, ep, (C*)c_out, (C*)dc_out); break;
-    case 4: k_proj_gather<R, 4><<<grid, 256, 0, st>>>((const C*)psi, N3, pt, (R)dV, ep, (C*)c_out, (C*)dc_out); break;
-    case 9: k_proj_gather<R, 9><<<grid, 256, 0, st>>>((const C*)psi, N3, pt, (R)dV, ep, (C*)c_out, (C*)dc_out); break;
+    case 1: PG_CASE(1);
+    case 4: PG_CASE(4);
+    case 9: PG_CASE(9);
     default: return cudaErrorInvalidValue;
   }
+#undef PG_CASE
+#undef PG_ARGS
   return cudaGetLastError();
 }
 
@@ -1177,8 +1328,11 @@ cudaError_t launch_atom_sums(cudaStream_t st, size_t N3, int natoms, const doubl
 #define TDDFT_INST(R)                                                                                           \
   template cudaError_t launch_fft_xy<R>(cudaStream_t, int, const void*, void*, int, const void*, bool);                       \
   template cudaError_t launch_fft_z<R>(cudaStream_t, int, void*, int, const void*, int, const ZParams&);          \
+  template cudaError_t launch_phase_table<R>(cudaStream_t, size_t, int, const R*, const EpiParams&, void*);      \
+  template cudaError_t launch_beta_table<R>(cudaStream_t, size_t, const R*, const int*, const ProjTables<R>&,    \
+                                            R*);                                                                \
   template cudaError_t launch_proj_gather<R>(cudaStream_t, int, const void*, int, const ProjTables<R>&, double,  \
-                                             const EpiParams&, void*, void*);                                   \
+                                             const EpiParams&, void*, int*, void*, void*);                      \
   template cudaError_t launch_density<R>(cudaStream_t, size_t, const void*, int, const double*, double*,         \
                                          double*);                                                                \
   template cudaError_t launch_convert_in<R>(cudaStream_t, size_t, const double2*, void*);                        \
