@@ -1054,7 +1054,7 @@ template <typename R> tddft_status one_step(tddft_ctx* c) {
   for (int it = 0; it < c->n_sc; ++it) {
     if ((s = density<R>(c, c->psi, rnext))) return s;
     if (c->sc_tol > 0.0) {
-      if ((s = c->launch(KC_OTHER, "sc diff", [&] { return launch_max_abs_diff(c->st, 4 * c->N3, rnext, rprev, c->red); })))
+      if ((s = c->launch(KC_OTHER, "sc diff", [&] { return launch_max_abs_diff(c->st, 4 * c->N3, rnext, rprev, c->red, c->red_part); })))
         return s;
       double d = 0.0;
       if ((s = c->cuda(cudaMemcpyAsync(&d, c->red, sizeof(double), cudaMemcpyDeviceToHost, c->st), "sc read"))) return s;
@@ -1926,7 +1926,7 @@ tddft_status create_impl(tddft_ctx* c, const tddft_cell* cell, const tddft_grid*
     return s;
   if (c->natoms > 0) {
     if ((s = c->alloc(&c->owner, N3 * sizeof(int), "voronoi owner")) ||
-        (s = c->alloc(&c->atom_sums, 4 * (size_t)c->natoms * 8, "atom sums")))
+        (s = c->alloc(&c->atom_sums, (4 * (size_t)c->natoms + atom_sums_part_doubles(c->natoms)) * 8, "atom sums")))
       return s;
     if ((s = c->launch(KC_OTHER, "voronoi owner", [&] {
            return launch_voronoi_owner(c->st, c->N, c->L, c->natoms, pos_d, c->owner);
@@ -2172,7 +2172,7 @@ tddft_status tddft_atom_moments(tddft_handle h, double* M, double* N) {
   if (!h->have_states) return h->fail(TDDFT_ERR_STATE, "no states loaded");
   if (h->natoms == 0) return TDDFT_OK;
   tddft_status s = h->launch(KC_OTHER, "atom sums", [&] {
-    return launch_atom_sums(h->st, h->N3, h->natoms, h->rho, h->owner, h->atom_sums);
+    return launch_atom_sums(h->st, h->N3, h->natoms, h->rho, h->owner, h->atom_sums, h->atom_sums + 4 * (size_t)h->natoms);
   });
   if (s) return s;
   std::vector<double> out(4 * (size_t)h->natoms);
@@ -2205,7 +2205,7 @@ tddft_status tddft_torques(tddft_handle h, double* soc, double* xc, double* zeem
          })))
       return s;
   }
-  if ((s = h->launch(KC_OTHER, "xc torque", [&] { return launch_xc_torque(h->st, h->N3, h->rho, h->vxc4, h->tq + 3 * nkb); })))
+  if ((s = h->launch(KC_OTHER, "xc torque", [&] { return launch_xc_torque(h->st, h->N3, h->rho, h->vxc4, h->tq + 3 * nkb, h->red_part); })))
     return s;
   std::vector<double> out(3 * (size_t)nkb + 6);
   if ((s = h->cuda(cudaMemcpyAsync(out.data(), h->tq, out.size() * 8, cudaMemcpyDeviceToHost, h->st), "torque read")) ||

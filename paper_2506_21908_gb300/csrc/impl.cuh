@@ -174,7 +174,8 @@ cudaError_t launch_field_sums(cudaStream_t st, size_t N3, const double* rho, con
                               const double* vH, const double* exc, const double* vxc4, const double* V,
                               const double* B, double* out, double* part);  // part: field_sums_part_doubles()
 size_t field_sums_part_doubles();
-cudaError_t launch_max_abs_diff(cudaStream_t st, size_t n, const double* a, const double* b, double* out);
+// part: field_sums_part_doubles() scratch, as below.
+cudaError_t launch_max_abs_diff(cudaStream_t st, size_t n, const double* a, const double* b, double* out, double* part);
 cudaError_t launch_check_window(cudaStream_t st, size_t N3, const double* V, double lo, double hi,
                                 double kin_max, double nl_bound, int* flag);
 // n and m (4 N3 doubles: n, m_x, m_y, m_z) from rho_v.
@@ -249,8 +250,11 @@ cudaError_t launch_voronoi_owner(cudaStream_t st, int N, const double* L, int na
 template <typename R>
 cudaError_t launch_soc_torque(cudaStream_t st, int nkb, int natoms, int M, const void* c, const double2* T,
                               double* out);
-cudaError_t launch_xc_torque(cudaStream_t st, size_t N3, const double* rho, const double* vxc4, double* out6);
-cudaError_t launch_atom_sums(cudaStream_t st, size_t N3, int natoms, const double* rho, const int* owner, double* out);
+cudaError_t launch_xc_torque(cudaStream_t st, size_t N3, const double* rho, const double* vxc4, double* out6,
+                             double* part);
+size_t atom_sums_part_doubles(int natoms);
+cudaError_t launch_atom_sums(cudaStream_t st, size_t N3, int natoms, const double* rho, const int* owner, double* out,
+                             double* part);
 
 // ---------------------------------------------------------------- adjoint launchers
 template <typename R>

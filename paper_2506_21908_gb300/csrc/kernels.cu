@@ -976,8 +976,19 @@ __device__ double block_sum(double v, double* sh) {
   return t;  // valid in thread 0
 }
 
+// out[i] = sum over parts of part[parts][nval]: one warp per value, lanes stride over the parts (a
+// single thread per value waits for one load after the other: 50 us for 304 parts).
+__global__ void k_parts_total(int nparts, int nval, const double* __restrict__ part, double* __restrict__ out) {
+  const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (i >= nval) return;
+  double s = 0.0;
+  for (int b = lane; b < nparts; b += 32) s += part[(size_t)b * nval + i];
+  s = warp_sum(s);
+  if (lane == 0) out[i] = s;
+}
+
 // out2[band] = sum over npts of conj(a) b (complex, double accumulation) in two passes: CTA
-// (chunk, band) sums a fixed range of points, then one thread per band adds the chunks in
+// (chunk, band) sums a fixed range of points, then one warp per band adds the chunks in a fixed
 // order (deterministic, and every SM busy).
 constexpr int kDotChunks = 64;
 template <typename R>
@@ -1014,22 +1025,26 @@ __global__ void __launch_bounds__(256) k_band_dot_part(size_t npts, const typena
   }
 }
 __global__ void k_band_dot_sum(int nbands, const double* __restrict__ part, double* out2) {
-  const int band = blockIdx.x * blockDim.x + threadIdx.x;
+  const int band = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (band >= nbands) return;
   double re = 0.0, im = 0.0;
-  for (int ch = 0; ch < kDotChunks; ++ch) {
+  for (int ch = lane; ch < kDotChunks; ch += 32) {
     re += part[((size_t)band * kDotChunks + ch) * 2];
     im += part[((size_t)band * kDotChunks + ch) * 2 + 1];
   }
-  out2[2 * band] = re;
-  out2[2 * band + 1] = im;
+  re = warp_sum(re);
+  im = warp_sum(im);
+  if (lane == 0) {
+    out2[2 * band] = re;
+    out2[2 * band + 1] = im;
+  }
 }
 template <typename R>
 cudaError_t launch_band_dot(cudaStream_t st, size_t npts, int nbands, const void* a, const void* b, double* out2,
                             double* part) {
   using C = typename CT<R>::type;
   k_band_dot_part<R><<<dim3(kDotChunks, nbands), 256, 0, st>>>(npts, (const C*)a, (const C*)b, part);
-  k_band_dot_sum<<<(nbands + 127) / 128, 128, 0, st>>>(nbands, part, out2);
+  k_band_dot_sum<<<(nbands + 3) / 4, 128, 0, st>>>(nbands, part, out2);
   return cudaGetLastError();
 }
 size_t band_dot_part_doubles(int nbands) { return (size_t)nbands * kDotChunks * 2; }
@@ -1088,34 +1103,9 @@ cudaError_t launch_soc_torque(cudaStream_t st, int nkb, int natoms, int M, const
   return cudaGetLastError();
 }
 
-// int b_xc x m and int m (without dV) from rho_v and the XC 4-vector [vbar + b_z, vbar - b_z,
-// 2 b_x, -2 b_y]; one block, fixed order.
-__global__ void __launch_bounds__(1024)
-k_xc_torque(size_t N3, const double* __restrict__ rho, const double* __restrict__ vxc4, double* out) {
-  __shared__ double sh[32];
-  double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-  for (size_t r = threadIdx.x; r < N3; r += 1024) {
-    const double r0 = rho[r], r1 = rho[N3 + r], r2 = rho[2 * N3 + r], r3 = rho[3 * N3 + r];
-    const double mx = 2.0 * r2, my = -2.0 * r3, mz = r0 - r1;
-    const double bz = 0.5 * (vxc4[r] - vxc4[N3 + r]), bx = 0.5 * vxc4[2 * N3 + r], by = -0.5 * vxc4[3 * N3 + r];
-    acc[0] += by * mz - bz * my;
-    acc[1] += bz * mx - bx * mz;
-    acc[2] += bx * my - by * mx;
-    acc[3] += mx; acc[4] += my; acc[5] += mz;
-  }
-  for (int i = 0; i < 6; ++i) {
-    const double t = block_sum<1024>(acc[i], sh);
-    if (threadIdx.x == 0) out[i] = t;
-  }
-}
-cudaError_t launch_xc_torque(cudaStream_t st, size_t N3, const double* rho, const double* vxc4, double* out6) {
-  k_xc_torque<<<1, 1024, 0, st>>>(N3, rho, vxc4, out6);
-  return cudaGetLastError();
-}
-
 // Field integrals (without dV): [0] v_loc n, [1] v_H n, [2] e_xc, [3..5] m, [6] n, [7] B.m,
 // [8] <rho_v, V_v^xc>, [9] count of non-finite rho values.  Two passes: each of kFieldBlocks
-// CTAs sums a fixed range of points, then one CTA adds the block partials in order.
+// CTAs sums a fixed range of points, then one CTA adds the block partials in a fixed order.
 constexpr int kFieldBlocks = 304;
 __global__ void __launch_bounds__(256)
 k_field_sums_part(size_t N3, const double* __restrict__ rho, const double* __restrict__ vloc, const double* __restrict__ vH,
@@ -1143,38 +1133,89 @@ k_field_sums_part(size_t N3, const double* __restrict__ rho, const double* __res
     if (threadIdx.x == 0) part[(size_t)blockIdx.x * 10 + i] = t;
   }
 }
-__global__ void k_field_sums_total(const double* __restrict__ part, double* out) {
-  const int i = threadIdx.x;
-  if (i >= 10) return;
-  double s = 0.0;
-  for (int b = 0; b < kFieldBlocks; ++b) s += part[(size_t)b * 10 + i];
-  out[i] = s;
-}
 cudaError_t launch_field_sums(cudaStream_t st, size_t N3, const double* rho, const double* vloc, const double* vH,
                               const double* exc, const double* vxc4, const double* /*V*/, const double* B, double* out,
                               double* part) {
   k_field_sums_part<<<kFieldBlocks, 256, 0, st>>>(N3, rho, vloc, vH, exc, vxc4, B[0], B[1], B[2], part);
-  k_field_sums_total<<<1, 32, 0, st>>>(part, out);
+  k_parts_total<<<1, 320, 0, st>>>(kFieldBlocks, 10, part, out);
   return cudaGetLastError();
 }
 size_t field_sums_part_doubles() { return (size_t)kFieldBlocks * 10; }
 
-__global__ void __launch_bounds__(1024) k_max_abs_diff(size_t n, const double* a, const double* b, double* out) {
-  __shared__ double sh[32];
+// int b_xc x m and int m (without dV) from rho_v and the XC 4-vector [vbar + b_z, vbar - b_z,
+// 2 b_x, -2 b_y], in the two passes of the field sums.  (One CTA over all points took most of a
+// report's reductions: 1.1 ms at 64^3.)
+__global__ void __launch_bounds__(256)
+k_xc_torque_part(size_t N3, const double* __restrict__ rho, const double* __restrict__ vxc4, double* part) {
+  __shared__ double sh[8];
+  double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  const size_t len = (N3 + kFieldBlocks - 1) / kFieldBlocks;
+  const size_t lo = (size_t)blockIdx.x * len, hi = lo + len < N3 ? lo + len : N3;
+  for (size_t r = lo + threadIdx.x; r < hi; r += 256) {
+    const double r0 = rho[r], r1 = rho[N3 + r], r2 = rho[2 * N3 + r], r3 = rho[3 * N3 + r];
+    const double mx = 2.0 * r2, my = -2.0 * r3, mz = r0 - r1;
+    const double bz = 0.5 * (vxc4[r] - vxc4[N3 + r]), bx = 0.5 * vxc4[2 * N3 + r], by = -0.5 * vxc4[3 * N3 + r];
+    acc[0] += by * mz - bz * my;
+    acc[1] += bz * mx - bx * mz;
+    acc[2] += bx * my - by * mx;
+    acc[3] += mx; acc[4] += my; acc[5] += mz;
+  }
+  for (int i = 0; i < 6; ++i) {
+    const double t = block_sum<256>(acc[i], sh);
+    if (threadIdx.x == 0) part[(size_t)blockIdx.x * 6 + i] = t;
+  }
+}
+cudaError_t launch_xc_torque(cudaStream_t st, size_t N3, const double* rho, const double* vxc4, double* out6,
+                             double* part) {
+  k_xc_torque_part<<<kFieldBlocks, 256, 0, st>>>(N3, rho, vxc4, part);
+  k_parts_total<<<1, 192, 0, st>>>(kFieldBlocks, 6, part, out6);
+  return cudaGetLastError();
+}
+
+// Sums of the three N3-fields of g, the same two passes.
+__global__ void __launch_bounds__(256) k_sum3_part(size_t N3, const double* __restrict__ g, double* part) {
+  __shared__ double sh[8];
+  const size_t len = (N3 + kFieldBlocks - 1) / kFieldBlocks;
+  const size_t lo = (size_t)blockIdx.x * len, hi = lo + len < N3 ? lo + len : N3;
+  double acc[3] = {0.0, 0.0, 0.0};
+  for (size_t r = lo + threadIdx.x; r < hi; r += 256)
+    for (int a = 0; a < 3; ++a) acc[a] += g[a * N3 + r];
+  for (int a = 0; a < 3; ++a) {
+    const double t = block_sum<256>(acc[a], sh);
+    if (threadIdx.x == 0) part[(size_t)blockIdx.x * 3 + a] = t;
+  }
+}
+cudaError_t launch_sum3(cudaStream_t st, size_t N3, const double* g, double* out, double* part) {
+  k_sum3_part<<<kFieldBlocks, 256, 0, st>>>(N3, g, part);
+  k_parts_total<<<1, 96, 0, st>>>(kFieldBlocks, 3, part, out);
+  return cudaGetLastError();
+}
+
+__global__ void __launch_bounds__(256) k_max_abs_diff(size_t n, const double* a, const double* b, double* part) {
+  __shared__ double sh[8];
   double m = 0.0;
-  for (size_t i = threadIdx.x; i < n; i += 1024) m = fmax(m, fabs(a[i] - b[i]));
+  for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (size_t)gridDim.x * 256)
+    m = fmax(m, fabs(a[i] - b[i]));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
-    for (int w = 0; w < 32; ++w) t = fmax(t, sh[w]);
-    *out = t;
+    for (int w = 0; w < 8; ++w) t = fmax(t, sh[w]);
+    part[blockIdx.x] = t;
   }
 }
-cudaError_t launch_max_abs_diff(cudaStream_t st, size_t n, const double* a, const double* b, double* out) {
-  k_max_abs_diff<<<1, 1024, 0, st>>>(n, a, b, out);
+__global__ void k_max_total(int nparts, const double* __restrict__ part, double* out) {
+  double m = 0.0;
+  for (int i = threadIdx.x; i < nparts; i += 32) m = fmax(m, part[i]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
+  if (threadIdx.x == 0) *out = m;
+}
+cudaError_t launch_max_abs_diff(cudaStream_t st, size_t n, const double* a, const double* b, double* out, double* part) {
+  k_max_abs_diff<<<kFieldBlocks, 256, 0, st>>>(n, a, b, part);
+  k_max_total<<<1, 32, 0, st>>>(kFieldBlocks, part, out);
   return cudaGetLastError();
 }
 
@@ -1247,13 +1288,19 @@ __global__ void __launch_bounds__(256) k_window_part(size_t N3, const double* __
   }
 }
 __global__ void k_window_total(int nparts, const double* __restrict__ part, double* out) {
-  if (threadIdx.x != 0) return;
   double vmin = 1e300, vmax = -1e300, bmax = 0.0;
-  for (int i = 0; i < nparts; ++i) {
+  for (int i = threadIdx.x; i < nparts; i += 32) {
     vmin = fmin(vmin, part[3 * i]);
     vmax = fmax(vmax, part[3 * i + 1]);
     bmax = fmax(bmax, part[3 * i + 2]);
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    vmin = fmin(vmin, __shfl_down_sync(0xffffffffu, vmin, o));
+    vmax = fmax(vmax, __shfl_down_sync(0xffffffffu, vmax, o));
+    bmax = fmax(bmax, __shfl_down_sync(0xffffffffu, bmax, o));
+  }
+  if (threadIdx.x != 0) return;
   out[0] = vmin;
   out[1] = vmax;
   out[2] = bmax;
@@ -1298,14 +1345,18 @@ cudaError_t launch_voronoi_owner(cudaStream_t st, int N, const double* L, int na
   return cudaGetLastError();
 }
 
-// out[a] = {sum m_x, sum m_y, sum m_z, sum n} over the points owned by atom a (one CTA per atom,
-// fixed order; multiply by dV on the host).
+// out[a] = {sum m_x, sum m_y, sum m_z, sum n} over the points owned by atom a (fixed order; multiply
+// by dV on the host): kAtomChunks CTAs per atom each scan a range of the grid's owners (one CTA per
+// atom over the whole grid left the chip idle), then one warp per atom adds their sums.
+constexpr int kAtomChunks = 32;
 __global__ void __launch_bounds__(256) k_atom_sums(size_t N3, const double* __restrict__ rho,
-                                                   const int* __restrict__ owner, double* __restrict__ out) {
+                                                   const int* __restrict__ owner, double* __restrict__ part) {
   __shared__ double sh[8];
   const int a = blockIdx.x;
+  const size_t len = (N3 + kAtomChunks - 1) / kAtomChunks;
+  const size_t lo = (size_t)blockIdx.y * len, hi = lo + len < N3 ? lo + len : N3;
   double acc[4] = {0, 0, 0, 0};
-  for (size_t r = threadIdx.x; r < N3; r += 256) {
+  for (size_t r = lo + threadIdx.x; r < hi; r += 256) {
     if (owner[r] != a) continue;
     const double r0 = rho[r], r1 = rho[N3 + r], r2 = rho[2 * N3 + r], r3 = rho[3 * N3 + r];
     acc[0] += 2.0 * r2;
@@ -1315,19 +1366,31 @@ __global__ void __launch_bounds__(256) k_atom_sums(size_t N3, const double* __re
   }
   for (int c = 0; c < 4; ++c) {
     const double t = block_sum<256>(acc[c], sh);
-    if (threadIdx.x == 0) out[4 * a + c] = t;
+    if (threadIdx.x == 0) part[((size_t)a * kAtomChunks + blockIdx.y) * 4 + c] = t;
     __syncthreads();
   }
 }
-cudaError_t launch_atom_sums(cudaStream_t st, size_t N3, int natoms, const double* rho, const int* owner, double* out) {
-  k_atom_sums<<<natoms, 256, 0, st>>>(N3, rho, owner, out);
+__global__ void k_atom_sums_total(int natoms, const double* __restrict__ part, double* __restrict__ out) {
+  const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;  // (atom, value)
+  if (i >= 4 * natoms) return;
+  const double s = warp_sum(part[((size_t)(i >> 2) * kAtomChunks + lane) * 4 + (i & 3)]);
+  if (lane == 0) out[i] = s;
+}
+size_t atom_sums_part_doubles(int natoms) { return (size_t)natoms * kAtomChunks * 4; }
+cudaError_t launch_atom_sums(cudaStream_t st, size_t N3, int natoms, const double* rho, const int* owner, double* out,
+                             double* part) {
+  static_assert(kAtomChunks == 32, "one lane per chunk");
+  k_atom_sums<<<dim3(natoms, kAtomChunks), 256, 0, st>>>(N3, rho, owner, part);
+  k_atom_sums_total<<<natoms, 128, 0, st>>>(natoms, part, out);
   return cudaGetLastError();
 }
 
 // ============================================================================ instantiations
 #define TDDFT_INST(R)                                                                                           \
   template cudaError_t launch_fft_xy<R>(cudaStream_t, int, const void*, void*, int, const void*, bool);                       \
-  template cudaError_t launch_fft_z<R>(cudaStream_t, int, void*, int, const void*, int, const ZParams&);          \
+  template cudaError_t launch_fft_z_kinetic<R>(cudaStream_t, int, void*, int, const void*, const void*,          \
+                                               const ZParams&);                                                 \
+  template cudaError_t launch_kin_tables<R>(cudaStream_t, int, int, const ZParams&, void*);                      \
   template cudaError_t launch_phase_table<R>(cudaStream_t, size_t, int, const R*, const EpiParams&, void*);      \
   template cudaError_t launch_beta_table<R>(cudaStream_t, size_t, const R*, const int*, const ProjTables<R>&,    \
                                             R*);                                                                \
