@@ -1388,9 +1388,7 @@ cudaError_t launch_atom_sums(cudaStream_t st, size_t N3, int natoms, const doubl
 // ============================================================================ instantiations
 #define TDDFT_INST(R)                                                                                           \
   template cudaError_t launch_fft_xy<R>(cudaStream_t, int, const void*, void*, int, const void*, bool);                       \
-  template cudaError_t launch_fft_z_kinetic<R>(cudaStream_t, int, void*, int, const void*, const void*,          \
-                                               const ZParams&);                                                 \
-  template cudaError_t launch_kin_tables<R>(cudaStream_t, int, int, const ZParams&, void*);                      \
+  template cudaError_t launch_fft_z<R>(cudaStream_t, int, void*, int, const void*, int, const ZParams&);          \
   template cudaError_t launch_phase_table<R>(cudaStream_t, size_t, int, const R*, const EpiParams&, void*);      \
   template cudaError_t launch_beta_table<R>(cudaStream_t, size_t, const R*, const int*, const ProjTables<R>&,    \
                                             R*);                                                                \
