@@ -564,45 +564,14 @@ cudaError_t launch_xc_adjoint(cudaStream_t st, size_t N3, const double* rho, con
 }
 
 // rbar[0], rbar[1] += vH-adjoint field (real part of the Hartree-transformed gv).
-__global__ void k_add_hartree_adjoint(size_t N3, const double2* __restrict__ h, double* __restrict__ rbar) {
+__global__ void k_add_hartree_adjoint(size_t N3, const double* __restrict__ h, double* __restrict__ rbar) {
   const size_t r = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= N3) return;
-  rbar[r] += h[r].x;
-  rbar[N3 + r] += h[r].x;
+  rbar[r] += h[r];
+  rbar[N3 + r] += h[r];
 }
-cudaError_t launch_add_hartree_adjoint(cudaStream_t st, size_t N3, const double2* h, double* rbar) {
+cudaError_t launch_add_hartree_adjoint(cudaStream_t st, size_t N3, const double* h, double* rbar) {
   k_add_hartree_adjoint<<<(unsigned)((N3 + 255) / 256), 256, 0, st>>>(N3, h, rbar);
-  return cudaGetLastError();
-}
-
-__global__ void k_real_field_to_complex(size_t n, const double* in, double2* out) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) out[i] = make_double2(in[i], 0.0);
-}
-cudaError_t launch_real_field_to_complex(cudaStream_t st, size_t N3, const double* in, double2* out) {
-  k_real_field_to_complex<<<(unsigned)((N3 + 255) / 256), 256, 0, st>>>(N3, in, out);
-  return cudaGetLastError();
-}
-
-// Deterministic single-CTA sums of the three b-cotangent fields.
-__global__ void __launch_bounds__(1024) k_sum3(size_t N3, const double* __restrict__ g, double* out) {
-  __shared__ double sh[32];
-  for (int a = 0; a < 3; ++a) {
-    double s = 0.0;
-    for (size_t r = threadIdx.x; r < N3; r += 1024) s += g[a * N3 + r];
-    s = warp_sum(s);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0.0;
-      for (int w = 0; w < 32; ++w) t += sh[w];
-      out[a] = t;
-    }
-    __syncthreads();
-  }
-}
-cudaError_t launch_sum3(cudaStream_t st, size_t N3, const double* g, double* out) {
-  k_sum3<<<1, 1024, 0, st>>>(N3, g, out);
   return cudaGetLastError();
 }
 

@@ -739,24 +739,19 @@ tddft_status upload(tddft_ctx* c, T** dst, const std::vector<T>& src, const char
 }
 
 // ------------------------------------------------------------------ potential pipeline
-tddft_status hartree(tddft_ctx* c, const double* rho) {
-  ZParams zp{};
-  const double pi = 3.14159265358979323846;
-  for (int a = 0; a < 3; ++a) zp.gs[a] = 2.0 * pi / c->L[a];
-  zp.scale = 1.0 / (double)c->N3;
-  tddft_status s;
-  if ((s = c->launch(KC_POT, "density to complex", [&] { return launch_density_to_complex(c->st, c->N3, rho, c->hart); }))) return s;
-  if ((s = c->launch(KC_POT, "hartree fft xy", [&] { return launch_fft_xy<double>(c->st, c->N, c->hart, c->hart, 1, c->tw64, false); }))) return s;
-  if ((s = c->launch(KC_POT, "hartree fft z", [&] { return launch_fft_z<double>(c->st, c->N, c->hart, 1, c->tw64, Z_POISSON, zp); }))) return s;
-  if ((s = c->launch(KC_POT, "hartree ifft xy", [&] { return launch_fft_xy<double>(c->st, c->N, c->hart, c->hart, 1, c->tw64, true); }))) return s;
-  return c->launch(KC_POT, "hartree real part", [&] { return launch_complex_real_part(c->st, c->N3, c->hart, c->vH, 1.0); });
+// out = v_H of in + in2 (in2 may be null).
+tddft_status hartree(tddft_ctx* c, const double* in, const double* in2, double* out) {
+  c->launches += kPoissonLaunches - 1;
+  return c->launch(KC_POT, "hartree", [&] {
+    return launch_poisson(c->st, c->N, in, in2, out, c->hart, c->tw64, nullptr, c->L);
+  });
 }
 
 // rho (4 x N3) -> V (FP64) and, in mixed precision, its FP32 copy.
 tddft_status potential(tddft_ctx* c, const double* rho, double tt, double* Vout, float* Vfout) {
   double A[3], B[3];
   c->fields(tt, A, B);
-  tddft_status s = hartree(c, rho);
+  tddft_status s = hartree(c, rho, rho + c->N3, c->vH);
   if (s) return s;
   return c->launch(KC_POT, "potential", [&] {
     return launch_potential(c->st, c->N3, rho, c->vH, c->vloc, B, c->xc, c->spin_mode, Vout, Vfout, c->exc, c->vxc4);
@@ -1231,17 +1226,10 @@ tddft_status cheb_adjoint(tddft_ctx* c, AdjWork& w, const std::vector<const void
 // Hartree (symmetric convolution) and the uniform Zeeman coupling mu_B B.sigma.
 tddft_status potential_adjoint(tddft_ctx* c, AdjWork& w, const double* rho, double gB[3]) {
   tddft_status s;
-  ZParams zp{};
-  const double pi = 3.14159265358979323846;
-  for (int a = 0; a < 3; ++a) zp.gs[a] = 2.0 * pi / c->L[a];
-  zp.scale = 1.0 / (double)c->N3;
   if ((s = c->launch(KC_POT, "xc adjoint", [&] { return launch_xc_adjoint(c->st, c->N3, rho, w.gV, c->xc, w.rbar, w.gvf, w.gbf); }))) return s;
-  if ((s = c->launch(KC_POT, "hartree adj in", [&] { return launch_real_field_to_complex(c->st, c->N3, w.gvf, c->hart); }))) return s;
-  if ((s = c->launch(KC_POT, "hartree adj xy", [&] { return launch_fft_xy<double>(c->st, c->N, c->hart, c->hart, 1, c->tw64, false); }))) return s;
-  if ((s = c->launch(KC_POT, "hartree adj z", [&] { return launch_fft_z<double>(c->st, c->N, c->hart, 1, c->tw64, Z_POISSON, zp); }))) return s;
-  if ((s = c->launch(KC_POT, "hartree adj ixy", [&] { return launch_fft_xy<double>(c->st, c->N, c->hart, c->hart, 1, c->tw64, true); }))) return s;
-  if ((s = c->launch(KC_POT, "hartree adj add", [&] { return launch_add_hartree_adjoint(c->st, c->N3, c->hart, w.rbar); }))) return s;
-  if ((s = c->launch(KC_POT, "b sums", [&] { return launch_sum3(c->st, c->N3, w.gbf, c->red); }))) return s;
+  if ((s = hartree(c, w.gvf, nullptr, w.gvf))) return s;
+  if ((s = c->launch(KC_POT, "hartree adj add", [&] { return launch_add_hartree_adjoint(c->st, c->N3, w.gvf, w.rbar); }))) return s;
+  if ((s = c->launch(KC_POT, "b sums", [&] { return launch_sum3(c->st, c->N3, w.gbf, c->red, c->red_part); }))) return s;
   double h[3];
   if ((s = c->cuda(cudaMemcpyAsync(h, c->red, sizeof(h), cudaMemcpyDeviceToHost, c->st), "b read"))) return s;
   if ((s = c->cuda(cudaStreamSynchronize(c->st), "b sync"))) return s;

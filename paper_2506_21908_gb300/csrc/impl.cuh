@@ -156,7 +156,12 @@ cudaError_t launch_density(cudaStream_t st, size_t N3, const void* psi, int nkb,
 cudaError_t launch_potential(cudaStream_t st, size_t N3, const double* rho, const double* vH,
                              const double* vloc, const double* B, int xc, int spin_mode, double* V, float* Vf,
                              double* exc, double* vxc4);
-cudaError_t launch_density_to_complex(cudaStream_t st, size_t N3, const double* rho, double2* out);
+// out = the Hartree potential of the real field in (+ in2, may be null); in and out may be the same
+// array.  g: N^3 / 2 complex scratch.  tw: exp(-2 pi i t / N), or null: then the solve forms them
+// in tw_out (N complex).  Five launches.
+constexpr int kPoissonLaunches = 5;
+cudaError_t launch_poisson(cudaStream_t st, int N, const double* in, const double* in2, double* out, double2* g,
+                           const double2* tw, double2* tw_out, const double* L);
 cudaError_t launch_complex_real_part(cudaStream_t st, size_t N3, const double2* in, double* out, double scale);
 cudaError_t launch_vloc_G(cudaStream_t st, int N, const double* L, int natoms, const double* pos,
                           const double* Zr, double omega, double2* out);
@@ -272,9 +277,8 @@ cudaError_t launch_nl_agrad_fused(cudaStream_t st, int N, const void* S, const v
                                   double f, double* part, double* out);
 cudaError_t launch_xc_adjoint(cudaStream_t st, size_t N3, const double* rho, const double* gV, int xc, double* rbar,
                               double* gvf, double* gbf);
-cudaError_t launch_add_hartree_adjoint(cudaStream_t st, size_t N3, const double2* h, double* rbar);
-cudaError_t launch_real_field_to_complex(cudaStream_t st, size_t N3, const double* in, double2* out);
-cudaError_t launch_sum3(cudaStream_t st, size_t N3, const double* g, double* out);
+cudaError_t launch_add_hartree_adjoint(cudaStream_t st, size_t N3, const double* h, double* rbar);
+cudaError_t launch_sum3(cudaStream_t st, size_t N3, const double* g, double* out, double* part);
 cudaError_t launch_accum_parts(cudaStream_t st, size_t count, const double* part, double f, double* out3);
 template <typename R>
 cudaError_t launch_density_adjoint(cudaStream_t st, size_t N3, int nkb, const void* psi, const double* rbar,

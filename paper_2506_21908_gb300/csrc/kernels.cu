@@ -857,15 +857,6 @@ cudaError_t launch_potential(cudaStream_t st, size_t N3, const double* rho, cons
   return cudaGetLastError();
 }
 
-// (rho_uu + rho_dd, 0): the total density as a complex field for the Poisson solve.
-__global__ void k_density_to_complex(size_t n, const double* rho, double2* out) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) out[i] = make_double2(rho[i] + rho[n + i], 0.0);
-}
-cudaError_t launch_density_to_complex(cudaStream_t st, size_t N3, const double* rho, double2* out) {
-  k_density_to_complex<<<(unsigned)((N3 + 255) / 256), 256, 0, st>>>(N3, rho, out);
-  return cudaGetLastError();
-}
 __global__ void k_complex_real_part(size_t n, const double2* in, double* out, double scale) {
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = in[i].x * scale;

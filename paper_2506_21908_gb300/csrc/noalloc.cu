@@ -25,17 +25,6 @@ constexpr int kMaxDevices = 64;
 std::mutex g_mutex;
 double2* g_scratch_ptr[kMaxDevices] = {nullptr};
 
-__global__ void k_noalloc_prepare(size_t n3, int N, const double* __restrict__ dens, double2* __restrict__ field,
-                                  double2* __restrict__ tw) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n3) field[i] = make_double2(dens[i], 0.0);
-  if (i < (size_t)N) {
-    double s, c;
-    sincospi(-2.0 * (double)i / (double)N, &s, &c);  // exp(-2 pi i t / N)
-    tw[i] = make_double2(c, s);
-  }
-}
-
 }  // namespace
 
 namespace tddft {
@@ -84,23 +73,11 @@ extern "C" tddft_status tddft_hartree_noalloc(const double* n_dev, double* vH_de
     scratch = g_scratch_ptr[dev];
   }
   cudaStream_t st = (cudaStream_t)stream;
-  const size_t n3 = (size_t)n * n * n;
   double2* field = scratch;
   double2* tw = scratch + kFieldElems;
   // every field element and twiddle used below is written first, so stale contents of the
   // shared array from an earlier call never leak into the result
-  k_noalloc_prepare<<<(unsigned)((n3 + 255) / 256), 256, 0, st>>>(n3, n, n_dev, field, tw);
-  if ((e = cudaGetLastError()) != cudaSuccess) goto fail;
-  {
-    ZParams zp{};
-    const double pi = 3.14159265358979323846;
-    for (int a = 0; a < 3; ++a) zp.gs[a] = 2.0 * pi / L[a];
-    zp.scale = 1.0 / (double)n3;
-    if ((e = launch_fft_xy<double>(st, n, field, field, 1, tw, false)) != cudaSuccess) goto fail;
-    if ((e = launch_fft_z<double>(st, n, field, 1, tw, Z_POISSON, zp)) != cudaSuccess) goto fail;
-    if ((e = launch_fft_xy<double>(st, n, field, field, 1, tw, true)) != cudaSuccess) goto fail;
-    if ((e = launch_complex_real_part(st, n3, field, vH_dev, 1.0)) != cudaSuccess) goto fail;
-  }
+  if ((e = launch_poisson(st, n, n_dev, nullptr, vH_dev, field, nullptr, tw, L)) != cudaSuccess) goto fail;
   return TDDFT_OK;
 fail:
   set_global_error(std::string("tddft_hartree_noalloc: launch failed: ") + cudaGetErrorString(e));
