@@ -181,7 +181,7 @@ k_fft_z2_current(typename CT<R>::type* __restrict__ U, const typename CT<R>::typ
   constexpr size_t ZS = (size_t)N * N;
   for (int i = threadIdx.x; i < N; i += NT) {
     tw[i] = twg[i];
-    const double qx = zp.gs[0] * freq<N>(i) + zp.shift[k][0];
+    const double qx = zp.gs[0] * freq<N>(kx_at<N>(i)) + zp.shift[k][0];
     const double qz = zp.gs[2] * freq<N>(i) + zp.shift[k][2];
     kx[i] = (R)(0.5 * qx * qx * zp.scale);
     kz[i] = (R)(0.5 * qz * qz * zp.scale);

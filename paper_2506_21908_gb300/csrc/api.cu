@@ -222,6 +222,9 @@ struct tddft_ctx {
   void *g_row = nullptr, *s_row = nullptr, *nrm = nullptr, *Dmat = nullptr;
   void *g_ph = nullptr, *s_ph = nullptr;      // phases exp(i (k + A).d) at A = ph_A
   void *g_beta = nullptr, *s_beta = nullptr;  // FP64 projector values
+  void* kin_tab = nullptr;                    // kinetic factors [nk][3][N] at A = kin_A
+  bool kin_valid = false;
+  double kin_A[3] = {0, 0, 0};
   bool ph_valid = false;
   double ph_A[3] = {0, 0, 0};
   void* gpart = nullptr;                      // gather partial sums of the chunks, and their counters
@@ -811,8 +814,16 @@ template <typename R> tddft_status kinetic(tddft_ctx* c, const void* in, void* o
   const int nbatch = 2 * c->nkb;
   const double by = 2.0 * nbatch * (double)c->N3 * 2 * sizeof(R);
   tddft_status s;
+  // the kinetic factors depend on A, the k-points and the cell only: formed when A changes
+  if (!c->kin_valid || A[0] != c->kin_A[0] || A[1] != c->kin_A[1] || A[2] != c->kin_A[2]) {
+    c->kin_valid = false;
+    if ((s = c->launch(KC_FFT_Z, "kinetic tables", [&] { return launch_kin_tables<R>(c->st, c->N, c->nk, zp, c->kin_tab); })))
+      return s;
+    for (int a = 0; a < 3; ++a) c->kin_A[a] = A[a];
+    c->kin_valid = true;
+  }
   if ((s = c->launch(KC_FFT_XY, "fft xy", [&] { return xy_pass<R>(c, in, out, nbatch, false); }, by))) return s;
-  if ((s = c->launch(KC_FFT_Z, "fft z", [&] { return launch_fft_z<R>(c->st, c->N, out, nbatch, c->tw, Z_KIN, zp); }, by))) return s;
+  if ((s = c->launch(KC_FFT_Z, "fft z", [&] { return launch_fft_z_kinetic<R>(c->st, c->N, out, nbatch, c->tw, c->kin_tab, zp); }, by))) return s;
   return c->launch(KC_FFT_XY, "ifft xy", [&] { return xy_pass<R>(c, out, out, nbatch, true); }, by);
 }
 
@@ -1879,7 +1890,9 @@ tddft_status create_impl(tddft_ctx* c, const tddft_cell* cell, const tddft_grid*
     c->stage_elems = std::min(c->psi_elems(), (size_t)(64u << 20) / sizeof(double2));
     if ((s = c->alloc(&c->stage, c->stage_elems * sizeof(double2), "stage"))) return s;
   }
-  if ((s = upload(c, &c->wf_d, c->wf, "weights"))) return s;
+  if ((s = upload(c, &c->wf_d, c->wf, "weights")) ||
+      (s = c->alloc(&c->kin_tab, 3 * (size_t)c->nk * c->N * rs, "kinetic tables")))
+    return s;
   if (density_groups(N3, c->nkb) > 1 &&
       (s = c->alloc(&c->rho_part, (size_t)density_groups(N3, c->nkb) * 4 * N3 * 8, "density partials")))
     return s;
@@ -1920,8 +1933,7 @@ tddft_status create_impl(tddft_ctx* c, const tddft_cell* cell, const tddft_grid*
       return s;
   }
   if ((s = c->launch(KC_OTHER, "vloc G", [&] { return launch_vloc_G(c->st, c->N, c->L, c->natoms, pos_d, zr_d, c->omega, c->hart); }))) return s;
-  ZParams zp{};
-  if ((s = c->launch(KC_OTHER, "vloc ifft z", [&] { return launch_fft_z<double>(c->st, c->N, c->hart, 1, c->tw64, Z_INV_ONLY, zp); }))) return s;
+  if ((s = c->launch(KC_OTHER, "vloc ifft z", [&] { return launch_fft_z_inverse(c->st, c->N, c->hart, 1, c->tw64); }))) return s;
   if ((s = c->launch(KC_OTHER, "vloc ifft xy", [&] { return launch_fft_xy<double>(c->st, c->N, c->hart, c->hart, 1, c->tw64, true); }))) return s;
   if ((s = c->launch(KC_OTHER, "vloc real", [&] { return launch_complex_real_part(c->st, N3, c->hart, c->vloc, 1.0); }))) return s;
 

@@ -322,11 +322,6 @@ template <> struct TwoFactor<48> { static constexpr bool ok = true; static const
 template <> struct TwoFactor<64> { static constexpr bool ok = true; static constexpr int R1 = 8, R2 = 8; };
 template <> struct TwoFactor<96> { static constexpr bool ok = true; static constexpr int R1 = 8, R2 = 12; };
 
-// Row pitch of a two-factor xy plane in shared memory: congruent to 8 modulo 16 elements, so that
-// the in-row exchange (8 lanes per row, columns rotated by K0) and the column accesses are both
-// free of bank conflicts.
-template <int N> struct TFPitch { static constexpr int value = (N % 16 == 8) ? N : (N % 16 == 0 ? N + 8 : N + 1); };
-
 // A side, forward: v[n1] = x[n0 + R1 n1] -> v[K0] = E[K0][n0].
 template <typename C, int N, bool INV> struct TF;
 template <typename C, int N> struct TF<C, N, false> {
@@ -349,4 +344,131 @@ template <typename C, int N> struct TF<C, N, true> {
   }
   // A side, inverse: v[K0] = E[K0][n0] -> v[n1] = x[n0 + R1 n1].
   __device__ __forceinline__ static void a_side(C* v, int, const C*) { SmallDFT<C, R2, true>::run(v); }
+};
+
+// ---------------------------------------------------------------------------- xy plane in shared memory
+//
+// The x axis of the spectrum is kept in the order in which the in-place exchange leaves it: cell
+// p = K0 R1 + (K1 + K0) mod R1 of a row holds kx = K0 + R2 K1 (kx_at).  Nobody needs the natural
+// order (the z passes take their kx factors in this order and the inverse starts from it), and so
+// the x B side writes back to the cells it read: no barrier, and one item's registers at a time.
+template <int N> __host__ __device__ __forceinline__ int kx_at(int p) {
+  if constexpr (TwoFactor<N>::ok) {
+    constexpr int R1 = TwoFactor<N>::R1, R2 = TwoFactor<N>::R2;
+    const int k0 = p / R1;
+    return k0 + R2 * ((p - k0 * R1 - k0 + 4 * R1) % R1);
+  } else {
+    return p;
+  }
+}
+
+// Threads of the plane passes: warp w owns RPW rows, so that its x items (RPW R1 and RPW R2) fill
+// whole warps (one of 24^2's sides to 75 %) and the x axis needs no CTA barrier, and the y items fill
+// whole CTAs.
+template <int N> struct XYThreads;
+template <> struct XYThreads<96> { static constexpr int value = 384; };
+template <> struct XYThreads<64> { static constexpr int value = 256; };
+template <> struct XYThreads<48> { static constexpr int value = 96; };
+template <> struct XYThreads<32> { static constexpr int value = 128; };
+template <> struct XYThreads<24> { static constexpr int value = 96; };
+template <> struct XYThreads<16> { static constexpr int value = 64; };
+
+// Plane in shared memory with row pitch P.  The 8 cells of a work item and the 8 items of a row touch
+// 64-byte (FP32) blocks; two neighbouring rows must not meet in the same banks.  SWZ (FP32, P a
+// multiple of 16) exchanges neighbouring blocks of 8 cells in odd rows; without it the pitch is
+// congruent to 8 modulo 16.  FP64 blocks are 128 bytes: no conflict at any pitch.
+template <typename C, int N, int P, bool SWZ> struct XYPlane {
+  static constexpr int R1 = TwoFactor<N>::R1, R2 = TwoFactor<N>::R2;
+  static constexpr int NT = XYThreads<N>::value, RPW = N / (NT / 32);
+  static constexpr int XA = RPW * R1 / 32, XB = (RPW * R2 + 31) / 32;  // x passes of a warp
+  static constexpr int YA = N * R1 / NT, YB = (N * R2 + NT - 1) / NT;  // y passes of the CTA
+  static_assert(RPW * (NT / 32) == N && RPW * R1 % 32 == 0 && N * R1 % NT == 0 && 32 % R1 == 0, "whole warps");
+  static_assert(!SWZ || (P % 16 == 0 && R1 % 2 == 0), "swizzle");
+
+  // cell of element j of block k0 (R1 cells) in row y
+  __device__ __forceinline__ static int cell(int y, int k0, int j) {
+    int c = k0 * R1 + ((j + k0) % R1);
+    if constexpr (SWZ) c ^= (y & 1) << 3;
+    return y * P + c;
+  }
+  // cell of column x in row r
+  __device__ __forceinline__ static int col(int r, int x) {
+    if constexpr (SWZ) x ^= (r & 1) << 3;
+    return r * P + x;
+  }
+  // x, A side of one warp: rows from src (global memory, or natural-order rows of pitch SP in this very
+  // buffer), exchange cells out.  A pass covers whole rows, so reading them before the first write
+  // of the pass is enough.
+  template <typename S>
+  __device__ __forceinline__ static void x_a_fwd(C* s, const S* src, int sp, const C* tw, int warp, int lane) {
+#pragma unroll
+    for (int p = 0; p < XA; ++p) {
+      const int i = lane + 32 * p, yl = i / R1, n0 = i - yl * R1, y = warp * RPW + yl;
+      C v[R2];
+#pragma unroll
+      for (int q = 0; q < R2; ++q) v[q] = src[y * sp + n0 + R1 * q];
+      __syncwarp();
+      TF<C, N, false>::a_side(v, n0, tw);
+#pragma unroll
+      for (int k0 = 0; k0 < R2; ++k0) s[cell(y, k0, n0)] = v[k0];
+    }
+  }
+  // x, B side of one warp, in place (forward: E -> X, inverse: X -> E)
+  template <bool INV> __device__ __forceinline__ static void x_b(C* s, const C* tw, int warp, int lane) {
+#pragma unroll
+    for (int p = 0; p < XB; ++p) {
+      const int i = lane + 32 * p;
+      if (RPW * R2 % 32 == 0 || i < RPW * R2) {
+        const int yl = i / R2, k0 = i - yl * R2, y = warp * RPW + yl;
+        C u[R1];
+#pragma unroll
+        for (int j = 0; j < R1; ++j) u[j] = s[cell(y, k0, j)];
+        TF<C, N, INV>::b_side(u, k0, tw);
+#pragma unroll
+        for (int j = 0; j < R1; ++j) s[cell(y, k0, j)] = u[j];
+      }
+    }
+  }
+  // x, A side of one warp, inverse: exchange cells to global rows
+  __device__ __forceinline__ static void x_a_inv(const C* s, C* o, const C* tw, int warp, int lane) {
+#pragma unroll
+    for (int p = 0; p < XA; ++p) {
+      const int i = lane + 32 * p, yl = i / R1, n0 = i - yl * R1, y = warp * RPW + yl;
+      C v[R2];
+#pragma unroll
+      for (int k0 = 0; k0 < R2; ++k0) v[k0] = s[cell(y, k0, n0)];
+      TF<C, N, true>::a_side(v, n0, tw);
+#pragma unroll
+      for (int q = 0; q < R2; ++q) o[y * N + n0 + R1 * q] = v[q];
+    }
+  }
+  // y, A side in place: item (x, n0), x fastest; rows n0 + R1 q and K0 R1 + n0 are the same ones
+  template <bool INV> __device__ __forceinline__ static void y_a(C* s, const C* tw) {
+#pragma unroll
+    for (int p = 0; p < YA; ++p) {
+      const int i = threadIdx.x + p * NT, n0 = i / N, x = i - n0 * N;
+      C v[R2];
+#pragma unroll
+      for (int q = 0; q < R2; ++q) v[q] = s[INV ? col(q * R1 + n0, x) : col(n0 + R1 * q, x)];
+      TF<C, N, INV>::a_side(v, n0, tw);
+#pragma unroll
+      for (int q = 0; q < R2; ++q) s[col(q * R1 + n0, x)] = v[q];
+    }
+  }
+  // y, B side, forward: to global rows
+  __device__ __forceinline__ static void y_b_fwd(const C* s, C* o, const C* tw) {
+#pragma unroll
+    for (int p = 0; p < YB; ++p) {
+      const int i = threadIdx.x + p * NT;
+      if (N * R2 % NT == 0 || i < N * R2) {
+        const int k0 = i / N, x = i - k0 * N;
+        C u[R1];
+#pragma unroll
+        for (int n0 = 0; n0 < R1; ++n0) u[n0] = s[col(k0 * R1 + n0, x)];
+        TF<C, N, false>::b_side(u, k0, tw);
+#pragma unroll
+        for (int k1 = 0; k1 < R1; ++k1) o[(k0 + R2 * k1) * N + x] = u[k1];
+      }
+    }
+  }
 };

@@ -1,7 +1,7 @@
 // xy pass of the kinetic term with its planes brought into shared memory by the bulk
 // asynchronous copy engine (FP32, two-factor sizes).
 //
-// The plain two-factor pass reads its plane from HBM into registers, so the bytes in flight are
+// The register-fed pass reads its plane from HBM into registers, so the bytes in flight are
 // bounded by the warps resident on the SM.  Here each CTA is persistent and double-buffers whole
 // planes: while it transforms plane j in one buffer, the row copies of plane j + grid
 // (`cp.async.bulk`, one 16-byte-aligned row each, completion counted in bytes on an mbarrier)
@@ -38,36 +38,27 @@ __device__ __forceinline__ void issue_rows(const float2* g, size_t stride, float
   for (int row = lane; row < N; row += 32) bulk_copy(buf + row * P, g + (size_t)row * stride, ROW, bar);
 }
 
-// Threads and resident CTAs: 256 threads; the two 36 KB buffers of a 64^2 plane allow three
-// CTAs per SM.  (512 threads at two CTAs per SM, one item per thread and side, were slower:
-// 0.190 against 0.161 ms per pass at 64^3 x 208 components.)  At 96^2 the two 78 KB buffers leave
-// one CTA per SM, and the register-fed pass is faster (7.2 against 9.0 ms per pass at 96^3 x 2048
-// components), so 96 takes that pass.
-template <int N> struct XyTmaThreads { static constexpr int value = 256; };
-template <int N> struct XyTmaBlocks { static constexpr int value = 4; };
+// Row pitch of the two buffers (rows arrive as they are: no swizzle).
+template <int N> struct TmaPitch { static constexpr int value = (N % 16 == 8) ? N : N + 8; };
+
+// Resident CTAs asked of the register allocator; the two 36 KB buffers of a 64^2 plane allow three.
+// At 96^2 the two 78 KB buffers would leave one CTA per SM: 96 takes the register-fed pass.
+template <int N> struct XyTmaBlocks { static constexpr int value = 8; };
 template <> struct XyTmaBlocks<64> { static constexpr int value = 3; };
-template <> struct XyTmaBlocks<48> { static constexpr int value = 3; };
+template <> struct XyTmaBlocks<48> { static constexpr int value = 5; };
 
 }  // namespace
 
-// Barriers.  A stage whose items read and write the same cells (the y A side in both
-// directions, whose rows n0 + R1 q are also its output rows K0 R1 + n0) runs in place without
-// one.  A stage whose items share a row (the x sides) only needs the row's items, which sit on
-// neighbouring lanes of one warp when the item count per row divides 32 and the CTA size.
+// The transform is that of k_fft_xy2 (XYPlane) with its first side reading the buffer in place: the
+// forward x A side rows by warp, the inverse y B side with every read of the plane before the first
+// write.
 template <int N, bool INV>
-__global__ void __launch_bounds__(XyTmaThreads<N>::value, XyTmaBlocks<N>::value)
+__global__ void __launch_bounds__(XYThreads<N>::value, XyTmaBlocks<N>::value)
 k_fft_xy2_tma(const float2* src, float2* dst, const float2* __restrict__ twg, int nplanes, int* err) {
   using C = float2;
-  using T = TF<C, N, INV>;
-  constexpr int NT = XyTmaThreads<N>::value;
-  constexpr int R1 = TwoFactor<N>::R1, R2 = TwoFactor<N>::R2;
-  constexpr int RS = TFPitch<N>::value;
-  constexpr int IA = N * R1, IB = N * R2;
-  constexpr int PA = (IA + NT - 1) / NT, PB = (IB + NT - 1) / NT;
-  constexpr bool ROW1 = (32 % R1 == 0) && (NT % R1 == 0);  // x A-side rows within a warp
-  constexpr bool ROW2 = (32 % R2 == 0) && (NT % R2 == 0);  // x B-side rows within a warp
-  constexpr bool ROW12 = ROW1 && R1 == R2;                 // and on the same lanes for both sides
-  static_assert(ROW1, "R1 divides the warp");
+  constexpr int RS = TmaPitch<N>::value;
+  using PL = XYPlane<C, N, RS, false>;
+  constexpr int R1 = PL::R1, R2 = PL::R2, NT = PL::NT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* tw = reinterpret_cast<C*>(smem_raw);
   C* buf0 = tw + N;
@@ -80,8 +71,6 @@ k_fft_xy2_tma(const float2* src, float2* dst, const float2* __restrict__ twg, in
   __syncthreads();
   int pl = blockIdx.x;
   if (pl < nplanes && warp == 0) issue_rows<N, RS>(src + (size_t)pl * N * N, N, buf0, bar0, lane);
-  C v[PA][R2];
-  C u[PB][R1];
   // Buffer schedule: at the start of plane j the copies of plane j + grid go to the other buffer,
   // whose last reader (plane j - grid) ended with the CTA barrier closing the previous step.
   for (int it = 0; pl < nplanes; ++it, pl += gridDim.x) {
@@ -91,151 +80,43 @@ k_fft_xy2_tma(const float2* src, float2* dst, const float2* __restrict__ twg, in
     if (nx < nplanes && warp == 0) issue_rows<N, RS>(src + (size_t)nx * N * N, N, sb ? buf0 : buf1, sb ? bar0 : bar1, lane);
     bulk_wait(sb ? bar1 : bar0, (uint32_t)(it >> 1) & 1u, err, 2);
     C* o = dst + (size_t)pl * N * N;
-    if (!INV) {
-      // x, A side in place: item (y, n0); a row's items share a warp
-#pragma unroll
-      for (int p = 0; p < PA; ++p) {
-        const int i = threadIdx.x + p * NT;
-        if (IA % NT == 0 || i < IA) {
-          const int y = i / R1, n0 = i - y * R1;
-#pragma unroll
-          for (int q = 0; q < R2; ++q) v[p][q] = s[y * RS + n0 + R1 * q];
-        }
-      }
+    if constexpr (!INV) {
+      PL::x_a_fwd(s, s, RS, tw, warp, lane);
       __syncwarp();
-#pragma unroll
-      for (int p = 0; p < PA; ++p) {
-        const int i = threadIdx.x + p * NT;
-        if (IA % NT == 0 || i < IA) {
-          const int y = i / R1, n0 = i - y * R1;
-          T::a_side(v[p], n0, tw);
-#pragma unroll
-          for (int k0 = 0; k0 < R2; ++k0) s[y * RS + k0 * R1 + (n0 + k0) % R1] = v[p][k0];
-        }
-      }
-      if constexpr (ROW12) __syncwarp(); else __syncthreads();
-      // x, B side: item (y, K0)
-#pragma unroll
-      for (int p = 0; p < PB; ++p) {
-        const int i = threadIdx.x + p * NT;
-        if (IB % NT == 0 || i < IB) {
-          const int y = i / R2, k0 = i - y * R2;
-#pragma unroll
-          for (int n0 = 0; n0 < R1; ++n0) u[p][n0] = s[y * RS + k0 * R1 + (n0 + k0) % R1];
-        }
-      }
-      if constexpr (ROW2) __syncwarp(); else __syncthreads();
-#pragma unroll
-      for (int p = 0; p < PB; ++p) {
-        const int i = threadIdx.x + p * NT;
-        if (IB % NT == 0 || i < IB) {
-          const int y = i / R2, k0 = i - y * R2;
-          T::b_side(u[p], k0, tw);
-#pragma unroll
-          for (int k1 = 0; k1 < R1; ++k1) s[y * RS + k0 + R2 * k1] = u[p][k1];
-        }
-      }
+      PL::template x_b<false>(s, tw, warp, lane);
       __syncthreads();
-      // y, A side in place: item (x, n0)
-#pragma unroll
-      for (int p = 0; p < PA; ++p) {
-        const int i = threadIdx.x + p * NT;
-        if (IA % NT == 0 || i < IA) {
-          const int n0 = i / N, x = i - n0 * N;
-#pragma unroll
-          for (int q = 0; q < R2; ++q) v[p][q] = s[(n0 + R1 * q) * RS + x];
-          T::a_side(v[p], n0, tw);
-#pragma unroll
-          for (int k0 = 0; k0 < R2; ++k0) s[(k0 * R1 + n0) * RS + x] = v[p][k0];
-        }
-      }
+      PL::template y_a<false>(s, tw);
       __syncthreads();
-      // y, B side: item (x, K0) -> HBM
-#pragma unroll
-      for (int p = 0; p < PB; ++p) {
-        const int i = threadIdx.x + p * NT;
-        if (IB % NT == 0 || i < IB) {
-          const int k0 = i / N, x = i - k0 * N;
-#pragma unroll
-          for (int n0 = 0; n0 < R1; ++n0) u[p][n0] = s[(k0 * R1 + n0) * RS + x];
-          T::b_side(u[p], k0, tw);
-#pragma unroll
-          for (int k1 = 0; k1 < R1; ++k1) o[(k0 + R2 * k1) * N + x] = u[p][k1];
-        }
-      }
+      PL::y_b_fwd(s, o, tw);
     } else {
-      // y, B side in place: item (x, K0); a column's items sit in several warps, so every read of
-      // the plane precedes the first write
+      // y, B side in place: item (x, K0)
+      C u[PL::YB][R1];
 #pragma unroll
-      for (int p = 0; p < PB; ++p) {
+      for (int p = 0; p < PL::YB; ++p) {
         const int i = threadIdx.x + p * NT;
-        if (IB % NT == 0 || i < IB) {
+        if (N * R2 % NT == 0 || i < N * R2) {
           const int k0 = i / N, x = i - k0 * N;
 #pragma unroll
-          for (int k1 = 0; k1 < R1; ++k1) u[p][k1] = s[(k0 + R2 * k1) * RS + x];
+          for (int k1 = 0; k1 < R1; ++k1) u[p][k1] = s[PL::col(k0 + R2 * k1, x)];
         }
       }
       __syncthreads();
 #pragma unroll
-      for (int p = 0; p < PB; ++p) {
+      for (int p = 0; p < PL::YB; ++p) {
         const int i = threadIdx.x + p * NT;
-        if (IB % NT == 0 || i < IB) {
+        if (N * R2 % NT == 0 || i < N * R2) {
           const int k0 = i / N, x = i - k0 * N;
-          T::b_side(u[p], k0, tw);
+          TF<C, N, true>::b_side(u[p], k0, tw);
 #pragma unroll
-          for (int n0 = 0; n0 < R1; ++n0) s[(k0 * R1 + n0) * RS + x] = u[p][n0];
+          for (int n0 = 0; n0 < R1; ++n0) s[PL::col(k0 * R1 + n0, x)] = u[p][n0];
         }
       }
       __syncthreads();
-      // y, A side in place: item (x, n0)
-#pragma unroll
-      for (int p = 0; p < PA; ++p) {
-        const int i = threadIdx.x + p * NT;
-        if (IA % NT == 0 || i < IA) {
-          const int n0 = i / N, x = i - n0 * N;
-#pragma unroll
-          for (int k0 = 0; k0 < R2; ++k0) v[p][k0] = s[(k0 * R1 + n0) * RS + x];
-          T::a_side(v[p], n0, tw);
-#pragma unroll
-          for (int n1 = 0; n1 < R2; ++n1) s[(n0 + R1 * n1) * RS + x] = v[p][n1];
-        }
-      }
+      PL::template y_a<true>(s, tw);
       __syncthreads();
-      // x, B side: item (y, K0)
-#pragma unroll
-      for (int p = 0; p < PB; ++p) {
-        const int i = threadIdx.x + p * NT;
-        if (IB % NT == 0 || i < IB) {
-          const int y = i / R2, k0 = i - y * R2;
-#pragma unroll
-          for (int k1 = 0; k1 < R1; ++k1) u[p][k1] = s[y * RS + k0 + R2 * k1];
-        }
-      }
-      if constexpr (ROW2) __syncwarp(); else __syncthreads();
-#pragma unroll
-      for (int p = 0; p < PB; ++p) {
-        const int i = threadIdx.x + p * NT;
-        if (IB % NT == 0 || i < IB) {
-          const int y = i / R2, k0 = i - y * R2;
-          T::b_side(u[p], k0, tw);
-#pragma unroll
-          for (int n0 = 0; n0 < R1; ++n0) s[y * RS + k0 * R1 + (n0 + k0) % R1] = u[p][n0];
-        }
-      }
-      if constexpr (ROW12) __syncwarp(); else __syncthreads();
-      // x, A side -> HBM: item (y, n0)
-#pragma unroll
-      for (int p = 0; p < PA; ++p) {
-        const int i = threadIdx.x + p * NT;
-        if (IA % NT == 0 || i < IA) {
-          const int y = i / R1, n0 = i - y * R1;
-#pragma unroll
-          for (int k0 = 0; k0 < R2; ++k0) v[p][k0] = s[y * RS + k0 * R1 + (n0 + k0) % R1];
-          T::a_side(v[p], n0, tw);
-#pragma unroll
-          for (int n1 = 0; n1 < R2; ++n1) o[y * N + n0 + R1 * n1] = v[p][n1];
-        }
-      }
+      PL::template x_b<true>(s, tw, warp, lane);
+      __syncwarp();
+      PL::x_a_inv(s, o, tw, warp, lane);
     }
     __syncthreads();
   }
@@ -246,7 +127,7 @@ bool fft_xy_tma_supported(int N) { return N == 16 || N == 24 || N == 32 || N == 
 template <int N>
 static cudaError_t xy_tma_n(cudaStream_t st, const void* src, void* dst, int nbatch, const void* tw, bool inv,
                             int* err) {
-  const size_t smem = (size_t)(N + 2 * N * TFPitch<N>::value) * sizeof(float2) + 2 * sizeof(uint64_t);
+  const size_t smem = (size_t)(N + 2 * N * TmaPitch<N>::value) * sizeof(float2) + 2 * sizeof(uint64_t);
   auto kf = inv ? k_fft_xy2_tma<N, true> : k_fft_xy2_tma<N, false>;
   static int per_sm[2] = {0, 0};
   static int sms = 0;
@@ -258,12 +139,12 @@ static cudaError_t xy_tma_n(cudaStream_t st, const void* src, void* dst, int nba
     int dev = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, kf, XyTmaThreads<N>::value, smem)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, kf, XYThreads<N>::value, smem)) != cudaSuccess) return e;
     if (ps < 1) return cudaErrorInvalidConfiguration;
   }
   const int nplanes = N * nbatch;
   const int grid = std::min(nplanes, sms * ps);
-  kf<<<grid, XyTmaThreads<N>::value, smem, st>>>((const float2*)src, (float2*)dst, (const float2*)tw, nplanes, err);
+  kf<<<grid, XYThreads<N>::value, smem, st>>>((const float2*)src, (float2*)dst, (const float2*)tw, nplanes, err);
   return cudaGetLastError();
 }
 

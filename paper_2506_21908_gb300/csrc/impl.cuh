@@ -16,7 +16,7 @@ constexpr int kNumCls = 8;     // profiling classes
 enum KernelClass { KC_FFT_XY = 0, KC_FFT_Z = 1, KC_EPI = 2, KC_PROJ = 3, KC_DENS = 4, KC_POT = 5, KC_OTHER = 6,
                    KC_SCATTER = 7 };
 
-// Multiplier of the z pass: kinetic 1/2|G + s_k|^2 * scale, Poisson 4 pi / G^2 * scale.
+// Multiplier of the z pass: kinetic 1/2|G + s_k|^2 * scale.
 struct ZParams {
   double gs[3];               // 2 pi / L_a
   double scale;
@@ -24,7 +24,7 @@ struct ZParams {
   double shift[kMaxK][3];     // k + A(t) per k-point
 };
 
-enum ZMode { Z_KIN = 0, Z_POISSON = 1, Z_INV_ONLY = 2 };
+enum ZMode { Z_KIN = 0, Z_INV_ONLY = 1 };
 
 // Chebyshev / Taylor epilogue modes.
 enum EpiMode { EPI_APPLY = 0, EPI_FIRST = 1, EPI_RECUR = 2, EPI_TAYLOR = 3, EPI_ADJ = 4, EPI_ADJ0 = 5 };
@@ -116,6 +116,7 @@ template <typename R> struct ProjTables {
 __host__ __device__ constexpr int beta_pitch(int nlm) { return nlm == 1 ? 1 : (nlm + 1) / 2 * 2; }
 
 // ---------------------------------------------------------------- launchers
+// xy transform of every plane; the x axis of the transform is in the order kx_at (fft.cuh).
 template <typename R>
 cudaError_t launch_fft_xy(cudaStream_t st, int N, const void* src, void* dst, int nbatch, const void* tw, bool inv);
 // FP32 xy pass over persistent CTAs whose planes arrive by bulk asynchronous copies into
@@ -124,9 +125,13 @@ cudaError_t launch_fft_xy(cudaStream_t st, int N, const void* src, void* dst, in
 bool fft_xy_tma_supported(int N);
 cudaError_t launch_fft_xy_tma(cudaStream_t st, int N, const void* src, void* dst, int nbatch, const void* tw, bool inv,
                               int* err);
+// z transform, multiplication by the kinetic factors, inverse z transform in place.  tab: the tables
+// of launch_kin_tables for these k-points and A (3 nk N reals; unused at n = 8 and 12).
 template <typename R>
-cudaError_t launch_fft_z(cudaStream_t st, int N, void* data, int nbatch, const void* tw, int mode,
-                         const ZParams& zp);
+cudaError_t launch_fft_z_kinetic(cudaStream_t st, int N, void* data, int nbatch, const void* tw, const void* tab,
+                                 const ZParams& zp);
+template <typename R> cudaError_t launch_kin_tables(cudaStream_t st, int N, int nk, const ZParams& zp, void* out);
+cudaError_t launch_fft_z_inverse(cudaStream_t st, int N, double2* data, int nbatch, const double2* tw);
 // out[k][e] = exp(i shift_k.d_e) from the compact rows; beta tables [entries][beta_pitch(nlm)], the
 // entries of atom a at g_ptr[a] (atom == null) or with their atom listed (scatter order).
 template <typename R>

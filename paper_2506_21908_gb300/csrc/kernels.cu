@@ -1,8 +1,8 @@
 // sm_103a kernels of the spinor propagation step.
 //
 //   k_fft_xy     one z-plane of one spinor component: 2D FFT along x then y in shared memory
-//   k_fft_z      one y-slab of one component: FFT along z, multiply (kinetic 1/2|G+k+A|^2 or
-//                Poisson 4 pi / G^2), inverse FFT along z -- the kinetic term of Eq. HNC-SDFT
+//   k_fft_z      one y-slab of one component: FFT along z, multiply by 1/2|G+k+A|^2, inverse FFT
+//                along z -- the kinetic term of Eq. HNC-SDFT
 //   k_proj_gather  c_{a,p,sigma} = sum_{r in S_a} beta~_p(r)^* psi_sigma(r) dV and D_a c
 //                (the contraction of the separable projectors, Eq. Vps with the L.S block)
 //   (k_epilogue, the pointwise Hamiltonian and Chebyshev update, is in epilogue.cu)
@@ -10,6 +10,7 @@
 //   k_potential  locally collinear LSDA (Eqs. LC+ALDA2, LC+ALDA) and assembly of V_v
 //   reductions   deterministic fixed-order block reductions for energies and norms
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
 
 #include "fft.cuh"
@@ -43,28 +44,17 @@ k_fft_xy(const typename CT<R>::type* src, typename CT<R>::type* dst, const typen
 
 // Per-axis multiplier tables for the z pass: the kinetic factor 1/2 |G + s|^2 scale is
 // tx[x] + ty[y] + tz[z] with ta[i] = 1/2 (g_a f(i) + s_a)^2 scale (computed in FP64, stored in R).
-template <typename R, int N, int MODE>
+template <typename R, int N>
 __device__ __forceinline__ void z_tables(R* tx, R* tz, R* ty, const ZParams& zp, int y, int k) {
   for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    if (MODE == Z_KIN) {
-      const double qx = zp.gs[0] * freq<N>(i) + zp.shift[k][0];
-      const double qz = zp.gs[2] * freq<N>(i) + zp.shift[k][2];
-      tx[i] = (R)(0.5 * qx * qx * zp.scale);
-      tz[i] = (R)(0.5 * qz * qz * zp.scale);
-    } else {
-      const double gx = zp.gs[0] * freq<N>(i), gz = zp.gs[2] * freq<N>(i);
-      tx[i] = (R)(gx * gx);
-      tz[i] = (R)(gz * gz);
-    }
+    const double qx = zp.gs[0] * freq<N>(i) + zp.shift[k][0];
+    const double qz = zp.gs[2] * freq<N>(i) + zp.shift[k][2];
+    tx[i] = (R)(0.5 * qx * qx * zp.scale);
+    tz[i] = (R)(0.5 * qz * qz * zp.scale);
   }
   if (threadIdx.x == 0) {
-    if (MODE == Z_KIN) {
-      const double qy = zp.gs[1] * freq<N>(y) + zp.shift[k][1];
-      *ty = (R)(0.5 * qy * qy * zp.scale);
-    } else {
-      const double gy = zp.gs[1] * freq<N>(y);
-      *ty = (R)(gy * gy);
-    }
+    const double qy = zp.gs[1] * freq<N>(y) + zp.shift[k][1];
+    *ty = (R)(0.5 * qy * qy * zp.scale);
   }
 }
 
@@ -85,7 +75,7 @@ k_fft_z(typename CT<R>::type* __restrict__ data, const typename CT<R>::type* __r
   const int b = blockIdx.y;
   const size_t base = (size_t)b * N * N * N + (size_t)y * N;
   for (int i = threadIdx.x; i < N; i += NT) tw[i] = twg[i];
-  if (MODE != Z_INV_ONLY) z_tables<R, N, MODE>(tx, tz, ty, zp, y, (MODE == Z_KIN) ? b / zp.comps_per_k : 0);
+  if (MODE != Z_INV_ONLY) z_tables<R, N>(tx, tz, ty, zp, y, b / zp.comps_per_k);
   slab_load<N, NT, RS>(s, data + base, (size_t)N * N);
   __syncthreads();
   if (MODE != Z_INV_ONLY) {
@@ -93,14 +83,7 @@ k_fft_z(typename CT<R>::type* __restrict__ data, const typename CT<R>::type* __r
     const R tyv = *ty;
     for (int i = threadIdx.x; i < N * N; i += NT) {
       const int z = i / N, x = i - z * N;
-      R m;
-      if (MODE == Z_KIN) {
-        m = tx[x] + tyv + tz[z];
-      } else {
-        const double g2 = (double)tx[x] + (double)tyv + (double)tz[z];
-        m = (R)(g2 > 0.0 ? 4.0 * 3.14159265358979323846 / g2 * zp.scale : 0.0);
-      }
-      s[z * RS + x] = cscale(s[z * RS + x], m);
+      s[z * RS + x] = cscale(s[z * RS + x], tx[x] + tyv + tz[z]);
     }
     __syncthreads();
   }
@@ -110,230 +93,158 @@ k_fft_z(typename CT<R>::type* __restrict__ data, const typename CT<R>::type* __r
 
 // ---------------------------------------------------------------- two-factor passes (N = R1 R2)
 
+// Resident CTAs per SM asked of the register allocator (FP32; what the dense planes and slabs
+// allow).  FP64 is bound by its arithmetic and keeps its registers.
+template <typename R, int N> struct XYBlocks { static constexpr int value = 1; };
+template <> struct XYBlocks<float, 96> { static constexpr int value = 3; };
+template <> struct XYBlocks<float, 64> { static constexpr int value = 5; };
+template <> struct XYBlocks<float, 48> { static constexpr int value = 10; };
+template <> struct XYBlocks<float, 32> { static constexpr int value = 8; };
+template <> struct XYBlocks<float, 24> { static constexpr int value = 10; };
+template <> struct XYBlocks<float, 16> { static constexpr int value = 16; };
+
 // xy transform of one z-plane with one shared-memory exchange per axis: the x transform's A side
 // reads global memory directly, the y transform's B side writes it directly (forward); the
-// inverse runs the steps in the opposite order.  Column of the in-row exchange: K0 R1 + (n0 +
-// K0) mod R1 (a rotation, so that the 8 lanes of a row hit distinct banks on both sides).
-// Barriers: the y A side reads and writes the same rows of its item (n0 + R1 q = K0 R1 + n0)
-// and runs in place without one; the x sides touch one row per item group, whose items sit on
-// neighbouring lanes of a warp when their count divides 32, so a warp barrier orders them.
+// inverse runs the steps in the opposite order.  The x axis is warp-local and in place (XYPlane), so
+// two CTA barriers remain, and the dense swizzled plane lets three CTAs of 96^2 share an SM.
 template <typename R, int N, bool INV>
-__global__ void __launch_bounds__(FFTThreads<N>::value, FFTMinBlocks<R, N>::value)
+__global__ void __launch_bounds__(XYThreads<N>::value, XYBlocks<R, N>::value)
 k_fft_xy2(const typename CT<R>::type* src, typename CT<R>::type* dst, const typename CT<R>::type* __restrict__ twg) {
   using C = typename CT<R>::type;
-  using T = TF<C, N, INV>;
-  constexpr int NT = FFTThreads<N>::value;
-  constexpr int R1 = TwoFactor<N>::R1, R2 = TwoFactor<N>::R2;
-  constexpr int RS = TFPitch<N>::value;
-  constexpr int IA = N * R1, IB = N * R2;                 // A / B items of one axis
-  constexpr int PA = (IA + NT - 1) / NT, PB = (IB + NT - 1) / NT;
-  constexpr bool ROW1 = (32 % R1 == 0) && (NT % R1 == 0);  // x A-side rows within a warp
-  constexpr bool ROW2 = (32 % R2 == 0) && (NT % R2 == 0);  // x B-side rows within a warp
-  constexpr bool ROW12 = ROW1 && R1 == R2;                 // and on the same lanes for both sides
+  using PL = XYPlane<C, N, N, sizeof(R) == 4 && N % 16 == 0>;
+  constexpr int R1 = PL::R1, R2 = PL::R2, NT = PL::NT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* tw = reinterpret_cast<C*>(smem_raw);
   C* s = tw + N;
   const size_t base = ((size_t)blockIdx.y * N + blockIdx.x) * (size_t)(N * N);
   const C* g = src + base;
   C* o = dst + base;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int i = threadIdx.x; i < N; i += NT) tw[i] = twg[i];
   __syncthreads();
-  C v[PA][R2];
-  C u[PB][R1];
-  if (!INV) {
-    // x, A side: item (y, n0), n0 fastest
-#pragma unroll
-    for (int p = 0; p < PA; ++p) {
-      const int i = threadIdx.x + p * NT;
-      if (IA % NT == 0 || i < IA) {
-        const int y = i / R1, n0 = i - y * R1;
-#pragma unroll
-        for (int q = 0; q < R2; ++q) v[p][q] = g[y * N + n0 + R1 * q];
-        T::a_side(v[p], n0, tw);
-#pragma unroll
-        for (int k0 = 0; k0 < R2; ++k0) s[y * RS + k0 * R1 + (n0 + k0) % R1] = v[p][k0];
-      }
-    }
-    if constexpr (ROW12) __syncwarp(); else __syncthreads();
-    // x, B side: item (y, K0)
-#pragma unroll
-    for (int p = 0; p < PB; ++p) {
-      const int i = threadIdx.x + p * NT;
-      if (IB % NT == 0 || i < IB) {
-        const int y = i / R2, k0 = i - y * R2;
-#pragma unroll
-        for (int n0 = 0; n0 < R1; ++n0) u[p][n0] = s[y * RS + k0 * R1 + (n0 + k0) % R1];
-      }
-    }
-    if constexpr (ROW2) __syncwarp(); else __syncthreads();
-#pragma unroll
-    for (int p = 0; p < PB; ++p) {
-      const int i = threadIdx.x + p * NT;
-      if (IB % NT == 0 || i < IB) {
-        const int y = i / R2, k0 = i - y * R2;
-        T::b_side(u[p], k0, tw);
-#pragma unroll
-        for (int k1 = 0; k1 < R1; ++k1) s[y * RS + k0 + R2 * k1] = u[p][k1];
-      }
-    }
+  if constexpr (!INV) {
+    PL::x_a_fwd(s, g, N, tw, warp, lane);
+    __syncwarp();
+    PL::template x_b<false>(s, tw, warp, lane);
     __syncthreads();
-    // y, A side in place: item (x, n0), x fastest; rows n0 + R1 q in, K0 R1 + n0 out (the same)
-#pragma unroll
-    for (int p = 0; p < PA; ++p) {
-      const int i = threadIdx.x + p * NT;
-      if (IA % NT == 0 || i < IA) {
-        const int n0 = i / N, x = i - n0 * N;
-#pragma unroll
-        for (int q = 0; q < R2; ++q) v[p][q] = s[(n0 + R1 * q) * RS + x];
-        T::a_side(v[p], n0, tw);
-#pragma unroll
-        for (int k0 = 0; k0 < R2; ++k0) s[(k0 * R1 + n0) * RS + x] = v[p][k0];
-      }
-    }
+    PL::template y_a<false>(s, tw);
     __syncthreads();
-    // y, B side: item (x, K0) -> global
-#pragma unroll
-    for (int p = 0; p < PB; ++p) {
-      const int i = threadIdx.x + p * NT;
-      if (IB % NT == 0 || i < IB) {
-        const int k0 = i / N, x = i - k0 * N;
-#pragma unroll
-        for (int n0 = 0; n0 < R1; ++n0) u[p][n0] = s[(k0 * R1 + n0) * RS + x];
-        T::b_side(u[p], k0, tw);
-#pragma unroll
-        for (int k1 = 0; k1 < R1; ++k1) o[(k0 + R2 * k1) * N + x] = u[p][k1];
-      }
-    }
+    PL::y_b_fwd(s, o, tw);
   } else {
     // y, B side from global: item (x, K0)
 #pragma unroll
-    for (int p = 0; p < PB; ++p) {
+    for (int p = 0; p < PL::YB; ++p) {
       const int i = threadIdx.x + p * NT;
-      if (IB % NT == 0 || i < IB) {
+      if (N * R2 % NT == 0 || i < N * R2) {
         const int k0 = i / N, x = i - k0 * N;
+        C u[R1];
 #pragma unroll
-        for (int k1 = 0; k1 < R1; ++k1) u[p][k1] = g[(k0 + R2 * k1) * N + x];
-        T::b_side(u[p], k0, tw);
+        for (int k1 = 0; k1 < R1; ++k1) u[k1] = g[(k0 + R2 * k1) * N + x];
+        TF<C, N, true>::b_side(u, k0, tw);
 #pragma unroll
-        for (int n0 = 0; n0 < R1; ++n0) s[(k0 * R1 + n0) * RS + x] = u[p][n0];
+        for (int n0 = 0; n0 < R1; ++n0) s[PL::col(k0 * R1 + n0, x)] = u[n0];
       }
     }
     __syncthreads();
-    // y, A side in place: item (x, n0)
-#pragma unroll
-    for (int p = 0; p < PA; ++p) {
-      const int i = threadIdx.x + p * NT;
-      if (IA % NT == 0 || i < IA) {
-        const int n0 = i / N, x = i - n0 * N;
-#pragma unroll
-        for (int k0 = 0; k0 < R2; ++k0) v[p][k0] = s[(k0 * R1 + n0) * RS + x];
-        T::a_side(v[p], n0, tw);
-#pragma unroll
-        for (int n1 = 0; n1 < R2; ++n1) s[(n0 + R1 * n1) * RS + x] = v[p][n1];
-      }
-    }
+    PL::template y_a<true>(s, tw);
     __syncthreads();
-    // x, B side: item (y, K0)
-#pragma unroll
-    for (int p = 0; p < PB; ++p) {
-      const int i = threadIdx.x + p * NT;
-      if (IB % NT == 0 || i < IB) {
-        const int y = i / R2, k0 = i - y * R2;
-#pragma unroll
-        for (int k1 = 0; k1 < R1; ++k1) u[p][k1] = s[y * RS + k0 + R2 * k1];
-      }
-    }
-    if constexpr (ROW2) __syncwarp(); else __syncthreads();
-#pragma unroll
-    for (int p = 0; p < PB; ++p) {
-      const int i = threadIdx.x + p * NT;
-      if (IB % NT == 0 || i < IB) {
-        const int y = i / R2, k0 = i - y * R2;
-        T::b_side(u[p], k0, tw);
-#pragma unroll
-        for (int n0 = 0; n0 < R1; ++n0) s[y * RS + k0 * R1 + (n0 + k0) % R1] = u[p][n0];
-      }
-    }
-    if constexpr (ROW12) __syncwarp(); else __syncthreads();
-    // x, A side -> global: item (y, n0)
-#pragma unroll
-    for (int p = 0; p < PA; ++p) {
-      const int i = threadIdx.x + p * NT;
-      if (IA % NT == 0 || i < IA) {
-        const int y = i / R1, n0 = i - y * R1;
-#pragma unroll
-        for (int k0 = 0; k0 < R2; ++k0) v[p][k0] = s[y * RS + k0 * R1 + (n0 + k0) % R1];
-        T::a_side(v[p], n0, tw);
-#pragma unroll
-        for (int n1 = 0; n1 < R2; ++n1) o[y * N + n0 + R1 * n1] = v[p][n1];
-      }
-    }
+    PL::template x_b<true>(s, tw, warp, lane);
+    __syncwarp();
+    PL::x_a_inv(s, o, tw, warp, lane);
   }
 }
 
-// z transform + kinetic multiply + inverse z transform of one y-slab, one exchange each way:
-// A side (x, n0) reads global memory along z, B side (x, K0) transforms, multiplies by
-// tx[x] + ty + tz[kz] and transforms back in registers, A side writes global memory.
+// Columns, threads and CTAs per SM of the z pass: a column's transform touches no other column, so a
+// CTA takes 32 columns (16, 24 or 48 at those sizes), few enough threads that the barriers of one
+// CTA leave the others of the SM running.
+template <int N> struct ZCols { static constexpr int value = N % 32 == 0 ? 32 : N; };
+template <int N> struct ZThreads { static constexpr int value = N % 32 == 0 ? 128 : (N == 16 ? 64 : 96); };
+template <typename R, int N> struct ZBlocks { static constexpr int value = 1; };
+template <> struct ZBlocks<float, 96> { static constexpr int value = 7; };
+template <> struct ZBlocks<float, 64> { static constexpr int value = 8; };
+template <> struct ZBlocks<float, 48> { static constexpr int value = 8; };
+template <> struct ZBlocks<float, 32> { static constexpr int value = 8; };
+template <> struct ZBlocks<float, 24> { static constexpr int value = 8; };
+template <> struct ZBlocks<float, 16> { static constexpr int value = 16; };
+
+// Kinetic factors 1/2 (g_a f + s_a)^2 scale of every k-point, per axis in the order of the passes (x by
+// kx_at), [nk][3][N]: formed in FP64 once per A(t) (a CTA forming its own spent an eighth of the
+// FP64 pipe on them).
 template <typename R, int N>
-__global__ void __launch_bounds__(FFTThreads<N>::value, FFTMinBlocks<R, N>::value)
-k_fft_z2_kin(typename CT<R>::type* __restrict__ data, const typename CT<R>::type* __restrict__ twg, ZParams zp) {
+__global__ void k_kin_tables(ZParams zp, R* __restrict__ out) {
+  const int k = blockIdx.x;
+  for (int i = threadIdx.x; i < 3 * N; i += blockDim.x) {
+    const int a = i / N, j = i - a * N;
+    const double q = zp.gs[a] * freq<N>(a == 0 ? kx_at<N>(j) : j) + zp.shift[k][a];
+    out[(size_t)k * 3 * N + i] = (R)(0.5 * q * q * zp.scale);
+  }
+}
+
+// z transform + kinetic multiply + inverse z transform of one slab (y, columns), one exchange each
+// way: A side (x, n0) reads global memory along z, B side (x, K0) transforms, multiplies by
+// tx[x] + ty[y] + tz[kz] and transforms back in registers, A side writes global memory.
+template <typename R, int N>
+__global__ void __launch_bounds__(ZThreads<N>::value, ZBlocks<R, N>::value)
+k_fft_z2_kin(typename CT<R>::type* __restrict__ data, const typename CT<R>::type* __restrict__ twg,
+             const R* __restrict__ tab, int comps_per_k) {
   using C = typename CT<R>::type;
   using TFW = TF<C, N, false>;
   using TIN = TF<C, N, true>;
-  constexpr int NT = FFTThreads<N>::value;
+  constexpr int NT = ZThreads<N>::value, CW = ZCols<N>::value;
   constexpr int R1 = TwoFactor<N>::R1, R2 = TwoFactor<N>::R2;
-  constexpr int IA = N * R1, IB = N * R2;
+  constexpr int IA = CW * R1, IB = CW * R2;
   constexpr int PA = (IA + NT - 1) / NT, PB = (IB + NT - 1) / NT;
+  __shared__ C tw[N];
+  __shared__ R tz[N];
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* tw = reinterpret_cast<C*>(smem_raw);
-  C* s = tw + N;                                  // [K0 R1 + n0][x], dense
-  R* tx = reinterpret_cast<R*>(s + N * N);
-  R* tz = tx + N;
-  R* ty = tz + N;
-  const int y = blockIdx.x;
+  C* s = reinterpret_cast<C*>(smem_raw);          // [K0 R1 + n0][x], dense
+  const int y = blockIdx.x / (N / CW), x0 = (blockIdx.x - y * (N / CW)) * CW;
   const int b = blockIdx.y;
-  C* g = data + (size_t)b * N * N * N + (size_t)y * N;
+  C* g = data + (size_t)b * N * N * N + (size_t)y * N + x0;
   constexpr size_t ZS = (size_t)N * N;
-  for (int i = threadIdx.x; i < N; i += NT) tw[i] = twg[i];
-  z_tables<R, N, Z_KIN>(tx, tz, ty, zp, y, b / zp.comps_per_k);
   C v[PA][R2];
 #pragma unroll
   for (int p = 0; p < PA; ++p) {
     const int i = threadIdx.x + p * NT;
     if (IA % NT == 0 || i < IA) {
-      const int n0 = i / N, x = i - n0 * N;
+      const int n0 = i / CW, x = i - n0 * CW;
 #pragma unroll
       for (int q = 0; q < R2; ++q) v[p][q] = g[(size_t)(n0 + R1 * q) * ZS + x];
     }
   }
+  const R* tk = tab + (size_t)(b / comps_per_k) * 3 * N;
+  for (int i = threadIdx.x; i < N; i += NT) {
+    tw[i] = twg[i];
+    tz[i] = tk[2 * N + i];
+  }
+  const R tyv = tk[N + y];
   __syncthreads();  // tables
 #pragma unroll
   for (int p = 0; p < PA; ++p) {
     const int i = threadIdx.x + p * NT;
     if (IA % NT == 0 || i < IA) {
-      const int n0 = i / N, x = i - n0 * N;
+      const int n0 = i / CW, x = i - n0 * CW;
       TFW::a_side(v[p], n0, tw);
 #pragma unroll
-      for (int k0 = 0; k0 < R2; ++k0) s[(k0 * R1 + n0) * N + x] = v[p][k0];
+      for (int k0 = 0; k0 < R2; ++k0) s[(k0 * R1 + n0) * CW + x] = v[p][k0];
     }
   }
   __syncthreads();
-  const R tyv = *ty;
 #pragma unroll
   for (int p = 0; p < PB; ++p) {
     const int i = threadIdx.x + p * NT;
     if (IB % NT == 0 || i < IB) {
-      const int k0 = i / N, x = i - k0 * N;
+      const int k0 = i / CW, x = i - k0 * CW;
       C u[R1];
 #pragma unroll
-      for (int n0 = 0; n0 < R1; ++n0) u[n0] = s[(k0 * R1 + n0) * N + x];
+      for (int n0 = 0; n0 < R1; ++n0) u[n0] = s[(k0 * R1 + n0) * CW + x];
       TFW::b_side(u, k0, tw);
-      const R txy = tx[x] + tyv;
+      const R txy = tk[x0 + x] + tyv;
 #pragma unroll
       for (int k1 = 0; k1 < R1; ++k1) u[k1] = cscale(u[k1], txy + tz[k0 + R2 * k1]);
       TIN::b_side(u, k0, tw);
 #pragma unroll
-      for (int n0 = 0; n0 < R1; ++n0) s[(k0 * R1 + n0) * N + x] = u[n0];
+      for (int n0 = 0; n0 < R1; ++n0) s[(k0 * R1 + n0) * CW + x] = u[n0];
     }
   }
   __syncthreads();
@@ -341,78 +252,93 @@ k_fft_z2_kin(typename CT<R>::type* __restrict__ data, const typename CT<R>::type
   for (int p = 0; p < PA; ++p) {
     const int i = threadIdx.x + p * NT;
     if (IA % NT == 0 || i < IA) {
-      const int n0 = i / N, x = i - n0 * N;
+      const int n0 = i / CW, x = i - n0 * CW;
+      C w[R2];
 #pragma unroll
-      for (int k0 = 0; k0 < R2; ++k0) v[p][k0] = s[(k0 * R1 + n0) * N + x];
-      TIN::a_side(v[p], n0, tw);
+      for (int k0 = 0; k0 < R2; ++k0) w[k0] = s[(k0 * R1 + n0) * CW + x];
+      TIN::a_side(w, n0, tw);
 #pragma unroll
-      for (int n1 = 0; n1 < R2; ++n1) g[(size_t)(n0 + R1 * n1) * ZS + x] = v[p][n1];
+      for (int n1 = 0; n1 < R2; ++n1) g[(size_t)(n0 + R1 * n1) * ZS + x] = w[n1];
     }
   }
 }
 
-template <typename R, int N>
-static cudaError_t fft_xy_n(cudaStream_t st, const void* src, void* data, int nbatch, const void* tw, bool inv) {
+// Opt in to a kernel's dynamic shared memory, once per device (the attribute calls cost more host time
+// than the launch).
+template <typename K> static cudaError_t opt_in_smem(K kf, size_t smem, std::atomic<unsigned long long>& done) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned long long bit = 1ull << (dev & 63);
+  if (done.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+  if ((e = cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(kf, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
+  return e;
+}
+
+template <typename R, int N, bool INV>
+static cudaError_t fft_xy_ni(cudaStream_t st, const void* src, void* data, int nbatch, const void* tw) {
   using C = typename CT<R>::type;
-  dim3 grid(N, nbatch);
+  static std::atomic<unsigned long long> done{0};
+  cudaError_t e;
   if constexpr (TwoFactor<N>::ok) {
-    const size_t smem2 = (size_t)(N + N * TFPitch<N>::value) * sizeof(C);
-    auto kf = inv ? k_fft_xy2<R, N, true> : k_fft_xy2<R, N, false>;
-    cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
-    cudaFuncSetAttribute(kf, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-    kf<<<grid, FFTThreads<N>::value, smem2, st>>>((const C*)src, (C*)data, (const C*)tw);
-    return cudaGetLastError();
-  }
-  const size_t smem = (size_t)(N + N * (N + 1)) * sizeof(C);
-  if (inv) {
-    auto kf = k_fft_xy<R, N, true>;
-    cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(kf, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-    kf<<<grid, FFTThreads<N>::value, smem, st>>>((const C*)src, (C*)data, (const C*)tw);
+    const size_t smem = (size_t)(N + N * N) * sizeof(C);
+    auto kf = k_fft_xy2<R, N, INV>;
+    if ((e = opt_in_smem(kf, smem, done)) != cudaSuccess) return e;
+    kf<<<dim3(N, nbatch), XYThreads<N>::value, smem, st>>>((const C*)src, (C*)data, (const C*)tw);
   } else {
-    auto kf = k_fft_xy<R, N, false>;
-    cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(kf, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-    kf<<<grid, FFTThreads<N>::value, smem, st>>>((const C*)src, (C*)data, (const C*)tw);
+    const size_t smem = (size_t)(N + N * (N + 1)) * sizeof(C);
+    auto kf = k_fft_xy<R, N, INV>;
+    if ((e = opt_in_smem(kf, smem, done)) != cudaSuccess) return e;
+    kf<<<dim3(N, nbatch), FFTThreads<N>::value, smem, st>>>((const C*)src, (C*)data, (const C*)tw);
   }
   return cudaGetLastError();
+}
+template <typename R, int N>
+static cudaError_t fft_xy_n(cudaStream_t st, const void* src, void* data, int nbatch, const void* tw, bool inv) {
+  return inv ? fft_xy_ni<R, N, true>(st, src, data, nbatch, tw) : fft_xy_ni<R, N, false>(st, src, data, nbatch, tw);
 }
 
 template <typename R, int N, int MODE>
-static cudaError_t fft_z_nm(cudaStream_t st, void* data, int nbatch, const void* tw, const ZParams& zp) {
+static cudaError_t fft_z_nm(cudaStream_t st, void* data, int nbatch, const void* tw, const void* tab, const ZParams& zp) {
   using C = typename CT<R>::type;
-  const size_t smem = (size_t)(N + N * N) * sizeof(C) + (2 * N + 2) * sizeof(R);
+  static std::atomic<unsigned long long> done{0};
+  cudaError_t e;
   if constexpr (MODE == Z_KIN && TwoFactor<N>::ok) {
+    constexpr int CW = ZCols<N>::value;
+    const size_t smem = (size_t)N * CW * sizeof(C);
     auto kf = k_fft_z2_kin<R, N>;
-    cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(kf, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+    if ((e = opt_in_smem(kf, smem, done)) != cudaSuccess) return e;
+    kf<<<dim3(N * (N / CW), nbatch), ZThreads<N>::value, smem, st>>>((C*)data, (const C*)tw, (const R*)tab, zp.comps_per_k);
+  } else {
+    const size_t smem = (size_t)(N + N * N) * sizeof(C) + (2 * N + 2) * sizeof(R);
+    auto kf = k_fft_z<R, N, MODE>;
+    if ((e = opt_in_smem(kf, smem, done)) != cudaSuccess) return e;
     kf<<<dim3(N, nbatch), FFTThreads<N>::value, smem, st>>>((C*)data, (const C*)tw, zp);
-    return cudaGetLastError();
   }
-  auto kf = k_fft_z<R, N, MODE>;
-  cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  cudaFuncSetAttribute(kf, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-  kf<<<dim3(N, nbatch), FFTThreads<N>::value, smem, st>>>((C*)data, (const C*)tw, zp);
   return cudaGetLastError();
 }
-
-template <typename R, int N>
-static cudaError_t fft_z_n(cudaStream_t st, void* data, int nbatch, const void* tw, int mode, const ZParams& zp) {
-  switch (mode) {
-    case Z_KIN: return fft_z_nm<R, N, Z_KIN>(st, data, nbatch, tw, zp);
-    case Z_POISSON: return fft_z_nm<R, N, Z_POISSON>(st, data, nbatch, tw, zp);
-    default: return fft_z_nm<R, N, Z_INV_ONLY>(st, data, nbatch, tw, zp);
-  }
-}
-
 
 template <typename R>
 cudaError_t launch_fft_xy(cudaStream_t st, int N, const void* src, void* data, int nbatch, const void* tw, bool inv) {
   TDDFT_DISPATCH_N(N, (fft_xy_n<R, NN>(st, src, data, nbatch, tw, inv)));
 }
 template <typename R>
-cudaError_t launch_fft_z(cudaStream_t st, int N, void* data, int nbatch, const void* tw, int mode, const ZParams& zp) {
-  TDDFT_DISPATCH_N(N, (fft_z_n<R, NN>(st, data, nbatch, tw, mode, zp)));
+cudaError_t launch_fft_z_kinetic(cudaStream_t st, int N, void* data, int nbatch, const void* tw, const void* tab,
+                                 const ZParams& zp) {
+  TDDFT_DISPATCH_N(N, (fft_z_nm<R, NN, Z_KIN>(st, data, nbatch, tw, tab, zp)));
+}
+cudaError_t launch_fft_z_inverse(cudaStream_t st, int N, double2* data, int nbatch, const double2* tw) {
+  const ZParams zp{};
+  TDDFT_DISPATCH_N(N, (fft_z_nm<double, NN, Z_INV_ONLY>(st, data, nbatch, tw, nullptr, zp)));
+}
+template <typename R, int N> static cudaError_t kin_tables_n(cudaStream_t st, int nk, const ZParams& zp, void* out) {
+  k_kin_tables<R, N><<<nk, 128, 0, st>>>(zp, (R*)out);
+  return cudaGetLastError();
+}
+template <typename R> cudaError_t launch_kin_tables(cudaStream_t st, int N, int nk, const ZParams& zp, void* out) {
+  TDDFT_DISPATCH_N(N, (kin_tables_n<R, NN>(st, nk, zp, out)));
 }
 
 // ============================================================================ projectors
@@ -867,14 +793,14 @@ cudaError_t launch_complex_real_part(cudaStream_t st, size_t N3, const double2* 
 }
 
 // V_loc(G) = sum_a [-4 pi Z / G^2 exp(-G^2 rc^2 / 4) exp(-i G.R_a)] / Omega, G = 0: sum_a pi Z rc^2 / Omega.
-__global__ void k_vloc_G(int N, double gx0, double gy0, double gz0, int natoms, const double* __restrict__ pos,
+template <int N>
+__global__ void k_vloc_G(double gx0, double gy0, double gz0, int natoms, const double* __restrict__ pos,
                          const double* __restrict__ Zr, double omega, double2* __restrict__ out) {
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   const size_t N3 = (size_t)N * N * N;
   if (i >= N3) return;
   const int x = (int)(i % N), y = (int)((i / N) % N), z = (int)(i / ((size_t)N * N));
-  auto fq = [N](int j) { return j < N / 2 ? j : j - N; };
-  const double gx = gx0 * fq(x), gy = gy0 * fq(y), gz = gz0 * fq(z);
+  const double gx = gx0 * freq<N>(kx_at<N>(x)), gy = gy0 * freq<N>(y), gz = gz0 * freq<N>(z);  // order of the xy pass
   const double g2 = gx * gx + gy * gy + gz * gz;
   const double kPi = 3.14159265358979323846;
   double re = 0.0, im = 0.0;
@@ -888,13 +814,17 @@ __global__ void k_vloc_G(int N, double gx0, double gy0, double gz0, int natoms, 
   }
   out[i] = make_double2(re / omega, im / omega);
 }
+template <int N>
+static cudaError_t vloc_G_n(cudaStream_t st, const double* L, int natoms, const double* pos, const double* Zr,
+                            double omega, double2* out) {
+  const double kPi = 3.14159265358979323846;
+  k_vloc_G<N><<<(unsigned)(((size_t)N * N * N + 255) / 256), 256, 0, st>>>(2 * kPi / L[0], 2 * kPi / L[1], 2 * kPi / L[2],
+                                                                           natoms, pos, Zr, omega, out);
+  return cudaGetLastError();
+}
 cudaError_t launch_vloc_G(cudaStream_t st, int N, const double* L, int natoms, const double* pos, const double* Zr,
                           double omega, double2* out) {
-  const size_t N3 = (size_t)N * N * N;
-  const double kPi = 3.14159265358979323846;
-  k_vloc_G<<<(unsigned)((N3 + 255) / 256), 256, 0, st>>>(N, 2 * kPi / L[0], 2 * kPi / L[1], 2 * kPi / L[2], natoms,
-                                                         pos, Zr, omega, out);
-  return cudaGetLastError();
+  TDDFT_DISPATCH_N(N, (vloc_G_n<NN>(st, L, natoms, pos, Zr, omega, out)));
 }
 
 // ============================================================================ conversions
@@ -1379,7 +1309,9 @@ cudaError_t launch_atom_sums(cudaStream_t st, size_t N3, int natoms, const doubl
 // ============================================================================ instantiations
 #define TDDFT_INST(R)                                                                                           \
   template cudaError_t launch_fft_xy<R>(cudaStream_t, int, const void*, void*, int, const void*, bool);                       \
-  template cudaError_t launch_fft_z<R>(cudaStream_t, int, void*, int, const void*, int, const ZParams&);          \
+  template cudaError_t launch_fft_z_kinetic<R>(cudaStream_t, int, void*, int, const void*, const void*,          \
+                                               const ZParams&);                                                 \
+  template cudaError_t launch_kin_tables<R>(cudaStream_t, int, int, const ZParams&, void*);                      \
   template cudaError_t launch_phase_table<R>(cudaStream_t, size_t, int, const R*, const EpiParams&, void*);      \
   template cudaError_t launch_beta_table<R>(cudaStream_t, size_t, const R*, const int*, const ProjTables<R>&,    \
                                             R*);                                                                \
