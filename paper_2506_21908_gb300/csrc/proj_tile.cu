@@ -157,6 +157,16 @@ __device__ __forceinline__ void tmem_ld8_async(uint32_t taddr, uint32_t* r) {
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                : "r"(taddr));
 }
+__device__ __forceinline__ void tmem_ld4_async(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
+}
+// W = 4 or 8 columns; tmem_regs_ready as above.
+template <int W> __device__ __forceinline__ void tmem_ld_async(uint32_t taddr, uint32_t* r) {
+  if constexpr (W == 4) tmem_ld4_async(taddr, r);
+  else tmem_ld8_async(taddr, r);
+}
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // After tmem_wait_ld: ties the loaded registers to a point after the wait, so that no use of them
 // is scheduled before it.
@@ -164,8 +174,9 @@ __device__ __forceinline__ void tmem_regs_ready(uint32_t* r) {
   asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
                "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]));
 }
-__device__ __forceinline__ void tmem_regs_ready8(uint32_t* r) {
-  asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]));
+template <int W> __device__ __forceinline__ void tmem_regs_ready_n(uint32_t* r) {
+  asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]));
+  if constexpr (W == 8) asm volatile("" : "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]));
 }
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float* v) {
   asm volatile(
@@ -571,12 +582,15 @@ k_tile_reduce(const float* __restrict__ part, TileDev td, int groups, int comps_
 //
 // Bound by HBM as long as enough loads are in flight: one CTA holds the SM (its 512
 // tensor-memory columns), so 16 worker warps drain it, four to each lane quarter of the tensor
-// memory, and the first spinors of a tile are requested before the wait for its products.
+// memory, inputs are requested before the wait for the tile's products, and the projector table
+// and the next tiles' rows (into L2) are on their way while X is built.
 // At the large supercell with 128 spinors the mean launch went from 2676 us (3.2 TB/s, 8 warps,
 // complex coefficients) to 1927 us (4.5 TB/s).
 constexpr int ST_WARPS = 16;                  // worker warps
-constexpr int ST_NT = 32 * (ST_WARPS + 2);    // + MMA warp + copy warp
-constexpr int ST_MMA_WARP = ST_WARPS, ST_COPY_WARP = ST_WARPS + 1;
+constexpr int ST_NT = 32 * (ST_WARPS + 3);    // + MMA warp + copy warp + prefetch warp
+constexpr int ST_MMA_WARP = ST_WARPS, ST_COPY_WARP = ST_WARPS + 1, ST_PF_WARP = ST_WARPS + 2;
+
+__device__ __forceinline__ void prefetch_l2_line(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 template <int EK, int TERMS, int AK>
 __global__ void __launch_bounds__(ST_NT, 1)
@@ -589,7 +603,8 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
   constexpr int STAGE = NPART * PT_PART;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  __shared__ uint64_t bar_full[2], bar_empty[2], bar_accf[2], bar_acce[2], bar_fin;
+  __shared__ uint64_t bar_full[2], bar_empty[2], bar_accf[2], bar_acce[2], bar_x, bar_fin;
+  __shared__ volatile int progress;  // tile the first drain warp is at (paces the prefetches)
   __shared__ uint32_t tmem_base;
   __shared__ volatile int abort_flag;
   __shared__ float2 px[32], py[8], pz[8];
@@ -622,7 +637,9 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
       bar_init(sm_addr(&bar_accf[s]), 1);
       bar_init(sm_addr(&bar_acce[s]), 32 * ST_WARPS);
     }
+    bar_init(sm_addr(&bar_x), 32 * ST_WARPS);
     bar_init(sm_addr(&bar_fin), 1);
+    progress = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   phase_tables(px, py, pz, BX, td, ep.shift[k]);
@@ -699,8 +716,8 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
       if constexpr (TERMS == 3) put<EK>(xpart(j / EPR, 1), row, j % EPR, 0u);
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    pt_arrive(sm_addr(&bar_x));
   }
-  __syncthreads();
 
   const int nchunk = ntile * kch;
   if (warp == ST_COPY_WARP) {
@@ -722,6 +739,7 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
   } else if (warp == ST_MMA_WARP) {
     if (lane == 0 && has_nl) {
       const uint32_t id = idesc<EK>(2 * SC);
+      if (!pt_wait(sm_addr(&bar_x), 0)) abort_flag = 1;
       for (int t = 0; t < ntile && !abort_flag; ++t) {
         const int acc = t & 1;
         if (t >= 2 && !pt_wait(sm_addr(&bar_acce[acc]), ((t >> 1) - 1) & 1)) { abort_flag = 1; break; }
@@ -750,6 +768,29 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
       mma_commit(sm_addr(&bar_fin));
       if (!pt_wait(sm_addr(&bar_fin), 0)) atomicOr(err, 1);
     }
+  } else if (warp == ST_PF_WARP) {
+    if constexpr (AK == 0 || AK == 1) {
+      // ---- the spinor rows of the tiles ahead of the drain, into L2: two tiles before the X build has
+      // finished, then one tile ahead.  The drain's loads then wait for L2 and not for HBM, and HBM is
+      // busy while the CTA starts.  Only a pace: nothing waits for this warp.  (With both accumulators
+      // the rows of two tiles of every SM no longer stay in L2, and the form is faster without.)
+      const bool rec = ep.mode == EPI_RECUR;
+      const float2* arr[4] = {io.Tk, io.kin, rec ? io.Tkm1 : nullptr, AK == 1 && !ep.init1 ? io.acc1 : nullptr};
+      // one 128-byte line (16 points) per lane; a row of BX points is one or two lines
+      const int lpr = BX / 16, lines = 8;  // lines per row, lines per tile and component
+      const int total = min(SC, comps_per_k - comp0) * lines;
+      for (int t = 0; t < ntile; ++t) {
+        for (int poll = 0; poll < (1 << 14) && progress < t - 1 && !abort_flag; ++poll) __nanosleep(200);
+        for (int i = lane; i < total; i += 32) {
+          const int comp = i >> 3, l = i & 7, row = t * (lines / lpr) + l / lpr;
+          const size_t o = ((size_t)k * comps_per_k + comp0 + comp) * N3 +
+                           ((size_t)(z0 + (row >> 3)) * N + (y0 + (row & 7))) * N + x0 + (l % lpr) * 16;
+#pragma unroll
+          for (int a = 0; a < 4; ++a)
+            if (arr[a]) prefetch_l2_line(arr[a] + o);
+        }
+      }
+    }
   } else {
     // ---- drain: thread = point of the tile (lane quarter of the warp); the four warps of a
     // quarter take a fourth of the components each, eight (four spinors) at a time;
@@ -761,147 +802,178 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
     const bool rec = ep.mode == EPI_RECUR;
     const bool use1 = AK >= 1 && ep.use_acc1, use2 = AK >= 2 && ep.use_acc2;
     const bool ld1 = use1 && !ep.init1, ld2 = use2 && !ep.init2;
-    // spinors loaded at a time; the accumulator forms hold fewer, for registers
-    constexpr int NB = AK == 0 ? 4 : 2;
-    float2 pu[NB], pd[NB], ku[NB], kd[NB], qu[NB], qd[NB], au[NB], ad[NB], bu[NB], bd[NB];
-    for (int t = 0; t < ntile; ++t) {
-      const int acc = t & 1;
+    // Without accumulators a step takes four spinors, requested together (the first of a tile before
+    // the wait for its products).  The accumulator forms have registers for two: their steps take
+    // one, and the inputs of the next step, over the end of the tile, are requested before this one
+    // is computed (two register sets; a pair of steps reads its V_NL together).  At 48^3 x 1024
+    // spinors: 1.40 ms without accumulators (1.56 ms in the paired form), 3.45 ms with two
+    // (3.76 ms two at a time).
+    constexpr bool PAIRED = AK >= 1;
+    constexpr int NB = PAIRED ? 1 : 4;
+    constexpr int W = PAIRED ? 4 : 8;  // components whose V_NL is read together
+    const float2 z2 = make_float2(0.f, 0.f);
+    struct In {
+      float2 pu[NB], pd[NB], ku[NB], kd[NB], qu[NB], qd[NB], au[NB], ad[NB], bu[NB], bd[NB];
+    } in0, in1;
+    auto point = [&](int t) -> size_t {
       const int p = t * 128 + row;
       const int lx = p % BX, ly = (p / BX) & 7, lz = p / (BX * 8);
-      const size_t idx = ((size_t)(z0 + lz) * N + (y0 + ly)) * N + (x0 + lx);
+      return ((size_t)(z0 + lz) * N + (y0 + ly)) * N + (x0 + lx);
+    };
+    const size_t group = ((size_t)k * comps_per_k + comp0) * N3;
+    // every input of NB spinors from component cu0 on, at point idx
+    auto load = [&](In& f, size_t idx, int cu0) {
+#pragma unroll
+      for (int j = 0; j < NB; ++j) {
+        const int cu = cu0 + 2 * j;
+        f.pu[j] = f.pd[j] = f.ku[j] = f.kd[j] = f.qu[j] = f.qd[j] = f.au[j] = f.ad[j] = f.bu[j] = f.bd[j] = z2;
+        if (comp0 + cu < comps_per_k) {
+          const size_t ou = group + idx + (size_t)cu * N3, od = ou + N3;
+          f.pu[j] = io.Tk[ou]; f.pd[j] = io.Tk[od];
+          f.ku[j] = io.kin[ou]; f.kd[j] = io.kin[od];
+          if (rec) { f.qu[j] = io.Tkm1[ou]; f.qd[j] = io.Tkm1[od]; }
+          if (ld1) { f.au[j] = io.acc1[ou]; f.ad[j] = io.acc1[od]; }
+          if (ld2) { f.bu[j] = io.acc2[ou]; f.bd[j] = io.acc2[od]; }
+        }
+      }
+    };
+    auto load_v = [&](size_t idx) { return make_float4(io.V[idx], io.V[N3 + idx], io.V[2 * N3 + idx], io.V[3 * N3 + idx]); };
+    float4 vn = make_float4(0.f, 0.f, 0.f, 0.f);
+    if constexpr (PAIRED) {
+      load(in0, point(0), cbeg);
+      vn = load_v(point(0));
+    }
+    for (int t = 0; t < ntile; ++t) {
+      const int acc = t & 1;
+      if (AK >= 0 && threadIdx.x == 0) progress = t;
+      const int p = t * 128 + row;
+      const int lx = p % BX, ly = (p / BX) & 7, lz = p / (BX * 8);
+      const size_t idx = point(t);
       const uint32_t tb = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * 2 * SC);
-      const size_t base = ((size_t)k * comps_per_k + comp0) * N3 + idx;  // component comp0 at this point
-      const float2 z2 = make_float2(0.f, 0.f);
-      // every input of NB spinors from component cu0 on
-      auto load = [&](int cu0) {
+      const size_t base = group + idx;  // component comp0 at this point
+      if constexpr (AK == 0) {
+        load(in0, idx, cbeg);
+        vn = load_v(idx);
+      }
+      const float V0 = vn.x, V1 = vn.y, hx = 0.5f * vn.z, hy = 0.5f * vn.w;
+      const float2 ph = cm(cm(px[lx], py[ly]), pz[lz]);
+      const float2 phc = make_float2(ph.x, -ph.y);
+      // one step: the Chebyshev epilogue of spinor components cu0 .. at this point, V_NL in re, im
+      auto step = [&](const In& f, int cu0, const float* re, const float* im) {
 #pragma unroll
         for (int j = 0; j < NB; ++j) {
           const int cu = cu0 + 2 * j;
-          pu[j] = pd[j] = ku[j] = kd[j] = qu[j] = qd[j] = au[j] = ad[j] = bu[j] = bd[j] = z2;
-          if (comp0 + cu < comps_per_k) {
-            const size_t ou = base + (size_t)cu * N3, od = ou + N3;
-            pu[j] = io.Tk[ou]; pd[j] = io.Tk[od];
-            ku[j] = io.kin[ou]; kd[j] = io.kin[od];
-            if (rec) { qu[j] = io.Tkm1[ou]; qd[j] = io.Tkm1[od]; }
-            if (ld1) { au[j] = io.acc1[ou]; ad[j] = io.acc1[od]; }
-            if (ld2) { bu[j] = io.acc2[ou]; bd[j] = io.acc2[od]; }
-          }
+          if (comp0 + cu >= comps_per_k) continue;
+          const size_t ou = base + (size_t)cu * N3, od = ou + N3;
+          const float2 vu = cm(make_float2(re[2 * j], im[2 * j]), phc);
+          const float2 vd = cm(make_float2(re[2 * j + 1], im[2 * j + 1]), phc);
+          float2 hu = make_float2(f.ku[j].x + vu.x, f.ku[j].y + vu.y);
+          float2 hd = make_float2(f.kd[j].x + vd.x, f.kd[j].y + vd.y);
+          const float2 u = f.pu[j], d = f.pd[j], qu = f.qu[j], qd = f.qd[j];
+          hu = make_float2(hu.x + V0 * u.x + hx * d.x - hy * d.y, hu.y + V0 * u.y + hx * d.y + hy * d.x);
+          hd = make_float2(hd.x + V1 * d.x + hx * u.x + hy * u.y, hd.y + V1 * d.y + hx * u.y - hy * u.x);
+          // the series constants as float pairs (split_constants); T_1 without the factor 2 and
+          // without T_{-1} (zero here)
+          const float c2 = rec ? 2.f : 1.f;
+          const float2 tu = make_float2(c2 * shifted_f(hu.x, u.x, ep.f_c, ep.f_id) - qu.x,
+                                        c2 * shifted_f(hu.y, u.y, ep.f_c, ep.f_id) - qu.y);
+          const float2 td = make_float2(c2 * shifted_f(hd.x, d.x, ep.f_c, ep.f_id) - qd.x,
+                                        c2 * shifted_f(hd.y, d.y, ep.f_c, ep.f_id) - qd.y);
+          io.Tout[ou] = tu;
+          io.Tout[od] = td;
+          // accumulators: up to three terms (T_{k-1}, T_k, T_{k+1}) at once in float-float
+          // arithmetic, rounded once, as in k_epilogue
+          auto upd = [&](float2* accp, int init, int fin, float2 xu, float2 xd, const float* cmf, const float* c0f,
+                         const float* c1f, const float* rf, const float* phf) {
+            if (init) xu = xd = z2;
+            float2 lu = z2, ld = z2;
+            if constexpr (AK < 3) {
+              const bool odd = ep.odd;
+              ff_rmadd(xu, lu, tu, rf + 4, !odd);
+              ff_rmadd(xd, ld, td, rf + 4, !odd);
+              ff_rmadd(xu, lu, u, rf + 2, odd);
+              ff_rmadd(xd, ld, d, rf + 2, odd);
+              if (rec) {
+                ff_rmadd(xu, lu, qu, rf, !odd);
+                ff_rmadd(xd, ld, qd, rf, !odd);
+              }
+              if (fin) {
+                accp[ou] = ff_phase(xu, lu, phf);
+                accp[od] = ff_phase(xd, ld, phf);
+                return;
+              }
+            } else {
+              ff_cmadd(xu, lu, tu, c1f);
+              ff_cmadd(xd, ld, td, c1f);
+              ff_cmadd(xu, lu, u, c0f);
+              ff_cmadd(xd, ld, d, c0f);
+              if (rec) {
+                ff_cmadd(xu, lu, qu, cmf);
+                ff_cmadd(xd, ld, qd, cmf);
+              }
+            }
+            accp[ou] = make_float2(xu.x + lu.x, xu.y + lu.y);
+            accp[od] = make_float2(xd.x + ld.x, xd.y + ld.y);
+          };
+          if (use1) upd(io.acc1, ep.init1, ep.fin1, f.au[j], f.ad[j], ep.f_am, ep.f_a0, ep.f_a1, ep.f_ra, ep.f_ph1);
+          if (use2) upd(io.acc2, ep.init2, ep.fin2, f.bu[j], f.bd[j], ep.f_bm, ep.f_b0, ep.f_b1, ep.f_rb, ep.f_ph2);
         }
       };
-      float V0 = 0.f, V1 = 0.f, hx = 0.f, hy = 0.f;
-      if constexpr (AK >= 0) {
-        load(cbeg);
-        V0 = io.V[idx];
-        V1 = io.V[N3 + idx];
-        hx = 0.5f * io.V[2 * N3 + idx];
-        hy = 0.5f * io.V[3 * N3 + idx];
-      }
-      const float2 ph = cm(cm(px[lx], py[ly]), pz[lz]);
-      const float2 phc = make_float2(ph.x, -ph.y);
       if (has_nl) {
         if (!pt_wait(sm_addr(&bar_accf[acc]), (t >> 1) & 1)) abort_flag = 1;
         if (__any_sync(0xffffffffu, abort_flag != 0)) break;
         asm volatile("tcgen05.fence::after_thread_sync;");
       }
 #pragma unroll 1
-      for (int c0 = cbeg; c0 < cend; c0 += 8) {
-        float re[8], im[8];
+      for (int c0 = cbeg; c0 < cend; c0 += W) {
+        if constexpr (PAIRED) load(in1, idx, c0 + W / 2);
+        float re[W], im[W];
         if (has_nl) {
           auto part = [&](uint32_t col, float* o) {
-            uint32_t h[8];
-            tmem_ld8_async(tb + col, h);
+            uint32_t h[W];
+            tmem_ld_async<W>(tb + col, h);
             if constexpr (TERMS == 3) {
-              uint32_t l[8];
-              tmem_ld8_async(tb + 256u + col, l);
+              uint32_t l[W];
+              tmem_ld_async<W>(tb + 256u + col, l);
               tmem_wait_ld();
-              tmem_regs_ready8(h);
-              tmem_regs_ready8(l);
+              tmem_regs_ready_n<W>(h);
+              tmem_regs_ready_n<W>(l);
 #pragma unroll
-              for (int j = 0; j < 8; ++j) o[j] = __uint_as_float(h[j]) + __uint_as_float(l[j]);
+              for (int j = 0; j < W; ++j) o[j] = __uint_as_float(h[j]) + __uint_as_float(l[j]);
             } else {
               tmem_wait_ld();
-              tmem_regs_ready8(h);
+              tmem_regs_ready_n<W>(h);
 #pragma unroll
-              for (int j = 0; j < 8; ++j) o[j] = __uint_as_float(h[j]);
+              for (int j = 0; j < W; ++j) o[j] = __uint_as_float(h[j]);
             }
           };
           part((uint32_t)c0, re);
           part((uint32_t)(SC + c0), im);
-          if (c0 + 8 >= cend) {
+          if (c0 + W >= cend) {
             asm volatile("tcgen05.fence::before_thread_sync;");
             pt_arrive(sm_addr(&bar_acce[acc]));
           }
         } else {
 #pragma unroll
-          for (int j = 0; j < 8; ++j) re[j] = im[j] = 0.f;
+          for (int j = 0; j < W; ++j) re[j] = im[j] = 0.f;
         }
         if constexpr (AK < 0) {
 #pragma unroll
-          for (int j = 0; j < 8; ++j)
+          for (int j = 0; j < W; ++j)
             if (comp0 + c0 + j < comps_per_k) out[base + (size_t)(c0 + j) * N3] = cm(make_float2(re[j], im[j]), phc);
+        } else if constexpr (!PAIRED) {
+          if (c0 != cbeg) load(in0, idx, c0);
+          step(in0, c0, re, im);
         } else {
-#pragma unroll
-          for (int b = 0; b < 8; b += 2 * NB) {
-            if (c0 + b != cbeg) load(c0 + b);
-#pragma unroll
-            for (int j = 0; j < NB; ++j) {
-              const int cu = c0 + b + 2 * j;
-              if (comp0 + cu >= comps_per_k) continue;
-              const size_t ou = base + (size_t)cu * N3, od = ou + N3;
-              const float2 vu = cm(make_float2(re[b + 2 * j], im[b + 2 * j]), phc);
-              const float2 vd = cm(make_float2(re[b + 2 * j + 1], im[b + 2 * j + 1]), phc);
-              float2 hu = make_float2(ku[j].x + vu.x, ku[j].y + vu.y);
-              float2 hd = make_float2(kd[j].x + vd.x, kd[j].y + vd.y);
-              const float2 u = pu[j], d = pd[j];
-              hu = make_float2(hu.x + V0 * u.x + hx * d.x - hy * d.y, hu.y + V0 * u.y + hx * d.y + hy * d.x);
-              hd = make_float2(hd.x + V1 * d.x + hx * u.x + hy * u.y, hd.y + V1 * d.y + hx * u.y - hy * u.x);
-              // the series constants as float pairs (split_constants); T_1 without the factor 2 and
-              // without T_{-1} (zero here)
-              const float f = rec ? 2.f : 1.f;
-              const float2 tu = make_float2(f * shifted_f(hu.x, u.x, ep.f_c, ep.f_id) - qu[j].x,
-                                            f * shifted_f(hu.y, u.y, ep.f_c, ep.f_id) - qu[j].y);
-              const float2 td = make_float2(f * shifted_f(hd.x, d.x, ep.f_c, ep.f_id) - qd[j].x,
-                                            f * shifted_f(hd.y, d.y, ep.f_c, ep.f_id) - qd[j].y);
-              io.Tout[ou] = tu;
-              io.Tout[od] = td;
-              // accumulators: up to three terms (T_{k-1}, T_k, T_{k+1}) at once in float-float
-              // arithmetic, rounded once, as in k_epilogue
-              auto upd = [&](float2* accp, int init, int fin, float2 xu, float2 xd, const float* cmf, const float* c0f,
-                             const float* c1f, const float* rf, const float* phf) {
-                if (init) xu = xd = z2;
-                float2 lu = z2, ld = z2;
-                if constexpr (AK < 3) {
-                  const bool odd = ep.odd;
-                  ff_rmadd(xu, lu, tu, rf + 4, !odd);
-                  ff_rmadd(xd, ld, td, rf + 4, !odd);
-                  ff_rmadd(xu, lu, u, rf + 2, odd);
-                  ff_rmadd(xd, ld, d, rf + 2, odd);
-                  if (rec) {
-                    ff_rmadd(xu, lu, qu[j], rf, !odd);
-                    ff_rmadd(xd, ld, qd[j], rf, !odd);
-                  }
-                  if (fin) {
-                    accp[ou] = ff_phase(xu, lu, phf);
-                    accp[od] = ff_phase(xd, ld, phf);
-                    return;
-                  }
-                } else {
-                  ff_cmadd(xu, lu, tu, c1f);
-                  ff_cmadd(xd, ld, td, c1f);
-                  ff_cmadd(xu, lu, u, c0f);
-                  ff_cmadd(xd, ld, d, c0f);
-                  if (rec) {
-                    ff_cmadd(xu, lu, qu[j], cmf);
-                    ff_cmadd(xd, ld, qd[j], cmf);
-                  }
-                }
-                accp[ou] = make_float2(xu.x + lu.x, xu.y + lu.y);
-                accp[od] = make_float2(xd.x + ld.x, xd.y + ld.y);
-              };
-              if (use1) upd(io.acc1, ep.init1, ep.fin1, au[j], ad[j], ep.f_am, ep.f_a0, ep.f_a1, ep.f_ra, ep.f_ph1);
-              if (use2) upd(io.acc2, ep.init2, ep.fin2, bu[j], bd[j], ep.f_bm, ep.f_b0, ep.f_b1, ep.f_rb, ep.f_ph2);
-            }
+          step(in0, c0, re, im);
+          if (c0 + W < cend) {
+            load(in0, idx, c0 + W);
+          } else if (t + 1 < ntile) {
+            const size_t nidx = point(t + 1);
+            load(in0, nidx, cbeg);
+            vn = load_v(nidx);
           }
+          step(in1, c0 + W / 2, re + W / 2, im + W / 2);
         }
       }
     }
