@@ -229,6 +229,7 @@ struct tddft_ctx {
   double ph_A[3] = {0, 0, 0};
   void* gpart = nullptr;                      // gather partial sums of the chunks, and their counters
   int* gcount = nullptr;
+  int* s_order = nullptr;                     // FP64: points by falling number of projector entries
   // bookkeeping
   std::string err;
   long long launches = 0;
@@ -256,6 +257,7 @@ struct tddft_ctx {
     p.nrm = (const R*)nrm;
     p.g_ph = g_ph;
     p.s_ph = s_ph;
+    p.s_order = s_order;
     p.g_beta = (const R*)g_beta;
     p.s_beta = (const R*)s_beta;
     const double pi = 3.14159265358979323846;  // the constants of solid_harmonics()
@@ -1995,6 +1997,14 @@ tddft_status create_impl(tddft_ctx* c, const tddft_cell* cell, const tddft_grid*
         (s = c->cuda(cudaMemset(c->gcount, 0, ncnt), "gather counters init")))
       return s;
     if (c->prec == TDDFT_FP64) {
+      // points by falling number of entries, each class in grid order (counting sort)
+      int most = 0;
+      for (size_t i = 0; i < N3; ++i) most = std::max(most, ht.s_ptr[i + 1] - ht.s_ptr[i]);
+      std::vector<int> start(most + 2, 0), order(N3);
+      for (size_t i = 0; i < N3; ++i) start[most - (ht.s_ptr[i + 1] - ht.s_ptr[i]) + 1]++;
+      for (int j = 0; j <= most; ++j) start[j + 1] += start[j];
+      for (size_t i = 0; i < N3; ++i) order[start[most - (ht.s_ptr[i + 1] - ht.s_ptr[i])]++] = (int)i;
+      if ((s = upload(c, &c->s_order, order, "point order"))) return s;
       const size_t bb = ne * beta_pitch(c->nlm) * sizeof(double);
       if ((s = c->alloc(&c->g_beta, bb, "projector values")) || (s = c->alloc(&c->s_beta, bb, "projector values"))) return s;
       const ProjTables<double> pt = c->tables<double>();

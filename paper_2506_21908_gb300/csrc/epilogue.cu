@@ -16,9 +16,12 @@ namespace tddft {
 
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
-// Each thread takes two items: two neighbouring grid points of one spinor (SP = 0, 16-byte
+// Each thread takes two items: two grid points of one spinor (SP = 0; in FP32 neighbours, 16-byte
 // accesses) or one grid point of two spinors of one k-point (SP = 1, 8-byte accesses), whose
-// projector scatter then walks the point's entries once for both.  The D c of the CTA's
+// projector scatter then walks the point's entries once for both.  FP64 takes the points in the
+// order pt.s_order, by falling number of projector entries: the FP64 pipe is its bound, and a warp
+// costs its longest lane (rows of x cross the spheres' edges: 106 FP64 instructions per point and
+// spinor where 72 are needed; 64^3 x 13 spinors 782 -> 440 us).  The D c of the CTA's
 // spinor(s) for every atom is staged in shared memory when it is small.
 // AK selects the accumulator code compiled in: 0 = Chebyshev term without accumulator update,
 // 1 = Chebyshev term updating accumulator 1, 2 = both, with the exponential's real coefficients;
@@ -51,22 +54,31 @@ k_epilogue(const typename CT<R>::type* __restrict__ kin, const typename CT<R>::t
     __syncthreads();
   }
   const C* dcb = (NLM > 0 && ep.dc_staged) ? dcs : dcg;
-  const size_t r = (SP ? 1 : 2) * ((size_t)blockIdx.x * blockDim.x + threadIdx.x);
-  if (r >= N3) return;
+  const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  size_t r = SP ? tid : 2 * tid, step = SP ? 2 * N3 : 1;  // the first item's point, and the way to the second
+  if constexpr (sizeof(R) == 8) {
+    // SP = 0: points i and i + 32 of the order, so that a warp's accesses stay together
+    const size_t i = SP ? tid : (tid & ~(size_t)31) * 2 + (tid & 31);
+    if (i >= N3) return;
+    r = pt.s_order ? (size_t)pt.s_order[i] : i;
+    if constexpr (!SP) step = (pt.s_order ? (size_t)pt.s_order[i + 32] : i + 32) - r;
+  } else {
+    if (r >= N3) return;
+  }
   const size_t ou = (size_t)(2 * kb) * N3 + r, od = ou + N3;
   // the thread's two items of an array at offset o (up) or o + N3 (down)
-  const size_t step = 2 * N3;
+  constexpr bool APART = SP || sizeof(R) == 8;  // two accesses, else one of both
   auto ld = [&](const C* b, size_t o) -> Pair<C> {
-    if constexpr (SP) return Pair<C>{b[o], b[o + step]};
+    if constexpr (APART) return Pair<C>{b[o], b[o + step]};
     else return ld2(b + o);
   };
   auto st = [&](C* b, size_t o, C x, C y) {
-    if constexpr (SP) { b[o] = x; b[o + step] = y; }
+    if constexpr (APART) { b[o] = x; b[o + step] = y; }
     else st2(b + o, x, y);
   };
   auto pf = [&](const C* b, size_t o) {
     prefetch_l2(b + o);
-    if constexpr (SP) prefetch_l2(b + o + step);
+    if constexpr (APART) prefetch_l2(b + o + step);
   };
   const Pair<C> pu2 = ld(Tk, ou), pd2 = ld(Tk, od);
   Pair<C> ku2 = ld(kin, ou), kd2 = ld(kin, od);
@@ -95,6 +107,12 @@ k_epilogue(const typename CT<R>::type* __restrict__ kin, const typename CT<R>::t
     if constexpr (SP) {
       const R v0 = V[r], v1 = V[N3 + r], v2 = V[2 * N3 + r], v3 = V[3 * N3 + r];
       h_point_2sp<R, NLM>(hu, hd, pu, pd, v0, v1, (R)0.5 * v2, (R)0.5 * v3, r, pt, dcb, dcb + ncoef, ph);
+    } else if constexpr (sizeof(R) == 8) {
+      const size_t r2 = r + step;
+      h_point<R, NLM>(hu[0], hd[0], pu[0], pd[0], V[r], V[N3 + r], (R)0.5 * V[2 * N3 + r], (R)0.5 * V[3 * N3 + r], r,
+                      pt, dcb, ph);
+      h_point<R, NLM>(hu[1], hd[1], pu[1], pd[1], V[r2], V[N3 + r2], (R)0.5 * V[2 * N3 + r2], (R)0.5 * V[3 * N3 + r2],
+                      r2, pt, dcb, ph);
     } else {
       const C v0 = *reinterpret_cast<const C*>(V + r), v1 = *reinterpret_cast<const C*>(V + N3 + r);
       const C v2 = *reinterpret_cast<const C*>(V + 2 * N3 + r), v3 = *reinterpret_cast<const C*>(V + 3 * N3 + r);
@@ -170,8 +188,14 @@ k_epilogue(const typename CT<R>::type* __restrict__ kin, const typename CT<R>::t
   } else {
     const C qus[2] = {qu0.a, qu0.b}, qds[2] = {qd0.a, qd0.b};
     for (int j = 0; j < 2; ++j) {
-      tu[j] = cmake<C>((R)2 * shf(hu[j].x, pu[j].x) - qus[j].x, (R)2 * shf(hu[j].y, pu[j].y) - qus[j].y);
-      td[j] = cmake<C>((R)2 * shf(hd[j].x, pd[j].x) - qds[j].x, (R)2 * shf(hd[j].y, pd[j].y) - qds[j].y);
+      if constexpr (sizeof(R) == 8) {
+        const R c = (R)ep.c, id2 = (R)(2.0 * ep.inv_delta);  // one multiply-add less than 2 shf - q
+        tu[j] = cmake<C>((hu[j].x - c * pu[j].x) * id2 - qus[j].x, (hu[j].y - c * pu[j].y) * id2 - qus[j].y);
+        td[j] = cmake<C>((hd[j].x - c * pd[j].x) * id2 - qds[j].x, (hd[j].y - c * pd[j].y) * id2 - qds[j].y);
+      } else {
+        tu[j] = cmake<C>((R)2 * shf(hu[j].x, pu[j].x) - qus[j].x, (R)2 * shf(hu[j].y, pu[j].y) - qus[j].y);
+        td[j] = cmake<C>((R)2 * shf(hd[j].x, pd[j].x) - qds[j].x, (R)2 * shf(hd[j].y, pd[j].y) - qds[j].y);
+      }
     }
   }
   st(Tout, ou, tu[0], tu[1]);

@@ -107,6 +107,7 @@ template <typename R> struct ProjTables {
   // (the FP64 pipe is the bound), the projector values [entries][beta_pitch(nlm)].
   const void* g_ph = nullptr;
   const void* s_ph = nullptr;
+  const int* s_order = nullptr;             // FP64: the grid points by falling number of entries
   const R* g_beta = nullptr;
   const R* s_beta = nullptr;
   R yc[4] = {};                             // solid-harmonic constants: l = 0, l = 1, l = 2 (xy, ...), l = 2 (3z^2 - r^2)
