@@ -805,25 +805,30 @@ cudaError_t epilogue(tddft_ctx* c, const void* kin, const void* Tk, const void* 
   return launch_epilogue<R>(c->st, c->N, kin, kin2, Tk, Tkm1, Tout, acc1, acc2, V, pt, dc, nkb, e);
 }
 
-// Kinetic part of H on all spinors: out = T in (three FFT passes).
-template <typename R> tddft_status kinetic(tddft_ctx* c, const void* in, void* out, const double A[3]) {
-  ZParams zp{};
+// Multiplier parameters of the z pass at k + A, with the tables formed when A changes (they depend
+// on A, the k-points and the cell only).
+template <typename R> tddft_status kin_params(tddft_ctx* c, const double A[3], ZParams& zp) {
   const double pi = 3.14159265358979323846;
   for (int a = 0; a < 3; ++a) zp.gs[a] = 2.0 * pi / c->L[a];
   zp.scale = 1.0 / (double)c->N3;
   zp.comps_per_k = 2 * c->nb;
   fill_shifts(c, A, zp.shift);
+  if (c->kin_valid && A[0] == c->kin_A[0] && A[1] == c->kin_A[1] && A[2] == c->kin_A[2]) return TDDFT_OK;
+  c->kin_valid = false;
+  tddft_status s = c->launch(KC_FFT_Z, "kinetic tables", [&] { return launch_kin_tables<R>(c->st, c->N, c->nk, zp, c->kin_tab); });
+  if (s) return s;
+  for (int a = 0; a < 3; ++a) c->kin_A[a] = A[a];
+  c->kin_valid = true;
+  return TDDFT_OK;
+}
+
+// Kinetic part of H on all spinors: out = T in (three FFT passes).
+template <typename R> tddft_status kinetic(tddft_ctx* c, const void* in, void* out, const double A[3]) {
+  ZParams zp{};
   const int nbatch = 2 * c->nkb;
   const double by = 2.0 * nbatch * (double)c->N3 * 2 * sizeof(R);
   tddft_status s;
-  // the kinetic factors depend on A, the k-points and the cell only: formed when A changes
-  if (!c->kin_valid || A[0] != c->kin_A[0] || A[1] != c->kin_A[1] || A[2] != c->kin_A[2]) {
-    c->kin_valid = false;
-    if ((s = c->launch(KC_FFT_Z, "kinetic tables", [&] { return launch_kin_tables<R>(c->st, c->N, c->nk, zp, c->kin_tab); })))
-      return s;
-    for (int a = 0; a < 3; ++a) c->kin_A[a] = A[a];
-    c->kin_valid = true;
-  }
+  if ((s = kin_params<R>(c, A, zp))) return s;
   if ((s = c->launch(KC_FFT_XY, "fft xy", [&] { return xy_pass<R>(c, in, out, nbatch, false); }, by))) return s;
   if ((s = c->launch(KC_FFT_Z, "fft z", [&] { return launch_fft_z_kinetic<R>(c->st, c->N, out, nbatch, c->tw, c->kin_tab, zp); }, by))) return s;
   return c->launch(KC_FFT_XY, "ifft xy", [&] { return xy_pass<R>(c, out, out, nbatch, true); }, by);
@@ -843,6 +848,22 @@ template <typename R> tddft_status phases(tddft_ctx* c, const double A[3], const
   for (int a = 0; a < 3; ++a) c->ph_A[a] = A[a];
   c->ph_valid = true;
   return TDDFT_OK;
+}
+
+// kdots[band] = {sum over the grid of Re conj(psi) T psi, 0} of the current states.
+template <typename R> tddft_status kinetic_energies(tddft_ctx* c, const double A[3], double* kdots) {
+  tddft_status s;
+  if (fft_z_energy_parts(c->N) == 0) {  // no energy pass: T psi, then its product with psi
+    if ((s = kinetic<R>(c, c->psi, c->tmp, A))) return s;
+    return c->launch(KC_OTHER, "kinetic dot", [&] { return launch_band_dot<R>(c->st, 2 * c->N3, c->nkb, c->psi, c->tmp, kdots, c->red_part); });
+  }
+  ZParams zp{};
+  if ((s = kin_params<R>(c, A, zp))) return s;
+  const double by = 2.0 * c->nkb * (double)c->N3 * 2 * sizeof(R);
+  if ((s = c->launch(KC_FFT_XY, "fft xy", [&] { return xy_pass<R>(c, c->psi, c->tmp, 2 * c->nkb, false); }, 2 * by))) return s;
+  return c->launch(KC_FFT_Z, "kinetic energy", [&] {
+    return launch_fft_z_energy<R>(c->st, c->N, c->tmp, c->nkb, c->tw, c->kin_tab, zp, c->red_part, kdots);
+  }, by);
 }
 
 template <typename R> tddft_status gather(tddft_ctx* c, const void* in, const double A[3], cudaStream_t sg = nullptr) {
@@ -1662,8 +1683,7 @@ template <typename R> tddft_status do_observables(tddft_ctx* c, double* n, doubl
   double* nle = kdots + 2 * nkb;
   if ((s = c->launch(KC_OTHER, "norms", [&] { return launch_band_dot<R>(c->st, 2 * c->N3, nkb, c->psi, c->psi, dots, c->red_part); }))) return s;
   // the kinetic and non-local energies only enter E: without E their passes are skipped
-  if (E && (s = kinetic<R>(c, c->psi, c->tmp, A))) return s;
-  if (E && (s = c->launch(KC_OTHER, "kinetic dot", [&] { return launch_band_dot<R>(c->st, 2 * c->N3, nkb, c->psi, c->tmp, kdots, c->red_part); }))) return s;
+  if (E && (s = kinetic_energies<R>(c, A, kdots))) return s;
   if (E && c->natoms > 0) {
     if ((s = gather<R>(c, c->psi, A))) return s;
     if ((s = c->launch(KC_OTHER, "nl energy", [&] { return launch_nl_energy<R>(c->st, nkb, c->natoms * 2 * c->nlm, c->cbuf, c->dcbuf, nle); }))) return s;
@@ -1922,7 +1942,7 @@ tddft_status create_impl(tddft_ctx* c, const tddft_cell* cell, const tddft_grid*
   if ((s = upload(c, &pos_d, c->pos.empty() ? std::vector<double>(3, 0.0) : c->pos, "pos")) || (s = upload(c, &zr_d, Zr, "Zr")))
     return s;
   if ((s = c->alloc(&c->tq, (3 * (size_t)c->nkb + 8) * sizeof(double), "torque sums"))) return s;
-  if ((s = c->alloc(&c->red_part, std::max(band_dot_part_doubles(c->nkb), field_sums_part_doubles()) * sizeof(double),
+  if ((s = c->alloc(&c->red_part, std::max({band_dot_part_doubles(c->nkb), field_sums_part_doubles(), (size_t)2 * c->nkb * fft_z_energy_parts(c->N)}) * sizeof(double),
                     "reduction partials")))
     return s;
   if (c->natoms > 0) {

@@ -263,6 +263,77 @@ k_fft_z2_kin(typename CT<R>::type* __restrict__ data, const typename CT<R>::type
   }
 }
 
+// Kinetic energy of one slab by Parseval: z transform of the xy transform (read only), then
+// sum |psi(G)|^2 1/2 |G + k + A|^2 scale over the slab's G, in the working precision over a work
+// item's R1 values and in FP64 above, to part[b][slab].  Half the passes of the kinetic operator
+// and its product with psi.
+template <typename R, int N>
+__global__ void __launch_bounds__(ZThreads<N>::value)
+k_fft_z2_energy(const typename CT<R>::type* __restrict__ data, const typename CT<R>::type* __restrict__ twg,
+                const R* __restrict__ tab, int comps_per_k, double* __restrict__ part) {
+  using C = typename CT<R>::type;
+  using TFW = TF<C, N, false>;
+  constexpr int NT = ZThreads<N>::value, CW = ZCols<N>::value;
+  constexpr int R1 = TwoFactor<N>::R1, R2 = TwoFactor<N>::R2;
+  constexpr int IA = CW * R1, IB = CW * R2;
+  constexpr int PA = (IA + NT - 1) / NT, PB = (IB + NT - 1) / NT;
+  __shared__ C tw[N];
+  __shared__ R tz[N];
+  __shared__ double red[NT / 32];
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* s = reinterpret_cast<C*>(smem_raw);  // [K0 R1 + n0][x], dense
+  const int y = blockIdx.x / (N / CW), x0 = (blockIdx.x - y * (N / CW)) * CW;
+  const int b = blockIdx.y;
+  const C* g = data + (size_t)b * N * N * N + (size_t)y * N + x0;
+  constexpr size_t ZS = (size_t)N * N;
+  const R* tk = tab + (size_t)(b / comps_per_k) * 3 * N;
+  for (int i = threadIdx.x; i < N; i += NT) {
+    tw[i] = twg[i];
+    tz[i] = tk[2 * N + i];
+  }
+  const R tyv = tk[N + y];
+  __syncthreads();  // tables
+#pragma unroll
+  for (int p = 0; p < PA; ++p) {
+    const int i = threadIdx.x + p * NT;
+    if (IA % NT == 0 || i < IA) {
+      const int n0 = i / CW, x = i - n0 * CW;
+      C v[R2];
+#pragma unroll
+      for (int q = 0; q < R2; ++q) v[q] = g[(size_t)(n0 + R1 * q) * ZS + x];
+      TFW::a_side(v, n0, tw);
+#pragma unroll
+      for (int k0 = 0; k0 < R2; ++k0) s[(k0 * R1 + n0) * CW + x] = v[k0];
+    }
+  }
+  __syncthreads();
+  double e = 0.0;
+#pragma unroll
+  for (int p = 0; p < PB; ++p) {
+    const int i = threadIdx.x + p * NT;
+    if (IB % NT == 0 || i < IB) {
+      const int k0 = i / CW, x = i - k0 * CW;
+      C u[R1];
+#pragma unroll
+      for (int n0 = 0; n0 < R1; ++n0) u[n0] = s[(k0 * R1 + n0) * CW + x];
+      TFW::b_side(u, k0, tw);
+      const R txy = tk[x0 + x] + tyv;
+      R t = (R)0;
+#pragma unroll
+      for (int k1 = 0; k1 < R1; ++k1) t += (u[k1].x * u[k1].x + u[k1].y * u[k1].y) * (txy + tz[k0 + R2 * k1]);
+      e += (double)t;
+    }
+  }
+  e = warp_sum(e);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = e;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int w = 0; w < NT / 32; ++w) t += red[w];
+    part[(size_t)b * gridDim.x + blockIdx.x] = t;
+  }
+}
+
 // Opt in to a kernel's dynamic shared memory, once per device (the attribute calls cost more host time
 // than the launch).
 template <typename K> static cudaError_t opt_in_smem(K kf, size_t smem, std::atomic<unsigned long long>& done) {
@@ -328,6 +399,57 @@ template <typename R>
 cudaError_t launch_fft_z_kinetic(cudaStream_t st, int N, void* data, int nbatch, const void* tw, const void* tab,
                                  const ZParams& zp) {
   TDDFT_DISPATCH_N(N, (fft_z_nm<R, NN, Z_KIN>(st, data, nbatch, tw, tab, zp)));
+}
+// Slabs per component of the energy pass (0: no such pass at this size).
+int fft_z_energy_parts(int N) {
+  switch (N) {
+    case 16: case 24: case 48: return N;  // ZCols = N
+    case 32: case 64: case 96: return N * (N / 32);
+    default: return 0;
+  }
+}
+template <typename R, int N>
+static cudaError_t fft_z_energy_n(cudaStream_t st, const void* data, int nbatch, const void* tw, const void* tab,
+                                  const ZParams& zp, double* part) {
+  if constexpr (TwoFactor<N>::ok) {
+    using C = typename CT<R>::type;
+    static std::atomic<unsigned long long> done{0};
+    constexpr int CW = ZCols<N>::value;
+    const size_t smem = (size_t)N * CW * sizeof(C);
+    auto kf = k_fft_z2_energy<R, N>;
+    cudaError_t e = opt_in_smem(kf, smem, done);
+    if (e != cudaSuccess) return e;
+    kf<<<dim3(N * (N / CW), nbatch), ZThreads<N>::value, smem, st>>>((const C*)data, (const C*)tw, (const R*)tab,
+                                                                     zp.comps_per_k, part);
+    return cudaGetLastError();
+  } else {
+    return cudaErrorInvalidValue;
+  }
+}
+// out2[band] = {sum of the band's per_band partials, 0}: one warp per band.
+__global__ void k_energy_sum(int nbands, int per_band, const double* __restrict__ part, double* __restrict__ out2) {
+  const int band = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (band >= nbands) return;
+  double t = 0.0;
+  for (int i = lane; i < per_band; i += 32) t += part[(size_t)band * per_band + i];
+  t = warp_sum(t);
+  if (lane == 0) {
+    out2[2 * band] = t;
+    out2[2 * band + 1] = 0.0;
+  }
+}
+template <typename R>
+static cudaError_t fft_z_energy(cudaStream_t st, int N, const void* data, int nbatch, const void* tw, const void* tab,
+                                const ZParams& zp, double* part) {
+  TDDFT_DISPATCH_N(N, (fft_z_energy_n<R, NN>(st, data, nbatch, tw, tab, zp, part)));
+}
+template <typename R>
+cudaError_t launch_fft_z_energy(cudaStream_t st, int N, const void* data, int nbands, const void* tw, const void* tab,
+                                const ZParams& zp, double* part, double* out2) {
+  cudaError_t e = fft_z_energy<R>(st, N, data, 2 * nbands, tw, tab, zp, part);
+  if (e != cudaSuccess) return e;
+  k_energy_sum<<<(nbands + 3) / 4, 128, 0, st>>>(nbands, 2 * fft_z_energy_parts(N), part, out2);
+  return cudaGetLastError();
 }
 cudaError_t launch_fft_z_inverse(cudaStream_t st, int N, double2* data, int nbatch, const double2* tw) {
   const ZParams zp{};
@@ -1311,6 +1433,8 @@ cudaError_t launch_atom_sums(cudaStream_t st, size_t N3, int natoms, const doubl
   template cudaError_t launch_fft_xy<R>(cudaStream_t, int, const void*, void*, int, const void*, bool);                       \
   template cudaError_t launch_fft_z_kinetic<R>(cudaStream_t, int, void*, int, const void*, const void*,          \
                                                const ZParams&);                                                 \
+  template cudaError_t launch_fft_z_energy<R>(cudaStream_t, int, const void*, int, const void*, const void*,       \
+                                              const ZParams&, double*, double*);                                \
   template cudaError_t launch_kin_tables<R>(cudaStream_t, int, int, const ZParams&, void*);                      \
   template cudaError_t launch_phase_table<R>(cudaStream_t, size_t, int, const R*, const EpiParams&, void*);      \
   template cudaError_t launch_beta_table<R>(cudaStream_t, size_t, const R*, const int*, const ProjTables<R>&,    \
