@@ -68,6 +68,7 @@ k_fft_xy2_tma(const float2* src, float2* dst, const float2* __restrict__ twg, in
   const uint32_t bar0 = sm_addr(&bars[0]), bar1 = sm_addr(&bars[1]);
   if (threadIdx.x == 0) bulk_init(bar0, bar1);
   for (int i = threadIdx.x; i < N; i += NT) tw[i] = twg[i];
+  pdl_wait();
   __syncthreads();
   int pl = blockIdx.x;
   if (pl < nplanes && warp == 0) issue_rows<N, RS>(src + (size_t)pl * N * N, N, buf0, bar0, lane);
@@ -144,8 +145,8 @@ static cudaError_t xy_tma_n(cudaStream_t st, const void* src, void* dst, int nba
   }
   const int nplanes = N * nbatch;
   const int grid = std::min(nplanes, sms * ps);
-  kf<<<grid, XYThreads<N>::value, smem, st>>>((const float2*)src, (float2*)dst, (const float2*)tw, nplanes, err);
-  return cudaGetLastError();
+  return launch_pdl(kf, dim3(grid), XYThreads<N>::value, smem, st, (const float2*)src, (float2*)dst, (const float2*)tw,
+                    nplanes, err);
 }
 
 cudaError_t launch_fft_xy_tma(cudaStream_t st, int N, const void* src, void* dst, int nbatch, const void* tw, bool inv,

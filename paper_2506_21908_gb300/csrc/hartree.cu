@@ -34,7 +34,6 @@ template <int N> struct LineTile {
   static constexpr int NT = TX * (R1 > R2 ? R1 : R2);  // one item per thread and side
 };
 
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // exp(-2 pi i t / N): from the table, or formed here when there is none (tw_out then receives it from
 // the first CTA for the passes that follow).
@@ -240,20 +239,6 @@ __global__ void __launch_bounds__(LineTile<N>::NT) k_poisson_z(C* __restrict__ g
     }
 }
 
-template <typename... K, typename... A>
-cudaError_t launch_pdl(void (*kf)(K...), dim3 grid, int nt, cudaStream_t st, A... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(nt);
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kf, static_cast<K>(args)...);
-}
-
 template <int N>
 cudaError_t poisson_n(cudaStream_t st, const double* in, const double* in2, double* out, double2* g, const double2* tw,
                       double2* tw_out, const ZParams& zp) {
@@ -262,12 +247,12 @@ cudaError_t poisson_n(cudaStream_t st, const double* in, const double* in2, doub
   const dim3 lines(N / L::TX, N / 2);
   const double2* twp = tw ? tw : tw_out;
   cudaError_t e;
-  if ((e = launch_pdl(k_poisson_x<N, false>, dim3(rows), L::NT, st, in, in2, g, nullptr, tw, tw_out)) != cudaSuccess ||
-      (e = launch_pdl(k_poisson_y<N, false>, lines, L::NT, st, g, twp)) != cudaSuccess ||
-      (e = launch_pdl(k_poisson_z<N>, dim3(N / L::TX, N / 2 + 1), L::NT, st, g, twp, zp)) != cudaSuccess ||
-      (e = launch_pdl(k_poisson_y<N, true>, lines, L::NT, st, g, twp)) != cudaSuccess)
+  if ((e = launch_pdl(k_poisson_x<N, false>, dim3(rows), L::NT, 0, st, in, in2, g, nullptr, tw, tw_out)) != cudaSuccess ||
+      (e = launch_pdl(k_poisson_y<N, false>, lines, L::NT, 0, st, g, twp)) != cudaSuccess ||
+      (e = launch_pdl(k_poisson_z<N>, dim3(N / L::TX, N / 2 + 1), L::NT, 0, st, g, twp, zp)) != cudaSuccess ||
+      (e = launch_pdl(k_poisson_y<N, true>, lines, L::NT, 0, st, g, twp)) != cudaSuccess)
     return e;
-  return launch_pdl(k_poisson_x<N, true>, dim3(rows), L::NT, st, nullptr, nullptr, g, out, twp, nullptr);
+  return launch_pdl(k_poisson_x<N, true>, dim3(rows), L::NT, 0, st, nullptr, nullptr, g, out, twp, nullptr);
 }
 
 }  // namespace

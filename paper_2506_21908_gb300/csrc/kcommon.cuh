@@ -14,6 +14,26 @@ template <int N> struct FFTThreads { static constexpr int value = (N >= 96) ? 38
 template <typename R, int N> struct FFTMinBlocks { static constexpr int value = 1; };
 template <int N> struct FFTMinBlocks<float, N> { static constexpr int value = (N <= 64) ? 1024 / FFTThreads<N>::value : 2; };
 
+// Programmatic dependent launch: the kernel may be set up before its predecessor on the stream has
+// ended, and calls pdl_wait() (which returns when it has, its writes visible) before it touches
+// memory the predecessor writes or reads.  2 us less between two short dependent kernels.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... K, typename... A>
+inline cudaError_t launch_pdl(void (*kf)(K...), dim3 grid, int nt, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(nt);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kf, static_cast<K>(args)...);
+}
+
 template <int N> __device__ __forceinline__ int freq(int i) { return i < N / 2 ? i : i - N; }
 
 // FP32 Chebyshev arithmetic with the series constants as float pairs hi + lo (see

@@ -121,6 +121,7 @@ k_fft_xy2(const typename CT<R>::type* src, typename CT<R>::type* dst, const type
   C* o = dst + base;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int i = threadIdx.x; i < N; i += NT) tw[i] = twg[i];
+  pdl_wait();
   __syncthreads();
   if constexpr (!INV) {
     PL::x_a_fwd(s, g, N, tw, warp, lane);
@@ -202,6 +203,8 @@ k_fft_z2_kin(typename CT<R>::type* __restrict__ data, const typename CT<R>::type
   const int b = blockIdx.y;
   C* g = data + (size_t)b * N * N * N + (size_t)y * N + x0;
   constexpr size_t ZS = (size_t)N * N;
+  for (int i = threadIdx.x; i < N; i += NT) tw[i] = twg[i];
+  pdl_wait();
   C v[PA][R2];
 #pragma unroll
   for (int p = 0; p < PA; ++p) {
@@ -213,10 +216,7 @@ k_fft_z2_kin(typename CT<R>::type* __restrict__ data, const typename CT<R>::type
     }
   }
   const R* tk = tab + (size_t)(b / comps_per_k) * 3 * N;
-  for (int i = threadIdx.x; i < N; i += NT) {
-    tw[i] = twg[i];
-    tz[i] = tk[2 * N + i];
-  }
+  for (int i = threadIdx.x; i < N; i += NT) tz[i] = tk[2 * N + i];
   const R tyv = tk[N + y];
   __syncthreads();  // tables
 #pragma unroll
@@ -357,7 +357,7 @@ static cudaError_t fft_xy_ni(cudaStream_t st, const void* src, void* data, int n
     const size_t smem = (size_t)(N + N * N) * sizeof(C);
     auto kf = k_fft_xy2<R, N, INV>;
     if ((e = opt_in_smem(kf, smem, done)) != cudaSuccess) return e;
-    kf<<<dim3(N, nbatch), XYThreads<N>::value, smem, st>>>((const C*)src, (C*)data, (const C*)tw);
+    return launch_pdl(kf, dim3(N, nbatch), XYThreads<N>::value, smem, st, (const C*)src, (C*)data, (const C*)tw);
   } else {
     const size_t smem = (size_t)(N + N * (N + 1)) * sizeof(C);
     auto kf = k_fft_xy<R, N, INV>;
@@ -381,7 +381,8 @@ static cudaError_t fft_z_nm(cudaStream_t st, void* data, int nbatch, const void*
     const size_t smem = (size_t)N * CW * sizeof(C);
     auto kf = k_fft_z2_kin<R, N>;
     if ((e = opt_in_smem(kf, smem, done)) != cudaSuccess) return e;
-    kf<<<dim3(N * (N / CW), nbatch), ZThreads<N>::value, smem, st>>>((C*)data, (const C*)tw, (const R*)tab, zp.comps_per_k);
+    return launch_pdl(kf, dim3(N * (N / CW), nbatch), ZThreads<N>::value, smem, st, (C*)data, (const C*)tw,
+                      (const R*)tab, zp.comps_per_k);
   } else {
     const size_t smem = (size_t)(N + N * N) * sizeof(C) + (2 * N + 2) * sizeof(R);
     auto kf = k_fft_z<R, N, MODE>;
