@@ -49,6 +49,7 @@ k_epilogue(const typename CT<R>::type* __restrict__ kin, const typename CT<R>::t
   const int k = kb / ep.nstates;
   const int ncoef = pt.natoms * 2 * NLM;
   const C* dcg = dc + (size_t)kb * ncoef;
+  pdl_wait();
   if (NLM > 0 && ep.dc_staged) {
     for (int i = threadIdx.x; i < (SP + 1) * ncoef; i += blockDim.x) dcs[i] = dcg[i];
     __syncthreads();
@@ -283,16 +284,15 @@ k_epilogue(const typename CT<R>::type* __restrict__ kin, const typename CT<R>::t
 }
 
 template <typename R, int NLM, int SP, typename... A>
-static void epi_ak(int ak, dim3 grid, size_t smem, cudaStream_t st, A... args) {
-  if (ak == 0) k_epilogue<R, NLM, 0, SP><<<grid, 256, smem, st>>>(args...);
-  else if (ak == 1) k_epilogue<R, NLM, 1, SP><<<grid, 256, smem, st>>>(args...);
-  else if (ak == 2) k_epilogue<R, NLM, 2, SP><<<grid, 256, smem, st>>>(args...);
-  else k_epilogue<R, NLM, 3, SP><<<grid, 256, smem, st>>>(args...);
+static cudaError_t epi_ak(int ak, dim3 grid, size_t smem, cudaStream_t st, A... args) {
+  if (ak == 0) return launch_pdl(k_epilogue<R, NLM, 0, SP>, grid, 256, smem, st, args...);
+  if (ak == 1) return launch_pdl(k_epilogue<R, NLM, 1, SP>, grid, 256, smem, st, args...);
+  if (ak == 2) return launch_pdl(k_epilogue<R, NLM, 2, SP>, grid, 256, smem, st, args...);
+  return launch_pdl(k_epilogue<R, NLM, 3, SP>, grid, 256, smem, st, args...);
 }
 template <typename R, int NLM, typename... A>
-static void epi_sp(bool sp, int ak, dim3 grid, size_t smem, cudaStream_t st, A... args) {
-  if (sp) epi_ak<R, NLM, 1>(ak, grid, smem, st, args...);
-  else epi_ak<R, NLM, 0>(ak, grid, smem, st, args...);
+static cudaError_t epi_sp(bool sp, int ak, dim3 grid, size_t smem, cudaStream_t st, A... args) {
+  return sp ? epi_ak<R, NLM, 1>(ak, grid, smem, st, args...) : epi_ak<R, NLM, 0>(ak, grid, smem, st, args...);
 }
 
 template <typename R>
@@ -315,14 +315,13 @@ cudaError_t launch_epilogue(cudaStream_t st, int N, const void* kin, const void*
   const int ak = (!cheb || (acc && !ep.real_coef)) ? 3 : (ep.use_acc2 ? 2 : (ep.use_acc1 ? 1 : 0));
 #define EPI_ARGS (const C*)kin, (const C*)kin2, (const C*)Tk, (const C*)Tkm1, (C*)Tout, (C*)acc1, (C*)acc2, V, N3, pt, (const C*)dc, epx
   switch (nlm) {
-    case 0: epi_sp<R, 0>(sp, ak, grid, smem, st, EPI_ARGS); break;
-    case 1: epi_sp<R, 1>(sp, ak, grid, smem, st, EPI_ARGS); break;
-    case 4: epi_sp<R, 4>(sp, ak, grid, smem, st, EPI_ARGS); break;
-    case 9: epi_sp<R, 9>(sp, ak, grid, smem, st, EPI_ARGS); break;
+    case 0: return epi_sp<R, 0>(sp, ak, grid, smem, st, EPI_ARGS);
+    case 1: return epi_sp<R, 1>(sp, ak, grid, smem, st, EPI_ARGS);
+    case 4: return epi_sp<R, 4>(sp, ak, grid, smem, st, EPI_ARGS);
+    case 9: return epi_sp<R, 9>(sp, ak, grid, smem, st, EPI_ARGS);
     default: return cudaErrorInvalidValue;
   }
 #undef EPI_ARGS
-  return cudaGetLastError();
 }
 
 

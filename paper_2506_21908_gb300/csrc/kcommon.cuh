@@ -1,5 +1,7 @@
 // Small device helpers shared by the kernel translation units.
 #pragma once
+#include <atomic>
+
 #include <cuda_runtime.h>
 
 namespace tddft {
@@ -18,6 +20,20 @@ template <int N> struct FFTMinBlocks<float, N> { static constexpr int value = (N
 // ended, and calls pdl_wait() (which returns when it has, its writes visible) before it touches
 // memory the predecessor writes or reads.  2 us less between two short dependent kernels.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Opt in to a kernel's dynamic shared memory, once per device (the attribute calls cost more host time
+// than the launch).
+template <typename K> inline cudaError_t opt_in_smem(K kf, size_t smem, std::atomic<unsigned long long>& done) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned long long bit = 1ull << (dev & 63);
+  if (done.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+  if ((e = cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(kf, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
+  return e;
+}
 
 template <typename... K, typename... A>
 inline cudaError_t launch_pdl(void (*kf)(K...), dim3 grid, int nt, size_t smem, cudaStream_t st, A... args) {

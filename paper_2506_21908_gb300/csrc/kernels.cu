@@ -10,7 +10,6 @@
 //   k_potential  locally collinear LSDA (Eqs. LC+ALDA2, LC+ALDA) and assembly of V_v
 //   reductions   deterministic fixed-order block reductions for energies and norms
 #include <algorithm>
-#include <atomic>
 #include <cstdint>
 
 #include "fft.cuh"
@@ -334,20 +333,6 @@ k_fft_z2_energy(const typename CT<R>::type* __restrict__ data, const typename CT
   }
 }
 
-// Opt in to a kernel's dynamic shared memory, once per device (the attribute calls cost more host time
-// than the launch).
-template <typename K> static cudaError_t opt_in_smem(K kf, size_t smem, std::atomic<unsigned long long>& done) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const unsigned long long bit = 1ull << (dev & 63);
-  if (done.load(std::memory_order_relaxed) & bit) return cudaSuccess;
-  if ((e = cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(kf, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
-  return e;
-}
-
 template <typename R, int N, bool INV>
 static cudaError_t fft_xy_ni(cudaStream_t st, const void* src, void* data, int nbatch, const void* tw) {
   using C = typename CT<R>::type;
@@ -480,13 +465,14 @@ k_phase_table(size_t nent, const R* __restrict__ rows, EpiParams ep, typename CT
   load_row<R, 4>(rows + e * 4, t);
   R sn, cs;
   sincos_r<R>((R)ep.shift[k][0] * t[0] + (R)ep.shift[k][1] * t[1] + (R)ep.shift[k][2] * t[2], &sn, &cs);
+  pdl_wait();
   out[(size_t)k * nent + e] = cmake<C>(cs, sn);
 }
 template <typename R>
 cudaError_t launch_phase_table(cudaStream_t st, size_t nent, int nk, const R* rows, const EpiParams& ep, void* out) {
   if (nent == 0) return cudaSuccess;
-  k_phase_table<R><<<dim3((unsigned)((nent + 255) / 256), nk), 256, 0, st>>>(nent, rows, ep, (typename CT<R>::type*)out);
-  return cudaGetLastError();
+  return launch_pdl(k_phase_table<R>, dim3((unsigned)((nent + 255) / 256), nk), 256, 0, st, nent, rows, ep,
+                    (typename CT<R>::type*)out);
 }
 
 // Projector values of every entry (once, at creation).
@@ -592,8 +578,9 @@ k_proj_gather(const typename CT<R>::type* __restrict__ psi, size_t N3, ProjTable
   C pc = zc, w[2 * SPN];
 #pragma unroll
   for (int j = 0; j < 2 * SPN; ++j) w[j] = zc;
+  const int r0 = (e < e1) ? pt.g_idx[e] : 0;
+  pdl_wait();
   if (e < e1) {
-    const int r0 = pt.g_idx[e];
     pc = ph[e];
 #pragma unroll
     for (int j = 0; j < 2 * SPN; ++j) w[j] = up[(size_t)j * N3 + r0];
@@ -712,13 +699,9 @@ cudaError_t launch_proj_gather(cudaStream_t st, int N, const void* psi, int nkb,
 #define PG_ARGS (const C*)psi, N3, pt, (R)dV, ep.nstates, chunks, (R*)part, counters, (C*)c_out, (C*)dc_out
 #define PG_CASE(NLM)                                                                         \
   if constexpr (sizeof(R) == 4) {                                                            \
-    if (spn == 2) {                                                                          \
-      k_proj_gather<R, NLM, 2><<<grid, PG_NT, 0, st>>>(PG_ARGS);                             \
-      break;                                                                                 \
-    }                                                                                        \
+    if (spn == 2) return launch_pdl(k_proj_gather<R, NLM, 2>, grid, PG_NT, 0, st, PG_ARGS);  \
   }                                                                                          \
-  k_proj_gather<R, NLM, 1><<<grid, PG_NT, 0, st>>>(PG_ARGS);                                 \
-  break
+  return launch_pdl(k_proj_gather<R, NLM, 1>, grid, PG_NT, 0, st, PG_ARGS)
   switch (pt.nlm) {
     case 1: PG_CASE(1);
     case 4: PG_CASE(4);
@@ -727,7 +710,6 @@ cudaError_t launch_proj_gather(cudaStream_t st, int N, const void* psi, int nkb,
   }
 #undef PG_CASE
 #undef PG_ARGS
-  return cudaGetLastError();
 }
 
 
@@ -745,6 +727,7 @@ k_density(const typename CT<R>::type* __restrict__ psi, size_t N3, int nkb, int 
   const int g = blockIdx.y;
   const int kb0 = (int)(((long long)nkb * g) / ngroups), kb1 = (int)(((long long)nkb * (g + 1)) / ngroups);
   double s[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};
+  pdl_wait();
   // FP32 spinors: bilinears of up to 8 bands are summed in FP32 (the inputs' own precision) and
   // each such partial sum is added to the FP64 accumulators; FP64 spinors: FP64 throughout
   constexpr int CH = sizeof(R) == 4 ? 8 : 1;
@@ -779,6 +762,7 @@ k_density(const typename CT<R>::type* __restrict__ psi, size_t N3, int nkb, int 
 __global__ void k_density_reduce(size_t n, int ngroups, const double* __restrict__ part, double* __restrict__ rho) {
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
+  pdl_wait();
   double t = 0.0;
   for (int g = 0; g < ngroups; ++g) t += part[(size_t)g * n + i];
   rho[i] = t;
@@ -799,11 +783,10 @@ cudaError_t launch_density(cudaStream_t st, size_t N3, const void* psi, int nkb,
   const int G = part ? density_groups(N3, nkb) : 1;
   const size_t nthreads = N3 / 2;
   dim3 grid((unsigned)((nthreads + 255) / 256), G);
-  k_density<R><<<grid, 256, 0, st>>>((const typename CT<R>::type*)psi, N3, nkb, G, wf, G == 1 ? rho : part);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_pdl(k_density<R>, grid, 256, 0, st, (const typename CT<R>::type*)psi, N3, nkb, G, wf,
+                             G == 1 ? rho : part);
   if (e != cudaSuccess || G == 1) return e;
-  k_density_reduce<<<(unsigned)((4 * N3 + 255) / 256), 256, 0, st>>>(4 * N3, G, part, rho);
-  return cudaGetLastError();
+  return launch_pdl(k_density_reduce, dim3((unsigned)((4 * N3 + 255) / 256)), 256, 0, st, 4 * N3, G, part, rho);
 }
 
 // ============================================================================ XC and potential
@@ -864,6 +847,7 @@ __global__ void k_potential(size_t N3, const double* __restrict__ rho, const dou
                             double* __restrict__ vxc4) {
   const size_t r = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= N3) return;
+  pdl_wait();
   const double r0 = rho[r], r1 = rho[N3 + r], r2 = rho[2 * N3 + r], r3 = rho[3 * N3 + r];
   const double n = r0 + r1, mx = 2.0 * r2, my = -2.0 * r3, mz = r0 - r1;
   double e = 0.0, vbar = 0.0, bx = 0.0, by = 0.0, bz = 0.0;
@@ -901,9 +885,8 @@ __global__ void k_potential(size_t N3, const double* __restrict__ rho, const dou
 
 cudaError_t launch_potential(cudaStream_t st, size_t N3, const double* rho, const double* vH, const double* vloc,
                              const double* B, int xc, int mode, double* V, float* Vf, double* exc, double* vxc4) {
-  k_potential<<<(unsigned)((N3 + 255) / 256), 256, 0, st>>>(N3, rho, vH, vloc, B[0], B[1], B[2], xc, mode, V, Vf, exc,
-                                                            vxc4);
-  return cudaGetLastError();
+  return launch_pdl(k_potential, dim3((unsigned)((N3 + 255) / 256)), 256, 0, st, N3, rho, vH, vloc, B[0], B[1], B[2],
+                    xc, mode, V, Vf, exc, vxc4);
 }
 
 __global__ void k_complex_real_part(size_t n, const double2* in, double* out, double scale) {
@@ -1268,6 +1251,7 @@ __global__ void k_check_window(size_t N3, const double* __restrict__ V, double l
                                double nl_bound, int* flag) {
   const size_t r = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= N3) return;
+  pdl_wait();
   const double v = 0.5 * (V[r] + V[N3 + r]);
   const double bz = 0.5 * (V[r] - V[N3 + r]), bx = 0.5 * V[2 * N3 + r], by = 0.5 * V[3 * N3 + r];
   const double b = sqrt(bx * bx + by * by + bz * bz);
@@ -1276,8 +1260,7 @@ __global__ void k_check_window(size_t N3, const double* __restrict__ V, double l
 }
 cudaError_t launch_check_window(cudaStream_t st, size_t N3, const double* V, double lo, double hi, double kin_max,
                                 double nl_bound, int* flag) {
-  k_check_window<<<(unsigned)((N3 + 255) / 256), 256, 0, st>>>(N3, V, lo, hi, kin_max, nl_bound, flag);
-  return cudaGetLastError();
+  return launch_pdl(k_check_window, dim3((unsigned)((N3 + 255) / 256)), 256, 0, st, N3, V, lo, hi, kin_max, nl_bound, flag);
 }
 
 // n = rho_uu + rho_dd and m = (2 Re rho_ud, -2 Im rho_ud, rho_uu - rho_dd) from rho_v, into

@@ -336,6 +336,7 @@ k_tile_gather(const float2* __restrict__ psi, int N, int comps_per_k, int groups
     // loads run two chunks ahead of the conversion: chunk c + 2 is requested before chunk c is
     // converted (wa: chunk c, wb: c + 1, wc: c + 2)
     V wa[CPW], wb[CPW], wc[CPW];
+    pdl_wait();
     load(0, wa);
     if (nch > 1) load(1, wb);
     for (int c = 0; c < nch; ++c) {
@@ -516,6 +517,7 @@ k_tile_reduce(const float* __restrict__ part, TileDev td, int groups, int comps_
   const int e0 = td.a_ptr[a], e1 = td.a_ptr[a + 1];
   const float* base = part + (size_t)kg * td.part_layer + (size_t)p * 128 + t;
   float2 acc = make_float2(0.f, 0.f);
+  pdl_wait();
   for (int b0 = e0; b0 < e1; b0 += kRedPh) {
     const int nb = min(kRedPh, e1 - b0);
     __syncthreads();
@@ -668,6 +670,7 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
   // gives both spin components of one spinor at one projector (index 2 p + sigma).
   if (warp < ST_WARPS) {
     const int tid = threadIdx.x;
+    pdl_wait();
     constexpr int SPG = SC / 2;                    // spinors per CTA
     const int total = nslot * SPG * nlm;
     const float4* dc4 = reinterpret_cast<const float4*>(dc);
@@ -778,6 +781,7 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
       const float2* arr[4] = {io.Tk, io.kin, rec ? io.Tkm1 : nullptr, AK == 1 && !ep.init1 ? io.acc1 : nullptr};
       // one 128-byte line (16 points) per lane; a row of BX points is one or two lines
       const int lpr = BX / 16, lines = 8;  // lines per row, lines per tile and component
+      pdl_wait();
       const int total = min(SC, comps_per_k - comp0) * lines;
       for (int t = 0; t < ntile; ++t) {
         for (int poll = 0; poll < (1 << 14) && progress < t - 1 && !abort_flag; ++poll) __nanosleep(200);
@@ -1009,14 +1013,14 @@ static cudaError_t gather_et(cudaStream_t st, int N, const void* psi, int nk, in
   const int groups = (comps_per_k + 63) / 64;
   const size_t smem = tile_gather_smem(TERMS);
   auto kf = k_tile_gather<EK, TERMS>;
-  cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  kf<<<dim3(nk * groups, td.nitems), PT_NT, smem, st>>>((const float2*)psi, N, comps_per_k, groups, td, ep, part, err);
-  cudaError_t e = cudaGetLastError();
+  static std::atomic<unsigned long long> done{0};
+  cudaError_t e = opt_in_smem(kf, smem, done);
   if (e != cudaSuccess) return e;
-  k_tile_reduce<<<dim3(td.natoms, nk * groups), 64 * td.nlm, 0, st>>>(part, td, groups, comps_per_k, nstates,
-                                                                      td.natoms, (float)dV, ep, Dmat, (float2*)c_out,
-                                                                      (float2*)dc_out);
-  return cudaGetLastError();
+  e = launch_pdl(kf, dim3(nk * groups, td.nitems), PT_NT, smem, st, (const float2*)psi, N, comps_per_k,
+                             groups, td, ep, part, err);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k_tile_reduce, dim3(td.natoms, nk * groups), 64 * td.nlm, 0, st, part, td, groups, comps_per_k,
+                    nstates, td.natoms, (float)dV, ep, Dmat, (float2*)c_out, (float2*)dc_out);
 }
 
 template <int EK, int TERMS, int AK>
@@ -1026,12 +1030,12 @@ static cudaError_t scatter_et(cudaStream_t st, int N, void* out, int nk, int nst
   const int comps_per_k = 2 * nstates;
   const int sgroups = (comps_per_k + SC - 1) / SC;
   const size_t smem = tile_scatter_smem(EK, TERMS, td.kch_max);
-  if (smem > 227 * 1024) return cudaErrorInvalidConfiguration;
+  if (smem > 224 * 1024) return cudaErrorInvalidConfiguration;
   auto kf = k_tile_scatter<EK, TERMS, AK>;
-  cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  kf<<<dim3(nk * sgroups, td.nitems), ST_NT, smem, st>>>((float2*)out, N, comps_per_k, sgroups, nstates, td.natoms,
-                                                         td, ep, (const float2*)dc, err, io);
-  return cudaGetLastError();
+  static std::atomic<unsigned long long> done{0};
+  if (cudaError_t e = opt_in_smem(kf, 224 * 1024, done)) return e;  // any handle's kch_max (at most 193 KB)
+  return launch_pdl(kf, dim3(nk * sgroups, td.nitems), ST_NT, smem, st, (float2*)out, N, comps_per_k, sgroups, nstates,
+                    td.natoms, td, ep, (const float2*)dc, err, io);
 }
 
 template <int AK>
