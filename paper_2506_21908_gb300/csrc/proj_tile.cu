@@ -622,7 +622,8 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
   const int brick = td.it_brick[it];
   const int bx = brick % td.nbx, by = (brick / td.nbx) % td.nby, bz = brick / (td.nbx * td.nby);
   const int x0 = bx * BX, y0 = by * 8, z0 = bz * 8;
-  const int ntile = BX * 64 / 128;
+  // this CTA's share of the brick's tiles (gridDim.z shares): t0 + 0 .. ntile - 1
+  const int t0 = (BX * 64 / 128) / gridDim.z * blockIdx.z, ntile = (BX * 64 / 128) / gridDim.z;
   const size_t N3 = (size_t)N * N * N;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nlm = td.nlm;
@@ -725,7 +726,7 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
   const int nchunk = ntile * kch;
   if (warp == ST_COPY_WARP) {
     if (lane == 0 && has_nl) {
-      const unsigned char* src = td.s_tab + td.it_soff[it];
+      const unsigned char* src = td.s_tab + td.it_soff[it] + (size_t)t0 * kch * NPART * PT_PART;
       int issued = 0;
       for (int j = 0; j < nchunk; ++j) {
         const int s = j & 1;
@@ -786,7 +787,7 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
       for (int t = 0; t < ntile; ++t) {
         for (int poll = 0; poll < (1 << 14) && progress < t - 1 && !abort_flag; ++poll) __nanosleep(200);
         for (int i = lane; i < total; i += 32) {
-          const int comp = i >> 3, l = i & 7, row = t * (lines / lpr) + l / lpr;
+          const int comp = i >> 3, l = i & 7, row = (t0 + t) * (lines / lpr) + l / lpr;
           const size_t o = ((size_t)k * comps_per_k + comp0 + comp) * N3 +
                            ((size_t)(z0 + (row >> 3)) * N + (y0 + (row & 7))) * N + x0 + (l % lpr) * 16;
 #pragma unroll
@@ -820,7 +821,7 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
       float2 pu[NB], pd[NB], ku[NB], kd[NB], qu[NB], qd[NB], au[NB], ad[NB], bu[NB], bd[NB];
     } in0, in1;
     auto point = [&](int t) -> size_t {
-      const int p = t * 128 + row;
+      const int p = (t0 + t) * 128 + row;
       const int lx = p % BX, ly = (p / BX) & 7, lz = p / (BX * 8);
       return ((size_t)(z0 + lz) * N + (y0 + ly)) * N + (x0 + lx);
     };
@@ -850,7 +851,7 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
     for (int t = 0; t < ntile; ++t) {
       const int acc = t & 1;
       if (AK >= 0 && threadIdx.x == 0) progress = t;
-      const int p = t * 128 + row;
+      const int p = (t0 + t) * 128 + row;
       const int lx = p % BX, ly = (p / BX) & 7, lz = p / (BX * 8);
       const size_t idx = point(t);
       const uint32_t tb = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * 2 * SC);
@@ -1034,7 +1035,13 @@ static cudaError_t scatter_et(cudaStream_t st, int N, void* out, int nk, int nst
   auto kf = k_tile_scatter<EK, TERMS, AK>;
   static std::atomic<unsigned long long> done{0};
   if (cudaError_t e = opt_in_smem(kf, 224 * 1024, done)) return e;  // any handle's kch_max (at most 193 KB)
-  return launch_pdl(kf, dim3(nk * sgroups, td.nitems), ST_NT, smem, st, (float2*)out, N, comps_per_k, sgroups, nstates,
+  // One CTA runs per SM: with few of them the last wave is a large part of the launch, so a brick's
+  // tiles are then shared by two CTAs, each building X for itself.  Up to four waves (152 SMs) of
+  // whole bricks two shares are faster (64^3 x 104 spinors, 3.4 waves: 441 -> 412 us per launch); four
+  // shares of 1.4 waves are slower than one (48^3 x 27: 80 -> 87 us).
+  const int ctas = nk * sgroups * td.nitems;
+  const int shares = ctas <= 608 ? 2 : 1;
+  return launch_pdl(kf, dim3(nk * sgroups, td.nitems, shares), ST_NT, smem, st, (float2*)out, N, comps_per_k, sgroups, nstates,
                     td.natoms, td, ep, (const float2*)dc, err, io);
 }
 
