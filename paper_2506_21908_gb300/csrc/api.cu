@@ -853,7 +853,7 @@ template <typename R> tddft_status phases(tddft_ctx* c, const double A[3], const
 // kdots[band] = {sum over the grid of Re conj(psi) T psi, 0} of the current states.
 template <typename R> tddft_status kinetic_energies(tddft_ctx* c, const double A[3], double* kdots) {
   tddft_status s;
-  if (fft_z_energy_parts(c->N) == 0) {  // no energy pass: T psi, then its product with psi
+  if (fft_z_energy_parts<R>(c->N) == 0) {  // no energy pass: T psi, then its product with psi
     if ((s = kinetic<R>(c, c->psi, c->tmp, A))) return s;
     return c->launch(KC_OTHER, "kinetic dot", [&] { return launch_band_dot<R>(c->st, 2 * c->N3, c->nkb, c->psi, c->tmp, kdots, c->red_part); });
   }
@@ -1942,7 +1942,7 @@ tddft_status create_impl(tddft_ctx* c, const tddft_cell* cell, const tddft_grid*
   if ((s = upload(c, &pos_d, c->pos.empty() ? std::vector<double>(3, 0.0) : c->pos, "pos")) || (s = upload(c, &zr_d, Zr, "Zr")))
     return s;
   if ((s = c->alloc(&c->tq, (3 * (size_t)c->nkb + 8) * sizeof(double), "torque sums"))) return s;
-  if ((s = c->alloc(&c->red_part, std::max({band_dot_part_doubles(c->nkb), field_sums_part_doubles(), (size_t)2 * c->nkb * fft_z_energy_parts(c->N)}) * sizeof(double),
+  if ((s = c->alloc(&c->red_part, std::max({band_dot_part_doubles(c->nkb), field_sums_part_doubles(), (size_t)2 * c->nkb * fft_z_energy_parts<double>(c->N)}) * sizeof(double),
                     "reduction partials")))
     return s;
   if (c->natoms > 0) {

@@ -133,8 +133,8 @@ cudaError_t launch_fft_z_kinetic(cudaStream_t st, int N, void* data, int nbatch,
                                  const ZParams& zp);
 // out2[band] = {sum over the grid and both components of Re conj(psi) T psi, 0} of every spinor from
 // its xy transform (Parseval: the sum over G of |psi(G)|^2 times the kinetic factor, scale 1 / N^3).
-// part: fft_z_energy_parts(N) doubles per component; no such pass where that is 0.
-int fft_z_energy_parts(int N);
+// part: fft_z_energy_parts<R>(N) doubles per component; no such pass where that is 0.
+template <typename R> int fft_z_energy_parts(int N);
 template <typename R>
 cudaError_t launch_fft_z_energy(cudaStream_t st, int N, const void* data, int nbands, const void* tw, const void* tab,
                                 const ZParams& zp, double* part, double* out2);

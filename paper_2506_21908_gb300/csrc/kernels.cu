@@ -156,9 +156,13 @@ k_fft_xy2(const typename CT<R>::type* src, typename CT<R>::type* dst, const type
 
 // Columns, threads and CTAs per SM of the z pass: a column's transform touches no other column, so a
 // CTA takes 32 columns (16, 24 or 48 at those sizes), few enough threads that the barriers of one
-// CTA leave the others of the SM running.
-template <int N> struct ZCols { static constexpr int value = N % 32 == 0 ? 32 : N; };
-template <int N> struct ZThreads { static constexpr int value = N % 32 == 0 ? 128 : (N == 16 ? 64 : 96); };
+// CTA leave the others of the SM running.  FP64: 8 columns (128-byte rows) and one warp, so that few
+// components still give every SM's FP64 pipe the same work (24^3 with 8 components: 192 CTAs of 24
+// columns on 152 SMs took 14.8 us, 576 of 8 take 9.9 us).
+template <typename R, int N> struct ZCols { static constexpr int value = sizeof(R) == 8 ? 8 : (N % 32 == 0 ? 32 : N); };
+template <typename R, int N> struct ZThreads {
+  static constexpr int value = sizeof(R) == 8 ? 32 : (N % 32 == 0 ? 128 : (N == 16 ? 64 : 96));
+};
 template <typename R, int N> struct ZBlocks { static constexpr int value = 1; };
 template <> struct ZBlocks<float, 96> { static constexpr int value = 7; };
 template <> struct ZBlocks<float, 64> { static constexpr int value = 8; };
@@ -184,13 +188,13 @@ __global__ void k_kin_tables(ZParams zp, R* __restrict__ out) {
 // way: A side (x, n0) reads global memory along z, B side (x, K0) transforms, multiplies by
 // tx[x] + ty[y] + tz[kz] and transforms back in registers, A side writes global memory.
 template <typename R, int N>
-__global__ void __launch_bounds__(ZThreads<N>::value, ZBlocks<R, N>::value)
+__global__ void __launch_bounds__(ZThreads<R, N>::value, ZBlocks<R, N>::value)
 k_fft_z2_kin(typename CT<R>::type* __restrict__ data, const typename CT<R>::type* __restrict__ twg,
              const R* __restrict__ tab, int comps_per_k) {
   using C = typename CT<R>::type;
   using TFW = TF<C, N, false>;
   using TIN = TF<C, N, true>;
-  constexpr int NT = ZThreads<N>::value, CW = ZCols<N>::value;
+  constexpr int NT = ZThreads<R, N>::value, CW = ZCols<R, N>::value;
   constexpr int R1 = TwoFactor<N>::R1, R2 = TwoFactor<N>::R2;
   constexpr int IA = CW * R1, IB = CW * R2;
   constexpr int PA = (IA + NT - 1) / NT, PB = (IB + NT - 1) / NT;
@@ -267,12 +271,12 @@ k_fft_z2_kin(typename CT<R>::type* __restrict__ data, const typename CT<R>::type
 // item's R1 values and in FP64 above, to part[b][slab].  Half the passes of the kinetic operator
 // and its product with psi.
 template <typename R, int N>
-__global__ void __launch_bounds__(ZThreads<N>::value)
+__global__ void __launch_bounds__(ZThreads<R, N>::value)
 k_fft_z2_energy(const typename CT<R>::type* __restrict__ data, const typename CT<R>::type* __restrict__ twg,
                 const R* __restrict__ tab, int comps_per_k, double* __restrict__ part) {
   using C = typename CT<R>::type;
   using TFW = TF<C, N, false>;
-  constexpr int NT = ZThreads<N>::value, CW = ZCols<N>::value;
+  constexpr int NT = ZThreads<R, N>::value, CW = ZCols<R, N>::value;
   constexpr int R1 = TwoFactor<N>::R1, R2 = TwoFactor<N>::R2;
   constexpr int IA = CW * R1, IB = CW * R2;
   constexpr int PA = (IA + NT - 1) / NT, PB = (IB + NT - 1) / NT;
@@ -362,11 +366,11 @@ static cudaError_t fft_z_nm(cudaStream_t st, void* data, int nbatch, const void*
   static std::atomic<unsigned long long> done{0};
   cudaError_t e;
   if constexpr (MODE == Z_KIN && TwoFactor<N>::ok) {
-    constexpr int CW = ZCols<N>::value;
+    constexpr int CW = ZCols<R, N>::value;
     const size_t smem = (size_t)N * CW * sizeof(C);
     auto kf = k_fft_z2_kin<R, N>;
     if ((e = opt_in_smem(kf, smem, done)) != cudaSuccess) return e;
-    return launch_pdl(kf, dim3(N * (N / CW), nbatch), ZThreads<N>::value, smem, st, (C*)data, (const C*)tw,
+    return launch_pdl(kf, dim3(N * (N / CW), nbatch), ZThreads<R, N>::value, smem, st, (C*)data, (const C*)tw,
                       (const R*)tab, zp.comps_per_k);
   } else {
     const size_t smem = (size_t)(N + N * N) * sizeof(C) + (2 * N + 2) * sizeof(R);
@@ -387,10 +391,14 @@ cudaError_t launch_fft_z_kinetic(cudaStream_t st, int N, void* data, int nbatch,
   TDDFT_DISPATCH_N(N, (fft_z_nm<R, NN, Z_KIN>(st, data, nbatch, tw, tab, zp)));
 }
 // Slabs per component of the energy pass (0: no such pass at this size).
-int fft_z_energy_parts(int N) {
+template <typename R> int fft_z_energy_parts(int N) {
   switch (N) {
-    case 16: case 24: case 48: return N;  // ZCols = N
-    case 32: case 64: case 96: return N * (N / 32);
+    case 16: return 16 * (16 / ZCols<R, 16>::value);
+    case 24: return 24 * (24 / ZCols<R, 24>::value);
+    case 32: return 32 * (32 / ZCols<R, 32>::value);
+    case 48: return 48 * (48 / ZCols<R, 48>::value);
+    case 64: return 64 * (64 / ZCols<R, 64>::value);
+    case 96: return 96 * (96 / ZCols<R, 96>::value);
     default: return 0;
   }
 }
@@ -400,12 +408,12 @@ static cudaError_t fft_z_energy_n(cudaStream_t st, const void* data, int nbatch,
   if constexpr (TwoFactor<N>::ok) {
     using C = typename CT<R>::type;
     static std::atomic<unsigned long long> done{0};
-    constexpr int CW = ZCols<N>::value;
+    constexpr int CW = ZCols<R, N>::value;
     const size_t smem = (size_t)N * CW * sizeof(C);
     auto kf = k_fft_z2_energy<R, N>;
     cudaError_t e = opt_in_smem(kf, smem, done);
     if (e != cudaSuccess) return e;
-    kf<<<dim3(N * (N / CW), nbatch), ZThreads<N>::value, smem, st>>>((const C*)data, (const C*)tw, (const R*)tab,
+    kf<<<dim3(N * (N / CW), nbatch), ZThreads<R, N>::value, smem, st>>>((const C*)data, (const C*)tw, (const R*)tab,
                                                                      zp.comps_per_k, part);
     return cudaGetLastError();
   } else {
@@ -434,7 +442,7 @@ cudaError_t launch_fft_z_energy(cudaStream_t st, int N, const void* data, int nb
                                 const ZParams& zp, double* part, double* out2) {
   cudaError_t e = fft_z_energy<R>(st, N, data, 2 * nbands, tw, tab, zp, part);
   if (e != cudaSuccess) return e;
-  k_energy_sum<<<(nbands + 3) / 4, 128, 0, st>>>(nbands, 2 * fft_z_energy_parts(N), part, out2);
+  k_energy_sum<<<(nbands + 3) / 4, 128, 0, st>>>(nbands, 2 * fft_z_energy_parts<R>(N), part, out2);
   return cudaGetLastError();
 }
 cudaError_t launch_fft_z_inverse(cudaStream_t st, int N, double2* data, int nbatch, const double2* tw) {
@@ -798,10 +806,10 @@ __device__ __forceinline__ void pw92_g(double rs, double sr, double isr, double 
   const double q0 = -2.0 * A * (1.0 + a1 * rs);
   const double q1 = 2.0 * A * sr * (b1 + sr * (b2 + sr * (b3 + sr * b4)));
   const double q1p = A * (b1 * isr + 2.0 * b2 + 3.0 * b3 * sr + 4.0 * b4 * rs);
-  const double iq1 = 1.0 / q1;
-  const double lg = log1p(iq1);
+  const double r = 1.0 / (q1 * (q1 + 1.0));  // one division: 1 / q1 = (q1 + 1) r
+  const double lg = log1p((q1 + 1.0) * r);
   *g = q0 * lg;
-  *dg = -2.0 * A * a1 * lg - q0 * q1p * iq1 / (q1 + 1.0);
+  *dg = -2.0 * A * a1 * lg - q0 * q1p * r;
 }
 
 // Slater exchange with spin scaling plus PW92 correlation on (nu, nd): energy density, v_up, v_dn.
@@ -841,7 +849,10 @@ __device__ void lsda_point(double nu, double nd, double* e, double* vu, double* 
   *vd = vxd + common - (z + 1.0) * dz;
 }
 
-__global__ void k_potential(size_t N3, const double* __restrict__ rho, const double* __restrict__ vH,
+// Bound by the FP64 pipe (some 600 instructions a point); small CTAs spread a small grid over the
+// SMs (24^3: 30 us on 54 CTAs of 256).
+constexpr int kPotThreads = 64;
+__global__ void __launch_bounds__(kPotThreads) k_potential(size_t N3, const double* __restrict__ rho, const double* __restrict__ vH,
                             const double* __restrict__ vloc, double Bx, double By, double Bz, int xc, int mode,
                             double* __restrict__ V, float* __restrict__ Vf, double* __restrict__ exc,
                             double* __restrict__ vxc4) {
@@ -885,7 +896,7 @@ __global__ void k_potential(size_t N3, const double* __restrict__ rho, const dou
 
 cudaError_t launch_potential(cudaStream_t st, size_t N3, const double* rho, const double* vH, const double* vloc,
                              const double* B, int xc, int mode, double* V, float* Vf, double* exc, double* vxc4) {
-  return launch_pdl(k_potential, dim3((unsigned)((N3 + 255) / 256)), 256, 0, st, N3, rho, vH, vloc, B[0], B[1], B[2],
+  return launch_pdl(k_potential, dim3((unsigned)((N3 + kPotThreads - 1) / kPotThreads)), kPotThreads, 0, st, N3, rho, vH, vloc, B[0], B[1], B[2],
                     xc, mode, V, Vf, exc, vxc4);
 }
 
@@ -1417,6 +1428,7 @@ cudaError_t launch_atom_sums(cudaStream_t st, size_t N3, int natoms, const doubl
   template cudaError_t launch_fft_xy<R>(cudaStream_t, int, const void*, void*, int, const void*, bool);                       \
   template cudaError_t launch_fft_z_kinetic<R>(cudaStream_t, int, void*, int, const void*, const void*,          \
                                                const ZParams&);                                                 \
+  template int fft_z_energy_parts<R>(int);                                                                      \
   template cudaError_t launch_fft_z_energy<R>(cudaStream_t, int, const void*, int, const void*, const void*,       \
                                               const ZParams&, double*, double*);                                \
   template cudaError_t launch_kin_tables<R>(cudaStream_t, int, int, const ZParams&, void*);                      \
