@@ -348,15 +348,17 @@ template <typename C, int N> struct TF<C, N, true> {
 
 // ---------------------------------------------------------------------------- xy plane in shared memory
 //
-// The x axis of the spectrum is kept in the order in which the in-place exchange leaves it: cell
-// p = K0 R1 + (K1 + K0) mod R1 of a row holds kx = K0 + R2 K1 (kx_at).  Nobody needs the natural
-// order (the z passes take their kx factors in this order and the inverse starts from it), and so
-// the x B side writes back to the cells it read: no barrier, and one item's registers at a time.
+// The x axis of the spectrum is kept in the order in which the in-place exchange leaves it: the block
+// of R1 cells K0 R1 .. holds kx = K0 + R2 K1 for K1 = 0 .. R1 - 1, its pairs of cells rotated by
+// K0 / 2 (kx_at).  Nobody needs the natural order (the z passes take their kx factors in this order
+// and the inverse starts from it), and so the x B side writes back to the cells it read: no barrier,
+// one item's registers at a time, and 16-byte accesses (FP32: pairs of cells), whose 8 lanes the
+// rotation spreads over the banks.
 template <int N> __host__ __device__ __forceinline__ int kx_at(int p) {
   if constexpr (TwoFactor<N>::ok) {
     constexpr int R1 = TwoFactor<N>::R1, R2 = TwoFactor<N>::R2;
-    const int k0 = p / R1;
-    return k0 + R2 * ((p - k0 * R1 - k0 + 4 * R1) % R1);
+    const int k0 = p / R1, r = p - k0 * R1;
+    return k0 + R2 * (2 * (((r >> 1) - (k0 >> 1) + 4 * R1) % (R1 / 2)) + (r & 1));
   } else {
     return p;
   }
@@ -373,6 +375,17 @@ template <> struct XYThreads<32> { static constexpr int value = 128; };
 template <> struct XYThreads<24> { static constexpr int value = 96; };
 template <> struct XYThreads<16> { static constexpr int value = 64; };
 
+__device__ __forceinline__ void ld_pair(const float2* p, float2& a, float2& b) {
+  const float4 v = *reinterpret_cast<const float4*>(p);
+  a = make_float2(v.x, v.y);
+  b = make_float2(v.z, v.w);
+}
+__device__ __forceinline__ void st_pair(float2* p, float2 a, float2 b) {
+  *reinterpret_cast<float4*>(p) = make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ void ld_pair(const double2* p, double2& a, double2& b) { a = p[0]; b = p[1]; }
+__device__ __forceinline__ void st_pair(double2* p, double2 a, double2 b) { p[0] = a; p[1] = b; }
+
 // Plane in shared memory with row pitch P.  The 8 cells of a work item and the 8 items of a row touch
 // 64-byte (FP32) blocks; two neighbouring rows must not meet in the same banks.  SWZ (FP32, P a
 // multiple of 16) exchanges neighbouring blocks of 8 cells in odd rows; without it the pitch is
@@ -385,9 +398,9 @@ template <typename C, int N, int P, bool SWZ> struct XYPlane {
   static_assert(RPW * (NT / 32) == N && RPW * R1 % 32 == 0 && N * R1 % NT == 0 && 32 % R1 == 0, "whole warps");
   static_assert(!SWZ || (P % 16 == 0 && R1 % 2 == 0), "swizzle");
 
-  // cell of element j of block k0 (R1 cells) in row y
+  // cell of element j of block k0 (R1 cells) in row y; elements 2 i and 2 i + 1 are neighbours
   __device__ __forceinline__ static int cell(int y, int k0, int j) {
-    int c = k0 * R1 + ((j + k0) % R1);
+    int c = k0 * R1 + 2 * (((j >> 1) + (k0 >> 1)) % (R1 / 2)) + (j & 1);
     if constexpr (SWZ) c ^= (y & 1) << 3;
     return y * P + c;
   }
@@ -422,10 +435,10 @@ template <typename C, int N, int P, bool SWZ> struct XYPlane {
         const int yl = i / R2, k0 = i - yl * R2, y = warp * RPW + yl;
         C u[R1];
 #pragma unroll
-        for (int j = 0; j < R1; ++j) u[j] = s[cell(y, k0, j)];
+        for (int j = 0; j < R1; j += 2) ld_pair(s + cell(y, k0, j), u[j], u[j + 1]);
         TF<C, N, INV>::b_side(u, k0, tw);
 #pragma unroll
-        for (int j = 0; j < R1; ++j) s[cell(y, k0, j)] = u[j];
+        for (int j = 0; j < R1; j += 2) st_pair(s + cell(y, k0, j), u[j], u[j + 1]);
       }
     }
   }

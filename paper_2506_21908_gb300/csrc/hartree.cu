@@ -107,7 +107,7 @@ k_poisson_x(const double* in, const double* in2, C* __restrict__ g, double* out,
       fwd_a<N>(v, n0, line, s, tw);
     }
     __syncthreads();
-      if (threadIdx.x < TX * R2) {
+    if (threadIdx.x < TX * R2) {
       const int line = threadIdx.x / R2, k0 = threadIdx.x - line * R2;
       C u[R1];
       fwd_b<N>(u, k0, line, s);
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(LineTile<N>::NT) k_poisson_y(C* __restrict__ g
       fwd_a<N>(v, j, line, s, tw);
     }
     __syncthreads();
-      if (j < R2) {
+    if (j < R2) {
       fwd_b<N>(u, j, line, s);
 #pragma unroll
       for (int k1 = 0; k1 < R1; ++k1) p[(size_t)(j + R2 * k1) * N + line] = u[k1];
@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(LineTile<N>::NT) k_poisson_y(C* __restrict__ g
       inv_b<N>(u, j, line, s, tw);
     }
     __syncthreads();
-      if (j < R1) {
+    if (j < R1) {
       inv_a<N>(v, j, line, s);
 #pragma unroll
       for (int q = 0; q < R2; ++q) p[(size_t)(j + R1 * q) * N + line] = v[q];
