@@ -49,23 +49,39 @@ k_epilogue(const typename CT<R>::type* __restrict__ kin, const typename CT<R>::t
   const int k = kb / ep.nstates;
   const int ncoef = pt.natoms * 2 * NLM;
   const C* dcg = dc + (size_t)kb * ncoef;
-  pdl_wait();
-  if (NLM > 0 && ep.dc_staged) {
-    for (int i = threadIdx.x; i < (SP + 1) * ncoef; i += blockDim.x) dcs[i] = dcg[i];
-    __syncthreads();
-  }
   const C* dcb = (NLM > 0 && ep.dc_staged) ? dcs : dcg;
   const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   size_t r = SP ? tid : 2 * tid, step = SP ? 2 * N3 : 1;  // the first item's point, and the way to the second
   if constexpr (sizeof(R) == 8) {
     // SP = 0: points i and i + 32 of the order, so that a warp's accesses stay together
     const size_t i = SP ? tid : (tid & ~(size_t)31) * 2 + (tid & 31);
-    if (i >= N3) return;
-    r = pt.s_order ? (size_t)pt.s_order[i] : i;
-    if constexpr (!SP) step = (pt.s_order ? (size_t)pt.s_order[i + 32] : i + 32) - r;
-  } else {
-    if (r >= N3) return;
+    if (i < N3) {
+      r = pt.s_order ? (size_t)pt.s_order[i] : i;
+      if constexpr (!SP) step = (pt.s_order ? (size_t)pt.s_order[i + 32] : i + 32) - r;
+    } else {
+      r = N3;
+    }
   }
+  // the entries of the first point (ea .. eb) and of the second (ec .. ed; in FP32 neighbours: ec = eb)
+  int ea = 0, eb = 0, ec = 0, ed = 0;
+  if (NLM > 0 && r < N3) {
+    ea = pt.s_ptr[r];
+    eb = pt.s_ptr[r + 1];
+    if constexpr (!SP) {
+      ec = sizeof(R) == 4 ? eb : pt.s_ptr[r + step];
+      ed = pt.s_ptr[r + step + 1];
+    }
+  }
+  pdl_wait();
+  if (NLM > 0 && ep.dc_staged) {
+    for (int i = threadIdx.x; i < (SP + 1) * ncoef; i += blockDim.x) dcs[i] = dcg[i];
+    __syncthreads();
+  }
+  if (r >= N3) return;
+  // FP32: one stream over both neighbours' entries
+  EntryStream<R, NLM> es(pt, reinterpret_cast<const C*>(pt.s_ph) + (size_t)k * pt.nent, ea,
+                         (SP || sizeof(R) == 8) ? eb : ed);
+  if constexpr (NLM > 0) es.start();
   const size_t ou = (size_t)(2 * kb) * N3 + r, od = ou + N3;
   // the thread's two items of an array at offset o (up) or o + N3 (down)
   constexpr bool APART = SP || sizeof(R) == 8;  // two accesses, else one of both
@@ -104,21 +120,27 @@ k_epilogue(const typename CT<R>::type* __restrict__ kin, const typename CT<R>::t
   const C pu[2] = {pu2.a, pu2.b}, pd[2] = {pd2.a, pd2.b};
   C hu[2] = {ku2.a, ku2.b}, hd[2] = {kd2.a, kd2.b};
   {
-    const C* ph = reinterpret_cast<const C*>(pt.s_ph) + (size_t)k * pt.nent;
     if constexpr (SP) {
-      const R v0 = V[r], v1 = V[N3 + r], v2 = V[2 * N3 + r], v3 = V[3 * N3 + r];
-      h_point_2sp<R, NLM>(hu, hd, pu, pd, v0, v1, (R)0.5 * v2, (R)0.5 * v3, r, pt, dcb, dcb + ncoef, ph);
-    } else if constexpr (sizeof(R) == 8) {
-      const size_t r2 = r + step;
-      h_point<R, NLM>(hu[0], hd[0], pu[0], pd[0], V[r], V[N3 + r], (R)0.5 * V[2 * N3 + r], (R)0.5 * V[3 * N3 + r], r,
-                      pt, dcb, ph);
-      h_point<R, NLM>(hu[1], hd[1], pu[1], pd[1], V[r2], V[N3 + r2], (R)0.5 * V[2 * N3 + r2], (R)0.5 * V[3 * N3 + r2],
-                      r2, pt, dcb, ph);
+      const R v0 = V[r], v1 = V[N3 + r], hx = (R)0.5 * V[2 * N3 + r], hy = (R)0.5 * V[3 * N3 + r];
+      for (int g = 0; g < 2; ++g) h_local<R>(hu[g], hd[g], pu[g], pd[g], v0, v1, hx, hy);
+      if constexpr (NLM > 0) h_scatter_2sp<R, NLM>(hu, hd, es, dcb, dcb + ncoef);
     } else {
-      const C v0 = *reinterpret_cast<const C*>(V + r), v1 = *reinterpret_cast<const C*>(V + N3 + r);
-      const C v2 = *reinterpret_cast<const C*>(V + 2 * N3 + r), v3 = *reinterpret_cast<const C*>(V + 3 * N3 + r);
-      h_point<R, NLM>(hu[0], hd[0], pu[0], pd[0], v0.x, v1.x, (R)0.5 * v2.x, (R)0.5 * v3.x, r, pt, dcb, ph);
-      h_point<R, NLM>(hu[1], hd[1], pu[1], pd[1], v0.y, v1.y, (R)0.5 * v2.y, (R)0.5 * v3.y, r + 1, pt, dcb, ph);
+      R v[4][2];
+      if constexpr (sizeof(R) == 8) {
+        for (int c = 0; c < 4; ++c) { v[c][0] = V[c * N3 + r]; v[c][1] = V[c * N3 + r + step]; }
+      } else {
+        for (int c = 0; c < 4; ++c) {
+          const C w = *reinterpret_cast<const C*>(V + c * N3 + r);
+          v[c][0] = w.x; v[c][1] = w.y;
+        }
+      }
+      for (int j = 0; j < 2; ++j)
+        h_local<R>(hu[j], hd[j], pu[j], pd[j], v[0][j], v[1][j], (R)0.5 * v[2][j], (R)0.5 * v[3][j]);
+      if constexpr (NLM > 0) {
+        h_scatter<R, NLM>(hu[0], hd[0], es, eb, dcb);
+        if constexpr (sizeof(R) == 8) { es.e = ec; es.end = ed; }
+        h_scatter<R, NLM>(hu[1], hd[1], es, ed, dcb);
+      }
     }
   }
   if (rec) { qu0 = ld(Tkm1, ou); qd0 = ld(Tkm1, od); }

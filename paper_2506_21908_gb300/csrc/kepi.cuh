@@ -75,24 +75,96 @@ __device__ __forceinline__ void entry_beta(size_t e, int a, const R* rows, const
   }
 }
 
-// Hamiltonian at one point for both spinor components: (hu, hd) holds the kinetic part on
-// entry; the 2x2 local potential and the projector scatter are added.
-template <typename R, int NLM>
-__device__ __forceinline__ void h_point(typename CT<R>::type& hu, typename CT<R>::type& hd, typename CT<R>::type pu,
-                                        typename CT<R>::type pd, R V0, R V1, R hx, R hy, size_t r,
-                                        const ProjTables<R>& pt, const typename CT<R>::type* dcb,
-                                        const typename CT<R>::type* ph) {
+// The projector entries of a thread's point(s) in scatter order, one entry ahead: the table row, phase
+// and atom of the next entry are requested before the current one is used (FP32, whose scatter is
+// bound by these dependent loads; FP64 is bound by its arithmetic and reads its longer rows in
+// place).  The first entry's loads are issued together with the spinors' (start).
+template <typename R, int NLM> struct EntryStream {
   using C = typename CT<R>::type;
+  const ProjTables<R>& pt;
+  const C* ph;
+  int e, end, a;
+  C pe;
+  float4 row;
+  __device__ __forceinline__ EntryStream(const ProjTables<R>& t, const C* p, int e0, int e1)
+      : pt(t), ph(p), e(e0), end(e1), a(0), pe(cmake<C>((R)0, (R)0)), row(make_float4(0.f, 0.f, 0.f, 0.f)) {}
+  __device__ __forceinline__ void start() {
+    if (sizeof(R) == 4 && e < end) fetch();
+  }
+  __device__ __forceinline__ void fetch() {
+    a = pt.s_atom[e];
+    pe = ph[e];
+    if constexpr (sizeof(R) == 4) row = __ldg(reinterpret_cast<const float4*>(pt.s_row) + e);
+  }
+  // projector values, phase and atom of the current entry; moves on to the next
+  __device__ __forceinline__ void next(R* bt, C& phase, int& atom) {
+    if constexpr (sizeof(R) == 8) {
+      fetch();
+      entry_beta<R, NLM>(e, a, pt.s_row, pt.s_beta, pt, bt);
+      phase = pe;
+      atom = a;
+      ++e;
+    } else {
+      const float4 t = row;
+      phase = pe;
+      atom = a;
+      ++e;
+      if (e < end) fetch();
+      R nl[4];
+      load_row<R, 4>(pt.nrm + (size_t)atom * 4, nl);
+      beta_values<R, NLM>(t.x, t.y, t.z, t.w, nl, pt.yc, bt);
+    }
+  }
+};
+
+// Local part of H at one point: (hu, hd) holds the kinetic part on entry; the 2x2 potential is added.
+template <typename R, typename C>
+__device__ __forceinline__ void h_local(C& hu, C& hd, C pu, C pd, R V0, R V1, R hx, R hy) {
   hu = cmake<C>(hu.x + V0 * pu.x + hx * pd.x - hy * pd.y, hu.y + V0 * pu.y + hx * pd.y + hy * pd.x);
   hd = cmake<C>(hd.x + V1 * pd.x + hx * pu.x + hy * pu.y, hd.y + V1 * pd.y + hx * pu.y - hy * pu.x);
-  if constexpr (NLM > 0) {
-    const int e0 = pt.s_ptr[r], e1 = pt.s_ptr[r + 1];
-    for (int e = e0; e < e1; ++e) {
-      const int a = pt.s_atom[e];
-      R bt[beta_pitch(NLM)];
-      const C pe = ph[e];
-      entry_beta<R, NLM>(e, a, pt.s_row, pt.s_beta, pt, bt);
-      const C* dca = dcb + (size_t)a * 2 * NLM;  // this spinor's D c of atom a, (up, dn) per p
+}
+
+// Projector scatter at one point for both spinor components: the entries of the stream before e1.
+template <typename R, int NLM>
+__device__ __forceinline__ void h_scatter(typename CT<R>::type& hu, typename CT<R>::type& hd, EntryStream<R, NLM>& es,
+                                          int e1, const typename CT<R>::type* dcb) {
+  using C = typename CT<R>::type;
+  while (es.e < e1) {
+    R bt[beta_pitch(NLM)];
+    C pe;
+    int a;
+    es.next(bt, pe, a);
+    const C* dca = dcb + (size_t)a * 2 * NLM;  // this spinor's D c of atom a, (up, dn) per p
+    R vux = 0, vuy = 0, vdx = 0, vdy = 0;
+#pragma unroll
+    for (int p = 0; p < NLM; ++p) {
+      const R bp = bt[p];
+      const Pair<C> cc = ld2(dca + 2 * p);
+      vux += bp * cc.a.x; vuy += bp * cc.a.y;
+      vdx += bp * cc.b.x; vdy += bp * cc.b.y;
+    }
+    const R cs = pe.x, sn = pe.y;
+    hu.x += vux * cs + vuy * sn; hu.y += vuy * cs - vux * sn;
+    hd.x += vdx * cs + vdy * sn; hd.y += vdy * cs - vdx * sn;
+  }
+}
+
+// The same for one point of two spinors of one k-point (index g = 0, 1): the projector entries
+// of the point, their beta values and phases are evaluated once for both spinors.
+template <typename R, int NLM>
+__device__ __forceinline__ void h_scatter_2sp(typename CT<R>::type (&hu)[2], typename CT<R>::type (&hd)[2],
+                                              EntryStream<R, NLM>& es, const typename CT<R>::type* dcb0,
+                                              const typename CT<R>::type* dcb1) {
+  using C = typename CT<R>::type;
+  while (es.e < es.end) {
+    R bt[beta_pitch(NLM)];
+    C pe;
+    int a;
+    es.next(bt, pe, a);
+    const R cs = pe.x, sn = pe.y;
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+      const C* dca = (g ? dcb1 : dcb0) + (size_t)a * 2 * NLM;
       R vux = 0, vuy = 0, vdx = 0, vdy = 0;
 #pragma unroll
       for (int p = 0; p < NLM; ++p) {
@@ -101,52 +173,8 @@ __device__ __forceinline__ void h_point(typename CT<R>::type& hu, typename CT<R>
         vux += bp * cc.a.x; vuy += bp * cc.a.y;
         vdx += bp * cc.b.x; vdy += bp * cc.b.y;
       }
-      const R cs = pe.x, sn = pe.y;
-      hu.x += vux * cs + vuy * sn; hu.y += vuy * cs - vux * sn;
-      hd.x += vdx * cs + vdy * sn; hd.y += vdy * cs - vdx * sn;
-    }
-  }
-}
-
-
-// The same for one point of two spinors of one k-point (index g = 0, 1): the projector entries
-// of the point, their beta values and phases are evaluated once for both spinors.
-template <typename R, int NLM>
-__device__ __forceinline__ void h_point_2sp(typename CT<R>::type (&hu)[2], typename CT<R>::type (&hd)[2],
-                                            const typename CT<R>::type (&pu)[2], const typename CT<R>::type (&pd)[2],
-                                            R V0, R V1, R hx, R hy, size_t r, const ProjTables<R>& pt,
-                                            const typename CT<R>::type* dcb0, const typename CT<R>::type* dcb1,
-                                            const typename CT<R>::type* ph) {
-  using C = typename CT<R>::type;
-#pragma unroll
-  for (int g = 0; g < 2; ++g) {
-    hu[g] = cmake<C>(hu[g].x + V0 * pu[g].x + hx * pd[g].x - hy * pd[g].y,
-                     hu[g].y + V0 * pu[g].y + hx * pd[g].y + hy * pd[g].x);
-    hd[g] = cmake<C>(hd[g].x + V1 * pd[g].x + hx * pu[g].x + hy * pu[g].y,
-                     hd[g].y + V1 * pd[g].y + hx * pu[g].y - hy * pu[g].x);
-  }
-  if constexpr (NLM > 0) {
-    const int e0 = pt.s_ptr[r], e1 = pt.s_ptr[r + 1];
-    for (int e = e0; e < e1; ++e) {
-      const int a = pt.s_atom[e];
-      R bt[beta_pitch(NLM)];
-      const C pe = ph[e];
-      entry_beta<R, NLM>(e, a, pt.s_row, pt.s_beta, pt, bt);
-      const R cs = pe.x, sn = pe.y;
-#pragma unroll
-      for (int g = 0; g < 2; ++g) {
-        const C* dca = (g ? dcb1 : dcb0) + (size_t)a * 2 * NLM;
-        R vux = 0, vuy = 0, vdx = 0, vdy = 0;
-#pragma unroll
-        for (int p = 0; p < NLM; ++p) {
-          const R bp = bt[p];
-          const Pair<C> cc = ld2(dca + 2 * p);
-          vux += bp * cc.a.x; vuy += bp * cc.a.y;
-          vdx += bp * cc.b.x; vdy += bp * cc.b.y;
-        }
-        hu[g].x += vux * cs + vuy * sn; hu[g].y += vuy * cs - vux * sn;
-        hd[g].x += vdx * cs + vdy * sn; hd[g].y += vdy * cs - vdx * sn;
-      }
+      hu[g].x += vux * cs + vuy * sn; hu[g].y += vuy * cs - vux * sn;
+      hd[g].x += vdx * cs + vdy * sn; hd[g].y += vdy * cs - vdx * sn;
     }
   }
 }
