@@ -422,7 +422,7 @@ cudaError_t launch_nl_agrad_fused(cudaStream_t st, int N, const void* S, const v
                                   double f, double* part, double* out) {
   using C = typename CT<R>::type;
   const size_t N3 = (size_t)N * N * N;
-  const int chunks = proj_chunks(pt.natoms, nkb, pt.nent);
+  const int chunks = proj_chunks(pt.natoms, nkb, pt.nent, 8);
   dim3 grid(pt.natoms * chunks, nkb);
 #define NLA_ARGS (const C*)S, (const C*)T, N3, pt, ep, chunks, (const C*)dcS, (const C*)dcT, part
   switch (pt.nlm) {

@@ -1420,7 +1420,7 @@ tddft_status do_backward(tddft_ctx* c, int nsteps, int ckpt, const double* dL_dr
   w.ncoef = (size_t)c->nkb * std::max(1, c->natoms) * 2 * c->nlm;
   const size_t cb = w.ncoef * 2 * sizeof(R);
   if ((s = tmp_alloc(c, db, &w.cS, cb, "cS")) || (s = tmp_alloc(c, db, &w.dcS, cb, "dcS")) ||
-      (s = tmp_alloc(c, db, &w.apart, (size_t)c->nkb * std::max(c->natoms, 1) * proj_chunks(c->natoms, c->nkb, c->n_entries) * 3 * 8, "agrad parts")) ||
+      (s = tmp_alloc(c, db, &w.apart, (size_t)c->nkb * std::max(c->natoms, 1) * proj_chunks(c->natoms, c->nkb, c->n_entries, 8) * 3 * 8, "agrad parts")) ||
       (s = tmp_alloc(c, db, &w.cT, cb, "cT")) || (s = tmp_alloc(c, db, &w.dcT, cb, "dcT")))
     return s;
   const int nck = (nsteps + ckpt - 1) / ckpt;

@@ -149,7 +149,7 @@ cudaError_t launch_beta_table(cudaStream_t st, size_t nent, const R* rows, const
                               R* out);
 // CTAs that share one (atom, spinor group) of the projector gather and of the projector-phase
 // gradient, and the scratch they need: partial sums (bytes) and zeroed counters (ints).
-int proj_chunks(int natoms, int ngroups, size_t nent);
+int proj_chunks(int natoms, int ngroups, size_t nent, size_t rsize);
 size_t proj_gather_part_bytes(int natoms, int nlm, int nk, int nstates, size_t nent, size_t rsize);
 size_t proj_gather_counters(int natoms, int nk, int nstates);
 template <typename R>
@@ -283,7 +283,7 @@ cudaError_t launch_fft_z_current(cudaStream_t st, int N, void* U, const void* W,
                                  const ZParams& zp, double* part);
 // Projector-phase A-gradient in one pass over the entries (replaces the moment gathers and
 // launch_nl_agrad): out[kb][a] += f sum_atoms sum_e d_a Im(e^{-i phi}[conj(S) w_T + conj(T) w_S]).
-// part: natoms x nkb x 3 doubles of scratch for each of proj_chunks(natoms, nkb, entries) chunks.
+// part: natoms x nkb x 3 doubles of scratch for each of proj_chunks(natoms, nkb, entries, 8) chunks.
 template <typename R>
 cudaError_t launch_nl_agrad_fused(cudaStream_t st, int N, const void* S, const void* T, int nkb,
                                   const ProjTables<R>& pt, const EpiParams& ep, const void* dcS, const void* dcT,

@@ -158,7 +158,7 @@ k_fft_xy2(const typename CT<R>::type* src, typename CT<R>::type* dst, const type
 // CTA takes 32 columns (16, 24 or 48 at those sizes), few enough threads that the barriers of one
 // CTA leave the others of the SM running.  FP64: 8 columns (128-byte rows) and one warp, so that few
 // components still give every SM's FP64 pipe the same work (24^3 with 8 components: 192 CTAs of 24
-// columns on 152 SMs took 14.8 us, 576 of 8 take 9.9 us).
+// columns on 152 SMs took 17.5 us with the launch, 576 of 8 take 14.2).
 template <typename R, int N> struct ZCols { static constexpr int value = sizeof(R) == 8 ? 8 : (N % 32 == 0 ? 32 : N); };
 template <typename R, int N> struct ZThreads {
   static constexpr int value = sizeof(R) == 8 ? 32 : (N % 32 == 0 ? 128 : (N == 16 ? 64 : 96));
@@ -682,16 +682,22 @@ k_proj_gather(const typename CT<R>::type* __restrict__ psi, size_t N3, ProjTable
 // Spinors per thread: two in FP32 where a k-point's states pair up, else one (FP64: registers).
 static int gather_spn(size_t rsize, int nstates) { return rsize == 4 && nstates % 2 == 0 ? 2 : 1; }
 
-// Enough CTAs for four per SM (608 on this chip), at least 256 entries each (two per thread).
-int proj_chunks(int natoms, int ngroups, size_t nent) {
+// Enough CTAs for four per SM (608 on this chip) of at least 256 entries each (two per thread); the
+// FP32 gather, whose CTAs wait for memory, goes on to four times as many of at least 2048 entries,
+// because the last, partly filled wave costs as much as a full one (64^3 x 104 spinors: 676 CTAs of
+// one chunk 107 us, 2704 of four 80 us; at 32^3 with 14 spinors chunks of 256 take 13.5 us with
+// 630 CTAs and 18.6 us with 1974).  The FP64 pipe stays busy with fewer.
+int proj_chunks(int natoms, int ngroups, size_t nent, size_t rsize) {
   const long long have = (long long)natoms * ngroups;
   if (have <= 0) return 1;
-  const long long want = (608 + have - 1) / have, most = (long long)(nent / (size_t)natoms) / 256;
-  return (int)std::max(1LL, std::min(want, std::min(most, 64LL)));
+  const long long per_atom = (long long)(nent / (size_t)natoms);
+  const long long fill = std::min((608 + have - 1) / have, per_atom / 256);
+  const long long waves = rsize == 4 ? std::min((2432 + have - 1) / have, per_atom / 2048) : 1;
+  return (int)std::max(1LL, std::min(64LL, std::max(fill, waves)));
 }
 size_t proj_gather_part_bytes(int natoms, int nlm, int nk, int nstates, size_t nent, size_t rsize) {
   const int spn = gather_spn(rsize, nstates), groups = nk * nstates / spn;
-  return (size_t)groups * natoms * proj_chunks(natoms, groups, nent) * spn * 4 * nlm * rsize;
+  return (size_t)groups * natoms * proj_chunks(natoms, groups, nent, rsize) * spn * 4 * nlm * rsize;
 }
 size_t proj_gather_counters(int natoms, int nk, int nstates) { return (size_t)natoms * nk * nstates; }
 
@@ -701,7 +707,7 @@ cudaError_t launch_proj_gather(cudaStream_t st, int N, const void* psi, int nkb,
   using C = typename CT<R>::type;
   if (pt.natoms == 0) return cudaSuccess;
   const int spn = gather_spn(sizeof(R), ep.nstates), groups = nkb / spn;
-  const int chunks = proj_chunks(pt.natoms, groups, pt.nent);
+  const int chunks = proj_chunks(pt.natoms, groups, pt.nent, sizeof(R));
   dim3 grid(pt.natoms * chunks, groups);
   const size_t N3 = (size_t)N * N * N;
 #define PG_ARGS (const C*)psi, N3, pt, (R)dV, ep.nstates, chunks, (R*)part, counters, (C*)c_out, (C*)dc_out
