@@ -231,7 +231,7 @@ template <> struct Split2<TILE_BF16> {
   }
 };
 
-constexpr int PT_WARPS = 8;                   // worker warps (16: 876 us against 677 at 96^3 x 128 spinors)
+constexpr int PT_WARPS = 8;                   // worker warps
 constexpr int PT_NT = 32 * (PT_WARPS + 2);    // + MMA warp + copy warp
 constexpr int PT_MMA_WARP = PT_WARPS, PT_COPY_WARP = PT_WARPS + 1;
 
@@ -292,6 +292,39 @@ k_tile_gather(const float2* __restrict__ psi, int N, int comps_per_k, int groups
     bar_init(sm_addr(&bar_drain), 32 * PT_WARPS);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  // Worker warps: each lane's point(s) of a chunk and the spinor components [warp CPW, + CPW) of the
+  // group there; the first two chunks are requested before the CTA's set-up.  Byte offsets of the
+  // group's components fit 32 bits, a lane's x and the rows of its chunks need no division, and two
+  // register sets alternate.  The kernel is bound by the chain MMA -> stage free -> conversion and
+  // copy -> MMA of its two stages, and by the MMAs' wait for P between groups: adding P into R before
+  // the next conversion instead of after it took 677 to 614 us (96^3, 128 atoms, 128 spinors) and 688
+  // to 650 us (48^3 x 1024).  (16 worker warps: 876 us.)
+  constexpr int PPL = (EPR == 64) ? 2 : 1;  // points per lane
+  using V = typename std::conditional<PPL == 2, float4, float2>::type;
+  const int bsh = BX == 32 ? 5 : 4, kk = lane * PPL, lx = kk & (BX - 1);
+  const int rpc = EPR >> bsh, row0 = kk >> bsh;  // grid rows per chunk, this lane's row in one
+  const char* gbase = reinterpret_cast<const char*>(psi + ((size_t)k * comps_per_k + comp0) * N3);
+  const uint32_t n3b = (uint32_t)N3 * (uint32_t)sizeof(float2);  // at most 64 n3b = 453 MB to a group
+  const uint32_t o0 = (uint32_t)warp * CPW * n3b + (uint32_t)((z0 * N + y0) * N + x0 + lx) * (uint32_t)sizeof(float2);
+  const int nvalid = min(CPW, comps_per_k - comp0 - warp * CPW);
+  auto load = [&](int c, V* w) {
+    const int row = c * rpc + row0;
+    const uint32_t o = o0 + (uint32_t)(((row >> 3) * N + (row & 7)) * N) * (uint32_t)sizeof(float2);
+#pragma unroll
+    for (int j = 0; j < CPW; ++j) {
+      V v;
+      if constexpr (PPL == 2) v = make_float4(0.f, 0.f, 0.f, 0.f);
+      else v = make_float2(0.f, 0.f);
+      if (j < nvalid) v = __ldg(reinterpret_cast<const V*>(gbase + (o + (uint32_t)j * n3b)));
+      w[j] = v;
+    }
+  };
+  V wa[CPW], wb[CPW];
+  if (warp < PT_WARPS) {
+    pdl_wait();
+    load(0, wa);
+    load(1, wb);
+  }
   phase_tables(px, py, pz, BX, td, ep.shift[k]);
   if (warp == PT_MMA_WARP) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sm_addr(&tmem_base)),
@@ -310,108 +343,78 @@ k_tile_gather(const float2* __restrict__ psi, int N, int comps_per_k, int groups
   const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
 
   if (warp < PT_WARPS) {
-    // ---- psi' = exp(i q.(r - r_b)) psi, split, into rows cl (re) and 64 + cl (im) of stage A.
-    constexpr int PPL = (EPR == 64) ? 2 : 1;  // points per lane
-    using V = typename std::conditional<PPL == 2, float4, float2>::type;
-    const int kk = lane * PPL;
-    const float2* base0 = psi + ((size_t)k * comps_per_k + comp0 + warp * CPW) * N3;
-    const int nvalid = min(CPW, comps_per_k - comp0 - warp * CPW);
-    auto point = [&](int c, int& lx, int& ly, int& lz) -> size_t {
-      const int p = c * EPR + kk;
-      lx = p % BX;
-      ly = (p / BX) & 7;
-      lz = p / (BX * 8);
-      return ((size_t)(z0 + lz) * N + (y0 + ly)) * N + (x0 + lx);
-    };
-    auto load = [&](int c, V* w) {
-      int lx, ly, lz;
-      const size_t idx = point(c, lx, ly, lz);
-#pragma unroll
-      for (int j = 0; j < CPW; ++j) {
-        V v;
-        if constexpr (PPL == 2) v = make_float4(0.f, 0.f, 0.f, 0.f);
-        else v = make_float2(0.f, 0.f);
-        if (j < nvalid) v = __ldg(reinterpret_cast<const V*>(base0 + (size_t)j * N3 + idx));
-        w[j] = v;
-      }
-    };
-    // loads run two chunks ahead of the conversion: chunk c + 2 is requested before chunk c is
-    // converted (wa: chunk c, wb: c + 1, wc: c + 2)
-    V wa[CPW], wb[CPW], wc[CPW];
-    pdl_wait();
-    load(0, wa);
-    if (nch > 1) load(1, wb);
-    for (int c = 0; c < nch; ++c) {
-      const int s = c & 1;
-      if (c + 2 < nch) load(c + 2, wc);
-      if (c >= 2 && !pt_wait(sm_addr(&bar_empty[s]), ((c >> 1) - 1) & 1)) abort_flag = 1;
-      if (__any_sync(0xffffffffu, abort_flag != 0)) break;
-      int lx, ly, lz;
-      point(c, lx, ly, lz);
-      const float2 ph0 = cm(cm(px[lx], py[ly]), pz[lz]);
-      const float2 ph1 = (PPL == 2) ? cm(cm(px[lx + 1], py[ly]), pz[lz]) : ph0;
-#pragma unroll
-      for (int j = 0; j < CPW; ++j) {
-        const int cl = warp * CPW + j;
-        if constexpr (PPL == 2) {
-          const float2 v0 = cm(make_float2(wa[j].x, wa[j].y), ph0);
-          const float2 v1 = cm(make_float2(wa[j].z, wa[j].w), ph1);
-          uint32_t rh, rl, ih, il;
-          Split2<EK>::two(v0.x, v1.x, rh, rl);
-          Split2<EK>::two(v0.y, v1.y, ih, il);
-          const uint32_t ore = sw128((uint32_t)cl * PT_ROWB + (uint32_t)(kk * 2));
-          const uint32_t oim = sw128((uint32_t)(64 + cl) * PT_ROWB + (uint32_t)(kk * 2));
-          *reinterpret_cast<uint32_t*>(stageA(s, 0) + ore) = rh;
-          *reinterpret_cast<uint32_t*>(stageA(s, 0) + oim) = ih;
-          if constexpr (TERMS == 3) {
-            *reinterpret_cast<uint32_t*>(stageA(s, 1) + ore) = rl;
-            *reinterpret_cast<uint32_t*>(stageA(s, 1) + oim) = il;
-          }
-        } else {
-          const float2 v0 = cm(make_float2(wa[j].x, wa[j].y), ph0);
-          uint32_t rh, rl, ih, il;
-          Split<EK>::two(v0.x, rh, rl);
-          Split<EK>::two(v0.y, ih, il);
-          put<EK>(stageA(s, 0), cl, kk, rh);
-          put<EK>(stageA(s, 0), 64 + cl, kk, ih);
-          if constexpr (TERMS == 3) {
-            put<EK>(stageA(s, 1), cl, kk, rl);
-            put<EK>(stageA(s, 1), 64 + cl, kk, il);
-          }
-        }
-      }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      pt_arrive(sm_addr(&bar_full[s]));
-#pragma unroll
-      for (int j = 0; j < CPW; ++j) {
-        wa[j] = wb[j];
-        wb[j] = wc[j];
-      }
-      // group g (1 <= g <= ngrp - 2) ended with chunk c - 2: add P into R before the next pass of
-      // this loop waits for the MMAs of the first chunk of group g + 1, which reuse P (the votes keep
-      // the warp together for the tensor-memory accesses)
+    // ---- psi' = exp(i q.(r - r_b)) psi, split, into rows cl (re) and 64 + cl (im) of stage A
+    const float2 px0 = px[lx], px1 = px[PPL == 2 ? lx + 1 : lx];
+    // one chunk from w; then the chunk after next is requested into w.  False: give up.
+    auto chunk = [&](int c, V* w) -> bool {
+      // group g (1 <= g <= ngrp - 2) ended with chunk c - 2: add P into R first of all, since the MMAs of
+      // chunk c - 1 (group g + 1), staged already, wait to reuse P (the votes keep the warp together
+      // for the tensor-memory accesses)
       const int gd = (c - 1) / CPG;
       if ((c - 1) % CPG == 0 && gd >= 2 && gd <= ngrp - 1) {
         if (!pt_wait(sm_addr(&bar_grp), (gd - 2) & 1)) abort_flag = 1;
-        if (__any_sync(0xffffffffu, abort_flag != 0)) break;
+        if (__any_sync(0xffffffffu, abort_flag != 0)) return false;
         asm volatile("tcgen05.fence::after_thread_sync;");
-        for (int c0 = cfirst; c0 < npad; c0 += CSTEP) {
-          uint32_t pv[16], rv[16];
-          tmem_ld16_async(accP + lane_off + (uint32_t)c0, pv);
-          tmem_ld16_async(accR + lane_off + (uint32_t)c0, rv);
-          tmem_wait_ld();
-          tmem_regs_ready(pv);
-          tmem_regs_ready(rv);
-          float sum[16];
+        for (int c0 = cfirst; c0 < npad; c0 += 2 * CSTEP) {  // two blocks of 16 columns at a time
+          const bool two = c0 + CSTEP < npad;
+          uint32_t pv[2][16], rv[2][16];
 #pragma unroll
-          for (int j = 0; j < 16; ++j) sum[j] = __uint_as_float(rv[j]) + __uint_as_float(pv[j]);
-          tmem_st16(accR + lane_off + (uint32_t)c0, sum);
+          for (int h = 0; h < 2; ++h)
+            if (h == 0 || two) {
+              tmem_ld16_async(accP + lane_off + (uint32_t)(c0 + h * CSTEP), pv[h]);
+              tmem_ld16_async(accR + lane_off + (uint32_t)(c0 + h * CSTEP), rv[h]);
+            }
+          tmem_wait_ld();
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            if (h == 0 || two) {
+              tmem_regs_ready(pv[h]);
+              tmem_regs_ready(rv[h]);
+              float sum[16];
+#pragma unroll
+              for (int j = 0; j < 16; ++j) sum[j] = __uint_as_float(rv[h][j]) + __uint_as_float(pv[h][j]);
+              tmem_st16(accR + lane_off + (uint32_t)(c0 + h * CSTEP), sum);
+            }
         }
         tmem_wait_st();
         asm volatile("tcgen05.fence::before_thread_sync;");
         pt_arrive(sm_addr(&bar_drain));
       }
-    }
+      const int s = c & 1;
+      if (c >= 2 && !pt_wait(sm_addr(&bar_empty[s]), ((c >> 1) - 1) & 1)) abort_flag = 1;
+      if (__any_sync(0xffffffffu, abort_flag != 0)) return false;
+      const int row = c * rpc + row0;
+      const float2 pyz = cm(py[row & 7], pz[row >> 3]);
+      const float2 ph0 = cm(px0, pyz), ph1 = PPL == 2 ? cm(px1, pyz) : ph0;
+      unsigned char* a0 = stageA(s, 0) + (warp * CPW) * PT_ROWB;
+#pragma unroll
+      for (int j = 0; j < CPW; ++j) {
+        // row j of this warp's eight: its swizzle is j
+        unsigned char* q = a0 + j * PT_ROWB + ((lane * 4) ^ (j << 4));
+        const float2 v0 = cm(make_float2(w[j].x, w[j].y), ph0);
+        uint32_t rh, rl, ih, il;
+        if constexpr (PPL == 2) {
+          const float2 v1 = cm(make_float2(w[j].z, w[j].w), ph1);
+          Split2<EK>::two(v0.x, v1.x, rh, rl);
+          Split2<EK>::two(v0.y, v1.y, ih, il);
+        } else {
+          Split<EK>::two(v0.x, rh, rl);
+          Split<EK>::two(v0.y, ih, il);
+        }
+        *reinterpret_cast<uint32_t*>(q) = rh;
+        *reinterpret_cast<uint32_t*>(q + 64 * PT_ROWB) = ih;
+        if constexpr (TERMS == 3) {
+          *reinterpret_cast<uint32_t*>(q + PT_PART) = rl;
+          *reinterpret_cast<uint32_t*>(q + PT_PART + 64 * PT_ROWB) = il;
+        }
+      }
+      if (c + 2 < nch) load(c + 2, w);
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      pt_arrive(sm_addr(&bar_full[s]));
+      return true;
+    };
+    for (int c = 0; c < nch; c += 2)  // nch is even
+      if (!chunk(c, wa) || !chunk(c + 1, wb)) break;
   } else if (warp == PT_COPY_WARP) {
     if (lane == 0) {
       // ---- projector values of the brick, chunk by chunk
