@@ -11,8 +11,9 @@
 // it occupies and by launch latency: with one CTA per plane (N CTAs on 152 SMs) it took 110 us at
 // 48^3.  Tiles of 8 lines give N^2 / 16 CTAs per pass, and each pass is set up while the one before
 // drains (programmatic dependent launch; every kernel waits for its predecessor before it touches
-// memory): 40 us at 48^3 and 47 us at 64^3, 51 and 58 us with plain launches.  Letting a pass start
-// its CTAs as soon as its predecessor's have started (an early trigger) is slower, 78 and 156 us.
+// memory): 40 us at 48^3 and 47 us at 64^3, 51 and 58 us with plain launches.  With its data requested
+// before the twiddles that it waits for with them, 39 and 46 us.  Letting a pass start its CTAs as
+// soon as its predecessor's have started (an early trigger) is slower, 78 and 156 us.
 #include "fft.cuh"
 #include "impl.cuh"
 #include "kcommon.cuh"
@@ -89,47 +90,47 @@ k_poisson_x(const double* in, const double* in2, C* __restrict__ g, double* out,
   __shared__ C tw[N], s[N * TX];
   if (!twg) twiddles<N>(tw, nullptr, nullptr);
   pdl_wait();
+  // every pass requests its data before the twiddles that it waits for with it
+  const size_t base = (size_t)blockIdx.x * TX * N;  // row (z, y) = blockIdx.x TX + line of the packed planes
+  const int line = threadIdx.x / (INV ? R2 : R1), j = threadIdx.x - line * (INV ? R2 : R1);  // k0 or n0
+  C v[R2], u[R1];
+  if constexpr (!INV) {
+    if (line < TX) {
+#pragma unroll
+      for (int q = 0; q < R2; ++q) {
+        const size_t i = base + line * N + j + R1 * q;
+        v[q] = make_double2(in[i], in[i + HALF]);
+        if (in2) v[q] = make_double2(v[q].x + in2[i], v[q].y + in2[i + HALF]);
+      }
+    }
+  } else {
+    if (line < TX) {
+#pragma unroll
+      for (int k1 = 0; k1 < R1; ++k1) u[k1] = g[base + line * N + j + R2 * k1];
+    }
+  }
   if (twg) twiddles<N>(tw, twg, nullptr);
   else if (tw_out && blockIdx.x == 0)
     for (int i = threadIdx.x; i < N; i += blockDim.x) tw_out[i] = tw[i];
   __syncthreads();
-  const size_t base = (size_t)blockIdx.x * TX * N;  // row (z, y) = blockIdx.x TX + line of the packed planes
   if constexpr (!INV) {
-    if (threadIdx.x < TX * R1) {
-      const int line = threadIdx.x / R1, n0 = threadIdx.x - line * R1;
-      C v[R2];
-#pragma unroll
-      for (int q = 0; q < R2; ++q) {
-        const size_t i = base + line * N + n0 + R1 * q;
-        v[q] = make_double2(in[i], in[i + HALF]);
-        if (in2) v[q] = make_double2(v[q].x + in2[i], v[q].y + in2[i + HALF]);
-      }
-      fwd_a<N>(v, n0, line, s, tw);
-    }
+    if (line < TX) fwd_a<N>(v, j, line, s, tw);
     __syncthreads();
     if (threadIdx.x < TX * R2) {
-      const int line = threadIdx.x / R2, k0 = threadIdx.x - line * R2;
-      C u[R1];
-      fwd_b<N>(u, k0, line, s);
+      const int lb = threadIdx.x / R2, k0 = threadIdx.x - lb * R2;
+      fwd_b<N>(u, k0, lb, s);
 #pragma unroll
-      for (int k1 = 0; k1 < R1; ++k1) g[base + line * N + k0 + R2 * k1] = u[k1];
+      for (int k1 = 0; k1 < R1; ++k1) g[base + lb * N + k0 + R2 * k1] = u[k1];
     }
   } else {
-    if (threadIdx.x < TX * R2) {
-      const int line = threadIdx.x / R2, k0 = threadIdx.x - line * R2;
-      C u[R1];
-#pragma unroll
-      for (int k1 = 0; k1 < R1; ++k1) u[k1] = g[base + line * N + k0 + R2 * k1];
-      inv_b<N>(u, k0, line, s, tw);
-    }
+    if (line < TX) inv_b<N>(u, j, line, s, tw);
     __syncthreads();
     if (threadIdx.x < TX * R1) {
-      const int line = threadIdx.x / R1, n0 = threadIdx.x - line * R1;
-      C v[R2];
-      inv_a<N>(v, n0, line, s);
+      const int la = threadIdx.x / R1, n0 = threadIdx.x - la * R1;
+      inv_a<N>(v, n0, la, s);
 #pragma unroll
       for (int q = 0; q < R2; ++q) {
-        const size_t i = base + line * N + n0 + R1 * q;
+        const size_t i = base + la * N + n0 + R1 * q;
         out[i] = v[q].x;
         out[i + HALF] = v[q].y;
       }
@@ -144,17 +145,21 @@ __global__ void __launch_bounds__(LineTile<N>::NT) k_poisson_y(C* __restrict__ g
   constexpr int R1 = L::R1, R2 = L::R2, TX = L::TX;
   __shared__ C tw[N], s[N * TX];
   pdl_wait();
-  twiddles<N>(tw, twg, nullptr);
-  __syncthreads();
   C* p = g + (size_t)blockIdx.y * N * N + blockIdx.x * TX;
   const int line = threadIdx.x % TX, j = threadIdx.x / TX;  // n0 (A side) or k0 (B side)
   C v[R2], u[R1];
-  if constexpr (!INV) {
-    if (j < R1) {
+  if (!INV && j < R1) {
 #pragma unroll
-      for (int q = 0; q < R2; ++q) v[q] = p[(size_t)(j + R1 * q) * N + line];
-      fwd_a<N>(v, j, line, s, tw);
-    }
+    for (int q = 0; q < R2; ++q) v[q] = p[(size_t)(j + R1 * q) * N + line];
+  }
+  if (INV && j < R2) {
+#pragma unroll
+    for (int k1 = 0; k1 < R1; ++k1) u[k1] = p[(size_t)(j + R2 * k1) * N + line];
+  }
+  twiddles<N>(tw, twg, nullptr);
+  __syncthreads();
+  if constexpr (!INV) {
+    if (j < R1) fwd_a<N>(v, j, line, s, tw);
     __syncthreads();
     if (j < R2) {
       fwd_b<N>(u, j, line, s);
@@ -162,11 +167,7 @@ __global__ void __launch_bounds__(LineTile<N>::NT) k_poisson_y(C* __restrict__ g
       for (int k1 = 0; k1 < R1; ++k1) p[(size_t)(j + R2 * k1) * N + line] = u[k1];
     }
   } else {
-    if (j < R2) {
-#pragma unroll
-      for (int k1 = 0; k1 < R1; ++k1) u[k1] = p[(size_t)(j + R2 * k1) * N + line];
-      inv_b<N>(u, j, line, s, tw);
-    }
+    if (j < R2) inv_b<N>(u, j, line, s, tw);
     __syncthreads();
     if (j < R1) {
       inv_a<N>(v, j, line, s);
@@ -191,23 +192,23 @@ __global__ void __launch_bounds__(LineTile<N>::NT) k_poisson_z(C* __restrict__ g
   const bool self_row = ky == 0 || ky == H;
   pdl_wait();
   if (self_row && x0 > H) return;
-  twiddles<N>(tw, twg, nullptr);
-  __syncthreads();
   const int line = threadIdx.x % TX, j = threadIdx.x / TX;
   const int kx = x0 + line, mx = (N - kx) % N, my = (N - ky) % N;
   const bool on = !self_row || kx <= H;
   C* gk = g + (size_t)ky * N + kx;
   C* gm = g + (size_t)my * N + mx;
+  C v[R2];
   if (on && j < R1) {
-    C v[R2];
 #pragma unroll
     for (int q = 0; q < R2; ++q) {
       const int z = j + R1 * q, jz = z < H ? z : z - H;
       const C a = gk[jz * P], b = gm[jz * P];  // b_j = (b.x, -b.y)
       v[q] = z < H ? make_double2(0.5 * (a.x + b.x), 0.5 * (a.y - b.y)) : make_double2(0.5 * (a.y + b.y), 0.5 * (b.x - a.x));
     }
-    fwd_a<N>(v, j, line, s, tw);
   }
+  twiddles<N>(tw, twg, nullptr);
+  __syncthreads();
+  if (on && j < R1) fwd_a<N>(v, j, line, s, tw);
   __syncthreads();
   C u[R1];
   if (on && j < R2) {
