@@ -227,6 +227,9 @@ struct tddft_ctx {
   double kin_A[3] = {0, 0, 0};
   bool ph_valid = false;
   double ph_A[3] = {0, 0, 0};
+  // Every call forms the tables it uses (a few us, once per value of A within the call): they are
+  // written in the call's own stream order, and a captured call carries their launches.
+  void new_call() { kin_valid = ph_valid = false; }
   void* gpart = nullptr;                      // gather partial sums of the chunks, and their counters
   int* gcount = nullptr;
   int* s_order = nullptr;                     // FP64: points by falling number of projector entries
@@ -805,8 +808,8 @@ cudaError_t epilogue(tddft_ctx* c, const void* kin, const void* Tk, const void* 
   return launch_epilogue<R>(c->st, c->N, kin, kin2, Tk, Tkm1, Tout, acc1, acc2, V, pt, dc, nkb, e);
 }
 
-// Multiplier parameters of the z pass at k + A, with the tables formed when A changes (they depend
-// on A, the k-points and the cell only).
+// Multiplier parameters of the z pass at k + A, with the tables formed when A changes within a call
+// (they depend on A, the k-points and the cell only).
 template <typename R> tddft_status kin_params(tddft_ctx* c, const double A[3], ZParams& zp) {
   const double pi = 3.14159265358979323846;
   for (int a = 0; a < 3; ++a) zp.gs[a] = 2.0 * pi / c->L[a];
@@ -836,7 +839,7 @@ template <typename R> tddft_status kinetic(tddft_ctx* c, const void* in, void* o
 
 // The phase tables of the CUDA-core projector kernels for this A, filled on the gather's stream: every
 // kernel that reads them follows a gather at the same A (on that stream or after its join).  They
-// depend on A, the k-points and the atoms only, so an unchanged A keeps them.
+// depend on A, the k-points and the atoms only, so an unchanged A keeps them within a call.
 template <typename R> tddft_status phases(tddft_ctx* c, const double A[3], const EpiParams& ep, cudaStream_t sg) {
   if (c->ph_valid && A[0] == c->ph_A[0] && A[1] == c->ph_A[1] && A[2] == c->ph_A[2]) return TDDFT_OK;
   c->ph_valid = false;
@@ -2128,6 +2131,7 @@ tddft_status tddft_set_fields(tddft_handle h, int nt, const double* t, const dou
 tddft_status tddft_set_states(tddft_handle h, const void* psi, int on_device, double t0) {
   if (!h) return TDDFT_ERR_ARG;
   if (!psi) return h->fail(TDDFT_ERR_ARG, "null psi");
+  h->new_call();
   return h->prec == TDDFT_FP64 ? do_set_states<double>(h, psi, on_device, t0) : do_set_states<float>(h, psi, on_device, t0);
 }
 
@@ -2141,6 +2145,7 @@ tddft_status tddft_get_states(tddft_handle h, void* psi, int on_device) {
 tddft_status tddft_set_states_c64(tddft_handle h, const void* psi, int on_device, double t0) {
   if (!h) return TDDFT_ERR_ARG;
   if (!psi) return h->fail(TDDFT_ERR_ARG, "null psi");
+  h->new_call();
   return h->prec == TDDFT_FP64 ? do_set_states<double>(h, psi, on_device, t0, true)
                                : do_set_states<float>(h, psi, on_device, t0, true);
 }
@@ -2156,6 +2161,7 @@ tddft_status tddft_step(tddft_handle h, int nsteps) {
   if (!h) return TDDFT_ERR_ARG;
   if (nsteps < 0) return h->fail(TDDFT_ERR_ARG, "nsteps must be >= 0");
   if (!h->have_states) return h->fail(TDDFT_ERR_STATE, "tddft_set_states must come first");
+  h->new_call();
   for (int i = 0; i < nsteps; ++i) {
     tddft_status s = h->prec == TDDFT_FP64 ? one_step<double>(h) : one_step<float>(h);
     if (s) return s;
@@ -2166,6 +2172,7 @@ tddft_status tddft_step(tddft_handle h, int nsteps) {
 tddft_status tddft_observables(tddft_handle h, double* n, double* m, double* E, double* M, double* norms) {
   if (!h) return TDDFT_ERR_ARG;
   if (!h->have_states) return h->fail(TDDFT_ERR_STATE, "no states loaded");
+  h->new_call();
   return h->prec == TDDFT_FP64 ? do_observables<double>(h, n, m, E, M, norms) : do_observables<float>(h, n, m, E, M, norms);
 }
 
@@ -2181,6 +2188,7 @@ tddft_status tddft_apply_hamiltonian(tddft_handle h, const void* in, void* out, 
   if (!h) return TDDFT_ERR_ARG;
   if (!in || !out || in == out) return h->fail(TDDFT_ERR_ARG, "bad in/out");
   if (!h->have_states) return h->fail(TDDFT_ERR_STATE, "no potential yet: call tddft_set_states first");
+  h->new_call();
   return h->prec == TDDFT_FP64 ? do_apply_h<double>(h, in, out, on_device) : do_apply_h<float>(h, in, out, on_device);
 }
 
@@ -2191,6 +2199,7 @@ tddft_status tddft_backward(tddft_handle h, int nsteps, int ckpt_every, const do
   if (h->spin_mode != TDDFT_SPIN_NONCOLLINEAR)
     return h->fail(TDDFT_ERR_UNSUPPORTED, "the adjoint covers the non-collinear mode only");
   if (!h->have_states) return h->fail(TDDFT_ERR_STATE, "tddft_set_states must come first");
+  h->new_call();
   return h->prec == TDDFT_FP64 ? do_backward<double>(h, nsteps, ckpt_every, dL_drho, loss, dL_dA, dL_dB)
                                : do_backward<float>(h, nsteps, ckpt_every, dL_drho, loss, dL_dA, dL_dB);
 }
@@ -2218,6 +2227,7 @@ tddft_status tddft_atom_moments(tddft_handle h, double* M, double* N) {
 tddft_status tddft_torques(tddft_handle h, double* soc, double* xc, double* zeeman) {
   if (!h) return TDDFT_ERR_ARG;
   if (!h->have_states) return h->fail(TDDFT_ERR_STATE, "no states loaded");
+  h->new_call();
   double A[3], B[3];
   h->fields(h->t, A, B);
   tddft_status s;

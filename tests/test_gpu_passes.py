@@ -92,6 +92,21 @@ def test_tables_follow_the_field(lib, precision):
     assert not np.array_equal(first[0], other[0])
 
 
+def test_every_call_forms_its_own_tables(lib):
+    """A call's launches do not depend on the calls before it."""
+    from paper_2506_21908_gb300 import _lib
+    wl, psi, _ = _system(16, 2, 3, 1)
+    h = _lib.TDDFT.from_workload(wl, precision=0, e_min=-30.0, e_max=250.0)
+    h.set_fields(wl.times, wl.A, wl.B)
+    h.set_states(psi, 0.0)
+    count = [h.info()["launches"]]
+    for _ in range(3):
+        h.apply_hamiltonian(psi)
+        count.append(h.info()["launches"])
+    h.close()
+    assert len(set(np.diff(count))) == 1
+
+
 def test_crank_nicolson_order_is_that_of_its_series(lib):
     """|rho| < 1 bounds the coefficients 4 |rho|^k / (beta |sqrt(x0^2 - 1)|): the FP64 order at 1e-16
     follows from the window and the step."""
