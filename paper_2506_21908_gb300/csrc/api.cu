@@ -1529,7 +1529,7 @@ void set_orders(tddft_ctx* c) {
     const int KM = 2048;
     auto cn = [&](double tau, int& K) {
       const cd alpha(1.0, 0.5 * tau * cc), x0 = cd(0.0, 1.0) * alpha / (0.5 * tau * dlt);
-      cd sq = std::sqrt(x0 * x0 - 1.0);
+      cd sq = std::sqrt(x0 - 1.0) * std::sqrt(x0 + 1.0);
       if (std::abs(x0 + sq) < std::abs(x0 - sq)) sq = -sq;
       const cd rho = 1.0 / (x0 + sq);
       const cd scale = cd(0.0, 4.0) / (0.5 * tau * dlt) / sq;  // 1 / (alpha + i beta x) = (i / beta) / (x0 - x)

@@ -124,6 +124,19 @@ def test_crank_nicolson_order_is_that_of_its_series(lib):
     assert K == int(np.nonzero(a >= 1e-16)[0].max())
 
 
+def test_crank_nicolson_with_a_vanishing_step_is_the_identity(lib):
+    from paper_2506_21908_gb300 import _lib
+    wl, psi, _ = _system(16, 1, 2, 1)
+    wl.dt = 1e-200
+    h = _lib.TDDFT.from_workload(wl, precision=0, exp_kind=2, e_min=-20.0, e_max=120.0)
+    h.set_states(psi, 0.0)
+    assert h.info()["K_full"] == 0
+    h.step(1)
+    out = h.get_states()
+    h.close()
+    assert rel(out, psi) <= 1e-15
+
+
 @pytest.mark.parametrize("nstates", [1, 33])
 def test_split_bricks_match_the_cuda_core_projectors(lib, nstates):
     """Bricks shared by two CTAs (fewer than 608) and a last component group of two: one step with the
