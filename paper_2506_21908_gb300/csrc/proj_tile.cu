@@ -265,7 +265,10 @@ k_tile_gather(const float2* __restrict__ psi, int N, int comps_per_k, int groups
   __shared__ float2 px[32], py[8], pz[8];
 
   // after a failed wait anywhere in the launch the remaining CTAs do nothing (the call reports it)
-  if (*reinterpret_cast<volatile int*>(err) & 1) return;
+  if (*reinterpret_cast<volatile int*>(err) & 1) {
+    pdl_wait();  // a launch never ends before its predecessor
+    return;
+  }
   const int kg = blockIdx.x, it = blockIdx.y;
   const int k = kg / groups, comp0 = (kg % groups) * 64;
   const int nslot = td.it_nslot[it], npad = td.it_npad[it];
@@ -617,7 +620,10 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
   __shared__ float2 px[32], py[8], pz[8];
   __shared__ float2 sph[256];  // exp(-i q.delta) per slot (at most 256 / nlm slots)
 
-  if (*reinterpret_cast<volatile int*>(err) & 1) return;
+  if (*reinterpret_cast<volatile int*>(err) & 1) {
+    pdl_wait();  // a launch never ends before its predecessor
+    return;
+  }
   const int kg = blockIdx.x, it = blockIdx.y;
   const int k = kg / sgroups, comp0 = (kg % sgroups) * SC;
   const int nslot = td.it_nslot[it], kch = td.it_kch[it];
