@@ -129,7 +129,7 @@ typedef struct {
  *   exp_kind  : TDDFT_EXP_CHEBYSHEV, TDDFT_EXP_TAYLOR, or TDDFT_EXP_CRANK_NICOLSON: the
  *               Cayley transform (1 + i tau H/2)^{-1} (1 - i tau H/2) in place of exp(-i tau H),
  *               applied through its own Chebyshev expansion on the spectral window (coefficients
- *               by Gauss-Chebyshev quadrature of the rational function, truncated like the
+ *               in closed form, truncated like the
  *               exponential's; equivalent to solving the linear system to that tolerance)
  *   exp_order : 0 = automatic (Chebyshev and Crank-Nicolson: smallest K with |a_k| < cheb_tol
  *               for all k > K, separately for dt and dt/2); > 0 = this order for every

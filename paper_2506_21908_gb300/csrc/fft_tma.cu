@@ -8,7 +8,7 @@
 // fill the other.  The first DFT stage reads the buffer in place; the rest of the transform is
 // that of k_fft_xy2 (one exchange per axis, the last stage writing HBM from registers), so the
 // results are the same bits.  (The z pass gains nothing from this form: with one exchange its
-// register-fed kernel keeps four CTAs per SM busy, against three for a double-buffered slab.)
+// register-fed kernel keeps more CTAs per SM busy than a double-buffered slab would leave.)
 //
 // Source and destination may be the same array: a CTA reads each plane (by the copy engine)
 // before it writes it, and no other CTA touches it.

@@ -2,7 +2,7 @@
 //
 //   k_fft_xy     one z-plane of one spinor component: 2D FFT along x then y in shared memory
 //   k_fft_z      one y-slab of one component: FFT along z, multiply by 1/2|G+k+A|^2, inverse FFT
-//                along z -- the kinetic term of Eq. HNC-SDFT
+//                along z -- the kinetic term of Eq. HNC-SDFT (k_fft_xy2, k_fft_z2_kin: two-factor sizes)
 //   k_proj_gather  c_{a,p,sigma} = sum_{r in S_a} beta~_p(r)^* psi_sigma(r) dV and D_a c
 //                (the contraction of the separable projectors, Eq. Vps with the L.S block)
 //   (k_epilogue, the pointwise Hamiltonian and Chebyshev update, is in epilogue.cu)

@@ -508,7 +508,8 @@ k_tile_gather(const float2* __restrict__ psi, int N, int comps_per_k, int groups
 // is used.  Bound by the latency of those loads: with one thread per component looping over the
 // projectors (64 threads, one pair at a time, 3 % of the warp slots) it took 241 us at the large
 // supercell with 32 spinors and 107 us at 64^3 with 48; gather and reduction together went from
-// 869 to 677 us per launch at the large supercell with 128 spinors.
+// 869 to 677 us per launch at the large supercell with 128 spinors (614 us with the gather's
+// groups added ahead of the conversion).
 constexpr int kRedPh = 256;
 __global__ void __launch_bounds__(64 * kMaxNLM)
 k_tile_reduce(const float* __restrict__ part, TileDev td, int groups, int comps_per_k, int nstates, int natoms,
