@@ -266,13 +266,16 @@ k_tile_gather(const float2* __restrict__ psi, int N, int comps_per_k, int groups
 
   // after a failed wait anywhere in the launch the remaining CTAs do nothing (the call reports it)
   if (*reinterpret_cast<volatile int*>(err) & 1) {
-    pdl_wait();  // a launch never ends before its predecessor
+    pdl_wait();  // a launch never ends before its predecessor, even if all its CTAs skip their work
     return;
   }
   const int kg = blockIdx.x, it = blockIdx.y;
   const int k = kg / groups, comp0 = (kg % groups) * 64;
   const int nslot = td.it_nslot[it], npad = td.it_npad[it];
-  if (nslot == 0) return;  // a brick no projector sphere reaches
+  if (nslot == 0) {  // a brick no projector sphere reaches
+    pdl_wait();
+    return;
+  }
   const int BX = td.BX;
   const int brick = td.it_brick[it];
   const int bx = brick % td.nbx, by = (brick / td.nbx) % td.nby, bz = brick / (td.nbx * td.nby);
@@ -628,7 +631,10 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
   const int kg = blockIdx.x, it = blockIdx.y;
   const int k = kg / sgroups, comp0 = (kg % sgroups) * SC;
   const int nslot = td.it_nslot[it], kch = td.it_kch[it];
-  if (AK < 0 && nslot == 0) return;  // nothing to add at this brick
+  if (AK < 0 && nslot == 0) {  // nothing to add at this brick
+    pdl_wait();
+    return;
+  }
   const bool has_nl = nslot > 0;
   const int BX = td.BX;
   const int brick = td.it_brick[it];

@@ -1,0 +1,54 @@
+"""GPU checks at the limits of what a handle accepts: spheres that hold no grid point, series of order 0
+and vanishing steps, the projector gather's splits that other tests' sizes do not reach, and calls that
+follow a refused one.  Against the FP64 oracle or a closed form."""
+import numpy as np
+import pytest
+
+from oracle import System
+from oracle.tddft import FieldTable
+from paper_2506_21908_gb300 import synthetic as S
+
+pytestmark = pytest.mark.gpu
+
+
+def rel(a, b):
+    return float(np.abs(np.asarray(a) - np.asarray(b)).max() / np.abs(np.asarray(b)).max())
+
+
+# FP64 1e-12 and FP32 2e-5 of the largest value: the bounds of the Hamiltonian apply at other systems.
+@pytest.mark.parametrize("precision,mode,tol", [(0, 0, 1e-12), (1, 1, 2e-5), (1, 2, 2e-5), (1, 3, 2e-5), (1, 4, 2e-5),
+                                                (1, 5, 2e-5)])
+def test_spheres_without_a_grid_point(lib, precision, mode, tol):
+    """Atoms between the grid points with a radius below their distance: no projector entry anywhere, so
+    every projector launch skips all of its blocks."""
+    from paper_2506_21908_gb300 import _lib
+    wl = S.small_parity(n=16, natoms=2, nstates=3, nk=2)
+    psi = S.small_parity_states(wl)
+    h0 = wl.L[0] / wl.n
+    wl.pos[:] = h0 * (np.array([[3, 5, 9], [12, 1, 6]]) + 0.5)
+    wl.r_cut = 0.5 * h0  # the nearest grid points are sqrt(3) / 2 spacings away
+    s = System.from_workload(wl)
+    A, B = FieldTable(wl.times, wl.A, wl.B).at(0.0)
+    V, _ = s.potential(s.rho_v(psi), B)
+    ref = s.apply_h(psi, V, A)
+    out = {}
+    for kind in (0, 1):  # Chebyshev (tensor cores: fused epilogue), Taylor (separate scatter)
+        h = _lib.TDDFT.from_workload(wl, precision=precision, proj_mode=mode, exp_kind=kind, e_min=-50.0, e_max=500.0)
+        h.set_fields(wl.times, wl.A, wl.B)
+        h.set_states(psi, 0.0)
+        assert rel(h.apply_hamiltonian(psi), ref) <= tol
+        assert np.abs(h.torques()["soc"]).max() == 0.0
+        h.step(1)
+        E = h.observables(fields=False)[2]
+        assert E["nl"] == 0.0
+        out[kind] = h.get_states()
+        if kind == 0 and precision == 0:
+            assert np.isfinite(h.backward(1, np.ones((4, wl.n ** 3)))[1]).all()
+        h.close()
+    # the same step by the CUDA-core form of the same precision
+    h = _lib.TDDFT.from_workload(wl, precision=precision, proj_mode=0 if precision == 0 else 1, e_min=-50.0, e_max=500.0)
+    h.set_fields(wl.times, wl.A, wl.B)
+    h.set_states(psi, 0.0)
+    h.step(1)
+    assert rel(out[0], h.get_states()) <= 2 * tol
+    h.close()
