@@ -37,11 +37,10 @@ template <int AK> struct EpiMinBlocks<float, AK> { static constexpr int value = 
 
 template <typename R, int NLM, int AK, int SP>
 __global__ void __launch_bounds__(256, EpiMinBlocks<R, AK>::value)
-k_epilogue(const typename CT<R>::type* __restrict__ kin, const typename CT<R>::type* __restrict__ kin2,
-           const typename CT<R>::type* Tk,
+k_epilogue(const typename CT<R>::type* kin, const typename CT<R>::type* kin2, const typename CT<R>::type* Tk,
            const typename CT<R>::type* Tkm1, typename CT<R>::type* Tout, typename CT<R>::type* acc1,
-           typename CT<R>::type* acc2, const R* __restrict__ V, size_t N3, ProjTables<R> pt,
-           const typename CT<R>::type* __restrict__ dc, EpiParams ep) {
+           typename CT<R>::type* acc2, const R* V, size_t N3, ProjTables<R> pt, const typename CT<R>::type* dc,
+           EpiParams ep) {
   using C = typename CT<R>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* dcs = reinterpret_cast<C*>(smem_raw);

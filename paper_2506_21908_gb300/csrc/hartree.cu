@@ -83,7 +83,7 @@ template <int N> __device__ __forceinline__ void inv_a(C* v, int n0, int line, c
 // inverse: real and imaginary parts of g back to the two planes of out.
 template <int N, bool INV>
 __global__ void __launch_bounds__(LineTile<N>::NT)
-k_poisson_x(const double* in, const double* in2, C* __restrict__ g, double* out, const C* __restrict__ twg, C* tw_out) {
+k_poisson_x(const double* in, const double* in2, C* g, double* out, const C* twg, C* tw_out) {
   using L = LineTile<N>;
   constexpr int R1 = L::R1, R2 = L::R2, TX = L::TX;
   constexpr size_t HALF = (size_t)N * N * N / 2;
@@ -140,7 +140,7 @@ k_poisson_x(const double* in, const double* in2, C* __restrict__ g, double* out,
 
 // y lines in place: TX neighbouring x of one packed plane (blockIdx.y).
 template <int N, bool INV>
-__global__ void __launch_bounds__(LineTile<N>::NT) k_poisson_y(C* __restrict__ g, const C* __restrict__ twg) {
+__global__ void __launch_bounds__(LineTile<N>::NT) k_poisson_y(C* g, const C* twg) {
   using L = LineTile<N>;
   constexpr int R1 = L::R1, R2 = L::R2, TX = L::TX;
   __shared__ C tw[N], s[N * TX];
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(LineTile<N>::NT) k_poisson_y(C* __restrict__ g
 // CTA: TX columns kx of the row ky = blockIdx.y <= N/2; rows 0 and N/2 mirror onto themselves, so
 // only their columns kx <= N/2 are taken (every mirror pair belongs to one line).
 template <int N>
-__global__ void __launch_bounds__(LineTile<N>::NT) k_poisson_z(C* __restrict__ g, const C* __restrict__ twg, ZParams zp) {
+__global__ void __launch_bounds__(LineTile<N>::NT) k_poisson_z(C* g, const C* twg, ZParams zp) {
   using L = LineTile<N>;
   constexpr int R1 = L::R1, R2 = L::R2, TX = L::TX, H = N / 2;
   constexpr size_t P = (size_t)N * N;

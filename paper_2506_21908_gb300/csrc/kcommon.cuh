@@ -19,6 +19,13 @@ template <int N> struct FFTMinBlocks<float, N> { static constexpr int value = (N
 // Programmatic dependent launch: the kernel may be set up before its predecessor on the stream has
 // ended, and calls pdl_wait() (which returns when it has, its writes visible) before it touches
 // memory the predecessor writes or reads.  2 us less between two short dependent kernels.
+//
+// A pointer that a kernel gets as const __restrict__, and a load by __ldg, promise the compiler that
+// nobody writes the data while the kernel lives; an unaliased pointer promises that pdl_wait() does
+// not concern it.  Either lets a load move above the wait.  So a kernel launched by launch_pdl
+// takes what any kernel of the chain writes through plain pointers and reads it by ordinary loads,
+// which the wait's memory clobber keeps behind it; the qualifiers are for the tables written at
+// creation only.  (Steps at 48^3, 64^3 and 96^3 measure the same within 0.4 % either way.)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Opt in to a kernel's dynamic shared memory, once per device (the attribute calls cost more host time

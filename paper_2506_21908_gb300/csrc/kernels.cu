@@ -189,8 +189,7 @@ __global__ void k_kin_tables(ZParams zp, R* __restrict__ out) {
 // tx[x] + ty[y] + tz[kz] and transforms back in registers, A side writes global memory.
 template <typename R, int N>
 __global__ void __launch_bounds__(ZThreads<R, N>::value, ZBlocks<R, N>::value)
-k_fft_z2_kin(typename CT<R>::type* __restrict__ data, const typename CT<R>::type* __restrict__ twg,
-             const R* __restrict__ tab, int comps_per_k) {
+k_fft_z2_kin(typename CT<R>::type* data, const typename CT<R>::type* __restrict__ twg, const R* tab, int comps_per_k) {
   using C = typename CT<R>::type;
   using TFW = TF<C, N, false>;
   using TIN = TF<C, N, true>;
@@ -198,6 +197,7 @@ k_fft_z2_kin(typename CT<R>::type* __restrict__ data, const typename CT<R>::type
   constexpr int R1 = TwoFactor<N>::R1, R2 = TwoFactor<N>::R2;
   constexpr int IA = CW * R1, IB = CW * R2;
   constexpr int PA = (IA + NT - 1) / NT, PB = (IB + NT - 1) / NT;
+  static_assert(NT % CW == 0, "a thread's items share one column");
   __shared__ C tw[N];
   __shared__ R tz[N];
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -220,7 +220,7 @@ k_fft_z2_kin(typename CT<R>::type* __restrict__ data, const typename CT<R>::type
   }
   const R* tk = tab + (size_t)(b / comps_per_k) * 3 * N;
   for (int i = threadIdx.x; i < N; i += NT) tz[i] = tk[2 * N + i];
-  const R tyv = tk[N + y];
+  const R txy = tk[x0 + threadIdx.x % CW] + tk[N + y];
   __syncthreads();  // tables
 #pragma unroll
   for (int p = 0; p < PA; ++p) {
@@ -242,7 +242,6 @@ k_fft_z2_kin(typename CT<R>::type* __restrict__ data, const typename CT<R>::type
 #pragma unroll
       for (int n0 = 0; n0 < R1; ++n0) u[n0] = s[(k0 * R1 + n0) * CW + x];
       TFW::b_side(u, k0, tw);
-      const R txy = tk[x0 + x] + tyv;
 #pragma unroll
       for (int k1 = 0; k1 < R1; ++k1) u[k1] = cscale(u[k1], txy + tz[k0 + R2 * k1]);
       TIN::b_side(u, k0, tw);
@@ -464,7 +463,7 @@ template <typename R> cudaError_t launch_kin_tables(cudaStream_t st, int N, int 
 // cost the gather, whose bound is the FP64 pipe).
 template <typename R>
 __global__ void __launch_bounds__(256)
-k_phase_table(size_t nent, const R* __restrict__ rows, EpiParams ep, typename CT<R>::type* __restrict__ out) {
+k_phase_table(size_t nent, const R* __restrict__ rows, EpiParams ep, typename CT<R>::type* out) {
   using C = typename CT<R>::type;
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= nent) return;
@@ -561,9 +560,8 @@ template <> struct GatherMinBlocks<float> { static constexpr int value = 4; };
 
 template <typename R, int NLM, int SPN>
 __global__ void __launch_bounds__(PG_NT, GatherMinBlocks<R>::value)
-k_proj_gather(const typename CT<R>::type* __restrict__ psi, size_t N3, ProjTables<R> pt, R dV, int nstates, int chunks,
-              R* __restrict__ part, int* __restrict__ counters, typename CT<R>::type* __restrict__ c_out,
-              typename CT<R>::type* __restrict__ dc_out) {
+k_proj_gather(const typename CT<R>::type* psi, size_t N3, ProjTables<R> pt, R dV, int nstates, int chunks, R* part,
+              int* counters, typename CT<R>::type* c_out, typename CT<R>::type* dc_out) {
   using C = typename CT<R>::type;
   constexpr int NS = 4 * NLM;    // reals per spinor: (re, im) x (up, dn) x NLM
   constexpr int NV = SPN * NS;
@@ -734,8 +732,7 @@ cudaError_t launch_proj_gather(cudaStream_t st, int N, const void* psi, int nkb,
 // added in a fixed order (deterministic result).
 template <typename R>
 __global__ void __launch_bounds__(256)
-k_density(const typename CT<R>::type* __restrict__ psi, size_t N3, int nkb, int ngroups,
-          const double* __restrict__ wf, double* __restrict__ out) {
+k_density(const typename CT<R>::type* psi, size_t N3, int nkb, int ngroups, const double* __restrict__ wf, double* out) {
   const size_t r = 2 * ((size_t)blockIdx.x * blockDim.x + threadIdx.x);
   if (r >= N3) return;
   const int g = blockIdx.y;
@@ -773,7 +770,7 @@ k_density(const typename CT<R>::type* __restrict__ psi, size_t N3, int nkb, int 
   for (int c = 0; c < 4; ++c) *reinterpret_cast<double2*>(o + c * N3 + r) = make_double2(s[0][c], s[1][c]);
 }
 
-__global__ void k_density_reduce(size_t n, int ngroups, const double* __restrict__ part, double* __restrict__ rho) {
+__global__ void k_density_reduce(size_t n, int ngroups, const double* part, double* rho) {
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   pdl_wait();
@@ -858,10 +855,8 @@ __device__ void lsda_point(double nu, double nd, double* e, double* vu, double* 
 // Bound by the FP64 pipe (some 600 instructions a point); small CTAs spread a small grid over the
 // SMs (24^3: 30 us on 54 CTAs of 256).
 constexpr int kPotThreads = 64;
-__global__ void __launch_bounds__(kPotThreads) k_potential(size_t N3, const double* __restrict__ rho, const double* __restrict__ vH,
-                            const double* __restrict__ vloc, double Bx, double By, double Bz, int xc, int mode,
-                            double* __restrict__ V, float* __restrict__ Vf, double* __restrict__ exc,
-                            double* __restrict__ vxc4) {
+__global__ void __launch_bounds__(kPotThreads) k_potential(size_t N3, const double* rho, const double* vH, const double* __restrict__ vloc, double Bx, double By,
+                            double Bz, int xc, int mode, double* V, float* Vf, double* exc, double* vxc4) {
   const size_t r = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= N3) return;
   pdl_wait();
@@ -1264,8 +1259,8 @@ cudaError_t launch_max_abs_diff(cudaStream_t st, size_t n, const double* a, cons
 }
 
 // Sets *flag when the local potential leaves [lo, hi] given the kinetic maximum and projector bound.
-__global__ void k_check_window(size_t N3, const double* __restrict__ V, double lo, double hi, double kin_max,
-                               double nl_bound, int* flag) {
+__global__ void k_check_window(size_t N3, const double* V, double lo, double hi, double kin_max, double nl_bound,
+                               int* flag) {
   const size_t r = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= N3) return;
   pdl_wait();

@@ -246,11 +246,21 @@ constexpr int PT_MMA_WARP = PT_WARPS, PT_COPY_WARP = PT_WARPS + 1;
 // falls with the length of a group.
 template <int TERMS> struct GatherGroups { static constexpr int CPG = (TERMS == 3) ? 4 : 8; };
 
+// Spinors, read once by a CTA: ordinary loads past L1, in program order with the waits (asm volatile),
+// since pdl_wait() has to precede them.  Requested after the arrival that the MMAs of the staged chunk
+// wait for, they take the gather from 615 to 600 us (96^3, 128 atoms, 128 spinors) and from 651 to
+// 632 us (48^3 x 1024) against read-only loads through L1; before that arrival 603 and 637 us.
+__device__ __forceinline__ void ld_stream(float4& v, const void* p) {
+  asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+}
+__device__ __forceinline__ void ld_stream(float2& v, const void* p) {
+  asm volatile("ld.global.cg.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+}
+
 // CTA (kg, item): 64 components (group g of k-point k) against the slots of one brick.
 template <int EK, int TERMS>
 __global__ void __launch_bounds__(PT_NT, 1)
-k_tile_gather(const float2* __restrict__ psi, int N, int comps_per_k, int groups, TileDev td, EpiParams ep,
-              float* __restrict__ part, int* __restrict__ err) {
+k_tile_gather(const float2* psi, int N, int comps_per_k, int groups, TileDev td, EpiParams ep, float* part, int* err) {
   constexpr int EPR = PT_ROWB / Elt<EK>::bytes;  // points per chunk (K elements per row)
   constexpr int NPART = (TERMS == 3) ? 2 : 1;
   constexpr int BPART = 256 * PT_ROWB;          // largest B part (N <= 256)
@@ -321,7 +331,7 @@ k_tile_gather(const float2* __restrict__ psi, int N, int comps_per_k, int groups
       V v;
       if constexpr (PPL == 2) v = make_float4(0.f, 0.f, 0.f, 0.f);
       else v = make_float2(0.f, 0.f);
-      if (j < nvalid) v = __ldg(reinterpret_cast<const V*>(gbase + (o + (uint32_t)j * n3b)));
+      if (j < nvalid) ld_stream(v, gbase + (o + (uint32_t)j * n3b));
       w[j] = v;
     }
   };
@@ -414,9 +424,9 @@ k_tile_gather(const float2* __restrict__ psi, int N, int comps_per_k, int groups
           *reinterpret_cast<uint32_t*>(q + PT_PART + 64 * PT_ROWB) = il;
         }
       }
-      if (c + 2 < nch) load(c + 2, w);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       pt_arrive(sm_addr(&bar_full[s]));
+      if (c + 2 < nch) load(c + 2, w);
       return true;
     };
     for (int c = 0; c < nch; c += 2)  // nch is even
@@ -515,9 +525,8 @@ k_tile_gather(const float2* __restrict__ psi, int N, int comps_per_k, int groups
 // groups added ahead of the conversion).
 constexpr int kRedPh = 256;
 __global__ void __launch_bounds__(64 * kMaxNLM)
-k_tile_reduce(const float* __restrict__ part, TileDev td, int groups, int comps_per_k, int nstates, int natoms,
-              float dV, EpiParams ep, const float* __restrict__ Dmat, float2* __restrict__ c_out,
-              float2* __restrict__ dc_out) {
+k_tile_reduce(const float* part, TileDev td, int groups, int comps_per_k, int nstates, int natoms, float dV,
+              EpiParams ep, const float* __restrict__ Dmat, float2* c_out, float2* dc_out) {
   const int a = blockIdx.x, kg = blockIdx.y;
   const int k = kg / groups, comp0 = (kg % groups) * 64;
   const int nlm = td.nlm;
@@ -549,8 +558,8 @@ k_tile_reduce(const float* __restrict__ part, TileDev td, int groups, int comps_
         re[j] = im[j] = 0.f;
         if (i + j < nb) {
           const float* src = base + so[i + j];
-          re[j] = __ldg(src);
-          im[j] = __ldg(src + 64);
+          re[j] = src[0];
+          im[j] = src[64];
         }
       }
 #pragma unroll
@@ -609,7 +618,7 @@ __device__ __forceinline__ void prefetch_l2_line(const void* p) { asm volatile("
 template <int EK, int TERMS, int AK>
 __global__ void __launch_bounds__(ST_NT, 1)
 k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, int natoms, TileDev td, EpiParams ep,
-               const float2* __restrict__ dc, int* __restrict__ err, EpiIO io) {
+               const float2* dc, int* err, EpiIO io) {
   constexpr int EPR = PT_ROWB / Elt<EK>::bytes;    // projector indices per K chunk
   constexpr int SC = (Elt<EK>::bytes == 4) ? 32 : 64;  // components per CTA
   constexpr int NPART = (TERMS == 3) ? 2 : 1;
@@ -707,7 +716,7 @@ k_tile_scatter(float2* out, int N, int comps_per_k, int sgroups, int nstates, in
           if (comp < comps_per_k) {
             const int a = td.slot_atom[(size_t)it * td.smax + sl];
             const size_t kb = (size_t)k * nstates + (comp >> 1);
-            f[u] = __ldg(dc4 + (kb * natoms + a) * nlm + p);
+            f[u] = dc4[(kb * natoms + a) * nlm + p];
           }
         }
       }

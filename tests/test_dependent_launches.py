@@ -61,3 +61,15 @@ def test_no_block_leaves_before_its_predecessor():
                 assert guard or before.strip().endswith("pdl_wait();"), (name, stmt)
             elif not re.match(r"\s*return;", body[m.end():]):
                 break
+
+
+# Written when a handle is created, before any launch of the chain: twiddles, weights, projector rows and
+# blocks, the local potential.  The Poisson kernels' twiddles may be written by the first of them.
+CREATED = {"twg", "wf", "rows", "vloc", "Dmat"}
+
+
+def test_what_a_predecessor_writes_is_not_promised_read_only():
+    for name, (params, body) in dependent_kernels().items():
+        allowed = set() if name.startswith("k_poisson") else CREATED
+        assert set(re.findall(r"__restrict__\s+(\w+)", params)) <= allowed, name
+        assert "__ldg(" not in body, name
