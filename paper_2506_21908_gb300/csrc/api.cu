@@ -960,6 +960,13 @@ static void acc_schedule(int k, int Ka, const std::vector<cd>& cf, const double*
   done = last + 1;
 }
 
+// acc = cf0 in, a series of order 0, which no epilogue updates; cf0 as hi + lo in FP32.
+template <typename R> tddft_status order0(tddft_ctx* c, const void* in, cd cf0, void* acc) {
+  const double hi[2] = {(double)(R)cf0.real(), (double)(R)cf0.imag()};
+  const double lo[2] = {cf0.real() - hi[0], cf0.imag() - hi[1]};
+  return c->launch(KC_OTHER, "order 0", [&] { return launch_seed<R>(c->st, c->psi_elems(), in, hi, in, lo, acc); });
+}
+
 // One Chebyshev series: T_k of H~ = (H - c)/Delta applied to `in`, accumulated with
 // coefficients cf1 (orders 0..K1) into acc1 and, when acc2 is set, cf2 (0..K2) into acc2.
 template <typename R>
@@ -988,6 +995,8 @@ tddft_status cheb_series(tddft_ctx* c, const void* in, const R* Vr, const double
   ep.real_coef = c->real_series ? 1 : 0;
   ep.ph1[0] = phase_of(cf1).real(); ep.ph1[1] = phase_of(cf1).imag();
   ep.ph2[0] = phase_of(cf2).real(); ep.ph2[1] = phase_of(cf2).imag();
+  if (K1 == 0 && (s = order0<R>(c, in, cf1[0], acc1))) return s;
+  if (acc2 && K2 == 0 && (s = order0<R>(c, in, cf2[0], acc2))) return s;
   for (int k = 0; k < K; ++k) {
     if ((s = kinetic_and_gather<R>(c, cur, A, !fuse))) return s;
     void* out;
@@ -1312,7 +1321,7 @@ tddft_status adjoint_step(tddft_ctx* c, AdjWork& w, const void* psi_n, double t0
   bool have_phibar = false;
   for (int j = c->n_sc; j >= 0; --j) {
     if ((s = c->cuda(cudaMemsetAsync(w.gV, 0, 4 * c->N3 * sizeof(double), c->st), "gV reset"))) return s;
-    std::vector<const void*> T(Kh);
+    std::vector<const void*> T(std::max(Kh, 1));
     T[0] = w.phi;
     for (int k = 1; k < Kh; ++k) T[k] = w.slots2[j][k];
     void* xbar = nullptr;
@@ -1332,7 +1341,7 @@ tddft_status adjoint_step(tddft_ctx* c, AdjWork& w, const void* psi_n, double t0
   }
   // ---- reverse through series 1 (shared terms for psi~ and phi) at t
   if ((s = c->cuda(cudaMemsetAsync(w.gV, 0, 4 * c->N3 * sizeof(double), c->st), "gV reset"))) return s;
-  std::vector<const void*> T(K1);
+  std::vector<const void*> T(std::max(K1, 1));
   T[0] = psi_n;
   for (int k = 1; k < K1; ++k) T[k] = w.slots1[k];
   void* xbar = nullptr;

@@ -52,3 +52,37 @@ def test_spheres_without_a_grid_point(lib, precision, mode, tol):
     h.step(1)
     assert rel(out[0], h.get_states()) <= 2 * tol
     h.close()
+
+
+# The order-0 coefficient is the mean of the exponential (or of the Cayley transform) over the window with
+# the Chebyshev weight.  psi takes the half step's coefficient twice; FP32 rounds three times (6e-8 each).
+# Orders: the exponential drops |J_1| < tol, the Cayley transform |a_1| < tol, about 2 |J_1|.
+@pytest.mark.parametrize("precision,tol", [(0, 1e-14), (1, 4e-7)])
+@pytest.mark.parametrize("kind,cheb_tol,orders", [(0, 0.05, (0, 0)), (0, 0.025, (1, 0)), (2, 0.1, (0, 0)), (2, 0.05, (1, 0))])
+def test_series_of_order_zero(lib, precision, tol, kind, cheb_tol, orders):
+    """Both orders 0, and the half step's alone: the states take the coefficient, the potential and the
+    density are those of the states, and nothing of them depends on the fields."""
+    from paper_2506_21908_gb300 import _lib
+    wl = S.small_parity(n=16, natoms=1, nstates=2, nk=1)
+    wl.dt = 1e-3
+    psi = S.small_parity_states(wl)
+    lo, hi = -20.0, 120.0
+    E = 0.5 * (lo + hi) + 0.5 * (hi - lo) * np.cos(np.pi * (np.arange(64) + 0.5) / 64)
+    tau = 0.5 * wl.dt
+    f = np.exp(-1j * tau * E) if kind == 0 else (1 - 0.5j * tau * E) / (1 + 0.5j * tau * E)
+    cf = f.mean()
+    h = _lib.TDDFT.from_workload(wl, precision=precision, exp_kind=kind, cheb_tol=cheb_tol, e_min=lo, e_max=hi)
+    h.set_fields(wl.times, wl.A, wl.B)
+    h.set_states(psi, 0.0)
+    assert (h.info()["K_full"], h.info()["K_half"]) == orders
+    h.step(1)
+    n, m, _, norms = h.observables()
+    assert rel(h.get_states(), cf * cf * psi) <= tol
+    assert np.abs(norms - abs(cf) ** 4).max() <= 2 * tol
+    s = System.from_workload(wl)
+    V, _ = s.potential(s.rho_v(cf * cf * psi), FieldTable(wl.times, wl.A, wl.B).at(wl.dt)[1])
+    assert rel(h.get_potential(), V) <= 4 * tol + 1e-12
+    h.set_states(psi, 0.0)
+    _, dA, dB = h.backward(1, np.random.default_rng(1).normal(size=(4, wl.n ** 3)))
+    assert not dA.any() and not dB.any()
+    h.close()
