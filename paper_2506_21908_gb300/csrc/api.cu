@@ -125,6 +125,11 @@ std::vector<double> bessel_j(int kmax, double z) {
     return J;
   }
   const double az = std::fabs(z);
+  if (az < 1e-50) {  // the recurrence below would overflow; 1 - J_0 and J_2 are below 1e-100
+    J[0] = 1.0;
+    if (kmax >= 1) J[1] = 0.5 * z;
+    return J;
+  }
   const int start = std::max(kmax, (int)az) + 60 + (int)(2.0 * std::sqrt(az + 1.0) * 10.0);
   std::vector<double> w(start + 2, 0.0);
   w[start + 1] = 0.0;

@@ -86,3 +86,25 @@ def test_series_of_order_zero(lib, precision, tol, kind, cheb_tol, orders):
     _, dA, dB = h.backward(1, np.random.default_rng(1).normal(size=(4, wl.n ** 3)))
     assert not dA.any() and not dB.any()
     h.close()
+
+
+# Every coefficient but the first vanishes and that one is 1: no rounding but the density's own.
+@pytest.mark.parametrize("kind", [0])
+@pytest.mark.parametrize("dt", [1e-60, -1e-200, 1e-310])
+@pytest.mark.parametrize("order", [0, 1, 4])
+def test_a_vanishing_step_is_the_identity(lib, kind, dt, order):
+    from paper_2506_21908_gb300 import _lib
+    wl = S.small_parity(n=16, natoms=1, nstates=2, nk=1)
+    wl.dt = dt
+    psi = S.small_parity_states(wl)
+    h = _lib.TDDFT.from_workload(wl, precision=0, exp_kind=kind, exp_order=order, e_min=-20.0, e_max=120.0)
+    h.set_states(psi, 0.0)
+    info = h.info()
+    assert (info["K_full"], info["K_half"]) == (order, order)
+    V = h.get_potential()
+    h.step(1)
+    norms = h.observables(fields=False)[3]
+    assert rel(h.get_states(), psi) <= 1e-15
+    assert rel(h.get_potential(), V) <= 1e-14
+    assert np.abs(norms - 1.0).max() <= 1e-12
+    h.close()
