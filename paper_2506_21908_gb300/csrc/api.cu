@@ -1538,15 +1538,14 @@ void set_orders(tddft_ctx* c) {
     // alpha = 1 + i tau c/2, beta = tau Delta/2, and the generating function of the Chebyshev
     // polynomials gives 1 / (x0 - x) = (1 + 2 sum_k rho^k T_k(x)) / sqrt(x0^2 - 1) for the pole
     // x0 = i alpha / beta off the window, rho = x0 - sqrt(x0^2 - 1) = 1 / (x0 + sqrt(x0^2 - 1)),
-    // |rho| < 1.  (A quadrature over 4096 nodes cost 63 ms of host time per exponential.)
+    // |rho| < 1.  In u = 1 / x0 = beta / (i alpha), which stays finite for any step, s = sqrt(1 - u^2)
+    // (Re s > 0): rho = u / (1 + s), and f = -1 + 2 / (alpha s) (1 + 2 sum_k rho^k T_k(x)).  (A
+    // quadrature over 4096 nodes cost 63 ms of host time per exponential.)
     const double tol = c->cheb_tol > 0 ? c->cheb_tol : (c->prec == TDDFT_FP64 ? 1e-16 : 1e-9);
     const int KM = 2048;
     auto cn = [&](double tau, int& K) {
-      const cd alpha(1.0, 0.5 * tau * cc), x0 = cd(0.0, 1.0) * alpha / (0.5 * tau * dlt);
-      cd sq = std::sqrt(x0 - 1.0) * std::sqrt(x0 + 1.0);
-      if (std::abs(x0 + sq) < std::abs(x0 - sq)) sq = -sq;
-      const cd rho = 1.0 / (x0 + sq);
-      const cd scale = cd(0.0, 4.0) / (0.5 * tau * dlt) / sq;  // 1 / (alpha + i beta x) = (i / beta) / (x0 - x)
+      const cd alpha(1.0, 0.5 * tau * cc), u = 0.5 * tau * dlt / (cd(0.0, 1.0) * alpha);
+      const cd sq = std::sqrt((1.0 - u) * (1.0 + u)), rho = u / (1.0 + sq), scale = 4.0 / (alpha * sq);
       std::vector<cd> a(KM);
       a[0] = 0.5 * scale - 1.0;
       cd r = rho;

@@ -89,7 +89,7 @@ def test_series_of_order_zero(lib, precision, tol, kind, cheb_tol, orders):
 
 
 # Every coefficient but the first vanishes and that one is 1: no rounding but the density's own.
-@pytest.mark.parametrize("kind", [0])
+@pytest.mark.parametrize("kind", [0, 2])
 @pytest.mark.parametrize("dt", [1e-60, -1e-200, 1e-310])
 @pytest.mark.parametrize("order", [0, 1, 4])
 def test_a_vanishing_step_is_the_identity(lib, kind, dt, order):
