@@ -125,28 +125,34 @@ k_fft_xy2_tma(const float2* src, float2* dst, const float2* __restrict__ twg, in
 
 bool fft_xy_tma_supported(int N) { return N == 16 || N == 24 || N == 32 || N == 48 || N == 64; }
 
+// CTAs of a full wave on the current device, asked once per device and kernel.
+template <int N, bool INV>
+static cudaError_t xy_tma_ni(cudaStream_t st, const void* src, void* dst, int nbatch, const void* tw, int* err) {
+  const size_t smem = (size_t)(N + 2 * N * TmaPitch<N>::value) * sizeof(float2) + 2 * sizeof(uint64_t);
+  auto kf = k_fft_xy2_tma<N, INV>;
+  static std::atomic<unsigned long long> done{0};
+  static std::atomic<int> wave[64];
+  int dev = 0;
+  cudaError_t e;
+  if ((e = opt_in_smem(kf, smem, done)) != cudaSuccess || (e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  int ctas = wave[dev & 63].load(std::memory_order_relaxed);
+  if (!ctas) {
+    int sms = 0, per_sm = 0;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kf, XYThreads<N>::value, smem)) != cudaSuccess)
+      return e;
+    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    ctas = sms * per_sm;
+    wave[dev & 63].store(ctas, std::memory_order_relaxed);
+  }
+  const int nplanes = N * nbatch;
+  return launch_pdl(kf, dim3(std::min(nplanes, ctas)), XYThreads<N>::value, smem, st, (const float2*)src, (float2*)dst,
+                    (const float2*)tw, nplanes, err);
+}
 template <int N>
 static cudaError_t xy_tma_n(cudaStream_t st, const void* src, void* dst, int nbatch, const void* tw, bool inv,
                             int* err) {
-  const size_t smem = (size_t)(N + 2 * N * TmaPitch<N>::value) * sizeof(float2) + 2 * sizeof(uint64_t);
-  auto kf = inv ? k_fft_xy2_tma<N, true> : k_fft_xy2_tma<N, false>;
-  static int per_sm[2] = {0, 0};
-  static int sms = 0;
-  int& ps = per_sm[inv ? 1 : 0];
-  if (!ps) {
-    cudaError_t e;
-    if ((e = cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-    cudaFuncSetAttribute(kf, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-    int dev = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, kf, XYThreads<N>::value, smem)) != cudaSuccess) return e;
-    if (ps < 1) return cudaErrorInvalidConfiguration;
-  }
-  const int nplanes = N * nbatch;
-  const int grid = std::min(nplanes, sms * ps);
-  return launch_pdl(kf, dim3(grid), XYThreads<N>::value, smem, st, (const float2*)src, (float2*)dst, (const float2*)tw,
-                    nplanes, err);
+  return inv ? xy_tma_ni<N, true>(st, src, dst, nbatch, tw, err) : xy_tma_ni<N, false>(st, src, dst, nbatch, tw, err);
 }
 
 cudaError_t launch_fft_xy_tma(cudaStream_t st, int N, const void* src, void* dst, int nbatch, const void* tw, bool inv,

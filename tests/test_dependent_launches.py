@@ -73,3 +73,11 @@ def test_what_a_predecessor_writes_is_not_promised_read_only():
         allowed = set() if name.startswith("k_poisson") else CREATED
         assert set(re.findall(r"__restrict__\s+(\w+)", params)) <= allowed, name
         assert "__ldg(" not in body, name
+
+
+def test_launchers_keep_no_unsynchronised_state():
+    """What a launcher remembers between calls (opted-in kernels, waves of a device) is shared by host
+    threads and devices: per-device atomics, no plain variable."""
+    for file, text in _sources().items():
+        local = re.findall(r"^[ \t]+static\s+(?!const\b|constexpr\b|std::atomic\b)[^;({]*[;={]", text, re.M)
+        assert not local, (file, local)
