@@ -167,6 +167,10 @@ typedef struct {
 
 /* Create a handle on the current CUDA device: validates the inputs, builds the G mesh,
  * the local potential, projector tables and L.S blocks, and allocates device memory.
+ * Per projector entry (a grid point in an atom's sphere) the handle holds two compact rows of four
+ * reals and, with CUDA-core projectors, two phases of every k-point (16 nk bytes in FP32-mixed, 32 nk
+ * in FP64) and in FP64 two rows of projector values ((lmax + 1)^2 rounded up to even, 160 bytes at
+ * lmax = 2).  96^3 with 128 atoms has 5.8 M entries: 1.5 GB in FP64 at one k-point.
  * *out receives the handle (NULL on failure). */
 tddft_status tddft_create(const tddft_cell* cell, const tddft_grid* grid, const tddft_atoms* atoms,
                           const tddft_projectors* proj, const tddft_params* params,
@@ -225,7 +229,8 @@ tddft_status tddft_apply_hamiltonian(tddft_handle h, const void* in, void* out, 
  * potential's dependence on the density through Hartree and the locally collinear LSDA
  * (analytic Jacobian), the velocity-gauge kinetic term and projector phases, and the Zeeman term.
  * Memory: spinor copies at every ckpt_every-th step (checkpoints), ckpt_every copies for the
- * recomputed segment, and one copy per Chebyshev term of a step, allocated for the call only.
+ * recomputed segment, one copy per Chebyshev term of a step, and with tensor-core projectors the
+ * phases of the CUDA-core gather (tddft_create), allocated for the call only.
  * Requires Chebyshev or Crank-Nicolson exponentials, sc_tol = 0, and two z-slabs of the grid in shared memory
  * (n <= 64 in FP64, n <= 96 in FP32-mixed); otherwise TDDFT_ERR_UNSUPPORTED.  The paper has no
  * adjoint; the loss and parameterisation follow the differentiation workload of this library. */
@@ -303,7 +308,7 @@ tddft_status tddft_profile_read(tddft_handle h, int ncls, double* ms, long long*
  * synchronising.
  *
  * It allocates nothing: no cudaMalloc, cudaFree or allocating library routine.  Its scratch
- * is one file-scope static device array of 64^3 + 64 complex FP64 values (4 MiB + 1 KiB),
+ * is one file-scope static device array of 64^3 / 2 + 64 complex FP64 values (2 MiB + 1 KiB),
  * present on every GPU that loads the library until the process exits.  Hence n must be one
  * of 8, 12, 16, 24, 32, 48, 64; larger grids return TDDFT_ERR_ARG.  The first call on a device
  * looks up that array's device address (cudaGetSymbolAddress) and keeps it for the life of the

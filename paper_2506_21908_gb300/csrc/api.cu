@@ -203,7 +203,7 @@ struct tddft_ctx {
   std::vector<void*> allocs;
   void *psi = nullptr, *phi = nullptr, *pred = nullptr, *Ta = nullptr, *Tb = nullptr, *tmp = nullptr;
   void *cbuf = nullptr, *dcbuf = nullptr, *tw = nullptr;
-  double2 *tw64 = nullptr, *hart = nullptr, *stage = nullptr;
+  double2 *tw64 = nullptr, *hart = nullptr, *stage = nullptr;  // hart: N^3 / 2, the packed planes of the Poisson solve
   size_t stage_elems = 0;
   double* rho_part = nullptr;  // band-group partial densities
   double *rho = nullptr, *rho2 = nullptr, *rho3 = nullptr, *V = nullptr, *Vnew = nullptr, *vloc = nullptr,
@@ -225,7 +225,7 @@ struct tddft_ctx {
   void* vnl = nullptr;         // V_NL T_k from the tensor-core scatter (spinor layout)
   int* tc_err = nullptr;     // wait errors: bit 1 tensor-core projector, bit 2 bulk-copy FFT pass
   void *g_row = nullptr, *s_row = nullptr, *nrm = nullptr, *Dmat = nullptr;
-  void *g_ph = nullptr, *s_ph = nullptr;      // phases exp(i (k + A).d) at A = ph_A
+  void *g_ph = nullptr, *s_ph = nullptr;      // phases exp(i (k + A).d) at A = ph_A (see proj_workspace)
   void *g_beta = nullptr, *s_beta = nullptr;  // FP64 projector values
   void* kin_tab = nullptr;                    // kinetic factors [nk][3][N] at A = kin_A
   bool kin_valid = false;
@@ -749,6 +749,21 @@ tddft_status upload(tddft_ctx* c, T** dst, const std::vector<T>& src, const char
   tddft_status s = c->alloc(dst, src.size() * sizeof(T), what);
   if (s) return s;
   return c->cuda(cudaMemcpy(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice), what);
+}
+
+// Phase tables, partial sums and counters of the CUDA-core gather.  A handle with tensor-core projectors
+// runs that gather in the reverse sweep alone and holds them for that call (do_backward): 16 nk bytes
+// per entry in FP32, 32 nk in FP64, and the partial sums.
+template <class F> tddft_status proj_workspace(tddft_ctx* c, F&& alloc) {
+  const size_t ph = c->n_entries * c->nk * 2 * c->rsize();
+  const size_t ncnt = proj_gather_counters(c->natoms, c->nk, c->nb) * sizeof(int);
+  tddft_status s;
+  if ((s = alloc(&c->g_ph, ph, "phases")) || (s = alloc(&c->s_ph, ph, "phases")) ||
+      (s = alloc(&c->gpart, proj_gather_part_bytes(c->natoms, c->nlm, c->nk, c->nb, c->n_entries, c->rsize()),
+                 "gather partials")) ||
+      (s = alloc(reinterpret_cast<void**>(&c->gcount), ncnt, "gather counters")))
+    return s;
+  return c->cuda(cudaMemsetAsync(c->gcount, 0, ncnt, c->st), "gather counters init");
 }
 
 // ------------------------------------------------------------------ potential pipeline
@@ -1403,6 +1418,15 @@ tddft_status do_backward(tddft_ctx* c, int nsteps, int ckpt, const double* dL_dr
   std::vector<double> gAt(3 * std::max<size_t>(nt, 1), 0.0), gBt(3 * std::max<size_t>(nt, 1), 0.0);
   DevBuf db;
   AdjWork w;
+  struct Borrowed {  // the gather's workspace of a tensor-core handle is the call's own (in db)
+    tddft_ctx* c;
+    ~Borrowed() {
+      if (!c->tile) return;
+      c->g_ph = c->s_ph = c->gpart = nullptr;
+      c->gcount = nullptr;
+      c->ph_valid = false;
+    }
+  } borrowed{c};
   const size_t pb = c->psi_elems() * 2 * sizeof(R);
   const size_t N3 = c->N3;
   const int K1 = std::max(c->K_full, c->K_half), Kh = c->K_half;
@@ -1439,6 +1463,8 @@ tddft_status do_backward(tddft_ctx* c, int nsteps, int ckpt, const double* dL_dr
   if ((s = tmp_alloc(c, db, &w.cS, cb, "cS")) || (s = tmp_alloc(c, db, &w.dcS, cb, "dcS")) ||
       (s = tmp_alloc(c, db, &w.apart, (size_t)c->nkb * std::max(c->natoms, 1) * proj_chunks(c->natoms, c->nkb, c->n_entries, 8) * 3 * 8, "agrad parts")) ||
       (s = tmp_alloc(c, db, &w.cT, cb, "cT")) || (s = tmp_alloc(c, db, &w.dcT, cb, "dcT")))
+    return s;
+  if (c->tile && (s = proj_workspace(c, [&](void** p, size_t b, const char* what) { return tmp_alloc(c, db, p, b, what); })))
     return s;
   const int nck = (nsteps + ckpt - 1) / ckpt;
   std::vector<void*> ck(std::max(nck, 1), nullptr), seg(ckpt, nullptr);
@@ -1920,7 +1946,7 @@ tddft_status create_impl(tddft_ctx* c, const tddft_cell* cell, const tddft_grid*
       (s = c->alloc(&c->rho3, 4 * N3 * 8, "rho3")) || (s = c->alloc(&c->V, 4 * N3 * 8, "V")) ||
       (s = c->alloc(&c->Vnew, 4 * N3 * 8, "Vnew")) || (s = c->alloc(&c->vloc, N3 * 8, "vloc")) ||
       (s = c->alloc(&c->vH, N3 * 8, "vH")) || (s = c->alloc(&c->exc, N3 * 8, "exc")) ||
-      (s = c->alloc(&c->vxc4, 4 * N3 * 8, "vxc4")) || (s = c->alloc(&c->hart, N3 * 16, "hartree")) ||
+      (s = c->alloc(&c->vxc4, 4 * N3 * 8, "vxc4")) || (s = c->alloc(&c->hart, N3 * 8, "hartree")) ||
       (s = c->alloc(&c->red, (16 + 5 * (size_t)c->nkb) * 8, "reductions")) || (s = c->alloc(&c->flag, 16, "flag")))
     return s;
   if (c->prec != TDDFT_FP64) {
@@ -1958,7 +1984,7 @@ tddft_status create_impl(tddft_ctx* c, const tddft_cell* cell, const tddft_grid*
   if ((s = upload(c, &pos_d, c->pos.empty() ? std::vector<double>(3, 0.0) : c->pos, "pos")) || (s = upload(c, &zr_d, Zr, "Zr")))
     return s;
   if ((s = c->alloc(&c->tq, (3 * (size_t)c->nkb + 8) * sizeof(double), "torque sums"))) return s;
-  if ((s = c->alloc(&c->red_part, std::max({band_dot_part_doubles(c->nkb), field_sums_part_doubles(), (size_t)2 * c->nkb * fft_z_energy_parts<double>(c->N)}) * sizeof(double),
+  if ((s = c->alloc(&c->red_part, std::max({band_dot_part_doubles(c->nkb), field_sums_part_doubles(), (size_t)2 * c->nkb * (c->prec == TDDFT_FP64 ? fft_z_energy_parts<double>(c->N) : fft_z_energy_parts<float>(c->N))}) * sizeof(double),
                     "reduction partials")))
     return s;
   if (c->natoms > 0) {
@@ -1970,10 +1996,11 @@ tddft_status create_impl(tddft_ctx* c, const tddft_cell* cell, const tddft_grid*
          })))
       return s;
   }
-  if ((s = c->launch(KC_OTHER, "vloc G", [&] { return launch_vloc_G(c->st, c->N, c->L, c->natoms, pos_d, zr_d, c->omega, c->hart); }))) return s;
-  if ((s = c->launch(KC_OTHER, "vloc ifft z", [&] { return launch_fft_z_inverse(c->st, c->N, c->hart, 1, c->tw64); }))) return s;
-  if ((s = c->launch(KC_OTHER, "vloc ifft xy", [&] { return launch_fft_xy<double>(c->st, c->N, c->hart, c->hart, 1, c->tw64, true); }))) return s;
-  if ((s = c->launch(KC_OTHER, "vloc real", [&] { return launch_complex_real_part(c->st, N3, c->hart, c->vloc, 1.0); }))) return s;
+  double2* field = static_cast<double2*>(c->tmp);  // a spinor's worth of FP32 is N^3 of these
+  if ((s = c->launch(KC_OTHER, "vloc G", [&] { return launch_vloc_G(c->st, c->N, c->L, c->natoms, pos_d, zr_d, c->omega, field); }))) return s;
+  if ((s = c->launch(KC_OTHER, "vloc ifft z", [&] { return launch_fft_z_inverse(c->st, c->N, field, 1, c->tw64); }))) return s;
+  if ((s = c->launch(KC_OTHER, "vloc ifft xy", [&] { return launch_fft_xy<double>(c->st, c->N, field, field, 1, c->tw64, true); }))) return s;
+  if ((s = c->launch(KC_OTHER, "vloc real", [&] { return launch_complex_real_part(c->st, N3, field, c->vloc, 1.0); }))) return s;
 
   // ---- projector tables
   HostTables ht;
@@ -2026,11 +2053,7 @@ tddft_status create_impl(tddft_ctx* c, const tddft_cell* cell, const tddft_grid*
         return s;
     }
     const size_t ne = c->n_entries;
-    const size_t part_bytes = proj_gather_part_bytes(c->natoms, c->nlm, c->nk, c->nb, ne, rs);
-    const size_t ncnt = proj_gather_counters(c->natoms, c->nk, c->nb) * sizeof(int);
-    if ((s = c->alloc(&c->g_ph, ne * c->nk * 2 * rs, "phases")) || (s = c->alloc(&c->s_ph, ne * c->nk * 2 * rs, "phases")) ||
-        (s = c->alloc(&c->gpart, part_bytes, "gather partials")) || (s = c->alloc(&c->gcount, ncnt, "gather counters")) ||
-        (s = c->cuda(cudaMemset(c->gcount, 0, ncnt), "gather counters init")))
+    if (!c->tile && (s = proj_workspace(c, [&](void** p, size_t b, const char* what) { return c->alloc(p, b, what); })))
       return s;
     if (c->prec == TDDFT_FP64) {
       // points by falling number of entries, each class in grid order (counting sort)

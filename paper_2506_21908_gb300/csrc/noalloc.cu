@@ -3,8 +3,8 @@
 // Some callers cannot call cudaMalloc: frameworks that reserve all device memory up front
 // and forbid further allocations, and latency-critical loops where an allocation's implicit
 // device synchronisation is not acceptable.  This entry point solves the same Poisson problem as
-// the library's own potential pipeline, but its scratch (one complex FP64 field and the
-// FFT twiddles) lives in a file-scope static device array instead of memory owned by a
+// the library's own potential pipeline, but its scratch (the real field's planes packed in pairs as
+// complex FP64, and the FFT twiddles) lives in a file-scope static device array instead of memory owned by a
 // handle.  The array exists on every GPU that loads the library, for the life of the
 // process.
 #include <mutex>
@@ -15,8 +15,8 @@
 namespace {
 
 constexpr int kNoAllocMaxN = 64;
-constexpr size_t kFieldElems = (size_t)kNoAllocMaxN * kNoAllocMaxN * kNoAllocMaxN;
-constexpr size_t kScratchElems = kFieldElems + kNoAllocMaxN;  // field + twiddles
+constexpr size_t kFieldElems = (size_t)kNoAllocMaxN * kNoAllocMaxN * kNoAllocMaxN / 2;  // packed planes
+constexpr size_t kScratchElems = kFieldElems + kNoAllocMaxN;  // + twiddles
 
 // Shared by every call on a device; its contents persist between calls.
 static __device__ __align__(256) double2 g_noalloc_scratch[kScratchElems];
@@ -43,7 +43,7 @@ extern "C" tddft_status tddft_hartree_noalloc(const double* n_dev, double* vH_de
   for (int v : ok) supported = supported || (v == n);
   if (!supported) {
     set_global_error("tddft_hartree_noalloc: n must be one of 8, 12, 16, 24, 32, 48, 64 (static scratch holds "
-                     "at most 64^3 complex values)");
+                     "the planes of at most 64^3 values)");
     return TDDFT_ERR_ARG;
   }
   if (!(L[0] > 0.0) || !(L[1] > 0.0) || !(L[2] > 0.0)) {

@@ -108,3 +108,49 @@ def test_a_vanishing_step_is_the_identity(lib, kind, dt, order):
     assert rel(h.get_potential(), V) <= 1e-14
     assert np.abs(norms - 1.0).max() <= 1e-12
     h.close()
+
+
+def test_tensor_core_handle_holds_no_gather_workspace(lib):
+    """The phases of the CUDA-core gather (16 bytes per entry and k-point) serve a tensor-core handle in
+    backward alone: creation takes no more per k-point than its spinor arrays and partial
+    products, backward gives back what it took, and its gradient tracks FP64 within the 1e-3 of the
+    FP32 path."""
+    import torch
+    from paper_2506_21908_gb300 import _lib
+    free = lambda: torch.cuda.mem_get_info()[0]  # noqa: E731
+    n, natoms, nk = 48, 8, 16
+    took = {}
+    for k in (1, nk):
+        wl = S.small_parity(n=n, natoms=natoms, nstates=1, nk=k, lmax=0)
+        torch.cuda.synchronize()
+        before = free()
+        h = _lib.TDDFT.from_workload(wl, precision=1, proj_mode=_lib.PROJ_F16X3, e_min=-20.0, e_max=300.0)
+        took[k] = before - free()
+        h.close()
+    entries = natoms * 4.0 / 3.0 * np.pi * (wl.r_cut * n / wl.L[0]) ** 3
+    phases = (nk - 1) * 16 * entries
+    arrays = (nk - 1) * 2 * n ** 3 * (7 * 8 + 16)  # seven of spinors and the staging of host states
+    arrays += 11 * 4 * n ** 3 * 8  # the band groups of the density at 16 spinors
+    partials = (nk - 1) * 2 * natoms * 108 * 512  # at most two images of an atom in each of the 108 bricks
+    assert took[nk] - took[1] <= arrays + partials + 0.5 * phases
+    wl = S.small_parity(n=16, natoms=2, nstates=2, nk=2)
+    wl.dt = 0.02
+    psi = S.small_parity_states(wl)
+    seed = np.zeros((4, wl.n ** 3))
+    seed[0], seed[1] = 1.0, -1.0
+    grad = []
+    for precision, mode in ((0, 0), (1, _lib.PROJ_F16X3)):
+        h = _lib.TDDFT.from_workload(wl, precision=precision, proj_mode=mode, e_min=-30.0, e_max=250.0)
+        h.set_fields(wl.times, wl.A, wl.B)
+        for _ in range(2):
+            h.set_states(psi, 0.0)
+            before = free()
+            grad.append(h.backward(2, seed)[1:])
+            assert free() >= before
+        h.step(1)  # the handle steps on as before
+        assert h.observables(fields=False)[2]["status"] == 0
+        h.close()
+    for a, b in ((grad[1], grad[0]), (grad[3], grad[2])):
+        assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+    for a, b in zip(grad[2], grad[0]):
+        assert np.abs(a - b).max() <= 1e-3 * np.abs(b).max()
