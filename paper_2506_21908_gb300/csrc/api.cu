@@ -282,6 +282,7 @@ struct tddft_ctx {
   }
   tddft_status cuda(cudaError_t e, const char* what) {
     if (e == cudaSuccess) return TDDFT_OK;
+    cudaGetLastError();  // reported here: a later call must not meet it again
     err = std::string(what) + ": " + cudaGetErrorString(e);
     return e == cudaErrorMemoryAllocation ? TDDFT_ERR_OOM : TDDFT_ERR_CUDA;
   }
@@ -289,6 +290,7 @@ struct tddft_ctx {
     void* q = nullptr;
     cudaError_t e = cudaMalloc(&q, bytes ? bytes : 16);
     if (e != cudaSuccess) {
+      cudaGetLastError();
       err = std::string("cudaMalloc ") + what + ": " + cudaGetErrorString(e);
       return TDDFT_ERR_OOM;
     }
@@ -1152,6 +1154,7 @@ template <typename T> tddft_status tmp_alloc(tddft_ctx* c, DevBuf& db, T** out, 
   void* q = nullptr;
   cudaError_t e = cudaMalloc(&q, bytes ? bytes : 16);
   if (e != cudaSuccess) {
+    cudaGetLastError();
     c->err = std::string("cudaMalloc ") + what + ": " + cudaGetErrorString(e);
     return TDDFT_ERR_OOM;
   }

@@ -80,6 +80,7 @@ extern "C" tddft_status tddft_hartree_noalloc(const double* n_dev, double* vH_de
   if ((e = launch_poisson(st, n, n_dev, nullptr, vH_dev, field, nullptr, tw, L)) != cudaSuccess) goto fail;
   return TDDFT_OK;
 fail:
+  cudaGetLastError();
   set_global_error(std::string("tddft_hartree_noalloc: launch failed: ") + cudaGetErrorString(e));
   return TDDFT_ERR_CUDA;
 }

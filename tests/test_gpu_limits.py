@@ -154,3 +154,21 @@ def test_tensor_core_handle_holds_no_gather_workspace(lib):
         assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
     for a, b in zip(grad[2], grad[0]):
         assert np.abs(a - b).max() <= 1e-3 * np.abs(b).max()
+
+
+def test_a_refused_allocation_is_not_met_again(lib):
+    """A handle beyond the device's memory is refused with TDDFT_ERR_OOM; the next one is created and steps
+    as if nothing had been asked (the runtime keeps an error until it is read)."""
+    from paper_2506_21908_gb300 import _lib
+    big = S.small_parity(n=96, natoms=0, nstates=32767, nk=1)  # one spinor array: 927 GB
+    wl = S.small_parity(n=16, natoms=2, nstates=2, nk=1)
+    psi = S.small_parity_states(wl)
+    for _ in range(2):
+        with pytest.raises(_lib.TddftError) as e:
+            _lib.TDDFT.from_workload(big, precision=0)
+        assert e.value.status == -3
+        h = _lib.TDDFT.from_workload(wl, precision=0, e_min=-30.0, e_max=250.0)
+        h.set_states(psi, 0.0)
+        h.step(1)
+        assert h.observables(fields=False)[2]["status"] == 0
+        h.close()
