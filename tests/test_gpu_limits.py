@@ -172,3 +172,23 @@ def test_a_refused_allocation_is_not_met_again(lib):
         h.step(1)
         assert h.observables(fields=False)[2]["status"] == 0
         h.close()
+
+
+# The gather's CTAs per atom (proj_chunks): one with two spinors per thread (about 190 entries per atom, no
+# partial sums), and the FP32 rule for more than 608 groups of an atom and a spinor pair (16 x 40 with
+# 12000 entries each: four).
+@pytest.mark.parametrize("precision,tol", [(0, 1e-12), (1, 2e-5)])
+@pytest.mark.parametrize("n,natoms,nstates", [(8, 1, 2), (8, 3, 4), (32, 16, 80)])
+def test_gather_splits(lib, precision, tol, n, natoms, nstates):
+    from paper_2506_21908_gb300 import _lib
+    wl = S.small_parity(n=n, natoms=natoms, nstates=nstates, nk=1, lmax=1)
+    psi = S.small_parity_states(wl)
+    s = System.from_workload(wl)
+    A, B = FieldTable(wl.times, wl.A, wl.B).at(wl.dt)
+    V, _ = s.potential(s.rho_v(psi), B)
+    ref = s.apply_h(psi, V, A)
+    h = _lib.TDDFT.from_workload(wl, precision=precision, e_min=-200.0, e_max=600.0)
+    h.set_fields(wl.times, wl.A, wl.B)
+    h.set_states(psi, wl.dt)
+    assert rel(h.apply_hamiltonian(psi), ref) <= tol
+    h.close()
