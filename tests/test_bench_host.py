@@ -49,6 +49,21 @@ def test_roofline_picks_the_dominant_class(tmp_path, monkeypatch):
     assert r["share"] == pytest.approx(0.75)
 
 
+def test_roofline_does_not_rank_times_shared_with_other_launches(tmp_path, monkeypatch):
+    """The gather's event times include the passes it runs beside; on one stream they are its own."""
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    prof = {"fft_xy": {"ms": 10.0, "launches": 4, "bytes": 4e9},
+            "proj_gather": {"ms": 50.0, "launches": 3, "bytes": 1e10},
+            "epilogue": {"ms": 30.0, "launches": 3, "bytes": 6e10}}
+    monkeypatch.delenv("TDDFT_NO_OVERLAP", raising=False)
+    r = bench.roofline_of(prof, 1000, "w")
+    assert r["kernel"] == "epilogue" and r["share"] == pytest.approx(0.75)
+    assert r["not_ranked"].startswith("proj_gather")
+    monkeypatch.setenv("TDDFT_NO_OVERLAP", "1")
+    r = bench.roofline_of(prof, 1000, "w")
+    assert r["kernel"] == "proj_gather" and r["not_ranked"] is None
+
+
 def test_committed_traffic_summaries_match_the_kernel_sources():
     """The committed summaries belong to the kernels in the tree (bench.py would drop them
     otherwise), and carry the keys bench.py reads."""
