@@ -6,15 +6,14 @@
 
 namespace tddft {
 
-// 96 = 8 x 12: 384 threads give every two-factor item loop (768 and 1152 items) and every
-// radix-stage butterfly loop (1152, 2304, 3072 butterflies) whole iterations.
+// Radix-stage passes (n = 8 and 12, and the FP64 inverse z transform of the local potential at every n):
+// at 96, 384 threads give every butterfly loop (1152, 2304, 3072 butterflies) whole iterations.
 template <int N> struct FFTThreads { static constexpr int value = (N >= 96) ? 384 : 256; };
 
-// Minimum resident CTAs per SM requested from the register allocator: several CTAs of the
-// FP32 passes up to 64^3 fit without spills, two of the FP32 96^3 passes (80 KB of shared
-// memory each); FP64 variants keep their registers.
-template <typename R, int N> struct FFTMinBlocks { static constexpr int value = 1; };
-template <int N> struct FFTMinBlocks<float, N> { static constexpr int value = (N <= 64) ? 1024 / FFTThreads<N>::value : 2; };
+// Minimum resident CTAs per SM requested of the register allocator for them: four in FP32, which fit
+// without spills; FP64 variants keep their registers.
+template <typename R> struct FFTMinBlocks { static constexpr int value = 1; };
+template <> struct FFTMinBlocks<float> { static constexpr int value = 4; };
 
 // Programmatic dependent launch: the kernel may be set up before its predecessor on the stream has
 // ended, and calls pdl_wait() (which returns when it has, its writes visible) before it touches

@@ -23,7 +23,7 @@ namespace tddft {
 // ============================================================================ FFT passes
 
 template <typename R, int N, bool INV>
-__global__ void __launch_bounds__(FFTThreads<N>::value, FFTMinBlocks<R, N>::value)
+__global__ void __launch_bounds__(FFTThreads<N>::value, FFTMinBlocks<R>::value)
 k_fft_xy(const typename CT<R>::type* src, typename CT<R>::type* dst, const typename CT<R>::type* __restrict__ twg) {
   using C = typename CT<R>::type;
   constexpr int NT = FFTThreads<N>::value;
@@ -58,7 +58,7 @@ __device__ __forceinline__ void z_tables(R* tx, R* tz, R* ty, const ZParams& zp,
 }
 
 template <typename R, int N, int MODE>
-__global__ void __launch_bounds__(FFTThreads<N>::value, FFTMinBlocks<R, N>::value)
+__global__ void __launch_bounds__(FFTThreads<N>::value, FFTMinBlocks<R>::value)
 k_fft_z(typename CT<R>::type* __restrict__ data, const typename CT<R>::type* __restrict__ twg, ZParams zp) {
   using C = typename CT<R>::type;
   constexpr int NT = FFTThreads<N>::value;
