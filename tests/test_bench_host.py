@@ -49,19 +49,38 @@ def test_roofline_picks_the_dominant_class(tmp_path, monkeypatch):
     assert r["share"] == pytest.approx(0.75)
 
 
-def test_roofline_does_not_rank_times_shared_with_other_launches(tmp_path, monkeypatch):
-    """The gather's event times include the passes it runs beside; on one stream they are its own."""
-    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
-    prof = {"fft_xy": {"ms": 10.0, "launches": 4, "bytes": 4e9},
-            "proj_gather": {"ms": 50.0, "launches": 3, "bytes": 1e10},
-            "epilogue": {"ms": 30.0, "launches": 3, "bytes": 6e10}}
-    monkeypatch.delenv("TDDFT_NO_OVERLAP", raising=False)
-    r = bench.roofline_of(prof, 1000, "w")
-    assert r["kernel"] == "epilogue" and r["share"] == pytest.approx(0.75)
-    assert r["not_ranked"].startswith("proj_gather")
-    monkeypatch.setenv("TDDFT_NO_OVERLAP", "1")
-    r = bench.roofline_of(prof, 1000, "w")
-    assert r["kernel"] == "proj_gather" and r["not_ranked"] is None
+def test_roofline_times_come_from_one_stream(monkeypatch):
+    """The profile behind the roofline is that of a handle created without overlap, and the switch is
+    back to what it was afterwards; profiling runs (--no-peaks) use the timed steps' own profile."""
+    import types
+    seen = []
+
+    class Handle:
+        @classmethod
+        def from_workload(cls, wl, **kw):
+            seen.append(os.environ.get("TDDFT_NO_OVERLAP"))
+            return cls()
+
+        def __getattr__(self, name):
+            return lambda *a: None
+
+    timed = {"proj_gather": {"ms": 50.0, "launches": 3, "bytes": 1e10}, "epilogue": {"ms": 30.0, "launches": 3, "bytes": 6e10}}
+    alone = {"proj_gather": {"ms": 10.0, "launches": 3, "bytes": 1e10}, "epilogue": {"ms": 30.0, "launches": 3, "bytes": 6e10}}
+    monkeypatch.setattr(bench, "timed_steps", lambda ctx, h, steps: (1.0, alone, 1))
+    lib = types.SimpleNamespace(TDDFT=Handle, FP32_MIXED=1)
+    wl = types.SimpleNamespace(times=None, A=None, B=None)
+    ctx = types.SimpleNamespace(stream=0)
+    for before in (None, "0"):
+        if before is None:
+            monkeypatch.delenv("TDDFT_NO_OVERLAP", raising=False)
+        else:
+            monkeypatch.setenv("TDDFT_NO_OVERLAP", before)
+        args = types.SimpleNamespace(no_peaks=False, proj=5)
+        r = bench.roofline_block(args, ctx, lib, wl, None, timed, 1000, "w")
+        assert r["kernel"] == "epilogue" and "one stream" in r["times"] and seen[-1] == "1"
+        assert os.environ.get("TDDFT_NO_OVERLAP") == before
+    args.no_peaks = True
+    assert bench.roofline_block(args, ctx, lib, wl, None, timed, 1000, "w")["kernel"] == "proj_gather" and len(seen) == 2
 
 
 def test_committed_traffic_summaries_match_the_kernel_sources():
